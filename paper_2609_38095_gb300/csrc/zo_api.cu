@@ -910,6 +910,34 @@ int zo_perturb_quadratic_loss(float* theta, const float* a, int64_t n, uint64_t 
   return e == cudaSuccess ? ZO_OK : cuda_fail(e, "perturb_quad_loss");
 }
 
+int64_t zo_quadratic_points_workspace_size(int32_t K) {
+  const int64_t points = 2 * static_cast<int64_t>(K < 1 ? 1 : K) + 1;
+  return points * zo::kQuadPointsMaxCtas * static_cast<int64_t>(sizeof(double)) + 8;  // the partials, then the ticket
+}
+
+int zo_quadratic_points(float* theta, const float* a, int64_t n, uint64_t seed, int32_t packing, int32_t K, double eps,
+                        double* losses, void* workspace, int64_t workspace_bytes, void* stream) {
+  if (n < 0 || losses == nullptr || (n > 0 && (theta == nullptr || a == nullptr)) || K < 1) return ZO_ERR_ARG;
+  if (K > ZO_MAX_PROBES) return ZO_ERR_TOO_MANY_PROBES;
+  if (packing != 0 && packing != zo::kPacking1 && packing != zo::kPacking8) return ZO_ERR_ARG;
+  const float scale = static_cast<float>(eps), mscale = static_cast<float>(-2.0 * eps);
+  if (!std::isfinite(scale) || !std::isfinite(mscale)) return ZO_ERR_ARG;
+  if (reinterpret_cast<uintptr_t>(theta) % sizeof(float) != 0 || reinterpret_cast<uintptr_t>(a) % sizeof(float) != 0)
+    return ZO_ERR_ALIGN;
+  if (workspace == nullptr || workspace_bytes < zo_quadratic_points_workspace_size(K)) return ZO_ERR_WORKSPACE;
+  if (reinterpret_cast<uintptr_t>(workspace) % sizeof(double) != 0) return ZO_ERR_ALIGN;
+  DeviceInfo* d = nullptr;
+  int rc = device_info(&d);
+  if (rc != ZO_OK) return rc;
+  double* partial = static_cast<double*>(workspace);
+  uint32_t* ticket =
+      reinterpret_cast<uint32_t*>(partial + (2 * static_cast<int64_t>(K) + 1) * zo::kQuadPointsMaxCtas);
+  cudaError_t e = zo::launch_quad_points(theta, a, n, expand_keys(seed), packing != 0 ? packing : g_packing.load(), K,
+                                         scale, mscale, losses, partial, ticket, d->sms,
+                                         static_cast<cudaStream_t>(stream));
+  return e == cudaSuccess ? ZO_OK : cuda_fail(e, "quad_points");
+}
+
 int zo_quadratic_loss_static(const float* theta, const float* a, int64_t n, double* out, void* stream) {
   if (n < 0 || out == nullptr || (n > 0 && (theta == nullptr || a == nullptr))) return ZO_ERR_ARG;
   if (n > ZO_QUADRATIC_LOSS_STATIC_MAX_N) return ZO_ERR_WORKSPACE;

@@ -15,6 +15,8 @@ constexpr int kThreads = 256;         // threads per block of the streaming kern
 constexpr int kMaxLossPartials = 2048;
 constexpr int kStaticLossPartials = 4096;   // fixed scratch of the allocation-free loss (32 KB)
 constexpr int kMaxQuadPassPartials = 4096;  // CTAs of the one-pass perturbation + loss
+constexpr int kQuadPointsMaxCtas = 256;     // CTAs of the launch that takes a step through all its forward points
+constexpr size_t kQuadPointsMaxSmem = 200 * 1024;  // and its shared memory per CTA
 constexpr int64_t kStaticLossSlice = 2048;  // elements per partial in that variant
 
 // f32v: the launch holds 32-byte aligned fp32 tensors (single-op kernel only).
@@ -55,5 +57,11 @@ cudaError_t launch_perturb_quad_loss(float* theta, const float* a, int64_t n, co
                                      const PerturbOp* ops, int nops, double* out, int out_copies, int64_t out_stride,
                                      double* partial, uint32_t* ticket, int max_partials, int num_sms,
                                      cudaStream_t stream);
+
+// Every forward point of a step: eps, meps the scales +eps and -2 eps; partial:
+// (2 K + 1) * kQuadPointsMaxCtas doubles; ticket: as above.
+cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const RoundKeys& keys, int packing, int K,
+                               float eps, float meps, double* losses, double* partial, uint32_t* ticket, int num_sms,
+                               cudaStream_t stream);
 
 }  // namespace zo

@@ -31,7 +31,8 @@ EXPORTS = ["zo_status_string", "zo_last_cuda_error", "zo_version", "zo_set_packi
            "zo_perturb", "zo_perturb2", "zo_perturb_pair", "zo_precondition",
            "zo_precondition_ex", "zo_update", "zo_update_ex", "zo_update_sequential", "zo_probe_bytes", "zo_probe_signs",
            "zo_quadratic_loss_workspace_size", "zo_quadratic_loss", "zo_quadratic_loss_static",
-           "zo_perturb_quadratic_loss_workspace_size", "zo_perturb_quadratic_loss"]
+           "zo_perturb_quadratic_loss_workspace_size", "zo_perturb_quadratic_loss",
+           "zo_quadratic_points_workspace_size", "zo_quadratic_points"]
 ZO_QUADRATIC_LOSS_STATIC_MAX_N = 8388608
 
 
@@ -83,6 +84,8 @@ def _lib():
             "zo_perturb_quadratic_loss_workspace_size": ([i64], i64),
             "zo_perturb_quadratic_loss": ([vp, vp, i64, u64, i32, i32, u32, f32, u32, f32, vp, i32, i64, vp, i64, vp],
                                           c.c_int),
+            "zo_quadratic_points_workspace_size": ([i32], i64),
+            "zo_quadratic_points": ([vp, vp, i64, u64, i32, i32, f64, vp, vp, i64, vp], c.c_int),
         }
         for name, (args, res) in sig.items():
             f = getattr(L, name)
@@ -471,6 +474,42 @@ class QuadraticPass:
                                                   ctypes.c_void_p(out_address), copies, stride, *self._ws,
                                                   _stream(self.device))
         _check("zo_perturb_quadratic_loss", rc)
+
+
+def quadratic_points_workspace_size(K: int) -> int:
+    return _lib().zo_quadratic_points_workspace_size(K)
+
+
+class QuadraticPoints:
+    """zo_quadratic_points with theta, a, the loss table and the workspace
+    checked once: a call takes theta through every forward point of a step
+    (+eps, -2 eps, +eps per probe) and writes the K x 3 loss table, in one
+    launch. The workspace is allocated zero-filled here, as the call requires.
+    packing: None follows the process default."""
+
+    def __init__(self, theta, a, losses, packing=None):
+        n = theta.numel()
+        if a.numel() != n:
+            raise ValueError("theta and a differ in size")
+        if packing not in (None, 1, 8):
+            raise ValueError("packing must be None, 1 or 8")
+        if losses.dim() != 2 or losses.shape[1] != 3:
+            raise ValueError("losses must have shape (K, 3)")
+        self.device = theta.device
+        K = losses.shape[0]
+        workspace = torch.zeros(quadratic_points_workspace_size(K), dtype=torch.uint8, device=self.device)
+        _same_device(self.device, a=a, losses=losses)
+        self._keep = (theta, a, losses, workspace)
+        self._args = (_dev_ptr(theta, torch.float32, "theta"), _dev_ptr(a, torch.float32, "a"), n)
+        self._out = (_dev_ptr(losses, torch.float64, "losses"), _dev_ptr(workspace), workspace.numel())
+        self.K = K
+        self.packing = packing or 0
+
+    def __call__(self, seed: int, eps: float):
+        with _on(self.device):
+            rc = _lib().zo_quadratic_points(*self._args, seed, self.packing, self.K, eps, *self._out,
+                                            _stream(self.device))
+        _check("zo_quadratic_points", rc)
 
 
 def perturb_quadratic_loss(theta, a, seed: int, ops, out=None, workspace=None, packing=None):

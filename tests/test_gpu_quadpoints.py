@@ -1,0 +1,121 @@
+"""zo_quadratic_points: every forward point of a step of the small workload in
+one launch, against the oracle's perturbations (bit for bit) and its fp64
+losses. Each loss is a sum of n exact or 2^-47-accurate terms, added as fp32
+pairs (relative error at most 2^-45 per addition of at most 8 + 40 in a
+thread, warp and CTA, and one per round), so 1e-12 of the sum of |terms| holds
+with room at these sizes."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_38095_gb300 import build as zo_build
+from paper_2609_38095_gb300 import workloads as W
+from paper_2609_38095_gb300 import zo
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    zo_build.build()
+    oracle.lib()
+
+
+def oracle_points(theta, a, seed, K, eps):
+    host, rows = [theta.copy()], []
+    l0 = oracle.quadratic_loss(host[0], a)
+    for k in range(K):
+        row = []
+        for scale in (eps, -2 * eps):
+            oracle.perturb(host, [W.DT_F32], seed, k, scale)
+            row.append(oracle.quadratic_loss(host[0], a))
+        oracle.perturb(host, [W.DT_F32], seed, k, eps)
+        rows.append(row + [l0])
+    return host[0], np.array(rows)
+
+
+def on_device(x, offset):
+    v = torch.zeros(x.size + offset, dtype=torch.float32, device="cuda")[offset:]
+    v.copy_(torch.from_numpy(x))
+    return v
+
+
+def run_points(th, a, seed, K, eps, offset=0, packing=None):
+    theta, ad = on_device(th, offset), on_device(a, offset)
+    table = torch.full((K, 3), -7.0, dtype=torch.float64, device="cuda")
+    q = zo.QuadraticPoints(theta, ad, table, packing=packing)
+    q(seed, eps)
+    first = (theta.cpu().numpy(), table.cpu().numpy())
+    theta.copy_(torch.from_numpy(th))   # the workspace is left ready: the same again, bit for bit
+    q(seed, eps)
+    assert np.array_equal(theta.cpu().numpy().view(np.uint32), first[0].view(np.uint32))
+    assert np.array_equal(table.cpu().numpy(), first[1], equal_nan=True)
+    return first
+
+
+def check(th, a, K, eps=1e-3, offset=0, packing=1):
+    seed = W.step_seed(th.size + K)
+    got_th, got = run_points(th, a, seed, K, eps, offset, packing)
+    with oracle.packing(packing):
+        want_th, want = oracle_points(th, a, seed, K, eps)
+    assert np.array_equal(got_th.view(np.uint32), want_th.view(np.uint32))
+    np.testing.assert_allclose(got, want, rtol=1e-12)
+
+
+@pytest.mark.parametrize("n,K", [(1, 1), (7, 3), (8, 4), (9, 5), (255, 8), (256, 9), (4097, 7), (100_003, 16),
+                                 (1 << 20, 8), (1_100_011, 2), (3_000_001, 3), (5000, 40), (3000, 130)])
+def test_points_parity(n, K):
+    rng = np.random.default_rng(n * 31 + K)
+    check(W.random_storage(rng, n, W.DT_F32), (10.0 ** rng.uniform(-2, 2, n)).astype(np.float32), K)
+
+
+@pytest.mark.parametrize("offset,packing", [(1, 1), (2, 8), (4, 8), (3, 1)])
+def test_points_views_and_packings(offset, packing):
+    rng = np.random.default_rng(offset)
+    n = 20_003
+    check(W.random_storage(rng, n, W.DT_F32), (10.0 ** rng.uniform(-2, 2, n)).astype(np.float32), 11, offset=offset,
+          packing=packing)
+
+
+def test_points_most_probes():
+    rng = np.random.default_rng(9)
+    check(W.random_storage(rng, 500, W.DT_F32), (10.0 ** rng.uniform(-2, 2, 500)).astype(np.float32),
+          zo.ZO_MAX_PROBES)
+
+
+def test_points_empty():
+    _, table = run_points(np.zeros(0, np.float32), np.zeros(0, np.float32), 1, 2, 1e-3)
+    assert np.all(table == 0.0)
+
+
+def test_points_weights_outside_the_exact_range():
+    """Zeros, tiny and huge weights and curvatures go to the fp64 terms; only
+    the values of their own size decide the sums they dominate."""
+    rng = np.random.default_rng(4)
+    n = 6000
+    a = (10.0 ** rng.uniform(-2, 2, n)).astype(np.float32)
+    for scale in (1e-25, 1e-12, 1e15, 1e18):
+        check((rng.standard_normal(n) * scale).astype(np.float32), a, 3, eps=scale / 16)
+    th = W.random_storage(rng, n, W.DT_F32)
+    th[::3] = 0.0
+    b = a.copy()
+    b[::5] = 0.0
+    b[1::7] *= np.float32(1e-20)
+    check(th, b, 5)
+    th[17], th[4000] = np.float32(3e38), np.float32(-2e30)
+    check(th, a, 2)
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_points_not_finite(value):
+    rng = np.random.default_rng(5)
+    th = W.random_storage(rng, 4099, W.DT_F32)
+    th[1234] = value
+    a = (10.0 ** rng.uniform(-2, 2, 4099)).astype(np.float32)
+    got_th, got = run_points(th, a, W.step_seed(1), 3, 1e-3)
+    want_th, want = oracle_points(th, a, W.step_seed(1), 3, 1e-3)
+    assert np.array_equal(got_th.view(np.uint32), want_th.view(np.uint32))
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
