@@ -85,15 +85,10 @@ constexpr int kTwoOpBlocksPerSm[kTwoOpCandidates] = {3, 4, 4};
 // eligible than one persistent wave (measured +3 % at K = 64 and 256).
 constexpr int kUpdateWaves = 4;
 
-// Packing-1 updates with up to 48 probe groups take the 8-probe-table kernel
-// (update_lut8_kernel); larger K and packing 8 take update_kernel. Measured
-// on the OPT-1.3B-shaped bf16 set against update_kernel: K = 8 1.08 vs 1.17
-// ms, K = 16 1.34 vs 1.60, K = 64 3.83 vs 4.21, K = 256 12.9 vs 14.7 (same
-// bits); on the OPT-30B-shaped fp16 set at K = 256 292 vs 332 ms.
-#ifndef ZO_LUT8_MIN_GROUPS
-#define ZO_LUT8_MIN_GROUPS 1
-#endif
-constexpr int kLut8MinGroups = ZO_LUT8_MIN_GROUPS;
+// Packing-1 updates with at most this many probe groups keep both groups'
+// tables in shared memory for the whole launch (update_lut8_small_kernel);
+// all others walk the groups chunk by chunk (update_lut8_kernel).
+constexpr int kSmallGroups = 2;
 
 // Per-device launch facts, filled once per device.
 struct DeviceInfo {
@@ -102,9 +97,8 @@ struct DeviceInfo {
   int two_op_bps[kTwoOpCandidates] = {};  // two-op perturb blocks per SM, by candidate
   int pair_bps = 0;                       // perturb_pair blocks per SM
   int shift_bps[2][3] = {};               // perturb_shift blocks per SM, by operation count and dtype
-  int update_bps[2][zo::kMaxGroups + 1] = {};  // by packing (1, 8) and probe-group count
-  int update_shift_bps[2][3][zo::kMaxGroups + 1] = {};  // update_shift_kernel: packing, dtype, group count
-  int lut8_bps[zo::kMaxGroups + 1] = {};  // update_lut8_kernel, by group count
+  int update_shift_bps[3][kSmallGroups + 1] = {};  // update_shift_kernel: dtype, group count
+  bool lut8_ready = false;                // the update kernels' shared-memory limits are raised
 };
 constexpr int kMaxDevices = 64;
 DeviceInfo g_dev[kMaxDevices];
@@ -146,12 +140,12 @@ int device_info(DeviceInfo** out) {
   return ZO_OK;
 }
 
-int update_shift_blocks_per_sm(DeviceInfo* d, int groups, int packing, uint8_t dt, int* out) {
+int update_shift_blocks_per_sm(DeviceInfo* d, int groups, uint8_t dt, int* out) {
   std::lock_guard<std::mutex> lock(g_dev_mu);
-  int& slot = d->update_shift_bps[packing == zo::kPacking8 ? 1 : 0][dt][groups];
+  int& slot = d->update_shift_bps[dt][groups];
   if (slot == 0) {
     int bps = 0;
-    cudaError_t e = zo::update_shift_blocks_per_sm(groups, packing, dt, &bps);
+    cudaError_t e = zo::update_shift_blocks_per_sm(groups, dt, &bps);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy(update_shift)");
     slot = bps > 0 ? bps : 1;
   }
@@ -159,31 +153,14 @@ int update_shift_blocks_per_sm(DeviceInfo* d, int groups, int packing, uint8_t d
   return ZO_OK;
 }
 
-// Also raises the kernel's dynamic shared-memory limit (once per device and
-// group count, before the first launch).
-int lut8_blocks_per_sm(DeviceInfo* d, int groups, int* out) {
+// Raises the update kernels' dynamic shared-memory limits, once per device.
+int lut8_ready(DeviceInfo* d) {
   std::lock_guard<std::mutex> lock(g_dev_mu);
-  int& slot = d->lut8_bps[groups];
-  if (slot == 0) {
-    int bps = 0;
-    cudaError_t e = zo::lut8_prepare(groups, &bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy(update_lut8)");
-    slot = bps > 0 ? bps : 1;
+  if (!d->lut8_ready) {
+    cudaError_t e = zo::lut8_prepare();
+    if (e != cudaSuccess) return cuda_fail(e, "shared-memory limit(update_lut8)");
+    d->lut8_ready = true;
   }
-  *out = slot;
-  return ZO_OK;
-}
-
-int update_blocks_per_sm(DeviceInfo* d, int groups, int packing, int* out) {
-  std::lock_guard<std::mutex> lock(g_dev_mu);
-  int& slot = d->update_bps[packing == zo::kPacking8 ? 1 : 0][groups];
-  if (slot == 0) {
-    int bps = 0;
-    cudaError_t e = zo::update_blocks_per_sm(groups, packing, &bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy(update)");
-    slot = bps > 0 ? bps : 1;
-  }
-  *out = slot;
   return ZO_OK;
 }
 
@@ -217,8 +194,10 @@ int validate_params(const zo_tensor* params, int32_t n, int* packing = nullptr) 
 // numbering every tensor starts on a multiple of kLaunchAlign blocks (see
 // TensorTable). Returns the first tensor not taken; *nblocks receives the
 // virtual blocks the launch covers (tab.blk_total its launch blocks).
+// slots: tensors off the 32-byte grid are flagged kShift and take 32 launch
+// blocks per 31 of their aligned chunks (update_lut8_kernel).
 int32_t fill_table(TensorTable& tab, const zo_tensor* params, int32_t t0, int32_t n, int64_t blk_base,
-                   int64_t* nblocks) {
+                   int64_t* nblocks, bool slots = false) {
   tab.n = 0;
   tab.blk_base = blk_base;
   int64_t b = 0;  // launch blocks so far
@@ -228,16 +207,23 @@ int32_t fill_table(TensorTable& tab, const zo_tensor* params, int32_t t0, int32_
     const zo_tensor& p = params[t];
     const int64_t nb = (p.numel + 15) / 16;
     const int64_t start = (b + zo::kLaunchAlign - 1) / zo::kLaunchAlign * zo::kLaunchAlign;
-    if (tab.n > 0 && start + nb >= zo::kMaxLaunchBlocks) break;
+    const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.ptr) % 32);
+    int64_t span = nb;  // launch blocks of the tensor
+    if (slots && off != 0 && nb > 0) {
+      const int64_t chunks = (p.numel + off / elem_size(p.dtype) + 15) / 16;
+      span = (chunks + zo::kShiftLanes - 1) / zo::kShiftLanes * zo::kLaunchAlign;
+    }
+    if (tab.n > 0 && start + span >= zo::kMaxLaunchBlocks) break;
     const int i = tab.n++;
     tab.vdelta[i] = static_cast<uint32_t>(start - v);
-    b = start + nb;
+    b = start + span;
     v += nb;
     tab.blk_end[i] = static_cast<uint32_t>(b);
     tab.ptr[i] = reinterpret_cast<uint64_t>(p.ptr);
     tab.numel[i] = p.numel;
     uint8_t fl = static_cast<uint8_t>(p.dtype);
-    if (reinterpret_cast<uintptr_t>(p.ptr) % 32 == 0) fl |= zo::kVec32;
+    if (off == 0) fl |= zo::kVec32;
+    if (slots && off != 0 && nb > 0) fl |= zo::kShift;
     tab.flags[i] = fl;
   }
   tab.blk_total = static_cast<uint32_t>(b);
@@ -735,42 +721,42 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  const bool lut8 = zo::lut8_supported(up.groups, up.packing) && up.groups >= kLut8MinGroups;
-  int bps = 1;
-  if (lut8) {
-    if ((rc = lut8_blocks_per_sm(d, up.groups, &bps)) != ZO_OK) return rc;
-  } else if ((rc = update_blocks_per_sm(d, up.groups, up.packing, &bps)) != ZO_OK) {
-    return rc;
-  }
+  const bool small = up.packing == zo::kPacking1 && up.groups <= kSmallGroups;
+  if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t blk = 0;
   for (int32_t t0 = 0; t0 < n_tensors;) {
     int64_t nb = 0;
-    t0 = fill_table(up.tab, params, t0, n_tensors, blk, &nb);
-    if (nb > 0) {
-      bool main_work = false;
-      const unsigned shift_types = mark_shift(up.tab, &main_work);
-      if (main_work && lut8) {
-        cudaError_t e = zo::launch_update_lut8(up, d->sms, bps, s);
-        if (e != cudaSuccess) return cuda_fail(e, "update_lut8_kernel");
-      } else if (main_work) {
-        cudaError_t e = zo::launch_update(up, grid_for(up.tab.blk_total, d->sms, bps * kUpdateWaves), s);
-        if (e != cudaSuccess) return cuda_fail(e, "update_kernel");
-      }
-      if (shift_types) tl_update_shift.u = up;
-      for (uint8_t dt = 0; dt < 3; ++dt) {
-        if (!(shift_types & (1u << dt))) continue;
-        const uint32_t groups = shift_groups(up.tab, dt, tl_update_shift.grp_end);
-        tl_update_shift.grp_total = groups;
-        int sbps = 1;
-        if ((rc = update_shift_blocks_per_sm(d, up.groups, up.packing, dt, &sbps)) != ZO_OK) return rc;
-        const int64_t want = (static_cast<int64_t>(groups) * 32 + zo::kThreads - 1) / zo::kThreads;
-        const int64_t cap = static_cast<int64_t>(d->sms) * sbps * kUpdateWaves;
-        cudaError_t e = zo::launch_update_shift(tl_update_shift, dt, static_cast<int>(want < cap ? want : cap), s);
-        if (e != cudaSuccess) return cuda_fail(e, "update_shift_kernel");
-      }
-    }
+    t0 = fill_table(up.tab, params, t0, n_tensors, blk, &nb, !small);
     blk += nb;
+    if (nb == 0) continue;
+    if (!small) {
+      bool any = false;  // a non-empty tensor that is not 16-bit and aligned
+      for (int i = 0; i < up.tab.n && !any; ++i)
+        any = up.tab.numel[i] > 0 &&
+              ((up.tab.flags[i] & zo::kShift) || (up.tab.flags[i] & zo::kDtypeMask) == zo::kF32);
+      cudaError_t e = zo::launch_update_lut8(up, any, d->sms, s);
+      if (e != cudaSuccess) return cuda_fail(e, "update_lut8_kernel");
+      continue;
+    }
+    bool main_work = false;
+    const unsigned shift_types = mark_shift(up.tab, &main_work);
+    if (main_work) {
+      cudaError_t e = zo::launch_update_lut8_small(up, d->sms, s);
+      if (e != cudaSuccess) return cuda_fail(e, "update_lut8_small_kernel");
+    }
+    if (shift_types) tl_update_shift.u = up;
+    for (uint8_t dt = 0; dt < 3; ++dt) {
+      if (!(shift_types & (1u << dt))) continue;
+      const uint32_t groups = shift_groups(up.tab, dt, tl_update_shift.grp_end);
+      tl_update_shift.grp_total = groups;
+      int sbps = 1;
+      if ((rc = update_shift_blocks_per_sm(d, up.groups, dt, &sbps)) != ZO_OK) return rc;
+      const int64_t want = (static_cast<int64_t>(groups) * 32 + zo::kThreads - 1) / zo::kThreads;
+      const int64_t cap = static_cast<int64_t>(d->sms) * sbps * kUpdateWaves;
+      cudaError_t e = zo::launch_update_shift(tl_update_shift, dt, static_cast<int>(want < cap ? want : cap), s);
+      if (e != cudaSuccess) return cuda_fail(e, "update_shift_kernel");
+    }
   }
   return ZO_OK;
 }

@@ -355,4 +355,42 @@ __device__ __forceinline__ int64_t virtual_block(const TensorTable& tab, int t, 
   return tab.blk_base + static_cast<int64_t>(b) - static_cast<int64_t>(tab.vdelta[t]);
 }
 
+// Helpers of the kernels that work on tensors off the 32-byte grid in aligned
+// chunks straddling two Philox blocks.
+// Bytes b .. b + 15 (b = 0..15) of the 32-byte string lo ++ hi.
+__device__ __forceinline__ uint4 window16(const uint4& lo, const uint4& hi, uint32_t b) {
+  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  uint32_t e[6], d[5];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) e[i] = (b & 8u) ? w[i + 2] : w[i];  // move by two words
+#pragma unroll
+  for (int i = 0; i < 5; ++i) d[i] = (b & 4u) ? e[i + 1] : e[i];  // and by one
+  const uint32_t sh = 8u * (b & 3u);
+  return make_uint4(__funnelshift_r(d[0], d[1], sh), __funnelshift_r(d[1], d[2], sh),
+                    __funnelshift_r(d[2], d[3], sh), __funnelshift_r(d[3], d[4], sh));
+}
+
+__device__ __forceinline__ uint4 shfl_up4(const uint4& x) {
+  return make_uint4(__shfl_up_sync(0xffffffffu, x.x, 1), __shfl_up_sync(0xffffffffu, x.y, 1),
+                    __shfl_up_sync(0xffffffffu, x.z, 1), __shfl_up_sync(0xffffffffu, x.w, 1));
+}
+
+// out[p] = (lo ++ hi)[s + p] for p = 0..15, s = 0..15: four stages of selects.
+__device__ __forceinline__ void window16f(const float (&lo)[16], const float (&hi)[16], uint32_t s,
+                                          float (&out)[16]) {
+  float t8[24], t4[20], t2[18];
+#pragma unroll
+  for (int i = 0; i < 24; ++i) {
+    const float a = i < 16 ? lo[i] : hi[i - 16];
+    const float b = i + 8 < 16 ? lo[i + 8] : hi[i - 8];
+    t8[i] = (s & 8u) ? b : a;
+  }
+#pragma unroll
+  for (int i = 0; i < 20; ++i) t4[i] = (s & 4u) ? t8[i + 4] : t8[i];
+#pragma unroll
+  for (int i = 0; i < 18; ++i) t2[i] = (s & 2u) ? t4[i + 2] : t4[i];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) out[i] = (s & 1u) ? t2[i + 1] : t2[i];
+}
+
 }  // namespace zo

@@ -345,24 +345,6 @@ __global__ void __launch_bounds__(256) perturb_kernel(const __grid_constant__ Pe
 // lane l - 1 by a shuffle: 32 Philox calls per 31 chunks, lane 0 only
 // generates. Chunks that cross the tensor's ends go element by element.
 // ---------------------------------------------------------------------------
-// Bytes b .. b + 15 (b = 0..15) of the 32-byte string lo ++ hi.
-__device__ __forceinline__ uint4 window16(const uint4& lo, const uint4& hi, uint32_t b) {
-  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-  uint32_t e[6], d[5];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) e[i] = (b & 8u) ? w[i + 2] : w[i];  // move by two words
-#pragma unroll
-  for (int i = 0; i < 5; ++i) d[i] = (b & 4u) ? e[i + 1] : e[i];  // and by one
-  const uint32_t sh = 8u * (b & 3u);
-  return make_uint4(__funnelshift_r(d[0], d[1], sh), __funnelshift_r(d[1], d[2], sh),
-                    __funnelshift_r(d[2], d[3], sh), __funnelshift_r(d[3], d[4], sh));
-}
-
-__device__ __forceinline__ uint4 shfl_up4(const uint4& x) {
-  return make_uint4(__shfl_up_sync(0xffffffffu, x.x, 1), __shfl_up_sync(0xffffffffu, x.y, 1),
-                    __shfl_up_sync(0xffffffffu, x.z, 1), __shfl_up_sync(0xffffffffu, x.w, 1));
-}
-
 // A chunk across an end of the tensor, element by element (not inlined: it
 // is rare and would otherwise hold registers in the vector path).
 template <int NOPS, uint8_t DT>
@@ -825,96 +807,6 @@ __device__ __forceinline__ void accumulate_block(float (&acc)[16], int64_t b, co
   }
 }
 
-// Packing 8: the sign of probe k is bit 0 of the element's byte of
-// Philox(b, k). Eight outputs (probes 8f..8f+7) are folded into the same
-// nibble layout as packing 1 -- bit 0 of every byte moved to bit i + 2 of the
-// low (i < 4) or high (i >= 4) offset word -- and looked up in the same tables.
-__device__ __forceinline__ void accumulate_block_p8(float (&acc)[16], int64_t b, const UpdateParams& P,
-                                                    uint32_t lut_base) {
-  const uint32_t blo = static_cast<uint32_t>(b), bhi = static_cast<uint32_t>(static_cast<uint64_t>(b) >> 32);
-  uint32_t frame = lut_base;
-  for (int f = 0; f < P.groups; ++f, frame += kFrameBytes) {
-    uint32_t lo4[4] = {0u, 0u, 0u, 0u}, hi4[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint4 x = philox10(blo, bhi, static_cast<uint32_t>(8 * f + i), 0u, P.keys);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        const uint32_t bits = word_of(x, m) & 0x01010101u;
-        if (i < 4)
-          lo4[m] |= bits << (i + 2);
-        else
-          hi4[m] |= bits << (i - 2);
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t sel = 0x7650u | static_cast<uint32_t>(j);
-        const float tlo = lds_lo(__byte_perm(lo4[m], frame, sel));
-        const float thi = lds_hi(__byte_perm(hi4[m], frame, sel));
-        acc[4 * m + j] = __fadd_rn(acc[4 * m + j], __fadd_rn(tlo, thi));
-      }
-    }
-  }
-}
-
-template <int PACK>
-__device__ __forceinline__ void accumulate_any(float (&acc)[16], int64_t b, const UpdateParams& P,
-                                               uint32_t lut_base) {
-  if constexpr (PACK == kPacking8)
-    accumulate_block_p8(acc, b, P, lut_base);
-  else
-    accumulate_block(acc, b, P, lut_base);
-}
-
-// One full, 32-byte aligned block: theta (16-bit) is loaded before the probe
-// loop so the load overlaps the arithmetic; the leading perturbation, when
-// present, is applied and rounded to storage before the probe sum is added.
-template <int PACK, uint8_t DT>
-__device__ __forceinline__ void update_block_vec(void* base, int64_t e0, int64_t b, const UpdateParams& P,
-                                                 uint32_t lut_base, bool do_sum) {
-  float acc[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) acc[m] = 0.0f;
-  if constexpr (DT == kF32) {
-    if (do_sum) accumulate_any<PACK>(acc, b, P, lut_base);
-    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-    if (P.has_pre) xp = block_bits(b, P.pre.ctr2, P.keys);
-    float* p = static_cast<float*>(base) + e0;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t v[8];
-      ld256(p + 8 * half, v);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        float th = __uint_as_float(v[r]);
-        if (P.has_pre) th = add_signed(th, xp, 8 * half + r, P.pre);
-        if (do_sum) th = __fadd_rn(th, acc[8 * half + r]);
-        v[r] = __float_as_uint(th);
-      }
-      st256(p + 8 * half, v);
-    }
-  } else {
-    uint16_t* p = static_cast<uint16_t*>(base) + e0;
-    uint32_t v[8];
-    ld256(p, v);
-    if (do_sum) accumulate_any<PACK>(acc, b, P, lut_base);
-    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-    if (P.has_pre) xp = block_bits(b, P.pre.ctr2, P.keys);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      if (P.has_pre) v[r] = pre_regs16<DT>(v[r], xp, r, P.pre);
-      if (do_sum) {
-        const float2 f = unpack2<DT>(v[r]);
-        v[r] = pack2<DT>(__fadd_rn(f.x, acc[2 * r]), __fadd_rn(f.y, acc[2 * r + 1]));
-      }
-    }
-    st256(p, v);
-  }
-}
-
 // Per-CTA prologue of the update kernels: a_k = fp32(coef_mul * c_k) for the
 // K probes (zero-padded to 8 * groups) and the per-quad partial-sum tables in
 // their frames. Returns false when the block has nothing to do (a failed
@@ -946,54 +838,6 @@ __device__ __forceinline__ bool update_prologue(const UpdateParams& P, unsigned 
   return true;
 }
 
-template <int PACK>
-__global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ UpdateParams P) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int skip;
-  uint32_t lut_base;
-  bool do_sum;
-  if (!update_prologue(P, smem, skip, lut_base, do_sum)) return;
-
-  const TensorTable& tab = P.tab;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  int t = 0;
-  for (uint32_t bl = blockIdx.x * blockDim.x + threadIdx.x; bl < tab.blk_total; bl += stride) {
-    t = advance_tensor(tab, t, bl);
-    const uint32_t tb = tensor_blk_begin(tab, t);
-    if (bl < tb) continue;  // padding between tensors
-    const int64_t e0 = static_cast<int64_t>(bl - tb) * 16;
-    const int64_t b = virtual_block(tab, t, bl);  // the Philox counter
-    const int64_t cnt = min(static_cast<int64_t>(16), tab.numel[t] - e0);
-    const uint8_t fl = tab.flags[t];
-    const uint8_t dt = fl & kDtypeMask;
-    void* base = reinterpret_cast<void*>(tab.ptr[t]);
-    if (cnt == 16 && (fl & kVec32)) {
-      if (dt == kBF16)
-        update_block_vec<PACK, kBF16>(base, e0, b, P, lut_base, do_sum);
-      else if (dt == kF16)
-        update_block_vec<PACK, kF16>(base, e0, b, P, lut_base, do_sum);
-      else
-        update_block_vec<PACK, kF32>(base, e0, b, P, lut_base, do_sum);
-    } else if (!(fl & kShift)) {  // kShift: an unaligned tensor, update_shift_kernel's
-      float acc[16];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) acc[m] = 0.0f;
-      if (do_sum) accumulate_any<PACK>(acc, b, P, lut_base);
-      uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-      if (P.has_pre) xp = block_bits(b, P.pre.ctr2, P.keys);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        if (i < cnt) {
-          float th = load_elem(base, dt, e0 + i);
-          if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
-          if (do_sum) th = __fadd_rn(th, acc[i]);
-          store_elem(base, dt, e0 + i, th);
-        }
-      }
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Fused update of unaligned tensors (kShift), in the 32-byte aligned chunks of
 // perturb_shift_kernel. Lane l sums the probes of block c = c0 - 1 + l (in
@@ -1002,25 +846,7 @@ __global__ void __launch_bounds__(256) update_kernel(const __grid_constant__ Upd
 // of the two blocks' sums, so every element gets the same fp32 value as in
 // update_kernel.
 // ---------------------------------------------------------------------------
-// out[p] = (lo ++ hi)[s + p] for p = 0..15, s = 0..15: four stages of selects.
-__device__ __forceinline__ void window16f(const float (&lo)[16], const float (&hi)[16], uint32_t s,
-                                          float (&out)[16]) {
-  float t8[24], t4[20], t2[18];
-#pragma unroll
-  for (int i = 0; i < 24; ++i) {
-    const float a = i < 16 ? lo[i] : hi[i - 16];
-    const float b = i + 8 < 16 ? lo[i + 8] : hi[i - 8];
-    t8[i] = (s & 8u) ? b : a;
-  }
-#pragma unroll
-  for (int i = 0; i < 20; ++i) t4[i] = (s & 4u) ? t8[i + 4] : t8[i];
-#pragma unroll
-  for (int i = 0; i < 18; ++i) t2[i] = (s & 2u) ? t4[i + 2] : t4[i];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) out[i] = (s & 1u) ? t2[i + 1] : t2[i];
-}
-
-template <int PACK, uint8_t DT>
+template <uint8_t DT>
 __device__ __forceinline__ void update_shift_group(const UpdateParams& P, uint32_t lut_base, bool do_sum, int t,
                                                    int64_t c_first) {
   constexpr int kElem = DT == kF32 ? 4 : 2;
@@ -1046,7 +872,7 @@ __device__ __forceinline__ void update_shift_group(const UpdateParams& P, uint32
     float own[16], below[16], sum[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) own[m] = 0.0f;
-    if (do_sum) accumulate_any<PACK>(own, vb0 + c, P, lut_base);
+    if (do_sum) accumulate_block(own, vb0 + c, P, lut_base);
 #pragma unroll
     for (int m = 0; m < 16; ++m) below[m] = __shfl_up_sync(0xffffffffu, own[m], 1);
     window16f(below, own, 16u - a, sum);
@@ -1092,7 +918,7 @@ __device__ __forceinline__ void update_shift_group(const UpdateParams& P, uint32
   }
 }
 
-template <int PACK, uint8_t DT>
+template <uint8_t DT>
 __global__ void __launch_bounds__(256) update_shift_kernel(const __grid_constant__ UpdateShiftParams S) {
   const UpdateParams& P = S.u;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1106,7 +932,7 @@ __global__ void __launch_bounds__(256) update_shift_kernel(const __grid_constant
   for (uint32_t g = warp; g < S.grp_total; g += nwarps) {  // the same g on every lane of the warp
     while (g >= S.grp_end[t]) ++t;
     const int64_t c_first = static_cast<int64_t>(g - (t == 0 ? 0u : S.grp_end[t - 1])) * kShiftGroup;
-    update_shift_group<PACK, DT>(P, lut_base, do_sum, t, c_first);
+    update_shift_group<DT>(P, lut_base, do_sum, t, c_first);
   }
 }
 
@@ -1215,38 +1041,24 @@ cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, 
   return cudaGetLastError();
 }
 
-template <int PACK>
-void launch_update_shift_pack(const UpdateShiftParams& p, uint8_t dt, int grid, size_t smem, cudaStream_t stream) {
-  if (dt == kBF16)
-    update_shift_kernel<PACK, kBF16><<<grid, kThreads, smem, stream>>>(p);
-  else if (dt == kF16)
-    update_shift_kernel<PACK, kF16><<<grid, kThreads, smem, stream>>>(p);
-  else
-    update_shift_kernel<PACK, kF32><<<grid, kThreads, smem, stream>>>(p);
-}
-
 cudaError_t launch_update_shift(const UpdateShiftParams& p, uint8_t dt, int grid, cudaStream_t stream) {
   const size_t smem = update_smem_bytes(p.u.groups);
-  if (p.u.packing == kPacking8)
-    launch_update_shift_pack<kPacking8>(p, dt, grid, smem, stream);
+  if (dt == kBF16)
+    update_shift_kernel<kBF16><<<grid, kThreads, smem, stream>>>(p);
+  else if (dt == kF16)
+    update_shift_kernel<kF16><<<grid, kThreads, smem, stream>>>(p);
   else
-    launch_update_shift_pack<kPacking1>(p, dt, grid, smem, stream);
+    update_shift_kernel<kF32><<<grid, kThreads, smem, stream>>>(p);
   return cudaGetLastError();
 }
 
-template <int PACK>
-cudaError_t update_shift_bps_pack(int groups, uint8_t dt, int* out) {
+cudaError_t update_shift_blocks_per_sm(int groups, uint8_t dt, int* out) {
   const size_t smem = update_smem_bytes(groups);
   if (dt == kBF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<PACK, kBF16>, kThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kBF16>, kThreads, smem);
   if (dt == kF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<PACK, kF16>, kThreads, smem);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<PACK, kF32>, kThreads, smem);
-}
-
-cudaError_t update_shift_blocks_per_sm(int groups, int packing, uint8_t dt, int* out) {
-  return packing == kPacking8 ? update_shift_bps_pack<kPacking8>(groups, dt, out)
-                              : update_shift_bps_pack<kPacking1>(groups, dt, out);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kF16>, kThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kF32>, kThreads, smem);
 }
 
 cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream) {
@@ -1256,14 +1068,6 @@ cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stre
 
 // Coefficients (32 bytes per group), alignment slack, one 256-byte frame per group.
 size_t update_smem_bytes(int groups) { return static_cast<size_t>(groups) * (32 + kFrameBytes) + kFrameBytes; }
-
-cudaError_t launch_update(const UpdateParams& p, int grid, cudaStream_t stream) {
-  if (p.packing == kPacking8)
-    update_kernel<kPacking8><<<grid, kThreads, update_smem_bytes(p.groups), stream>>>(p);
-  else
-    update_kernel<kPacking1><<<grid, kThreads, update_smem_bytes(p.groups), stream>>>(p);
-  return cudaGetLastError();
-}
 
 cudaError_t perturb_blocks_per_sm(int nops, int loop, int* out) {
   if (nops == 1)
@@ -1288,14 +1092,6 @@ cudaError_t shift_blocks_per_sm(int nops, uint8_t dt, int* out) {
 
 cudaError_t pair_blocks_per_sm(int* out) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_pair_kernel, kThreads, 0);
-}
-
-cudaError_t update_blocks_per_sm(int groups, int packing, int* out) {
-  if (packing == kPacking8)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_kernel<kPacking8>, kThreads,
-                                                         update_smem_bytes(groups));
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_kernel<kPacking1>, kThreads,
-                                                       update_smem_bytes(groups));
 }
 
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,

@@ -43,15 +43,6 @@
 namespace zo {
 
 constexpr uint32_t kLut8Region = 65536;   // 256 rows x 256 bytes: the tables of two groups
-constexpr int kLut8MaxGroups = 48;        // larger K takes update_kernel
-
-// Shared-memory request: two 64 KB regions starting on a 64 KB boundary of
-// the shared window, plus the coefficients, 4-probe tables and the chunk's
-// virtual blocks (lut8_side_bytes: at most 24 KB), placed in the slack below
-// the first region when they fit there (the window starts a few bytes in),
-// else after the second: 192 KB covers both cases.
-size_t lut8_smem_bytes(int) { return 3 * static_cast<size_t>(kLut8Region) + 16u; }
-
 __device__ __forceinline__ float lds_f32(uint32_t addr) {
   float v;
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
@@ -116,62 +107,68 @@ __device__ __forceinline__ void lut8_lookup(float (&acc)[16], const uint4& x, ui
   }
 }
 
-// A thread's block of the current chunk.
+// A thread's block of the current chunk, or, of a tensor off the 32-byte grid
+// (kShift), its 32-byte aligned chunk of sixteen elements: chunk c holds
+// elements 16c - a .. 16c - a + 15 (a = the base's offset from the boundary
+// below it, in elements), the tail of block c - 1 and the head of block c.
 struct Lut8Block {
-  int64_t b;       // virtual block (Philox counter)
-  int64_t e0;      // first element inside its tensor
+  int64_t b;       // virtual block whose probes the lane sums (Philox counter)
+  int64_t e0;      // first element of the block or chunk inside its tensor (below 0 in a tensor's first chunk)
+  int64_t numel;   // elements of the tensor
   void* base;      // tensor base pointer
-  int cnt;         // elements of the block (1..16)
+  uint32_t a;      // chunks: a; blocks: 0
   uint8_t fl;      // tensor flags
-  bool act;        // a block this kernel updates
-  bool vec16;      // full 32-byte aligned block of a 16-bit tensor (theta already in v)
+  bool act;        // there are elements here for this lane
+  bool vec;        // all sixteen, 32-byte aligned
 };
+
+// theta pair + the leading perturbation's signed scales, one packed add.
+__device__ __forceinline__ void add_signed2(float2& f, const uint4& x, int i, const PerturbOp& op) {
+  // the probe bit moved to bit 31 by a multiply (PerturbOp::mul): the
+  // multiply-add pipe instead of the integer ALU, the busier one here
+  fadd2_rn(f.x, f.y, __uint_as_float(op.nscale_bits ^ ((word_of(x, i >> 2) * op.mul[i & 3]) & 0x80000000u)),
+           __uint_as_float(op.nscale_bits ^ ((word_of(x, (i + 1) >> 2) * op.mul[(i + 1) & 3]) & 0x80000000u)));
+}
 
 template <uint8_t DT>
 __device__ __forceinline__ void lut8_apply16(uint32_t (&v)[8], const float (&acc)[16], const uint4& xp,
-                                             const UpdateParams& P, bool do_sum) {
+                                             const UpdateParams& P) {
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    if (P.has_pre) v[r] = pre_regs16<DT>(v[r], xp, r, P.pre);
-    if (do_sum) {
-      const float2 f = unpack2<DT>(v[r]);
-      v[r] = pack2<DT>(__fadd_rn(f.x, acc[2 * r]), __fadd_rn(f.y, acc[2 * r + 1]));
+    float2 f = unpack2<DT>(v[r]);
+    if (P.has_pre) {
+      add_signed2(f, xp, 2 * r, P.pre);
+      f = unpack2<DT>(pack2<DT>(f.x, f.y));  // the perturbed value is rounded to storage first
     }
+    fadd2_rn(f.x, f.y, acc[2 * r], acc[2 * r + 1]);
+    v[r] = pack2<DT>(f.x, f.y);
   }
 }
 
-// Apply the leading perturbation (if any) and the probe sums to a block that
-// is not a full, aligned 16-bit one: fp32 blocks and partial last blocks.
-__device__ __forceinline__ void lut8_apply_other(const Lut8Block& k, const float (&acc)[16], const UpdateParams& P,
-                                              bool do_sum) {
-  uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-  if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
-  const uint8_t dt = k.fl & kDtypeMask;
-  if (dt == kF32 && k.cnt == 16 && (k.fl & kVec32)) {
-    float* p = static_cast<float*>(k.base) + k.e0;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t v[8];
-      ld256(p + 8 * half, v);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        float th = __uint_as_float(v[r]);
-        if (P.has_pre) th = add_signed(th, xp, 8 * half + r, P.pre);
-        if (do_sum) th = __fadd_rn(th, acc[8 * half + r]);
-        v[r] = __float_as_uint(th);
-      }
-      st256(p + 8 * half, v);
-    }
-    return;
-  }
+// The same for sixteen fp32 weights: scalar adds, as in every fp32 path.
+__device__ __forceinline__ void lut8_apply32(uint32_t (&v)[16], const float (&acc)[16], const uint4& xp,
+                                             const UpdateParams& P) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
-    if (i < k.cnt) {
-      float th = load_elem(k.base, dt, k.e0 + i);
-      if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
-      if (do_sum) th = __fadd_rn(th, acc[i]);
-      store_elem(k.base, dt, k.e0 + i, th);
-    }
+    float th = __uint_as_float(v[i]);
+    if (P.has_pre) th = add_signed(th, xp, i, P.pre);
+    v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
+  }
+}
+
+// The same element by element, for a block or chunk across an end of its
+// tensor; do_sum false: the leading perturbation alone.
+__device__ __forceinline__ void lut8_apply_elements(const Lut8Block& k, const float (&acc)[16], const uint4& xp,
+                                                    const UpdateParams& P, bool do_sum) {
+  const uint8_t dt = k.fl & kDtypeMask;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int64_t e = k.e0 + i;
+    if (e < 0 || e >= k.numel) continue;
+    float th = load_elem(k.base, dt, e);
+    if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
+    if (do_sum) th = __fadd_rn(th, acc[i]);
+    store_elem(k.base, dt, e, th);
   }
 }
 
@@ -261,40 +258,36 @@ __device__ __forceinline__ void lut8_replicate4(uint32_t t4, uint32_t dst_t, int
   }
 }
 
-// A thread's tensor while its blocks stay inside it: the table is read again
-// only when a block leaves it.
-struct Lut8Cursor {
-  int t;
-  uint32_t tb, te;  // first and one-past-last launch block
-  int64_t numel;
-  void* base;
-  int64_t vbase;    // virtual block of launch block bl of this tensor, minus bl
-  uint8_t fl;
-};
-
-__device__ __forceinline__ void lut8_seek(const TensorTable& tab, Lut8Cursor& c, uint32_t bl) {
-  c.t = advance_tensor(tab, c.t, bl);
-  c.tb = tensor_blk_begin(tab, c.t);
-  c.te = tab.blk_end[c.t];
-  c.numel = tab.numel[c.t];
-  c.base = reinterpret_cast<void*>(tab.ptr[c.t]);
-  c.vbase = tab.blk_base - static_cast<int64_t>(tab.vdelta[c.t]);
-  c.fl = tab.flags[c.t];
-}
-
-// Block bl of the launch (bl only grows for a cursor): its tensor and place.
-__device__ __forceinline__ void lut8_block_info(const TensorTable& tab, Lut8Cursor& c, uint32_t bl, Lut8Block& k) {
-  k.act = bl < tab.blk_total;
-  k.vec16 = false;
-  if (!k.act) return;
-  if (bl >= c.te) lut8_seek(tab, c, bl);
-  k.fl = c.fl;
-  k.act = !(c.fl & kShift) && bl >= c.tb;
-  k.b = c.vbase + static_cast<int64_t>(bl);
-  k.e0 = static_cast<int64_t>(bl - c.tb) * 16;
-  k.cnt = static_cast<int>(min(static_cast<int64_t>(16), c.numel - k.e0));
-  k.base = c.base;
-  k.vec16 = k.act && k.cnt == 16 && (c.fl & kVec32) && (c.fl & kDtypeMask) != kF32;
+// Launch block bl, of tensor t: its place. (t of the warp's first block: every
+// tensor starts on a multiple of 32 launch blocks, so the 32 blocks of a warp
+// lie in one tensor or in the padding after it.) ANY: the launch may hold
+// kShift tensors. Of those each warp takes 31 chunks: lane l sums block
+// 31 w + l - 1 of the tensor and works on the chunk of that number, with the
+// sums of the block below from lane l - 1; lane 0 only sums.
+template <bool ANY>
+__device__ __forceinline__ Lut8Block lut8_block_info(const TensorTable& tab, int t, uint32_t bl) {
+  Lut8Block k;
+  const uint32_t tb = tensor_blk_begin(tab, t);
+  const uint32_t d = bl - tb;
+  k.fl = tab.flags[t];
+  k.numel = tab.numel[t];
+  k.base = reinterpret_cast<void*>(tab.ptr[t]);
+  k.a = 0u;
+  if (ANY && (k.fl & kShift)) {
+    const uint32_t lane = d & 31u;
+    k.a = static_cast<uint32_t>(tab.ptr[t] & 31u) / ((k.fl & kDtypeMask) == kF32 ? 4u : 2u);
+    const int64_t c = static_cast<int64_t>(d >> 5) * 31 + lane - 1;
+    k.b = virtual_block(tab, t, tb) + c;
+    k.e0 = 16 * c - k.a;
+    k.act = lane > 0 && k.e0 < k.numel;
+    k.vec = k.act && k.e0 >= 0 && k.e0 + 16 <= k.numel;
+  } else {
+    k.b = virtual_block(tab, t, bl);
+    k.e0 = static_cast<int64_t>(d) * 16;
+    k.act = bl < tab.blk_end[t];
+    k.vec = k.act && k.e0 + 16 <= k.numel && (k.fl & kVec32);
+  }
+  return k;
 }
 
 // Philox4x32-10 with rounds 0 and 1 split by what they depend on, for a
@@ -336,67 +329,207 @@ __device__ __forceinline__ BlockRound01 block_round01(uint32_t blo, const RoundK
   k.lpb1 = static_cast<uint32_t>(pb1);
   return k;
 }
-__device__ __forceinline__ uint4 philox_split(const BlockRound01& k, const GroupRound01& g, const RoundKeys& rk) {
-  uint32_t c0 = k.hpb1 ^ g.x0, c1 = k.lpb1, c2 = g.x2 ^ k.lpa0, c3 = g.lpa1;
+
+// A Philox call after its first two rounds.
+struct PhiloxState {
+  uint32_t c0, c1, c2, c3;
+};
+
+// A block's part of the counter: HIU, its round-0/1 products; otherwise the
+// counter itself.
+template <bool HIU>
+struct BlockCounter;
+template <>
+struct BlockCounter<true> {
+  BlockRound01 k;
+  // vr: the block's low word
+  __device__ __forceinline__ BlockCounter(uint32_t vr, int64_t, const RoundKeys& rk) : k(block_round01(vr, rk)) {}
+  __device__ __forceinline__ PhiloxState start(const GroupRound01& g, uint32_t, const RoundKeys&) const {
+    return {k.hpb1 ^ g.x0, k.lpb1, g.x2 ^ k.lpa0, g.lpa1};
+  }
+};
+template <>
+struct BlockCounter<false> {
+  uint32_t lo, hi;
+  // vr: the block's offset from `base`
+  __device__ __forceinline__ BlockCounter(uint32_t vr, int64_t base, const RoundKeys&) {
+    const uint64_t b = static_cast<uint64_t>(base + vr);
+    lo = static_cast<uint32_t>(b);
+    hi = static_cast<uint32_t>(b >> 32);
+  }
+  __device__ __forceinline__ PhiloxState start(const GroupRound01&, uint32_t q, const RoundKeys& rk) const {
+    PhiloxState s = {lo, hi, q, 0u};
+    philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[0], rk.k1[0]);
+    philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[1], rk.k1[1]);
+    return s;
+  }
+};
+
+__device__ __forceinline__ uint4 philox_finish(PhiloxState s, const RoundKeys& rk) {
 #pragma unroll
-  for (int r = 2; r < 10; ++r) philox_round(c0, c1, c2, c3, rk.k0[r], rk.k1[r]);
-  return make_uint4(c0, c1, c2, c3);
+  for (int r = 2; r < 10; ++r) philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[r], rk.k1[r]);
+  return make_uint4(s.c0, s.c1, s.c2, s.c3);
+}
+
+// The words whose byte m holds the signs of probes 8q .. 8q + 7 of element m
+// under packing 8: bit 0 of every byte of eight Philox calls, call i moved to
+// bit i; r01 holds the calls' group parts (HIU). Calls past probe K - 1 are
+// left out: their coefficients are 0 in the tables. A full group's calls run
+// in pairs, two independent chains of multiplies per thread: with the four
+// warps a scheduler has here, one chain leaves the multiply-add pipe waiting.
+__device__ __forceinline__ void fold_bits(uint4& y, const uint4& x, uint32_t i) {
+  const uint32_t m = 0x01010101u << i;
+  y.x |= (x.x << i) & m;
+  y.y |= (x.y << i) & m;
+  y.z |= (x.z << i) & m;
+  y.w |= (x.w << i) & m;
+}
+
+template <bool HIU>
+__device__ __forceinline__ uint4 group_words8(const BlockCounter<HIU>& kb, uint32_t q, uint32_t K, const uint4* r01,
+                                              const RoundKeys& keys) {
+  const auto start = [&](uint32_t k) {
+    GroupRound01 g = {0u, 0u, 0u};
+    if (HIU) {
+      const uint4 r = r01[k];
+      g = {r.x, r.y, r.z};
+    }
+    return kb.start(g, k, keys);
+  };
+  uint4 y = make_uint4(0u, 0u, 0u, 0u);
+  if (8u * q + 8u <= K) {
+#pragma unroll
+    for (uint32_t i = 0; i < 8u; i += 2u) {
+      PhiloxState s = start(8u * q + i), t = start(8u * q + i + 1u);
+#pragma unroll
+      for (int r = 2; r < 10; ++r) {
+        philox_round(s.c0, s.c1, s.c2, s.c3, keys.k0[r], keys.k1[r]);
+        philox_round(t.c0, t.c1, t.c2, t.c3, keys.k0[r], keys.k1[r]);
+      }
+      fold_bits(y, make_uint4(s.c0, s.c1, s.c2, s.c3), i);
+      fold_bits(y, make_uint4(t.c0, t.c1, t.c2, t.c3), i + 1u);
+    }
+  } else {
+#pragma unroll 1
+    for (uint32_t i = 0; 8u * q + i < K; ++i) fold_bits(y, philox_finish(start(8u * q + i), keys), i);
+  }
+  return y;
 }
 
 // One step of a probe-group pair: one block of this thread (its sums at TMEM
 // address ta) over group q and, when `two`, q + 1, the groups added in order.
 // Every lane takes part (an inactive lane's sums are never applied), so the
-// step has no per-lane branch; the group-q Philox call runs while the sums
-// come in from TMEM.
-template <bool FIRST>
-__device__ __forceinline__ void lut8_tm_step(uint32_t ta, int64_t b, uint32_t q, bool two, uint32_t frame,
+// step has no per-lane branch; the first group's Philox call runs while the
+// sums come from TMEM (FIRST: they start at zero).
+template <bool FIRST, bool HIU>
+__device__ __forceinline__ void lut8_tm_step(uint32_t ta, const BlockCounter<HIU>& kb, uint32_t q,
+                                             const GroupRound01& g0, const GroupRound01& g1, bool two, uint32_t frame,
                                              const RoundKeys& keys) {
   float acc[16];
   if (FIRST)
     zero16(acc);
   else
     tm_ld16(acc, ta);
-  const uint4 x0 = block_bits(b, q, keys);
+  const uint4 x0 = philox_finish(kb.start(g0, q, keys), keys);
   if (!FIRST) tm_wait_ld(acc);
   lut8_lookup(acc, x0, frame);
-  if (two) lut8_lookup(acc, block_bits(b, q + 1u, keys), frame | 128u);
+  if (two) lut8_lookup(acc, philox_finish(kb.start(g1, q + 1u, keys), keys), frame | 128u);
   tm_st16(ta, acc);
 }
 
-// The same step for a launch whose blocks share the counter's high word:
-// blo is the block's low word, g0 / g1 the groups' round-0/1 parts.
-template <bool FIRST>
-__device__ __forceinline__ void lut8_tm_step_split(uint32_t ta, uint32_t blo, const GroupRound01& g0,
-                                                   const GroupRound01& g1, bool two, uint32_t frame,
-                                                   const RoundKeys& keys) {
+// Rounds 2-9 of one Philox call (s: in, its state; out, its words) and, two
+// elements per round, the lookups of a group whose words x are known, added
+// to acc in element order; the additions trail the loads by a round. WAIT:
+// acc may still be on its way from TMEM and is waited for before the first.
+template <bool WAIT>
+__device__ __forceinline__ void philox_with_lookups(PhiloxState& s, float (&acc)[16], const uint4& x, uint32_t frame,
+                                                    const RoundKeys& rk) {
+  float p0 = 0.0f, p1 = 0.0f;
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+    const int e = 2 * (r - 2);
+    const uint32_t w = word_of(x, e >> 2);
+    const uint32_t a0 = __byte_perm(w, frame, 0x7604u | (static_cast<uint32_t>(e & 3) << 4));
+    const uint32_t a1 = __byte_perm(w, frame, 0x7604u | (static_cast<uint32_t>((e + 1) & 3) << 4));
+    const float n0 = lds_f32(a0), n1 = lds_f32(a1);
+    philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[r], rk.k1[r]);
+    if (WAIT && r == 3) tm_wait_ld(acc);
+    if (r > 2) fadd2_rn(acc[e - 2], acc[e - 1], p0, p1);
+    p0 = n0;
+    p1 = n1;
+  }
+  fadd2_rn(acc[14], acc[15], p0, p1);
+}
+
+// One step with the words one group ahead (x: those of group q of this block
+// on entry, of group qn of the next block on return): each Philox call runs
+// among the lookups of the group before it, so a warp mixes the multiplies of
+// the one with the byte-permutes and shared loads of the other instead of
+// waiting for each pipe in turn.
+template <bool FIRST, bool HIU>
+__device__ __forceinline__ void lut8_tm_step_ahead(uint32_t ta, uint4& x, BlockCounter<HIU>& kb, uint32_t q,
+                                                   const GroupRound01& g1, const BlockCounter<HIU>& next, uint32_t qn,
+                                                   const GroupRound01& gn, uint32_t frame, const RoundKeys& keys) {
   float acc[16];
   if (FIRST)
     zero16(acc);
   else
     tm_ld16(acc, ta);
-  const BlockRound01 k = block_round01(blo, keys);
-  const uint4 x0 = philox_split(k, g0, keys);
-  if (!FIRST) tm_wait_ld(acc);
+  PhiloxState s = kb.start(g1, q + 1u, keys);
+  philox_with_lookups<!FIRST>(s, acc, x, frame, keys);
+  x = make_uint4(s.c0, s.c1, s.c2, s.c3);
+  kb = next;
+  s = kb.start(gn, qn, keys);
+  philox_with_lookups<false>(s, acc, x, frame | 128u, keys);
+  x = make_uint4(s.c0, s.c1, s.c2, s.c3);
+  tm_st16(ta, acc);
+}
+
+// One step under packing 8.
+template <bool HIU>
+__device__ __forceinline__ void lut8_tm_step8(uint32_t ta, const BlockCounter<HIU>& kb, uint32_t q, uint32_t K,
+                                              const uint4* r01, bool two, uint32_t frame, const RoundKeys& keys) {
+  const uint4 x0 = group_words8(kb, q, K, r01, keys);
+  float acc[16];
+  if (q == 0u)
+    zero16(acc);
+  else
+    tm_get16(acc, ta);
   lut8_lookup(acc, x0, frame);
-  if (two) lut8_lookup(acc, philox_split(k, g1, keys), frame | 128u);
+  if (two) lut8_lookup(acc, group_words8(kb, q + 1u, K, r01, keys), frame | 128u);
   tm_st16(ta, acc);
 }
 
 // Shared memory besides the two regions: coefficients (8 per group), 4-probe
-// tables (32 per group) and the chunk's virtual blocks (one per thread and
-// block), below the first region when they fit there, else after the second.
-__host__ __device__ constexpr uint32_t lut8_side_bytes(int groups, int bpt) {
-  return 160u * static_cast<uint32_t>(groups) + 4u * kLut8Threads * static_cast<uint32_t>(bpt);
+// tables (32 per group), under packing 8 the probes' Philox group parts (16
+// bytes each), and the tensors of the chunk's blocks (one per warp and block),
+// below the first region when they fit there, else after the second.
+__host__ __device__ constexpr uint32_t lut8_side_bytes(int groups, int bpt, bool pack8) {
+  return (pack8 ? 288u : 160u) * static_cast<uint32_t>(groups) +
+         4u * static_cast<uint32_t>(kLut8Threads / 32 * bpt);
 }
 // Placed after the second region only when the slack below the first is
 // smaller than it, so the layout ends within 2 * side + 128 KB of the window's
-// start: inside the 192 KB request while side <= 32 KB.
-static_assert(lut8_side_bytes(kLut8MaxGroups, 8) <= kLut8Region / 2, "side data must fit the request");
+// start.
+constexpr size_t lut8_smem_bytes(bool pack8) {
+  const size_t after = 2 * static_cast<size_t>(kLut8Region) + 2 * lut8_side_bytes(kMaxGroups, 8, pack8) + 16u;
+  const size_t below = 3 * static_cast<size_t>(kLut8Region) + 16u;
+  return after > below ? after : below;
+}
+static_assert(lut8_smem_bytes(true) <= 226 * 1024, "side data must fit the shared memory of an SM");
 
 // HIU: every virtual block of the launch has the same counter high word (any
 // launch below 2^36 weights), so the steps use the split Philox and a 32-bit
 // block word (OPT-30B-shaped set, K = 256: 245.3 -> 235.9 ms, same bits).
-template <int BPT, bool HIU>
+// ANY: the launch may hold fp32 tensors and tensors off the 32-byte grid. An
+// instantiation of its own: with their code in the same kernel the loop over
+// the pairs is 2-3 % slower (registers), though it is the same source.
+// AHEAD: the steps run with the words one group ahead (lut8_tm_step_ahead):
+// faster from 24 groups on (OPT-30B-shaped layers, K = 256: 10.08 -> 9.95 ms,
+// K = 1024 on the OPT-1.3B-shaped set: 40.1 -> 39.6 ms), slower below (K = 64:
+// 4.23 -> 4.30 ms on Qwen3-8B-shaped layers), where the two groups' own calls
+// overlap enough and the last pair weighs more.
+template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD>
 __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __grid_constant__ UpdateParams P) {
   constexpr int THREADS = kLut8Threads;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -406,11 +539,12 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
   const int NP = (G + 1) / 2;  // group pairs: groups 2p, 2p + 1 share one region
   const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
   const uint32_t region0 = (sbase + kLut8Region - 1u) & ~(kLut8Region - 1u);
-  const uint32_t side = lut8_side_bytes(G, BPT);
+  const uint32_t side = lut8_side_bytes(G, BPT, PACK8);
   const uint32_t hdr = region0 - sbase >= side ? sbase : region0 + 2u * kLut8Region;
   float* a_s = reinterpret_cast<float*>(smem + (hdr - sbase));  // 8 G coefficients
   float* t4 = a_s + 8 * G;                                      // 32 G 4-probe partials
-  uint32_t* vr_s = reinterpret_cast<uint32_t*>(t4 + 32 * G);     // BPT x THREADS virtual blocks
+  uint4* r01_s = reinterpret_cast<uint4*>(t4 + 32 * G);         // packing 8: 8 G group parts
+  int* t_s = reinterpret_cast<int*>(PACK8 ? static_cast<void*>(r01_s + 8 * G) : static_cast<void*>(r01_s));
 
   if (threadIdx.x == 0) skip_s = (P.status != nullptr && *P.status != 0);
   for (int k = threadIdx.x; k < 8 * G; k += THREADS)
@@ -418,147 +552,259 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
   __syncthreads();
   const bool skip = skip_s != 0;
   if (skip && !P.has_pre) return;
-  const bool do_sum = !skip;  // a failed preconditioner still gets the leading perturbation
-  const uint32_t warp = threadIdx.x >> 5;
+  const TensorTable& tab = P.tab;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (skip) {  // a failed preconditioner: the leading perturbation alone
+    int t = 0;
+    for (uint32_t bl = blockIdx.x * THREADS + threadIdx.x; bl - lane < tab.blk_total; bl += gridDim.x * THREADS) {
+      t = advance_tensor(tab, t, bl - lane);
+      const Lut8Block k = lut8_block_info<ANY>(tab, t, bl);
+      uint4 xp = block_bits(k.b, P.pre.ctr2, P.keys);
+      if (ANY && (k.fl & kShift)) xp = window16(shfl_up4(xp), xp, 16u - k.a);
+      if (k.vec && (k.fl & kDtypeMask) != kF32) {
+        uint16_t* p = static_cast<uint16_t*>(k.base) + k.e0;
+        uint32_t v[8];
+        ld256(p, v);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          v[r] = (k.fl & kDtypeMask) == kBF16 ? pre_regs16<kBF16>(v[r], xp, r, P.pre) : pre_regs16<kF16>(v[r], xp, r, P.pre);
+        st256(p, v);
+      } else if (k.act) {
+        float none[16];
+        zero16(none);
+        lut8_apply_elements(k, none, xp, P, false);
+      }
+    }
+    return;
+  }
   const uint32_t t4_s = hdr + 32u * G;
   const uint32_t dst_t = 256u * (threadIdx.x >> 3) + 16u * (threadIdx.x & 7u);
-  uint32_t trow = 0;
-  if (do_sum) {
-    for (int e = threadIdx.x; e < 32 * G; e += THREADS) {
-      const float* a = a_s + 8 * (e >> 5) + ((e & 16) ? 4 : 0);
-      t4[e] = quad_partial(a, static_cast<uint32_t>(e) & 15u);
-    }
-    __syncthreads();
-    lut8_replicate4<THREADS>(t4_s, region0 + dst_t, 0, G > 1);
-    if (warp == 0) {
-      __syncwarp();
-      const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&tmem_s));
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(kTmemCols)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tm_fence_before();
-    __syncthreads();
-    tm_fence_after();
-    // TMEM lane 32 (warp mod 4) + lane id, columns from 128 (warp / 4)
-    trow = tmem_s + (((warp & 3u) * 32u) << 16) + (warp >> 2) * 128u;
+  const uint32_t bhi = static_cast<uint32_t>(static_cast<uint64_t>(tab.blk_base) >> 32);
+  for (int e = threadIdx.x; e < 32 * G; e += THREADS) {
+    const float* a = a_s + 8 * (e >> 5) + ((e & 16) ? 4 : 0);
+    t4[e] = quad_partial(a, static_cast<uint32_t>(e) & 15u);
   }
+  if (PACK8 && HIU) {
+    for (int k = threadIdx.x; k < 8 * G; k += THREADS) {
+      const GroupRound01 g = group_round01(static_cast<uint32_t>(k), bhi, P.keys);
+      r01_s[k] = make_uint4(g.x0, g.x2, g.lpa1, 0u);
+    }
+  }
+  __syncthreads();
+  lut8_replicate4<THREADS>(t4_s, region0 + dst_t, 0, G > 1);
+  if (warp == 0) {
+    __syncwarp();
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&tmem_s));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tm_fence_before();
+  __syncthreads();
+  tm_fence_after();
+  // TMEM lane 32 (warp mod 4) + lane id, columns from 128 (warp / 4)
+  const uint32_t trow = tmem_s + (((warp & 3u) * 32u) << 16) + (warp >> 2) * 128u;
 
-  const TensorTable& tab = P.tab;
-  const uint32_t lane = threadIdx.x & 31u;
   constexpr uint32_t chunk = static_cast<uint32_t>(THREADS * BPT);
   const uint32_t per_round = gridDim.x * chunk;
   const uint32_t rounds = (tab.blk_total + per_round - 1u) / per_round;
   uint32_t cur = 0;  // region holding the current pair (0 or 1)
-  Lut8Cursor cur0;   // tensor cursor at this thread's first block of the chunk
-  cur0.t = 0;
-  cur0.te = 0;       // nothing cached yet: the first block seeks
+  int t = 0;         // tensor of the warp's latest block
+  const auto counter_word = [&](const Lut8Block& k) {
+    return static_cast<uint32_t>(HIU ? static_cast<uint64_t>(k.b) : static_cast<uint64_t>(k.b - tab.blk_base));
+  };
 
   for (uint32_t rnd = 0; rnd < rounds; ++rnd) {
     // this thread's blocks of the chunk: cb, cb + THREADS, ..
     const uint32_t cb = (rnd * gridDim.x + blockIdx.x) * chunk + threadIdx.x;
-    if (do_sum) {
-      uint32_t wact = 0;  // blocks of the chunk that some lane of the warp sums
-      Lut8Cursor c = cur0;
+    int jn = 0;          // blocks of the warp inside the launch
+    uint32_t vr[BPT];    // their counter words (registers: 2-6 % faster than shared memory)
 #pragma unroll
-      for (int j = 0; j < BPT; ++j) {
-        Lut8Block k;
-        lut8_block_info(tab, c, cb + static_cast<uint32_t>(j * THREADS), k);
-        // HIU: the virtual block's low word; otherwise its offset from blk_base
-        vr_s[j * THREADS + threadIdx.x] =
-            k.act ? static_cast<uint32_t>(HIU ? static_cast<uint64_t>(k.b) : static_cast<uint64_t>(k.b - tab.blk_base))
-                  : 0u;
-        if (__any_sync(0xFFFFFFFFu, k.act)) wact |= 1u << j;
-        // theta is read after all pairs: bring it into L2 meanwhile
-        if (k.vec16) asm volatile("prefetch.L2 [%0];" ::"l"(static_cast<uint16_t*>(k.base) + k.e0));
-      }
-      for (int pr = 0; pr < NP; ++pr) {
-        const uint32_t frame = ((region0 + cur * kLut8Region) & 0xFFFF0000u) | (lane << 2);
-        const uint32_t q = 2u * static_cast<uint32_t>(pr);
-        const bool two = static_cast<int>(q) + 1 < G;
-        const auto run = [&](auto first) {
-          if constexpr (HIU) {
-            const uint32_t bhi = static_cast<uint32_t>(static_cast<uint64_t>(tab.blk_base) >> 32);
-            const GroupRound01 g0 = group_round01(q, bhi, P.keys);
-            const GroupRound01 g1 = group_round01(q + 1u, bhi, P.keys);
-#pragma unroll
-            for (int j = 0; j < BPT; ++j) {
-              if (!((wact >> j) & 1u)) continue;  // no lane of the warp has this block
-              const uint32_t blo = vr_s[j * THREADS + threadIdx.x];
-              lut8_tm_step_split<decltype(first)::value>(trow + 16u * static_cast<uint32_t>(j), blo, g0, g1, two,
-                                                         frame, P.keys);
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < BPT; ++j) {
-              if (!((wact >> j) & 1u)) continue;  // no lane of the warp has this block
-              const int64_t b = tab.blk_base + vr_s[j * THREADS + threadIdx.x];
-              lut8_tm_step<decltype(first)::value>(trow + 16u * static_cast<uint32_t>(j), b, q, two, frame, P.keys);
-            }
-          }
-        };
-        if (pr == 0)
-          run(std::true_type());
-        else
-          run(std::false_type());
-        tm_wait_st();  // this pair's sums are in TMEM before the next pair reads them
-        if (NP > 1) {
-          // the next pair (wrapping to pair 0 for the next chunk) into the other region
-          const int qn = pr + 1 < NP ? static_cast<int>(q) + 2 : 0;
-          lut8_replicate4<THREADS>(t4_s, region0 + (cur ^ 1u) * kLut8Region + dst_t, qn, qn + 1 < G);
-          __syncthreads();
-          cur ^= 1u;
+    for (int j = 0; j < BPT; ++j) {
+      const uint32_t bl = cb + static_cast<uint32_t>(j * THREADS);
+      vr[j] = 0u;
+      if (bl - lane < tab.blk_total) {
+        jn = j + 1;
+        t = advance_tensor(tab, t, bl - lane);
+        const Lut8Block k = lut8_block_info<ANY>(tab, t, bl);
+        vr[j] = counter_word(k);
+        if (lane == 0) t_s[j * (THREADS / 32) + warp] = t;
+        // theta is read with the last pair: bring it into L2 meanwhile
+        if (k.vec) {
+          const bool f32 = ANY && (k.fl & kDtypeMask) == kF32;
+          const char* p = static_cast<const char*>(k.base) + k.e0 * (f32 ? 4 : 2);
+          asm volatile("prefetch.L2 [%0];" ::"l"(p));
+          if (f32) asm volatile("prefetch.L2 [%0];" ::"l"(p + 32));
         }
       }
     }
-    // Apply: each block's sums read back from TMEM and added to theta (in L2
-    // by now). Full aligned 16-bit blocks here; the rare others (fp32, partial
-    // last blocks) in a loop of their own, which keeps their code out of this one.
-    Lut8Cursor c = cur0;
-    bool others = false;
+    __syncwarp();
+    bool others = false;  // a block of the chunk goes element by element
+    uint4 ahead = make_uint4(0u, 0u, 0u, 0u);  // AHEAD: the next step's words
+    for (int pr = 0; pr < NP; ++pr) {
+      const uint32_t frame = ((region0 + cur * kLut8Region) & 0xFFFF0000u) | (lane << 2);
+      const uint32_t q = 2u * static_cast<uint32_t>(pr);
+      const bool two = static_cast<int>(q) + 1 < G;
+      const GroupRound01 g0 = group_round01(q, bhi, P.keys);
+      const GroupRound01 g1 = group_round01(q + 1u, bhi, P.keys);
+      if (pr + 1 < NP) {
+        if constexpr (PACK8) {
 #pragma unroll 1
-    for (int j = 0; j < BPT; ++j) {
-      Lut8Block k;
-      lut8_block_info(tab, c, cb + static_cast<uint32_t>(j * THREADS), k);
-      others |= k.act && !k.vec16;
-      uint32_t v[8];
-      if (k.vec16) ld256(static_cast<uint16_t*>(k.base) + k.e0, v);
-      float acc[16];
-      zero16(acc);
-      if (do_sum && __any_sync(0xFFFFFFFFu, k.vec16)) tm_get16(acc, trow + 16u * static_cast<uint32_t>(j));
-      if (k.vec16) {
-        uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-        if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
-        if ((k.fl & kDtypeMask) == kBF16)
-          lut8_apply16<kBF16>(v, acc, xp, P, do_sum);
-        else
-          lut8_apply16<kF16>(v, acc, xp, P, do_sum);
-        st256(static_cast<uint16_t*>(k.base) + k.e0, v);
+          for (int j = 0; j < jn; ++j) {
+            const Lut8Block k = lut8_block_info<ANY>(tab, t_s[j * (THREADS / 32) + warp],
+                                                     cb + static_cast<uint32_t>(j * THREADS));
+            lut8_tm_step8<HIU>(trow + 16u * static_cast<uint32_t>(j),
+                               BlockCounter<HIU>(counter_word(k), tab.blk_base, P.keys), q,
+                               static_cast<uint32_t>(P.K), r01_s, two, frame, P.keys);
+          }
+        } else {
+          const auto run_ahead = [&](auto first) {
+            if (jn == 0) return;
+            const GroupRound01 g2 = group_round01(q + 2u, bhi, P.keys);
+            BlockCounter<HIU> kb(vr[0], tab.blk_base, P.keys);
+            if (decltype(first)::value) ahead = philox_finish(kb.start(g0, q, P.keys), P.keys);
+#pragma unroll
+            for (int j = 0; j < BPT; ++j) {
+              if (j >= jn) break;
+              const bool wrap = j + 1 == jn;  // next: block 0 of the next pair
+              const GroupRound01 gn = {wrap ? g2.x0 : g0.x0, wrap ? g2.x2 : g0.x2, wrap ? g2.lpa1 : g0.lpa1};
+              lut8_tm_step_ahead<decltype(first)::value, HIU>(
+                  trow + 16u * static_cast<uint32_t>(j), ahead, kb, q, g1,
+                  BlockCounter<HIU>(wrap ? vr[0] : vr[j + 1 < BPT ? j + 1 : 0], tab.blk_base, P.keys),
+                  wrap ? q + 2u : q, gn, frame, P.keys);
+            }
+          };
+          const auto run = [&](auto first) {
+            if constexpr (AHEAD) {
+              run_ahead(first);
+            } else {
+#pragma unroll
+              for (int j = 0; j < BPT; ++j) {
+                if (j >= jn) break;
+                lut8_tm_step<decltype(first)::value, HIU>(trow + 16u * static_cast<uint32_t>(j),
+                                                          BlockCounter<HIU>(vr[j], tab.blk_base, P.keys), q, g0, g1,
+                                                          two, frame, P.keys);
+              }
+            }
+          };
+          if (pr == 0)
+            run(std::true_type());
+          else
+            run(std::false_type());
+        }
+        tm_wait_st();  // this pair's sums are in TMEM before the next pair reads them
+      } else {
+        // The last pair applies the sums to theta as they complete: the loads
+        // are issued before the block's lookups, which hide them, and theta's
+        // traffic spreads over the pair instead of coming in a phase of its
+        // own. Blocks across a tensor's end leave their sums in TMEM for a
+        // pass of their own.
+        const int pre_at = !P.has_pre ? 0 : PACK8 ? 3 : P.pre.ctr2 == q ? 1 : (two && P.pre.ctr2 == q + 1u) ? 2 : 3;
+#pragma unroll 1
+        for (int j = 0; j < jn; ++j) {
+          const uint32_t ta = trow + 16u * static_cast<uint32_t>(j);
+          const Lut8Block k = lut8_block_info<ANY>(tab, t_s[j * (THREADS / 32) + warp],
+                                                   cb + static_cast<uint32_t>(j * THREADS));
+          const bool f32 = ANY && (k.fl & kDtypeMask) == kF32;  // the same in all lanes
+          char* tp = static_cast<char*>(k.base) + k.e0 * (f32 ? 4 : 2);
+          uint32_t v[16];
+          uint32_t(&lo)[8] = *reinterpret_cast<uint32_t(*)[8]>(&v[0]);
+          uint32_t(&hi)[8] = *reinterpret_cast<uint32_t(*)[8]>(&v[8]);
+          if (k.vec) ld256(tp, lo);
+          if (ANY && k.vec && f32) ld256(tp + 32, hi);
+          const BlockCounter<HIU> kb(counter_word(k), tab.blk_base, P.keys);
+          float acc[16];
+          uint4 x, xp;  // xp: words of the leading perturbation: group q's, q + 1's or its own
+          if constexpr (PACK8) {
+            x = group_words8(kb, q, static_cast<uint32_t>(P.K), r01_s, P.keys);
+            if (pr == 0)
+              zero16(acc);
+            else
+              tm_get16(acc, ta);
+          } else {
+            tm_ld16(acc, ta);
+            if (AHEAD && j == 0)
+              x = ahead;
+            else
+              x = philox_finish(kb.start(g0, q, P.keys), P.keys);
+            tm_wait_ld(acc);
+          }
+          lut8_lookup(acc, x, frame);
+          xp = x;
+          if (two) {
+            x = PACK8 ? group_words8(kb, q + 1u, static_cast<uint32_t>(P.K), r01_s, P.keys)
+                      : philox_finish(kb.start(g1, q + 1u, P.keys), P.keys);
+            lut8_lookup(acc, x, frame | 128u);
+            if (pre_at == 2) xp = x;
+          }
+          if (__any_sync(0xFFFFFFFFu, k.act && !k.vec)) {
+            tm_st16(ta, acc);
+            others = true;
+          }
+          if (pre_at == 3) xp = block_bits(k.b, P.pre.ctr2, P.keys);
+          if (ANY && (k.fl & kShift)) {  // the same in all lanes
+            float below[16], own[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              own[i] = acc[i];
+              below[i] = __shfl_up_sync(0xFFFFFFFFu, acc[i], 1);
+            }
+            window16f(below, own, 16u - k.a, acc);
+            xp = window16(shfl_up4(xp), xp, 16u - k.a);
+          }
+          if (k.vec) {
+            if (ANY && f32) {
+              lut8_apply32(v, acc, xp, P);
+              st256(tp + 32, hi);
+            } else if ((k.fl & kDtypeMask) == kBF16) {
+              lut8_apply16<kBF16>(lo, acc, xp, P);
+            } else {
+              lut8_apply16<kF16>(lo, acc, xp, P);
+            }
+            st256(tp, lo);
+          }
+        }
+        if (others) {
+          tm_wait_st();
+#pragma unroll 1
+          for (int j = 0; j < jn; ++j) {
+            const Lut8Block k = lut8_block_info<ANY>(tab, t_s[j * (THREADS / 32) + warp],
+                                                     cb + static_cast<uint32_t>(j * THREADS));
+            const bool mine = k.act && !k.vec;
+            if (!__any_sync(0xFFFFFFFFu, mine)) continue;
+            float acc[16];
+            tm_get16(acc, trow + 16u * static_cast<uint32_t>(j));
+            uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+            if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
+            if (ANY && (k.fl & kShift)) {
+              float below[16], own[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                own[i] = acc[i];
+                below[i] = __shfl_up_sync(0xFFFFFFFFu, acc[i], 1);
+              }
+              window16f(below, own, 16u - k.a, acc);
+              xp = window16(shfl_up4(xp), xp, 16u - k.a);
+            }
+            if (mine) lut8_apply_elements(k, acc, xp, P, true);
+          }
+        }
+      }
+      if (NP > 1) {
+        // the next pair (wrapping to pair 0 for the next chunk) into the other region
+        const int qn = pr + 1 < NP ? static_cast<int>(q) + 2 : 0;
+        lut8_replicate4<THREADS>(t4_s, region0 + (cur ^ 1u) * kLut8Region + dst_t, qn, qn + 1 < G);
+        __syncthreads();
+        cur ^= 1u;
       }
     }
-    if (__any_sync(0xFFFFFFFFu, others)) {
-      Lut8Cursor c2 = cur0;
-#pragma unroll 1
-      for (int j = 0; j < BPT; ++j) {
-        Lut8Block k;
-        lut8_block_info(tab, c2, cb + static_cast<uint32_t>(j * THREADS), k);
-        const bool mine = k.act && !k.vec16;
-        float acc[16];
-        zero16(acc);
-        if (do_sum && __any_sync(0xFFFFFFFFu, mine)) tm_get16(acc, trow + 16u * static_cast<uint32_t>(j));
-        if (mine) lut8_apply_other(k, acc, P, do_sum);
-      }
-    }
-    cur0 = c;
   }
-  if (do_sum) {
-    tm_fence_before();
-    __syncthreads();
-    tm_fence_after();
-    if (warp == 0) {
-      __syncwarp();
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_s), "r"(kTmemCols) : "memory");
-    }
+  tm_fence_before();
+  __syncthreads();
+  tm_fence_after();
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_s), "r"(kTmemCols) : "memory");
   }
 }
 
@@ -612,14 +858,6 @@ __device__ __forceinline__ float2 small_sum2(const uint4& x0, const uint4& x1, u
   return make_float2(lo, hi);
 }
 
-// theta pair + the leading perturbation's signed scales, one packed add.
-__device__ __forceinline__ void add_signed2(float2& f, const uint4& x, int i, const PerturbOp& op) {
-  // the probe bit moved to bit 31 by a multiply (PerturbOp::mul): the
-  // multiply-add pipe instead of the integer ALU, the busier one here
-  fadd2_rn(f.x, f.y, __uint_as_float(op.nscale_bits ^ ((word_of(x, i >> 2) * op.mul[i & 3]) & 0x80000000u)),
-           __uint_as_float(op.nscale_bits ^ ((word_of(x, (i + 1) >> 2) * op.mul[(i + 1) & 3]) & 0x80000000u)));
-}
-
 template <uint8_t DT, bool TWO>
 __device__ __forceinline__ void small_block16(uint32_t (&v)[8], const uint4& x0, const uint4& x1, const uint4& xp,
                                               uint32_t frame, bool pre, const UpdateParams& P, bool do_sum) {
@@ -650,6 +888,50 @@ __device__ __forceinline__ void small_block16(uint32_t (&v)[8], const uint4& x0,
   }
 }
 
+// A block of the launch outside the vector loop.
+struct SmallBlock {
+  int64_t b;       // virtual block (Philox counter)
+  int64_t e0;      // first element inside its tensor
+  void* base;      // tensor base pointer
+  int cnt;         // elements of the block (1..16)
+  uint8_t fl;      // tensor flags
+};
+
+// Apply the leading perturbation (if any) and the probe sums to a block that
+// is not a full, aligned 16-bit one: fp32 blocks and partial last blocks.
+__device__ __forceinline__ void small_apply_other(const SmallBlock& k, const float (&acc)[16], const UpdateParams& P,
+                                              bool do_sum) {
+  uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+  if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
+  const uint8_t dt = k.fl & kDtypeMask;
+  if (dt == kF32 && k.cnt == 16 && (k.fl & kVec32)) {
+    float* p = static_cast<float*>(k.base) + k.e0;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t v[8];
+      ld256(p + 8 * half, v);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float th = __uint_as_float(v[r]);
+        if (P.has_pre) th = add_signed(th, xp, 8 * half + r, P.pre);
+        if (do_sum) th = __fadd_rn(th, acc[8 * half + r]);
+        v[r] = __float_as_uint(th);
+      }
+      st256(p + 8 * half, v);
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    if (i < k.cnt) {
+      float th = load_elem(k.base, dt, k.e0 + i);
+      if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
+      if (do_sum) th = __fadd_rn(th, acc[i]);
+      store_elem(k.base, dt, k.e0 + i, th);
+    }
+  }
+}
+
 // Any other block of the launch: fp32, a partial last block, padding, or an
 // unaligned tensor (update_shift_kernel's).
 template <int TAG>
@@ -658,14 +940,12 @@ __device__ __noinline__ void small_block_other(const TensorTable& tab, int t, ui
   const uint32_t tb = tensor_blk_begin(tab, t);
   const uint8_t fl = tab.flags[t];
   if ((fl & kShift) || b < tb) return;
-  Lut8Block k;
+  SmallBlock k;
   k.b = virtual_block(tab, t, b);
   k.e0 = static_cast<int64_t>(b - tb) * 16;
   k.cnt = static_cast<int>(min(static_cast<int64_t>(16), tab.numel[t] - k.e0));
   k.base = reinterpret_cast<void*>(tab.ptr[t]);
   k.fl = fl;
-  k.act = true;
-  k.vec16 = false;
   float acc[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
@@ -673,7 +953,7 @@ __device__ __noinline__ void small_block_other(const TensorTable& tab, int t, ui
     lut8_lookup(acc, block_bits(k.b, 0u, P.keys), frame);
     if (P.groups > 1) lut8_lookup(acc, block_bits(k.b, 1u, P.keys), frame | 128u);
   }
-  lut8_apply_other(k, acc, P, do_sum);
+  small_apply_other(k, acc, P, do_sum);
 }
 
 // Leading perturbation of the small kernel's instantiations: on a Philox word
@@ -776,55 +1056,50 @@ __global__ void __launch_bounds__(kSmallThreads, 1) update_lut8_small_kernel(con
   }
 }
 
-template <int BPT>
-cudaError_t launch_lut8_cfg(const UpdateParams& p, int grid, cudaStream_t stream) {
-  // every virtual block of the launch lies in [blk_base, blk_base + blk_total)
-  const uint64_t first = static_cast<uint64_t>(p.tab.blk_base);
-  const uint64_t last = first + (p.tab.blk_total > 0 ? p.tab.blk_total - 1u : 0u);
-  if ((first >> 32) == (last >> 32))
-    update_lut8_kernel<BPT, true><<<grid, kLut8Threads, lut8_smem_bytes(p.groups), stream>>>(p);
-  else
-    update_lut8_kernel<BPT, false><<<grid, kLut8Threads, lut8_smem_bytes(p.groups), stream>>>(p);
+template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
+cudaError_t launch_lut8_cfg(const UpdateParams& p, int sms, cudaStream_t stream) {
+  // one CTA per chunk of 512 * BPT blocks, at most one per SM
+  const int64_t chunk = static_cast<int64_t>(kLut8Threads) * BPT;
+  const int64_t want = (static_cast<int64_t>(p.tab.blk_total) + chunk - 1) / chunk;
+  const int grid = static_cast<int>(want < sms ? want : sms);
+  update_lut8_kernel<BPT, HIU, ANY, PACK8, AHEAD><<<grid, kLut8Threads, lut8_smem_bytes(PACK8), stream>>>(p);
   return cudaGetLastError();
 }
 
-template <int BPT>
-cudaError_t lut8_prepare_cfg(int groups, int* blocks_per_sm) {
-  // the limit covers every group count, so later launches with more groups still fit
-  cudaError_t e = cudaFuncSetAttribute(update_lut8_kernel<BPT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(lut8_smem_bytes(kLut8MaxGroups)));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(update_lut8_kernel<BPT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(lut8_smem_bytes(kLut8MaxGroups)));
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, update_lut8_kernel<BPT, false>, kLut8Threads,
-                                                       lut8_smem_bytes(groups));
+template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
+cudaError_t lut8_limit() {
+  return cudaFuncSetAttribute(update_lut8_kernel<BPT, HIU, ANY, PACK8, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(lut8_smem_bytes(PACK8)));
 }
 
-bool lut8_supported(int groups, int packing) { return packing == kPacking1 && groups >= 1 && groups <= kLut8MaxGroups; }
 
-cudaError_t lut8_prepare(int groups, int* blocks_per_sm) {
-  if (groups <= 2) {
-    const int lim = static_cast<int>(lut8_small_smem_bytes());
-    cudaError_t e = cudaSuccess;
-    const void* kernels[] = {
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, false>),
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, true>),
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, false>),
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, true>),
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, false>),
-        reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, true>)};
-    for (const void* k : kernels)
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, update_lut8_small_kernel<kPreRuntime, true>,
-                                                         kSmallThreads, lut8_small_smem_bytes());
-  }
-  cudaError_t e = lut8_prepare_cfg<2>(groups, blocks_per_sm);
-  if (e == cudaSuccess) e = lut8_prepare_cfg<4>(groups, blocks_per_sm);
-  if (e == cudaSuccess) e = lut8_prepare_cfg<8>(groups, blocks_per_sm);
+cudaError_t lut8_prepare() {
+  const int lim = static_cast<int>(lut8_small_smem_bytes());
+  cudaError_t e = cudaSuccess;
+  const void* kernels[] = {reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, false>),
+                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, true>),
+                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, false>),
+                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, true>),
+                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, false>),
+                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, true>)};
+  for (const void* k : kernels)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = lut8_limit<2, true, false, false>();
+  if (e == cudaSuccess) e = lut8_limit<4, true, false, false>();
+  if (e == cudaSuccess) e = lut8_limit<8, true, false, false>();
+  if (e == cudaSuccess) e = lut8_limit<8, true, false, false, true>();
+  if (e == cudaSuccess) e = lut8_limit<2, true, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<4, true, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<8, true, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<8, false, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<2, true, true, true>();
+  if (e == cudaSuccess) e = lut8_limit<4, true, true, true>();
+  if (e == cudaSuccess) e = lut8_limit<8, true, true, true>();
+  if (e == cudaSuccess) e = lut8_limit<8, false, true, true>();
   return e;
 }
+
+constexpr int kAheadGroups = 24;  // see AHEAD
 
 // Blocks per thread: the largest of 8, 4, 2 that still gives every SM a chunk.
 int lut8_bpt(uint32_t blk_total, int sms) {
@@ -833,44 +1108,54 @@ int lut8_bpt(uint32_t blk_total, int sms) {
   return 2;
 }
 
-
-cudaError_t launch_update_lut8(const UpdateParams& p, int sms, int blocks_per_sm, cudaStream_t stream) {
-  const int64_t total = p.tab.blk_total;
-  const int64_t cap = static_cast<int64_t>(sms) * blocks_per_sm;
-  if (p.groups <= 2) {
-    const int64_t want = (total + kSmallThreads - 1) / kSmallThreads;
-    const int g = static_cast<int>(want < cap ? want : cap);
-    const size_t sm = lut8_small_smem_bytes();
-    // with a leading perturbation: its Philox word one of the sums' or its own;
-    // without one, the run-time instantiation (faster there: its registers are
-    // laid out for the leading perturbation and it does not spill)
-    const bool two = p.groups == 2;
-    const int pre = !p.has_pre ? kPreRuntime
-                               : (p.pre.ctr2 == 0u || (p.pre.ctr2 == 1u && two) ? kPreShared : kPreOwn);
-    if (pre == kPreShared && two)
-      update_lut8_small_kernel<kPreShared, true><<<g, kSmallThreads, sm, stream>>>(p);
-    else if (pre == kPreShared)
-      update_lut8_small_kernel<kPreShared, false><<<g, kSmallThreads, sm, stream>>>(p);
-    else if (pre == kPreOwn && two)
-      update_lut8_small_kernel<kPreOwn, true><<<g, kSmallThreads, sm, stream>>>(p);
-    else if (pre == kPreOwn)
-      update_lut8_small_kernel<kPreOwn, false><<<g, kSmallThreads, sm, stream>>>(p);
-    else if (two)
-      update_lut8_small_kernel<kPreRuntime, true><<<g, kSmallThreads, sm, stream>>>(p);
-    else
-      update_lut8_small_kernel<kPreRuntime, false><<<g, kSmallThreads, sm, stream>>>(p);
-    return cudaGetLastError();
-  }
-  // one CTA per chunk of 512 * BPT blocks, at most the resident CTAs
-  const int bpt = lut8_bpt(p.tab.blk_total, sms);
-  const int64_t chunk = static_cast<int64_t>(kLut8Threads) * bpt;
-  const int64_t want = (total + chunk - 1) / chunk;
-  const int grid = static_cast<int>(want < cap ? want : cap);
+template <bool ANY, bool PACK8>
+cudaError_t launch_lut8_any(const UpdateParams& p, int bpt, int sms, cudaStream_t stream) {
   switch (bpt) {
-    case 8: return launch_lut8_cfg<8>(p, grid, stream);
-    case 4: return launch_lut8_cfg<4>(p, grid, stream);
-    default: return launch_lut8_cfg<2>(p, grid, stream);
+    case 8: return launch_lut8_cfg<8, true, ANY, PACK8>(p, sms, stream);
+    case 4: return launch_lut8_cfg<4, true, ANY, PACK8>(p, sms, stream);
+    default: return launch_lut8_cfg<2, true, ANY, PACK8>(p, sms, stream);
   }
+}
+
+cudaError_t launch_update_lut8_small(const UpdateParams& p, int sms, cudaStream_t stream) {
+  const int64_t want = (static_cast<int64_t>(p.tab.blk_total) + kSmallThreads - 1) / kSmallThreads;
+  const int g = static_cast<int>(want < sms ? want : sms);
+  const size_t sm = lut8_small_smem_bytes();
+  // with a leading perturbation: its Philox word one of the sums' or its own;
+  // without one, the run-time instantiation (faster there: its registers are
+  // laid out for the leading perturbation and it does not spill)
+  const bool two = p.groups == 2;
+  const int pre =
+      !p.has_pre ? kPreRuntime : (p.pre.ctr2 == 0u || (p.pre.ctr2 == 1u && two) ? kPreShared : kPreOwn);
+  if (pre == kPreShared && two)
+    update_lut8_small_kernel<kPreShared, true><<<g, kSmallThreads, sm, stream>>>(p);
+  else if (pre == kPreShared)
+    update_lut8_small_kernel<kPreShared, false><<<g, kSmallThreads, sm, stream>>>(p);
+  else if (pre == kPreOwn && two)
+    update_lut8_small_kernel<kPreOwn, true><<<g, kSmallThreads, sm, stream>>>(p);
+  else if (pre == kPreOwn)
+    update_lut8_small_kernel<kPreOwn, false><<<g, kSmallThreads, sm, stream>>>(p);
+  else if (two)
+    update_lut8_small_kernel<kPreRuntime, true><<<g, kSmallThreads, sm, stream>>>(p);
+  else
+    update_lut8_small_kernel<kPreRuntime, false><<<g, kSmallThreads, sm, stream>>>(p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream) {
+  const bool pack8 = p.packing == kPacking8;
+  // every virtual block that a lane sums lies in [blk_base, blk_base + blk_total), except the one below a
+  // tensor's first chunk, whose sums nothing uses
+  const uint64_t first = static_cast<uint64_t>(p.tab.blk_base);
+  const uint64_t last = first + (p.tab.blk_total > 0 ? p.tab.blk_total - 1u : 0u);
+  if ((first >> 32) != (last >> 32))
+    return pack8 ? launch_lut8_cfg<8, false, true, true>(p, sms, stream)
+                 : launch_lut8_cfg<8, false, true, false>(p, sms, stream);
+  const int bpt = lut8_bpt(p.tab.blk_total, sms);
+  if (pack8) return launch_lut8_any<true, true>(p, bpt, sms, stream);
+  if (any) return launch_lut8_any<true, false>(p, bpt, sms, stream);
+  if (bpt == 8 && p.groups >= kAheadGroups) return launch_lut8_cfg<8, true, false, false, true>(p, sms, stream);
+  return launch_lut8_any<false, false>(p, bpt, sms, stream);
 }
 
 }  // namespace zo
