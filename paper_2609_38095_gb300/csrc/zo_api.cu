@@ -81,10 +81,6 @@ constexpr int kTwoOpCandidates = 3;
 constexpr int kTwoOpLoop[kTwoOpCandidates] = {zo::kLoopRuns, zo::kLoopRuns, zo::kLoopBlocks};
 constexpr int kTwoOpBlocksPerSm[kTwoOpCandidates] = {3, 4, 4};
 
-// The update is issue-bound; four waves of its blocks per SM keep more warps
-// eligible than one persistent wave (measured +3 % at K = 64 and 256).
-constexpr int kUpdateWaves = 4;
-
 // Packing-1 updates with at most this many probe groups keep both groups'
 // tables in shared memory for the whole launch (update_lut8_small_kernel);
 // all others walk the groups chunk by chunk (update_lut8_kernel).
@@ -97,7 +93,6 @@ struct DeviceInfo {
   int two_op_bps[kTwoOpCandidates] = {};  // two-op perturb blocks per SM, by candidate
   int pair_bps = 0;                       // perturb_pair blocks per SM
   int shift_bps[2][3] = {};               // perturb_shift blocks per SM, by operation count and dtype
-  int update_shift_bps[3][kSmallGroups + 1] = {};  // update_shift_kernel: dtype, group count
   bool lut8_ready = false;                // the update kernels' shared-memory limits are raised
 };
 constexpr int kMaxDevices = 64;
@@ -137,19 +132,6 @@ int device_info(DeviceInfo** out) {
     d.sms = sms;
   }
   *out = &d;
-  return ZO_OK;
-}
-
-int update_shift_blocks_per_sm(DeviceInfo* d, int groups, uint8_t dt, int* out) {
-  std::lock_guard<std::mutex> lock(g_dev_mu);
-  int& slot = d->update_shift_bps[dt][groups];
-  if (slot == 0) {
-    int bps = 0;
-    cudaError_t e = zo::update_shift_blocks_per_sm(groups, dt, &bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy(update_shift)");
-    slot = bps > 0 ? bps : 1;
-  }
-  *out = slot;
   return ZO_OK;
 }
 
@@ -194,10 +176,15 @@ int validate_params(const zo_tensor* params, int32_t n, int* packing = nullptr) 
 // numbering every tensor starts on a multiple of kLaunchAlign blocks (see
 // TensorTable). Returns the first tensor not taken; *nblocks receives the
 // virtual blocks the launch covers (tab.blk_total its launch blocks).
-// slots: tensors off the 32-byte grid are flagged kShift and take 32 launch
-// blocks per 31 of their aligned chunks (update_lut8_kernel).
+// kSlots: tensors off the 32-byte grid are flagged kShift and take 32 launch
+// blocks per 31 of their aligned chunks (the update kernels). kItems: so, and
+// launch blocks are 32-byte items, of which fp32 tensors have two per block; a
+// tensor whose items alone exceed a launch is not taken.
+enum Numbering { kBlocks, kSlots, kItems };
+
 int32_t fill_table(TensorTable& tab, const zo_tensor* params, int32_t t0, int32_t n, int64_t blk_base,
-                   int64_t* nblocks, bool slots = false) {
+                   int64_t* nblocks, Numbering numbering = kBlocks) {
+  const bool slots = numbering != kBlocks;
   tab.n = 0;
   tab.blk_base = blk_base;
   int64_t b = 0;  // launch blocks so far
@@ -208,12 +195,13 @@ int32_t fill_table(TensorTable& tab, const zo_tensor* params, int32_t t0, int32_
     const int64_t nb = (p.numel + 15) / 16;
     const int64_t start = (b + zo::kLaunchAlign - 1) / zo::kLaunchAlign * zo::kLaunchAlign;
     const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.ptr) % 32);
-    int64_t span = nb;  // launch blocks of the tensor
+    const int64_t per = numbering == kItems && p.dtype == ZO_F32 ? 8 : 16;  // elements per launch block
+    int64_t span = (p.numel + per - 1) / per;  // launch blocks of the tensor
     if (slots && off != 0 && nb > 0) {
-      const int64_t chunks = (p.numel + off / elem_size(p.dtype) + 15) / 16;
+      const int64_t chunks = (p.numel + off / elem_size(p.dtype) + per - 1) / per;
       span = (chunks + zo::kShiftLanes - 1) / zo::kShiftLanes * zo::kLaunchAlign;
     }
-    if (tab.n > 0 && start + span >= zo::kMaxLaunchBlocks) break;
+    if ((tab.n > 0 || numbering == kItems) && start + span >= zo::kMaxLaunchBlocks) break;
     const int i = tab.n++;
     tab.vdelta[i] = static_cast<uint32_t>(start - v);
     b = start + span;
@@ -421,7 +409,6 @@ uint32_t shift_groups(const zo::TensorTable& tab, uint8_t dt, uint32_t* grp_end)
 }
 
 thread_local zo::ShiftParams tl_shift;
-thread_local zo::UpdateShiftParams tl_update_shift;
 
 int run_perturb(const zo_tensor* params, int32_t n, PerturbParams& pp, DeviceInfo* d, cudaStream_t s) {
   int loop = zo::kLoopBlocks, bps = d->perturb_bps, slot = -1;
@@ -567,7 +554,7 @@ int run_pair_shift(const zo::PairParams& pp, uint8_t dt, bool moved, DeviceInfo*
 
 thread_local PerturbParams tl_perturb;
 thread_local zo::PairParams tl_pair;
-thread_local UpdateParams tl_update;
+thread_local zo::SmallUpdateParams tl_update;
 
 }  // namespace
 
@@ -711,7 +698,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   if (n_tensors == 0) return rc;
   DeviceInfo* d = nullptr;
   if ((rc = device_info(&d)) != ZO_OK) return rc;
-  UpdateParams& up = tl_update;
+  UpdateParams& up = tl_update.u;
   up.keys = expand_keys(seed);
   up.coef = c;
   up.coef_mul = -(lr / static_cast<double>(K));
@@ -721,42 +708,25 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  const bool small = up.packing == zo::kPacking1 && up.groups <= kSmallGroups;
+  const bool few = up.packing == zo::kPacking1 && up.groups <= kSmallGroups;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t blk = 0;
   for (int32_t t0 = 0; t0 < n_tensors;) {
     int64_t nb = 0;
-    t0 = fill_table(up.tab, params, t0, n_tensors, blk, &nb, !small);
+    const int32_t first = t0;
+    t0 = fill_table(up.tab, params, first, n_tensors, blk, &nb, few ? kItems : kSlots);
+    const bool small = few && t0 > first && zo::one_high_word(up.tab);
+    if (few && !small) t0 = fill_table(up.tab, params, first, n_tensors, blk, &nb, kSlots);
     blk += nb;
     if (nb == 0) continue;
-    if (!small) {
-      bool any = false;  // a non-empty tensor that is not 16-bit and aligned
-      for (int i = 0; i < up.tab.n && !any; ++i)
-        any = up.tab.numel[i] > 0 &&
-              ((up.tab.flags[i] & zo::kShift) || (up.tab.flags[i] & zo::kDtypeMask) == zo::kF32);
-      cudaError_t e = zo::launch_update_lut8(up, any, d->sms, s);
-      if (e != cudaSuccess) return cuda_fail(e, "update_lut8_kernel");
-      continue;
-    }
-    bool main_work = false;
-    const unsigned shift_types = mark_shift(up.tab, &main_work);
-    if (main_work) {
-      cudaError_t e = zo::launch_update_lut8_small(up, d->sms, s);
-      if (e != cudaSuccess) return cuda_fail(e, "update_lut8_small_kernel");
-    }
-    if (shift_types) tl_update_shift.u = up;
-    for (uint8_t dt = 0; dt < 3; ++dt) {
-      if (!(shift_types & (1u << dt))) continue;
-      const uint32_t groups = shift_groups(up.tab, dt, tl_update_shift.grp_end);
-      tl_update_shift.grp_total = groups;
-      int sbps = 1;
-      if ((rc = update_shift_blocks_per_sm(d, up.groups, dt, &sbps)) != ZO_OK) return rc;
-      const int64_t want = (static_cast<int64_t>(groups) * 32 + zo::kThreads - 1) / zo::kThreads;
-      const int64_t cap = static_cast<int64_t>(d->sms) * sbps * kUpdateWaves;
-      cudaError_t e = zo::launch_update_shift(tl_update_shift, dt, static_cast<int>(want < cap ? want : cap), s);
-      if (e != cudaSuccess) return cuda_fail(e, "update_shift_kernel");
-    }
+    bool any = false;  // a non-empty tensor that is not 16-bit and aligned
+    for (int i = 0; i < up.tab.n && !any; ++i)
+      any = up.tab.numel[i] > 0 &&
+            ((up.tab.flags[i] & zo::kShift) || (up.tab.flags[i] & zo::kDtypeMask) == zo::kF32);
+    const cudaError_t e = small ? zo::launch_update_lut8_small(tl_update, any, d->sms, s)
+                                : zo::launch_update_lut8(up, any, d->sms, s);
+    if (e != cudaSuccess) return cuda_fail(e, small ? "update_lut8_small_kernel" : "update_lut8_kernel");
   }
   return ZO_OK;
 }

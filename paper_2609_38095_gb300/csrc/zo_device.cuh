@@ -160,12 +160,22 @@ struct UpdateParams {
   const int32_t* status;   // optional: when *status != 0 only `pre` is applied
 };
 
-// The fused update over the unaligned tensors of a launch (same chunking and
-// group counting as ShiftParams).
-struct UpdateShiftParams {
+// Philox rounds 0-1 as far as they depend on the probe group alone (the
+// launch's virtual blocks sharing the counter's high word).
+struct GroupRound01 {
+  uint32_t x0;    // lo(M1 q) ^ k0[1]
+  uint32_t x2;    // hi(M0 u) ^ k1[1], u = hi(M1 q) ^ bhi ^ k0[0]
+  uint32_t lpa1;  // lo(M0 u)
+};
+
+// The update at one or two probe groups: the groups' and the leading
+// perturbation's Philox parts beside it. In its table launch blocks are
+// 32-byte items: half blocks of fp32 tensors, and 32 per 31 aligned chunks of
+// tensors off the 32-byte grid (kShift).
+struct SmallUpdateParams {
   UpdateParams u;
-  uint32_t grp_total;
-  uint32_t grp_end[kMaxTensorsPerLaunch];
+  GroupRound01 g[2];
+  GroupRound01 gp;
 };
 
 // ---------------------------------------------------------------------------

@@ -26,17 +26,15 @@ cudaError_t launch_perturb_shift(const ShiftParams& p, uint8_t dt, int grid, cud
 cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream);
 // moved: theta at another offset from the 32-byte grid than plus and minus (16-bit only).
 cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, int grid, cudaStream_t stream);
-// Fused update: packing 1 and at most two probe groups (K <= 16), ...
-cudaError_t launch_update_lut8_small(const UpdateParams& p, int sms, cudaStream_t stream);
+// Fused update: packing 1, at most two probe groups (K <= 16) and virtual
+// blocks that share the counter's high word; ...
+cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream);
 // ... and every other one. any: the launch holds fp32 tensors or tensors off
 // the 32-byte grid (those flagged kShift, in slots of 32 launch blocks per 31
 // chunks).
 cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream);
 cudaError_t lut8_prepare();  // raises both kernels' shared-memory limits (once per device)
-// Tensors off the 32-byte grid at K <= 16.
-cudaError_t launch_update_shift(const UpdateShiftParams& p, uint8_t dt, int grid, cudaStream_t stream);
-cudaError_t update_shift_blocks_per_sm(int groups, uint8_t dt, int* out);
-size_t update_smem_bytes(int groups);
+bool one_high_word(const TensorTable& tab);  // of the launch's virtual blocks
 cudaError_t perturb_blocks_per_sm(int nops, int loop, int* out);
 cudaError_t shift_blocks_per_sm(int nops, uint8_t dt, int* out);
 cudaError_t pair_blocks_per_sm(int* out);

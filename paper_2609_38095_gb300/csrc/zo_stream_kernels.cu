@@ -751,192 +751,6 @@ __global__ void __launch_bounds__(256, 4) pair_shift_kernel(const __grid_constan
 }
 
 // ---------------------------------------------------------------------------
-// Fused K-probe update: theta <- rn(fp32(theta) + sum_k a_k z_k[g]).
-//
-// Byte m of Philox(b, q) holds the signs of probes 8q..8q+7 for element
-// 16b + m. Its low nibble indexes a 16-entry table of the fp32 partial sums
-//   T[n] = ((s0 a_{4h} + s1 a_{4h+1}) + s2 a_{4h+2}) + s3 a_{4h+3},
-//   s_j = +1 if bit j of n is set, else -1,
-// for probe quad h = 2q, the high nibble the table of quad 2q + 1. Each
-// element adds the two looked-up partials (low quad + high quad: the group's
-// 8-probe partial) to its fp32 accumulator, groups in increasing order: one
-// shared-memory load and one add per four probes instead of a select and an
-// add per probe. Probes K..8*groups-1 have a = 0. update_lut8_kernel adds the
-// same 8-probe partials in the same order, so both give the same bits.
-//
-// Shared-memory layout: probe group q owns a 256-byte frame starting on a
-// 256-byte boundary of the shared window; bytes [0, 64) hold the table of
-// quad 2q, [64, 128) the table of quad 2q + 1. Masking a Philox word once
-// with 0x3C3C3C3C (after a shift by 2) leaves four nibble*4 offsets in its
-// four bytes; one byte-permute then splices an offset under the frame's
-// upper bytes, giving the lookup address in a single instruction.
-// ---------------------------------------------------------------------------
-constexpr uint32_t kFrameBytes = 256;
-
-__device__ __forceinline__ float lds_lo(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-  return v;
-}
-
-__device__ __forceinline__ float lds_hi(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1+64];" : "=f"(v) : "r"(addr));
-  return v;
-}
-
-__device__ __forceinline__ void accumulate_block(float (&acc)[16], int64_t b, const UpdateParams& P,
-                                                 uint32_t lut_base) {
-  const uint32_t blo = static_cast<uint32_t>(b), bhi = static_cast<uint32_t>(static_cast<uint64_t>(b) >> 32);
-  uint32_t frame = lut_base;
-  for (int q = 0; q < P.groups; ++q, frame += kFrameBytes) {
-    const uint4 x = philox10(blo, bhi, static_cast<uint32_t>(q), 0u, P.keys);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const uint32_t w = word_of(x, m);
-      const uint32_t lo4 = (w << 2) & 0x3C3C3C3Cu;  // byte j: 4 * low nibble of byte j of w
-      const uint32_t hi4 = (w >> 2) & 0x3C3C3C3Cu;  // byte j: 4 * high nibble of byte j of w
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t sel = 0x7650u | static_cast<uint32_t>(j);  // byte j of the offsets, bytes 1-3 of the frame
-        const float tlo = lds_lo(__byte_perm(lo4, frame, sel));
-        const float thi = lds_hi(__byte_perm(hi4, frame, sel));
-        acc[4 * m + j] = __fadd_rn(acc[4 * m + j], __fadd_rn(tlo, thi));
-      }
-    }
-  }
-}
-
-// Per-CTA prologue of the update kernels: a_k = fp32(coef_mul * c_k) for the
-// K probes (zero-padded to 8 * groups) and the per-quad partial-sum tables in
-// their frames. Returns false when the block has nothing to do (a failed
-// preconditioner and no leading perturbation); do_sum is false when only the
-// leading perturbation applies.
-__device__ __forceinline__ bool update_prologue(const UpdateParams& P, unsigned char* smem, int& skip,
-                                                uint32_t& lut_base, bool& do_sum) {
-  float* a_s = reinterpret_cast<float*>(smem);  // 8 * groups coefficients (zero padded)
-  const uint32_t smem_sh = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-  lut_base = (smem_sh + 32u * P.groups + kFrameBytes - 1) & ~(kFrameBytes - 1);
-  float* lut = reinterpret_cast<float*>(smem + (lut_base - smem_sh));  // generic view of the frames
-  if (threadIdx.x == 0) skip = (P.status != nullptr && *P.status != 0);
-  const int npad = 8 * P.groups;
-  for (int k = threadIdx.x; k < npad; k += blockDim.x)
-    a_s[k] = k < P.K ? __double2float_rn(P.coef_mul * P.coef[k]) : 0.0f;
-  __syncthreads();
-  if (skip && !P.has_pre) return false;
-  do_sum = !skip;  // a failed preconditioner still gets the leading perturbation
-  for (int e = threadIdx.x; e < 32 * P.groups; e += blockDim.x) {
-    const int h = e >> 4, n = e & 15;
-    const float* a = a_s + 4 * h;
-    float s = (n & 1) ? a[0] : -a[0];
-    s = __fadd_rn(s, (n & 2) ? a[1] : -a[1]);
-    s = __fadd_rn(s, (n & 4) ? a[2] : -a[2]);
-    s = __fadd_rn(s, (n & 8) ? a[3] : -a[3]);
-    lut[(h >> 1) * (kFrameBytes / 4) + (h & 1) * 16 + n] = s;
-  }
-  __syncthreads();
-  return true;
-}
-
-// ---------------------------------------------------------------------------
-// Fused update of unaligned tensors (kShift), in the 32-byte aligned chunks of
-// perturb_shift_kernel. Lane l sums the probes of block c = c0 - 1 + l (in
-// block order, exactly as update_kernel does) and takes the sums of block
-// c - 1 from lane l - 1; chunk c's sixteen sums are elements 16 - a .. 31 - a
-// of the two blocks' sums, so every element gets the same fp32 value as in
-// update_kernel.
-// ---------------------------------------------------------------------------
-template <uint8_t DT>
-__device__ __forceinline__ void update_shift_group(const UpdateParams& P, uint32_t lut_base, bool do_sum, int t,
-                                                   int64_t c_first) {
-  constexpr int kElem = DT == kF32 ? 4 : 2;
-  constexpr int kWords = 16 * kElem / 4;
-  const TensorTable& tab = P.tab;
-  const uintptr_t ptr = tab.ptr[t];
-  const int64_t n = tab.numel[t];
-  const uint32_t a = static_cast<uint32_t>(ptr & 31u) / kElem;
-  char* chunk0 = reinterpret_cast<char*>(ptr - (ptr & 31u));
-  const int64_t nchunks = (n + a + 15) / 16;
-  const int64_t vb0 = virtual_block(tab, t, tensor_blk_begin(tab, t));
-  const int lane = static_cast<int>(threadIdx.x & 31u);
-#pragma unroll 1
-  for (int s = 0; s < kShiftSub; ++s) {
-    const int64_t c = c_first + s * kShiftLanes + lane - 1;
-    const bool full = shift_full(lane, c, a, n);
-    char* q = chunk0 + c * (16 * kElem);
-    uint32_t v[kWords];
-    if (full) {  // issued before the probe sums, which hide its latency
-      ld256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-      if constexpr (DT == kF32) ld256(q + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[8]));
-    }
-    float own[16], below[16], sum[16];
-#pragma unroll
-    for (int m = 0; m < 16; ++m) own[m] = 0.0f;
-    if (do_sum) accumulate_block(own, vb0 + c, P, lut_base);
-#pragma unroll
-    for (int m = 0; m < 16; ++m) below[m] = __shfl_up_sync(0xffffffffu, own[m], 1);
-    window16f(below, own, 16u - a, sum);
-    uint4 y = make_uint4(0u, 0u, 0u, 0u);
-    if (P.has_pre) {
-      const uint4 xp = block_bits(vb0 + c, P.pre.ctr2, P.keys);
-      y = window16(shfl_up4(xp), xp, 16u - a);
-    }
-    if (full) {
-      if constexpr (DT == kF32) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float th = __uint_as_float(v[i]);
-          if (P.has_pre) th = add_signed(th, y, i, P.pre);
-          if (do_sum) th = __fadd_rn(th, sum[i]);
-          v[i] = __float_as_uint(th);
-        }
-        st256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-        st256(q + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[8]));
-      } else {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          if (P.has_pre) v[r] = pre_regs16<DT>(v[r], y, r, P.pre);
-          if (do_sum) {
-            const float2 f = unpack2<DT>(v[r]);
-            v[r] = pack2<DT>(__fadd_rn(f.x, sum[2 * r]), __fadd_rn(f.y, sum[2 * r + 1]));
-          }
-        }
-        st256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-      }
-    } else if (lane > 0 && c >= 0 && c < nchunks) {  // a chunk across an end of the tensor
-      void* base = reinterpret_cast<void*>(ptr);
-#pragma unroll
-      for (int p = 0; p < 16; ++p) {
-        const int64_t e = 16 * c - a + p;
-        if (e < 0 || e >= n) continue;
-        float th = load_elem(base, DT, e);
-        if (P.has_pre) th = round_to_storage(DT, add_signed(th, y, p, P.pre));
-        if (do_sum) th = __fadd_rn(th, sum[p]);
-        store_elem(base, DT, e, th);
-      }
-    }
-  }
-}
-
-template <uint8_t DT>
-__global__ void __launch_bounds__(256) update_shift_kernel(const __grid_constant__ UpdateShiftParams S) {
-  const UpdateParams& P = S.u;
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int skip;
-  uint32_t lut_base;
-  bool do_sum;
-  if (!update_prologue(P, smem, skip, lut_base, do_sum)) return;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  int t = 0;
-  for (uint32_t g = warp; g < S.grp_total; g += nwarps) {  // the same g on every lane of the warp
-    while (g >= S.grp_end[t]) ++t;
-    const int64_t c_first = static_cast<int64_t>(g - (t == 0 ? 0u : S.grp_end[t - 1])) * kShiftGroup;
-    update_shift_group<DT>(P, lut_base, do_sum, t, c_first);
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Debug views: probe k packed one bit per element (Appendix F layout) and the
 // unpacked int8 signs, over a range of the virtual index space.
 // ---------------------------------------------------------------------------
@@ -1004,9 +818,9 @@ cudaError_t launch_perturb(const PerturbParams& p, int grid, int loop, bool f32v
 }
 
 static_assert(sizeof(PairParams) <= 32764, "pair table exceeds the kernel parameter space");
-static_assert(sizeof(ShiftParams) <= 32764 && sizeof(UpdateShiftParams) <= 32764 && sizeof(PairShiftParams) <= 32764,
+static_assert(sizeof(ShiftParams) <= 32764 && sizeof(PairShiftParams) <= 32764,
               "shift table exceeds the kernel parameter space");
-static_assert(sizeof(PerturbParams) <= 32764 && sizeof(UpdateParams) <= 32764,
+static_assert(sizeof(PerturbParams) <= 32764 && sizeof(SmallUpdateParams) <= 32764,
               "tensor table exceeds the kernel parameter space");
 
 template <int NOPS>
@@ -1041,33 +855,10 @@ cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_update_shift(const UpdateShiftParams& p, uint8_t dt, int grid, cudaStream_t stream) {
-  const size_t smem = update_smem_bytes(p.u.groups);
-  if (dt == kBF16)
-    update_shift_kernel<kBF16><<<grid, kThreads, smem, stream>>>(p);
-  else if (dt == kF16)
-    update_shift_kernel<kF16><<<grid, kThreads, smem, stream>>>(p);
-  else
-    update_shift_kernel<kF32><<<grid, kThreads, smem, stream>>>(p);
-  return cudaGetLastError();
-}
-
-cudaError_t update_shift_blocks_per_sm(int groups, uint8_t dt, int* out) {
-  const size_t smem = update_smem_bytes(groups);
-  if (dt == kBF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kBF16>, kThreads, smem);
-  if (dt == kF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kF16>, kThreads, smem);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, update_shift_kernel<kF32>, kThreads, smem);
-}
-
 cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream) {
   perturb_pair_kernel<<<grid, kThreads, 0, stream>>>(p);
   return cudaGetLastError();
 }
-
-// Coefficients (32 bytes per group), alignment slack, one 256-byte frame per group.
-size_t update_smem_bytes(int groups) { return static_cast<size_t>(groups) * (32 + kFrameBytes) + kFrameBytes; }
 
 cudaError_t perturb_blocks_per_sm(int nops, int loop, int* out) {
   if (nops == 1)

@@ -10,9 +10,8 @@
 // and T_hi likewise for probes 8q+4..8q+7, holds the group's fp32 partial sum
 // for every sign byte n. An element adds one looked-up value per group, groups
 // in increasing order: one byte-permute (the address), one shared load and
-// half a packed fp32x2 add per eight probes. update_kernel adds exactly these
-// partials in this order (as two 4-probe lookups), so the two kernels give
-// the same bits.
+// half a packed fp32x2 add per eight probes. Both kernels of this file add these
+// partials in this order, so they give the same bits.
 //
 // Bank conflicts. 32 lanes looking up random bytes of one 256-entry table
 // would collide on the 32 shared-memory banks, so every lane reads its own
@@ -33,8 +32,8 @@
 // the next pair's tables into the other; one barrier per pair separates the
 // two. The sums live in tensor memory (TMEM) between pairs, so the chunk is
 // not limited by registers: per pair, each 64 KB table copy and its barrier
-// serve 4096 blocks. With one or two groups (update_lut8_small_kernel) the
-// first region holds them for the whole launch and there is no chunking.
+// serve 4096 blocks. With one or two groups (update_lut8_small_kernel) shared
+// memory holds them for the whole launch and there is no chunking.
 #include <type_traits>
 
 #include "zo_device.cuh"
@@ -60,34 +59,6 @@ __device__ __forceinline__ float quad_partial(const float* a, uint32_t i) {
   s = __fadd_rn(s, (i & 4u) ? a[2] : -a[2]);
   s = __fadd_rn(s, (i & 8u) ? a[3] : -a[3]);
   return s;
-}
-
-// Copy the tables of groups q (and q + 1 when `two`) into the two halves of a
-// region. Each thread owns the same 16-byte pieces (four lane copies) of 2048 /
-// THREADS rows in every table: row n = p * THREADS / 8 + tid / 8, piece tid mod
-// 8, so eight consecutive threads fill one half row (each quarter-warp store
-// covers 128 contiguous bytes) and every address is a per-thread base plus a
-// constant. All loads are issued before the first store.
-//   src_t  shared address of t8 + 4 * (tid / 8)
-//   dst_t  region + 256 * (tid / 8) + 16 * (tid mod 8)
-template <int THREADS>
-__device__ __forceinline__ void lut8_replicate(uint32_t src_t, uint32_t dst_t, int q, bool two) {
-  constexpr int S = 2048 / THREADS;                // rows per thread and table
-  constexpr uint32_t kRowStep = THREADS / 8;       // rows between a thread's pieces
-  float v0[S], v1[S];
-  const uint32_t s0 = src_t + static_cast<uint32_t>(q) * 1024u;
-#pragma unroll
-  for (int p = 0; p < S; ++p) v0[p] = lds_f32(s0 + p * kRowStep * 4u);
-  if (two) {
-#pragma unroll
-    for (int p = 0; p < S; ++p) v1[p] = lds_f32(s0 + 1024u + p * kRowStep * 4u);
-  }
-#pragma unroll
-  for (int p = 0; p < S; ++p) sts_f32x4(dst_t + p * kRowStep * 256u, v0[p]);
-  if (two) {
-#pragma unroll
-    for (int p = 0; p < S; ++p) sts_f32x4(dst_t + 128u + p * kRowStep * 256u, v1[p]);
-  }
 }
 
 // Add group q's partial of the 16 elements of a block (Philox output x) to acc,
@@ -230,8 +201,13 @@ __device__ __forceinline__ void zero16(float (&a)[16]) {
 // Copy the tables of groups q (and q + 1 when `two`) into the two halves of a
 // region, forming each entry T8[n] = T_lo[n & 15] + T_hi[n >> 4] from the
 // group's 16-entry 4-probe tables (t4: T_lo then T_hi, 32 floats per group).
-// Rows and pieces as in lut8_replicate; a thread's rows are 64 apart, so
-// n & 15 is the same in all of them.
+// Each thread owns the same 16-byte pieces (four lane copies) of 2048 / THREADS
+// rows in every table: row n = p * THREADS / 8 + tid / 8, piece tid mod 8, so
+// eight consecutive threads fill one half row (each quarter-warp store covers
+// 128 contiguous bytes) and every address is a per-thread base plus a constant;
+// a thread's rows are 64 apart, so n & 15 is the same in all of them. All loads
+// are issued before the first store.
+//   dst_t  region + 256 * (tid / 8) + 16 * (tid mod 8)
 template <int THREADS>
 __device__ __forceinline__ void lut8_replicate4(uint32_t t4, uint32_t dst_t, int q, bool two) {
   constexpr int S = 2048 / THREADS;
@@ -299,17 +275,12 @@ __device__ __forceinline__ Lut8Block lut8_block_info(const TensorTable& tab, int
 // every block) and once per block (BlockRound01, shared by the pair's two
 // groups); only their xors and rounds 2-9 are per (block, group). The output
 // equals philox10(b_lo, bhi, q, 0) bit for bit.
-struct GroupRound01 {
-  uint32_t x0;    // lo(M1 q) ^ k0[1]
-  uint32_t x2;    // hi(M0 u) ^ k1[1], u = hi(M1 q) ^ bhi ^ k0[0]
-  uint32_t lpa1;  // lo(M0 u)
-};
 struct BlockRound01 {
   uint32_t lpa0;  // lo(M0 b_lo)
   uint32_t hpb1;  // hi(M1 v), v = hi(M0 b_lo) ^ k1[0]
   uint32_t lpb1;  // lo(M1 v)
 };
-__device__ __forceinline__ GroupRound01 group_round01(uint32_t q, uint32_t bhi, const RoundKeys& rk) {
+__host__ __device__ __forceinline__ GroupRound01 group_round01(uint32_t q, uint32_t bhi, const RoundKeys& rk) {
   const uint64_t pb0 = static_cast<uint64_t>(kPhiloxM1) * q;
   const uint32_t u = static_cast<uint32_t>(pb0 >> 32) ^ bhi ^ rk.k0[0];
   const uint64_t pa1 = static_cast<uint64_t>(kPhiloxM0) * u;
@@ -722,7 +693,10 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
             else
               tm_get16(acc, ta);
           } else {
-            tm_ld16(acc, ta);
+            if (!HIU && pr == 0)
+              zero16(acc);
+            else
+              tm_ld16(acc, ta);
             if (AHEAD && j == 0)
               x = ahead;
             else
@@ -809,248 +783,357 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
 }
 
 // ---------------------------------------------------------------------------
-// One or two probe groups (K <= 16): both tables stay in the first region for
-// the whole launch, so there is no chunking and no barrier. The kernel walks
-// blocks grid-stride like the perturbation passes, the next block's 256-bit
-// load issued before the current block is computed, and every element takes
-// its one or two lookups and is stored at once: the same sums, in the same
-// order (0 + T8_0 [+ T8_1]), as the chunked kernel. The leading perturbation
-// reuses the Philox word of its own group when it is one of the two. The group
-// count and the leading perturbation's case are template arguments: with
-// 64 registers a thread (1024 threads), the run-time flags cost 7-14 % of
-// the time of this issue-bound loop.
+// One or two probe groups (K <= 16): the tables stay in shared memory for the
+// whole launch, so there is no chunking and no barrier. The kernel walks
+// 32-byte items of theta grid-stride like the perturbation passes (sixteen
+// 16-bit or eight fp32 elements, half a Philox block), the next item's 256-bit
+// load issued before the current one is computed: the same sums, in the same
+// order (0 + T8_0 [+ T8_1]), as the chunk kernel.
+//
+// At K <= 16 the bound is one pass over HBM, 379 cycles per warp and item at
+// 2.07 GHz, and what the SM has to issue in that time: two Philox calls cost
+// about 180 (a 32x32->64 multiply holds the issue for four), so the rest has
+// to be short:
+//  * Philox rounds 0-1 split as in the chunk kernel, the groups' parts from
+//    the host (parameter space, no registers);
+//  * group 0's table holds 0 + T8_0, so its addition to 0 is gone;
+//  * with the leading perturbation's probe in the last group (the fused
+//    schedule's restore of probe K - 1), that group's entries are pairs (T8,
+//    the signed scale): one 64-bit lookup gives both, in place of a multiply
+//    and a logic operation per element. Its sums are scalar adds: packed ones
+//    would need the two elements' halves moved into register pairs first
+//    (0.95 against 0.90 ms at K = 16, 1.00 against 0.79 ms at K = 8).
+// OPT-1.3B-shaped bf16 set (one pass at the copy bandwidth: 0.775 ms), with
+// the leading perturbation: K = 8 0.845 -> 0.787 ms, K = 16 0.941 -> 0.903 ms
+// (fp16 0.962 -> 0.880); without it 0.822 -> 0.780 and 0.880 -> 0.810 ms. fp32
+// and tensors off the 32-byte grid ran element by element or in a kernel of
+// their own before: 205 M fp32 weights, K = 16: 0.332 -> 0.260 ms; 400 M bf16
+// weights in one flat buffer, K = 16: 0.749 -> 0.381 ms. Not adopted: a
+// prefetch of the item after the next into L2 (K = 16 -2 %, K = 8 +10 %).
 // ---------------------------------------------------------------------------
 constexpr int kSmallThreads = 1024;
-size_t lut8_small_smem_bytes() { return 2 * static_cast<size_t>(kLut8Region) + 16u; }
+constexpr size_t small_smem_bytes(bool pairs_and_two) {
+  return (pairs_and_two ? 3 : 2) * static_cast<size_t>(kLut8Region) + 16u;
+}
 
+__device__ __forceinline__ void lds_pair(uint32_t addr, float& a, float& b) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(addr));
+}
+
+// Shared address of element i's entry: its sign byte in byte i mod 4 of w.
+template <int I>
+__device__ __forceinline__ uint32_t entry_addr(uint32_t w, uint32_t frame) {
+  return __byte_perm(w, frame, 0x7604u | (static_cast<uint32_t>(I & 3) << 4));
+}
+
+// The leading perturbation in the small kernel: none, in the last group's
+// table, or with Philox words of its own.
+constexpr int kPreNone = 0, kPreTable = 1, kPreOwn = 2;
+
+// Sum of element I (t), and with kPreTable its leading perturbation (d).
+template <int I, int PRE, bool TWO>
+__device__ __forceinline__ void small_sums(uint32_t w0, uint32_t wl, uint32_t f0, uint32_t fl, float& t0, float& tl,
+                                           float& d) {
+  if constexpr (TWO) t0 = lds_f32(entry_addr<I>(w0, f0));
+  if constexpr (PRE == kPreTable)
+    lds_pair(entry_addr<I>(wl, fl), tl, d);
+  else
+    tl = lds_f32(entry_addr<I>(wl, fl));
+}
+
+// Sixteen 16-bit elements. x0, xl: words of group 0 and of the last group.
+template <uint8_t DT, int PRE, bool TWO, int R>
+__device__ __forceinline__ void small_pair16(uint32_t& v, const uint4& x0, const uint4& xl, const uint4& xp,
+                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
+  constexpr int e = 2 * R;
+  float2 f = unpack2<DT>(v);
+  float a0 = 0.0f, a1 = 0.0f, l0, l1, d0 = 0.0f, d1 = 0.0f;
+  small_sums<e, PRE, TWO>(word_of(x0, e >> 2), word_of(xl, e >> 2), f0, fl, a0, l0, d0);
+  small_sums<e + 1, PRE, TWO>(word_of(x0, e >> 2), word_of(xl, e >> 2), f0, fl, a1, l1, d1);
+  if constexpr (PRE != kPreNone) {
+    if constexpr (PRE == kPreTable) {
+      f.x = __fadd_rn(f.x, d0);
+      f.y = __fadd_rn(f.y, d1);
+    } else {
+      add_signed2(f, xp, e, P.pre);
+    }
+    f = unpack2<DT>(pack2<DT>(f.x, f.y));  // the perturbed value is rounded to storage first
+  }
+  if constexpr (PRE == kPreTable) {
+    if constexpr (TWO) {
+      l0 = __fadd_rn(a0, l0);
+      l1 = __fadd_rn(a1, l1);
+    }
+    f.x = __fadd_rn(f.x, l0);
+    f.y = __fadd_rn(f.y, l1);
+  } else if constexpr (TWO) {
+    fadd2_rn(a0, a1, l0, l1);
+    fadd2_rn(f.x, f.y, a0, a1);
+  } else {
+    fadd2_rn(f.x, f.y, l0, l1);
+  }
+  v = pack2<DT>(f.x, f.y);
+}
+
+template <uint8_t DT, int PRE, bool TWO>
+__device__ __forceinline__ void small_item16(uint32_t (&v)[8], const uint4& x0, const uint4& xl, const uint4& xp,
+                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
+  small_pair16<DT, PRE, TWO, 0>(v[0], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 1>(v[1], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 2>(v[2], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 3>(v[3], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 4>(v[4], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 5>(v[5], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 6>(v[6], x0, xl, xp, f0, fl, P);
+  small_pair16<DT, PRE, TWO, 7>(v[7], x0, xl, xp, f0, fl, P);
+}
+
+// One fp32 element (scalar adds, as every fp32 path).
+template <int PRE, bool TWO, int I>
+__device__ __forceinline__ void small_one32(uint32_t& v, const uint4& x0, const uint4& xl, const uint4& xp, uint32_t f0,
+                                            uint32_t fl, const UpdateParams& P) {
+  float th = __uint_as_float(v);
+  float a = 0.0f, l, d = 0.0f;
+  small_sums<I, PRE, TWO>(word_of(x0, I >> 2), word_of(xl, I >> 2), f0, fl, a, l, d);
+  if constexpr (PRE == kPreTable) th = __fadd_rn(th, d);
+  if constexpr (PRE == kPreOwn) th = add_signed(th, xp, I, P.pre);
+  v = __float_as_uint(__fadd_rn(th, TWO ? __fadd_rn(a, l) : l));
+}
+
+template <int PRE, bool TWO>
+__device__ __forceinline__ void small_item32(uint32_t (&v)[8], const uint4& x0, const uint4& xl, const uint4& xp,
+                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
+  small_one32<PRE, TWO, 0>(v[0], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 1>(v[1], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 2>(v[2], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 3>(v[3], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 4>(v[4], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 5>(v[5], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 6>(v[6], x0, xl, xp, f0, fl, P);
+  small_one32<PRE, TWO, 7>(v[7], x0, xl, xp, f0, fl, P);
+}
+
+// An item across an end of its tensor, element by element (not inlined: it
+// is rare and would otherwise hold registers in the loop). e0: the item's
+// first element; do_sum false: the leading perturbation alone.
+template <int PRE, bool TWO, bool ANY>
+__device__ __noinline__ void small_elements(void* base, uint8_t dt, int64_t e0, int64_t numel, uint4 x0, uint4 xl,
+                                            uint4 xp, uint32_t f0, uint32_t fl, bool do_sum, PerturbOp pre) {
+  const int per = dt == kF32 ? 8 : 16;
+#pragma unroll 1
+  for (int i = 0; i < per; ++i) {
+    const int64_t e = e0 + i;
+    if (e < 0 || e >= numel) continue;
+    const uint32_t sel = 0x7604u | (static_cast<uint32_t>(i & 3) << 4);
+    float th = load_elem(base, dt, e);
+    float a = 0.0f, l = 0.0f, d = 0.0f;
+    if (do_sum) {
+      if constexpr (TWO) a = lds_f32(__byte_perm(word_of(x0, i >> 2), f0, sel));
+      const uint32_t at = __byte_perm(word_of(xl, i >> 2), fl, sel);
+      if constexpr (PRE == kPreTable)
+        lds_pair(at, l, d);
+      else
+        l = lds_f32(at);
+    }
+    if (PRE != kPreNone) {
+      th = do_sum && PRE == kPreTable ? __fadd_rn(th, d) : add_signed(th, xp, i, pre);
+      th = round_to_storage(dt, th);
+    }
+    if (do_sum) th = __fadd_rn(th, TWO ? __fadd_rn(a, l) : l);
+    store_elem(base, dt, e, th);
+  }
+}
+
+// A warp's position in the table: its 32 items lie in one tensor.
 struct SmallCursor {
   int t;
-  uint32_t tb, te, n16;  // first and one-past-last launch block; full aligned 16-bit blocks from tb
-  uint32_t vd;           // launch block minus virtual block offset
-  uint16_t* tp;
-  uint8_t dt;
+  uint32_t tb, te;   // first and one-past-last launch item
+  uint32_t full;     // full aligned items from tb (0: tensors off the 32-byte grid)
+  uint32_t vb;       // low word of the virtual block of the tensor's first element
+  char* p;           // base pointer
+  uint8_t fl;        // flags
+  uint32_t a;        // kShift: the base's offset from the 32-byte boundary below it, in elements
 };
 
+template <bool ANY>
 __device__ __forceinline__ void small_seek(const TensorTable& tab, SmallCursor& c, uint32_t b) {
   c.t = advance_tensor(tab, c.t, b);
   c.tb = tensor_blk_begin(tab, c.t);
   c.te = tab.blk_end[c.t];
-  const uint8_t fl = tab.flags[c.t];
-  c.dt = fl & kDtypeMask;
-  c.n16 = ((fl & kVec32) && c.dt != kF32) ? static_cast<uint32_t>(tab.numel[c.t] / 16) : 0u;
-  c.vd = tab.vdelta[c.t];
-  c.tp = reinterpret_cast<uint16_t*>(tab.ptr[c.t]);
+  c.fl = tab.flags[c.t];
+  c.p = reinterpret_cast<char*>(tab.ptr[c.t]);
+  c.vb = static_cast<uint32_t>(static_cast<uint64_t>(virtual_block(tab, c.t, c.tb)));
+  const bool f32 = ANY && (c.fl & kDtypeMask) == kF32;
+  c.full = (c.fl & kVec32) ? static_cast<uint32_t>(tab.numel[c.t] / (f32 ? 8 : 16)) : 0u;
+  c.a = ANY ? static_cast<uint32_t>(tab.ptr[c.t] & 31u) / (f32 ? 4u : 2u) : 0u;
 }
 
-// Sums of elements e and e + 1 (e even) of a block, 0 + T8_0 [+ T8_1] each,
-// from the Philox words of groups 0 and 1, two elements per packed add.
-template <int E>
-__device__ __forceinline__ float2 small_sum2(const uint4& x0, const uint4& x1, uint32_t frame, bool two) {
-  constexpr uint32_t sel0 = 0x7604u | (static_cast<uint32_t>(E & 3) << 4);
-  constexpr uint32_t sel1 = 0x7604u | (static_cast<uint32_t>((E + 1) & 3) << 4);
-  float lo = 0.0f, hi = 0.0f;
-  const uint32_t w0 = word_of(x0, E >> 2);
-  fadd2_rn(lo, hi, lds_f32(__byte_perm(w0, frame, sel0)), lds_f32(__byte_perm(w0, frame, sel1)));
-  if (two) {
-    const uint32_t w1 = word_of(x1, E >> 2);
-    fadd2_rn(lo, hi, lds_f32(__byte_perm(w1, frame | 128u, sel0)), lds_f32(__byte_perm(w1, frame | 128u, sel1)));
-  }
-  return make_float2(lo, hi);
-}
-
-template <uint8_t DT, bool TWO>
-__device__ __forceinline__ void small_block16(uint32_t (&v)[8], const uint4& x0, const uint4& x1, const uint4& xp,
-                                              uint32_t frame, bool pre, const UpdateParams& P, bool do_sum) {
-  constexpr bool two = TWO;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    float2 f = unpack2<DT>(v[r]);
-    if (pre) {
-      add_signed2(f, xp, 2 * r, P.pre);
-      v[r] = pack2<DT>(f.x, f.y);  // the perturbed value is rounded to storage first
-      f = unpack2<DT>(v[r]);
-    }
-    if (do_sum) {
-      float2 acc;
-      switch (r) {  // element indices must be constants for the word and byte selects
-        case 0: acc = small_sum2<0>(x0, x1, frame, two); break;
-        case 1: acc = small_sum2<2>(x0, x1, frame, two); break;
-        case 2: acc = small_sum2<4>(x0, x1, frame, two); break;
-        case 3: acc = small_sum2<6>(x0, x1, frame, two); break;
-        case 4: acc = small_sum2<8>(x0, x1, frame, two); break;
-        case 5: acc = small_sum2<10>(x0, x1, frame, two); break;
-        case 6: acc = small_sum2<12>(x0, x1, frame, two); break;
-        default: acc = small_sum2<14>(x0, x1, frame, two); break;
-      }
-      fadd2_rn(f.x, f.y, acc.x, acc.y);
-      v[r] = pack2<DT>(f.x, f.y);
-    }
-  }
-}
-
-// A block of the launch outside the vector loop.
-struct SmallBlock {
-  int64_t b;       // virtual block (Philox counter)
-  int64_t e0;      // first element inside its tensor
-  void* base;      // tensor base pointer
-  int cnt;         // elements of the block (1..16)
-  uint8_t fl;      // tensor flags
+// A lane's item. Tensors off the 32-byte grid (kShift): each warp takes 31 of
+// their aligned 32-byte chunks, lane l the chunk 31 w + l - 1 and the signs of
+// the elements that fall into the block (fp32: half block) below from lane
+// l - 1; lane 0 only generates.
+struct SmallItem {
+  char* p;        // the item's address (full)
+  uint32_t blk;   // low word of the Philox block it generates
+  int64_t e0;     // its first element
+  bool upper;     // fp32: the block's upper half
+  bool full;      // all its elements exist, 32-byte aligned
+  bool act;       // some do
 };
 
-// Apply the leading perturbation (if any) and the probe sums to a block that
-// is not a full, aligned 16-bit one: fp32 blocks and partial last blocks.
-__device__ __forceinline__ void small_apply_other(const SmallBlock& k, const float (&acc)[16], const UpdateParams& P,
-                                              bool do_sum) {
-  uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-  if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
-  const uint8_t dt = k.fl & kDtypeMask;
-  if (dt == kF32 && k.cnt == 16 && (k.fl & kVec32)) {
-    float* p = static_cast<float*>(k.base) + k.e0;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t v[8];
-      ld256(p + 8 * half, v);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        float th = __uint_as_float(v[r]);
-        if (P.has_pre) th = add_signed(th, xp, 8 * half + r, P.pre);
-        if (do_sum) th = __fadd_rn(th, acc[8 * half + r]);
-        v[r] = __float_as_uint(th);
-      }
-      st256(p + 8 * half, v);
-    }
-    return;
+template <bool ANY>
+__device__ __forceinline__ SmallItem small_item(const TensorTable& tab, const SmallCursor& c, uint32_t b) {
+  SmallItem k;
+  const uint32_t d = b - c.tb;
+  if constexpr (!ANY) {
+    k.full = d < c.full;
+    k.act = b < c.te;
+    k.p = c.p + static_cast<size_t>(d) * 32;
+    k.blk = c.vb + d;
+    k.e0 = static_cast<int64_t>(d) * 16;
+    k.upper = false;
+  } else {
+    const bool f32 = (c.fl & kDtypeMask) == kF32;
+    const int per = f32 ? 8 : 16;
+    int64_t i = d;  // item number inside the tensor
+    if (c.fl & kShift) i = static_cast<int64_t>(d >> 5) * kShiftLanes + static_cast<int64_t>(d & 31u) - 1;
+    k.e0 = i * per - c.a;
+    const int64_t numel = tab.numel[c.t];
+    k.act = (c.fl & kShift) ? (d & 31u) != 0u && k.e0 < numel : b < c.te;
+    k.full = k.act && k.e0 >= 0 && k.e0 + per <= numel;
+    k.p = c.p + k.e0 * (f32 ? 4 : 2);
+    k.blk = c.vb + static_cast<uint32_t>(static_cast<uint64_t>(f32 ? i >> 1 : i));
+    k.upper = f32 && (i & 1) != 0;
   }
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    if (i < k.cnt) {
-      float th = load_elem(k.base, dt, k.e0 + i);
-      if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
-      if (do_sum) th = __fadd_rn(th, acc[i]);
-      store_elem(k.base, dt, k.e0 + i, th);
-    }
-  }
+  return k;
 }
 
-// Any other block of the launch: fp32, a partial last block, padding, or an
-// unaligned tensor (update_shift_kernel's).
-template <int TAG>
-__device__ __noinline__ void small_block_other(const TensorTable& tab, int t, uint32_t b, const UpdateParams& P,
-                                               uint32_t frame, bool do_sum) {
-  const uint32_t tb = tensor_blk_begin(tab, t);
-  const uint8_t fl = tab.flags[t];
-  if ((fl & kShift) || b < tb) return;
-  SmallBlock k;
-  k.b = virtual_block(tab, t, b);
-  k.e0 = static_cast<int64_t>(b - tb) * 16;
-  k.cnt = static_cast<int>(min(static_cast<int64_t>(16), tab.numel[t] - k.e0));
-  k.base = reinterpret_cast<void*>(tab.ptr[t]);
-  k.fl = fl;
-  float acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
-  if (do_sum) {
-    lut8_lookup(acc, block_bits(k.b, 0u, P.keys), frame);
-    if (P.groups > 1) lut8_lookup(acc, block_bits(k.b, 1u, P.keys), frame | 128u);
+// The sign words of an item's elements from its block's Philox words.
+__device__ __forceinline__ uint4 small_window(const SmallCursor& c, const SmallItem& k, uint4 x) {
+  if ((c.fl & kDtypeMask) == kF32) {  // the same in all lanes
+    uint2 y = k.upper ? make_uint2(x.z, x.w) : make_uint2(x.x, x.y);
+    if (c.fl & kShift) {  // bytes 8 - a .. 15 - a of (the half below) ++ (this half), a = 1..7
+      const uint32_t b0 = __shfl_up_sync(0xFFFFFFFFu, y.x, 1), b1 = __shfl_up_sync(0xFFFFFFFFu, y.y, 1);
+      const uint32_t s = 8u - c.a, sh = 8u * (s & 3u);
+      const uint32_t w0 = s >= 4u ? b1 : b0, w1 = s >= 4u ? y.x : b1, w2 = s >= 4u ? y.y : y.x;
+      y = make_uint2(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh));
+    }
+    return make_uint4(y.x, y.y, 0u, 0u);
   }
-  small_apply_other(k, acc, P, do_sum);
+  return (c.fl & kShift) ? window16(shfl_up4(x), x, 16u - c.a) : x;
 }
 
-// Leading perturbation of the small kernel's instantiations: on a Philox word
-// the sums also use (group 0 or 1), on its own word, or decided at run time
-// (no leading perturbation, or any).
-constexpr int kPreShared = 1, kPreOwn = 2, kPreRuntime = 3;
-
-template <int PRE, bool TWO>
-__global__ void __launch_bounds__(kSmallThreads, 1) update_lut8_small_kernel(const __grid_constant__ UpdateParams P) {
+// ANY: the launch may hold fp32 tensors (numbered in half blocks) and tensors
+// off the 32-byte grid (32 launch items per 31 chunks).
+template <int PRE, bool TWO, bool ANY>
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    update_lut8_small_kernel(const __grid_constant__ SmallUpdateParams S) {
+  const UpdateParams& P = S.u;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
-  const int G = P.groups;  // 1 or 2
+  constexpr int G = TWO ? 2 : 1;
+  constexpr uint32_t kRegions = TWO && PRE == kPreTable ? 2u : 1u;
   const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
   const uint32_t region0 = (sbase + kLut8Region - 1u) & ~(kLut8Region - 1u);
   // coefficients and unreplicated tables (2 KB at most) below the region, or after it when the window starts on
   // a 64 KB boundary
-  const uint32_t hdr = region0 - sbase >= 32u * G + 1024u * G ? sbase : region0 + kLut8Region;
+  const uint32_t hdr = region0 - sbase >= 32u * G + 1024u * G ? sbase : region0 + kRegions * kLut8Region;
   float* a_s = reinterpret_cast<float*>(smem + (hdr - sbase));
   float* t8 = a_s + 8 * G;
   if (threadIdx.x == 0) skip_s = (P.status != nullptr && *P.status != 0);
   for (int k = threadIdx.x; k < 8 * G; k += kSmallThreads)
     a_s[k] = k < P.K ? __double2float_rn(P.coef_mul * P.coef[k]) : 0.0f;
   __syncthreads();
-  const bool skip = skip_s != 0;
-  const bool has_pre = PRE == kPreRuntime ? P.has_pre : true;
-  if (skip && !has_pre) return;
-  const bool do_sum = !skip;
+  const bool do_sum = skip_s == 0;  // a failed preconditioner still gets the leading perturbation
+  if (!do_sum && PRE == kPreNone) return;
   if (do_sum) {
     for (int e = threadIdx.x; e < 256 * G; e += kSmallThreads) {
       const float* a = a_s + 8 * (e >> 8);
       const uint32_t n = static_cast<uint32_t>(e) & 255u;
-      t8[e] = __fadd_rn(quad_partial(a, n & 15u), quad_partial(a + 4, n >> 4));
+      const float v = __fadd_rn(quad_partial(a, n & 15u), quad_partial(a + 4, n >> 4));
+      t8[e] = e < 256 ? __fadd_rn(0.0f, v) : v;
     }
     __syncthreads();
-    const uint32_t src_t = hdr + 32u * G + 4u * (threadIdx.x >> 3);
-    const uint32_t dst_t = 256u * (threadIdx.x >> 3) + 16u * (threadIdx.x & 7u);
-    lut8_replicate<kSmallThreads>(src_t, region0 + dst_t, 0, G > 1);
+    // rows of 256 bytes. Pairs: (T8, signed scale) of the last group, lane l in 8-byte word l; plain tables: lane
+    // l in word l of the first (group 0, or the only group) or second (group 1) half of the row
+    constexpr int kPieces = 256 * 16;  // 16-byte pieces of a region
+    for (int i = threadIdx.x; i < kPieces; i += kSmallThreads) {
+      const uint32_t n = static_cast<uint32_t>(i) >> 4, piece = static_cast<uint32_t>(i) & 15u;
+      const uint32_t row = region0 + 256u * n + 16u * piece;
+      if constexpr (PRE == kPreTable) {
+        const float v = t8[256 * (G - 1) + n];
+        const float d = __uint_as_float(P.pre.nscale_bits ^ (((n >> P.pre.bit) & 1u) << 31));
+        const uint32_t at = row + (kRegions - 1u) * kLut8Region;
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" ::"r"(at), "f"(v), "f"(d) : "memory");
+        if (TWO && piece < 8u) sts_f32x4(row, t8[n]);
+      } else {
+        if (piece < 8u || TWO) sts_f32x4(row, t8[(piece < 8u ? 0 : 256) + n]);
+      }
+    }
     __syncthreads();
   }
   const TensorTable& tab = P.tab;
   const uint32_t total = tab.blk_total;
   const uint32_t stride = gridDim.x * kSmallThreads;
-  const uint32_t frame = (region0 & 0xFFFF0000u) | ((threadIdx.x & 31u) << 2);
-  constexpr bool two = TWO;
-  // the leading perturbation's Philox word: group 0's, group 1's, or its own
-  // the leading perturbation's Philox word: none (-1), group 0's or group 1's (0, 1), or its own (2)
-  const int pre_src = PRE == kPreOwn ? 2
-                      : PRE == kPreShared ? (P.pre.ctr2 == 1u ? 1 : 0)
-                      : (!P.has_pre ? -1 : (P.pre.ctr2 == 0u ? 0 : (P.pre.ctr2 == 1u && two ? 1 : 2)));
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t f0 = (region0 & 0xFFFF0000u) | (lane << 2);
+  const uint32_t fl = PRE == kPreTable ? ((region0 + (kRegions - 1u) * kLut8Region) & 0xFFFF0000u) | (lane << 3)
+                                       : (TWO ? f0 | 128u : f0);
   uint32_t b = blockIdx.x * kSmallThreads + threadIdx.x;
-  if (b >= total) return;
+  if (b - lane >= total) return;
   SmallCursor c;
   c.t = 0;
-  small_seek(tab, c, b);
-  int t = c.t;
-  uint8_t dt = c.dt;
-  uint32_t vd = c.vd;
-  bool fast = b - c.tb < c.n16;
-  uint16_t* p = c.tp + static_cast<size_t>(b - c.tb) * 16;
+  small_seek<ANY>(tab, c, b - lane);
+  if (!do_sum) {
+    for (; b - lane < total; b += stride) {
+      if (b - lane >= c.te) small_seek<ANY>(tab, c, b - lane);
+      const SmallItem k = small_item<ANY>(tab, c, b);
+      const BlockCounter<true> kb(k.blk, 0, P.keys);
+      uint4 xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
+      if (ANY) xp = small_window(c, k, xp);
+      if (k.act) small_elements<PRE, TWO, ANY>(c.p, c.fl & kDtypeMask, k.e0, tab.numel[c.t], xp, xp, xp, f0, fl, false, P.pre);
+    }
+    return;
+  }
+  SmallItem k = small_item<ANY>(tab, c, b);
   uint32_t v[8];
-  if (fast) ld256(p, v);
+  if (k.full) ld256(k.p, v);
   while (true) {
     const uint32_t bn = b + stride;
-    bool fastn = false;
-    uint16_t* pn = nullptr;
+    const bool more = bn - lane < total;
+    SmallCursor cn = c;
+    SmallItem kn = k;
     uint32_t vn[8];
-    if (bn < total) {
-      if (bn >= c.te) small_seek(tab, c, bn);
-      fastn = bn - c.tb < c.n16;
-      pn = c.tp + static_cast<size_t>(bn - c.tb) * 16;
-      if (fastn) ld256(pn, vn);
+    if (more) {
+      if (bn - lane >= c.te) small_seek<ANY>(tab, cn, bn - lane);
+      kn = small_item<ANY>(tab, cn, bn);
+      if (kn.full) ld256(kn.p, vn);
     }
-    if (fast) {
-      const int64_t vb = tab.blk_base + (b - vd);
-      uint4 x0 = make_uint4(0u, 0u, 0u, 0u), x1 = x0, xp = x0;
-      if (do_sum || pre_src == 0 || pre_src == 1) {
-        x0 = block_bits(vb, 0u, P.keys);
-        if (two) x1 = block_bits(vb, 1u, P.keys);
-      }
-      if (pre_src == 0) xp = x0;
-      if (pre_src == 1) xp = x1;
-      if (pre_src == 2) xp = block_bits(vb, P.pre.ctr2, P.keys);
-      if (dt == kBF16)
-        small_block16<kBF16, TWO>(v, x0, x1, xp, frame, has_pre, P, do_sum);
+    const BlockCounter<true> kb(k.blk, 0, P.keys);
+    uint4 x0 = philox_finish(kb.start(S.g[0], 0u, P.keys), P.keys);
+    uint4 xl = TWO ? philox_finish(kb.start(S.g[1], 1u, P.keys), P.keys) : x0;
+    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+    if (PRE == kPreOwn) xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
+    if (ANY) {
+      x0 = small_window(c, k, x0);
+      xl = TWO ? small_window(c, k, xl) : x0;
+      if (PRE == kPreOwn) xp = small_window(c, k, xp);
+    }
+    if (k.full) {
+      if (ANY && (c.fl & kDtypeMask) == kF32)
+        small_item32<PRE, TWO>(v, x0, xl, xp, f0, fl, P);
+      else if ((c.fl & kDtypeMask) == kBF16)
+        small_item16<kBF16, PRE, TWO>(v, x0, xl, xp, f0, fl, P);
       else
-        small_block16<kF16, TWO>(v, x0, x1, xp, frame, has_pre, P, do_sum);
-      st256(p, v);
-    } else {
-      small_block_other<2 * PRE + TWO>(tab, t, b, P, frame, do_sum);
+        small_item16<kF16, PRE, TWO>(v, x0, xl, xp, f0, fl, P);
+      st256(k.p, v);
+    } else if (k.act) {
+      small_elements<PRE, TWO, ANY>(c.p, c.fl & kDtypeMask, k.e0, tab.numel[c.t], x0, xl, xp, f0, fl, true, P.pre);
     }
-    if (bn >= total) break;
+    if (!more) break;
     b = bn;
-    t = c.t;
-    dt = c.dt;
-    vd = c.vd;
-    fast = fastn;
-    p = pn;
+    c = cn;
+    k = kn;
 #pragma unroll
     for (int r = 0; r < 8; ++r) v[r] = vn[r];
   }
@@ -1073,17 +1156,25 @@ cudaError_t lut8_limit() {
 }
 
 
+template <int PRE, bool TWO, bool ANY>
+cudaError_t small_limit() {
+  return cudaFuncSetAttribute(update_lut8_small_kernel<PRE, TWO, ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(small_smem_bytes(TWO && PRE == kPreTable)));
+}
+
+template <int PRE>
+cudaError_t small_limits() {
+  cudaError_t e = small_limit<PRE, false, false>();
+  if (e == cudaSuccess) e = small_limit<PRE, true, false>();
+  if (e == cudaSuccess) e = small_limit<PRE, false, true>();
+  if (e == cudaSuccess) e = small_limit<PRE, true, true>();
+  return e;
+}
+
 cudaError_t lut8_prepare() {
-  const int lim = static_cast<int>(lut8_small_smem_bytes());
-  cudaError_t e = cudaSuccess;
-  const void* kernels[] = {reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, false>),
-                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreShared, true>),
-                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, false>),
-                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreOwn, true>),
-                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, false>),
-                           reinterpret_cast<const void*>(update_lut8_small_kernel<kPreRuntime, true>)};
-  for (const void* k : kernels)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaError_t e = small_limits<kPreNone>();
+  if (e == cudaSuccess) e = small_limits<kPreTable>();
+  if (e == cudaSuccess) e = small_limits<kPreOwn>();
   if (e == cudaSuccess) e = lut8_limit<2, true, false, false>();
   if (e == cudaSuccess) e = lut8_limit<4, true, false, false>();
   if (e == cudaSuccess) e = lut8_limit<8, true, false, false>();
@@ -1117,38 +1208,52 @@ cudaError_t launch_lut8_any(const UpdateParams& p, int bpt, int sms, cudaStream_
   }
 }
 
-cudaError_t launch_update_lut8_small(const UpdateParams& p, int sms, cudaStream_t stream) {
-  const int64_t want = (static_cast<int64_t>(p.tab.blk_total) + kSmallThreads - 1) / kSmallThreads;
-  const int g = static_cast<int>(want < sms ? want : sms);
-  const size_t sm = lut8_small_smem_bytes();
-  // with a leading perturbation: its Philox word one of the sums' or its own;
-  // without one, the run-time instantiation (faster there: its registers are
-  // laid out for the leading perturbation and it does not spill)
-  const bool two = p.groups == 2;
-  const int pre =
-      !p.has_pre ? kPreRuntime : (p.pre.ctr2 == 0u || (p.pre.ctr2 == 1u && two) ? kPreShared : kPreOwn);
-  if (pre == kPreShared && two)
-    update_lut8_small_kernel<kPreShared, true><<<g, kSmallThreads, sm, stream>>>(p);
-  else if (pre == kPreShared)
-    update_lut8_small_kernel<kPreShared, false><<<g, kSmallThreads, sm, stream>>>(p);
-  else if (pre == kPreOwn && two)
-    update_lut8_small_kernel<kPreOwn, true><<<g, kSmallThreads, sm, stream>>>(p);
-  else if (pre == kPreOwn)
-    update_lut8_small_kernel<kPreOwn, false><<<g, kSmallThreads, sm, stream>>>(p);
-  else if (two)
-    update_lut8_small_kernel<kPreRuntime, true><<<g, kSmallThreads, sm, stream>>>(p);
+bool one_high_word(const TensorTable& tab) {
+  // every virtual block that a lane sums lies in [blk_base, blk_base + blk_total), except the one below a
+  // tensor's first chunk, whose sums nothing uses
+  const uint64_t first = static_cast<uint64_t>(tab.blk_base);
+  const uint64_t last = first + (tab.blk_total > 0 ? tab.blk_total - 1u : 0u);
+  return (first >> 32) == (last >> 32);
+}
+
+template <int PRE, bool TWO>
+void launch_small_cfg(const SmallUpdateParams& p, bool any, int grid, cudaStream_t stream) {
+  constexpr size_t sm = small_smem_bytes(TWO && PRE == kPreTable);
+  if (any)
+    update_lut8_small_kernel<PRE, TWO, true><<<grid, kSmallThreads, sm, stream>>>(p);
   else
-    update_lut8_small_kernel<kPreRuntime, false><<<g, kSmallThreads, sm, stream>>>(p);
+    update_lut8_small_kernel<PRE, TWO, false><<<grid, kSmallThreads, sm, stream>>>(p);
+}
+
+template <int PRE>
+void launch_small_pre(const SmallUpdateParams& p, bool any, int grid, cudaStream_t stream) {
+  if (p.u.groups == 2)
+    launch_small_cfg<PRE, true>(p, any, grid, stream);
+  else
+    launch_small_cfg<PRE, false>(p, any, grid, stream);
+}
+
+cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream) {
+  const UpdateParams& u = p.u;
+  const uint32_t bhi = static_cast<uint32_t>(static_cast<uint64_t>(u.tab.blk_base) >> 32);
+  p.g[0] = group_round01(0u, bhi, u.keys);
+  p.g[1] = group_round01(1u, bhi, u.keys);
+  p.gp = group_round01(u.pre.ctr2, bhi, u.keys);
+  const int64_t want = (static_cast<int64_t>(u.tab.blk_total) + kSmallThreads - 1) / kSmallThreads;
+  const int grid = static_cast<int>(want < sms ? want : sms);
+  if (!u.has_pre)
+    launch_small_pre<kPreNone>(p, any, grid, stream);
+  else if (u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups))
+    launch_small_pre<kPreTable>(p, any, grid, stream);
+  else
+    launch_small_pre<kPreOwn>(p, any, grid, stream);
   return cudaGetLastError();
 }
 
 cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream) {
   const bool pack8 = p.packing == kPacking8;
-  // every virtual block that a lane sums lies in [blk_base, blk_base + blk_total), except the one below a
-  // tensor's first chunk, whose sums nothing uses
-  const uint64_t first = static_cast<uint64_t>(p.tab.blk_base);
-  const uint64_t last = first + (p.tab.blk_total > 0 ? p.tab.blk_total - 1u : 0u);
-  if ((first >> 32) != (last >> 32))
+  // a launch of one or two groups comes here when the small kernel cannot take it: rare, on the general form
+  if (!one_high_word(p.tab) || (!pack8 && p.groups <= 2))
     return pack8 ? launch_lut8_cfg<8, false, true, true>(p, sms, stream)
                  : launch_lut8_cfg<8, false, true, false>(p, sms, stream);
   const int bpt = lut8_bpt(p.tab.blk_total, sms);
