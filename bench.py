@@ -112,8 +112,8 @@ def measured_peaks():
 # The sources each kernel is compiled from: a traffic figure stays valid
 # while they are unchanged.
 KERNEL_SOURCES = {
-    "perturb_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
-    "perturb2_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
+    "perturb_items_kernel<1>": ("zo_device.cuh", "zo_stream_kernels.cu"),
+    "perturb_items_kernel<2>": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "perturb_pair_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "update_lut8_kernel": ("zo_device.cuh", "zo_update_lut8.cu"),
 }
@@ -568,7 +568,7 @@ def run_tiny(args):
     ms_per_step = max_over_ranks(sum(a_.elapsed_time(b_) for a_, b_ in ev) / args.steps, world, dev)
     launches = q.library_launches_per_step()
     if schedule == "onepass":
-        calls = 2 * K + 1 + 2                                                # C-ABI calls per step
+        calls = 3                                                            # C-ABI calls per step
     else:
         calls = 2 * K + 1 + (2 * K if schedule == "fused" else 3 * K) + 2
     host_us_per_call = 1e6 * statistics.median(host_s) / calls
@@ -616,10 +616,10 @@ def run_tiny(args):
     peaks, peak_kind = measured_peaks()
     hbm_peak = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     # bytes the step must move: each weight pass reads and writes theta, each
-    # loss reads theta and a (onepass: a pass that perturbs and evaluates
-    # reads theta and a and writes theta)
+    # loss reads theta and a (onepass: one launch reads theta and a and writes
+    # theta for all forward points, then the update)
     if schedule == "onepass":
-        step_bytes = 2 * K * 3 * d * 4 + 2 * d * 4 + 2 * d * 4
+        step_bytes = 3 * d * 4 + 2 * d * 4
     else:
         passes = 2 * K + 1 if schedule == "fused" else 3 * K + 1
         step_bytes = passes * 2 * d * 4 + (2 * K + 1) * 2 * d * 4
@@ -763,7 +763,7 @@ def run_zo(args):
     K, eps, d = ps.K, ps.eps, ps.d
     params = W.allocate_params(ps, device=dev, view_offset=args.view_offset)
     plist = zo.ParamList(params)
-    shifted = any(t.data_ptr() % 32 for t in params)   # the perturbation passes use perturb_shift_kernel
+    shifted = any(t.data_ptr() % 32 for t in params)   # the pair pass uses pair_shift_kernel
 
     def like_param(t):
         """A buffer for theta +- eps z_k laid out like t (same offset into its own allocation)."""
@@ -777,7 +777,7 @@ def run_zo(args):
     c = torch.empty(K, dtype=torch.float64, device=dev)
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     stream = torch.cuda.current_stream(dev)
-    chunks = (len(params) + 1023) // 1024
+    chunks = (len(params) + 959) // 960   # tensors per launch
     pp = args.probe_parallel
     pair = args.schedule == "pair" or pp
     my_probes = K          # probes whose passes this rank runs
@@ -969,19 +969,15 @@ def run_zo(args):
                                             else "perturb_pair_kernel"), pair_ms, my_probes
         traffic, traffic_how = committed_traffic("perturb_pair_kernel", traffic_key)
     elif n2 > 0 and n2 * perturb2_ms > n1 * perturb_ms:
-        dom_kernel, dom_ms, dom_launches = ("perturb_shift_kernel<2, *> (zo_perturb2, tensors off the 32-byte grid)"
-                                            if shifted else
-                                            "perturb_kernel<2, *> (zo_perturb2, configuration tuned per list)",
-                                            perturb2_ms, n2)
-        traffic, traffic_how = committed_traffic("perturb2_kernel", traffic_key)
+        dom_kernel, dom_ms, dom_launches = "perturb_items_kernel<2> (zo_perturb2)", perturb2_ms, n2
+        traffic, traffic_how = committed_traffic("perturb_items_kernel<2>", traffic_key)
     else:
-        dom_kernel, dom_ms, dom_launches = ("perturb_shift_kernel<1, *> (zo_perturb, tensors off the 32-byte grid)"
-                                            if shifted else "perturb_kernel<1, 0> (zo_perturb)", perturb_ms, n1)
-        traffic, traffic_how = committed_traffic("perturb_kernel", traffic_key)
+        dom_kernel, dom_ms, dom_launches = "perturb_items_kernel<1> (zo_perturb)", perturb_ms, n1
+        traffic, traffic_how = committed_traffic("perturb_items_kernel<1>", traffic_key)
     dom_bytes = pair_bytes if pair else perturb_bytes
     # the update's DRAM bytes (one read and one write of theta, whatever K): the
     # 8-probe-table kernel's committed capture when it is the one this K runs
-    if args.packing == 1 and 16 < K <= 384 and not shifted:
+    if args.packing == 1 and K > 16 and not shifted:
         upd_traffic, upd_traffic_how = committed_traffic("update_lut8_kernel", traffic_key)
     else:
         upd_traffic, upd_traffic_how = None, "no capture committed for the update kernel this K runs"

@@ -6,16 +6,15 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include <cuda_runtime.h>
 
 #include "zo.h"
+#include "zo_items.h"
 #include "zo_launch.h"
 
 namespace {
 
-using zo::PerturbParams;
 using zo::RoundKeys;
 using zo::TensorTable;
 using zo::UpdateParams;
@@ -68,18 +67,10 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
   return op;
 }
 
-// Resident perturb blocks per SM. The passes are HBM-bound and each thread
-// keeps two 32-byte loads in flight. The single-op pass streams fastest with
-// four 256-thread blocks per SM (3 -> 90.6 %, 4 -> 97.7 %, 5 -> 93.0 % of the
-// copy bandwidth on the 60 GB OPT-30B-shaped set), the out-of-place pair pass
-// with three. The two-op pass has three candidate (loop, blocks per SM)
-// configurations, timed on the caller's list (TwoOpTuner below).
-constexpr int kPerturbBlocksPerSm = 4;
+// Resident blocks per SM of the pair pass: three of 256 threads stream fastest
+// (4 blocks per SM slower); pair_shift_kernel takes at most 64 registers.
 constexpr int kPairBlocksPerSm = 3;
-constexpr int kShiftBlocksPerSm = 4;   // pair_shift_kernel: 256 threads, at most 64 registers
-constexpr int kTwoOpCandidates = 3;
-constexpr int kTwoOpLoop[kTwoOpCandidates] = {zo::kLoopRuns, zo::kLoopRuns, zo::kLoopBlocks};
-constexpr int kTwoOpBlocksPerSm[kTwoOpCandidates] = {3, 4, 4};
+constexpr int kShiftBlocksPerSm = 4;
 
 // Packing-1 updates with at most this many probe groups keep both groups'
 // tables in shared memory for the whole launch (update_lut8_small_kernel);
@@ -89,10 +80,7 @@ constexpr int kSmallGroups = 2;
 // Per-device launch facts, filled once per device.
 struct DeviceInfo {
   int sms = 0;
-  int perturb_bps = 0;                    // single-op perturb blocks per SM
-  int two_op_bps[kTwoOpCandidates] = {};  // two-op perturb blocks per SM, by candidate
   int pair_bps = 0;                       // perturb_pair blocks per SM
-  int shift_bps[2][3] = {};               // perturb_shift blocks per SM, by operation count and dtype
   bool lut8_ready = false;                // the update kernels' shared-memory limits are raised
 };
 constexpr int kMaxDevices = 64;
@@ -111,24 +99,9 @@ int device_info(DeviceInfo** out) {
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     int bps = 0;
-    e = zo::perturb_blocks_per_sm(1, zo::kLoopBlocks, &bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy(perturb)");
-    d.perturb_bps = bps < 1 ? 1 : (bps < kPerturbBlocksPerSm ? bps : kPerturbBlocksPerSm);
-    for (int i = 0; i < kTwoOpCandidates; ++i) {
-      e = zo::perturb_blocks_per_sm(2, kTwoOpLoop[i], &bps);
-      if (e != cudaSuccess) return cuda_fail(e, "occupancy(perturb2)");
-      d.two_op_bps[i] = bps < 1 ? 1 : (bps < kTwoOpBlocksPerSm[i] ? bps : kTwoOpBlocksPerSm[i]);
-    }
     e = zo::pair_blocks_per_sm(&bps);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy(perturb_pair)");
     d.pair_bps = bps < 1 ? 1 : (bps < kPairBlocksPerSm ? bps : kPairBlocksPerSm);
-    for (int nops = 1; nops <= 2; ++nops) {
-      for (uint8_t dt = 0; dt < 3; ++dt) {
-        e = zo::shift_blocks_per_sm(nops, dt, &bps);
-        if (e != cudaSuccess) return cuda_fail(e, "occupancy(perturb_shift)");
-        d.shift_bps[nops - 1][dt] = bps < 1 ? 1 : bps;
-      }
-    }
     d.sms = sms;
   }
   *out = &d;
@@ -226,234 +199,59 @@ int grid_for(int64_t blocks, int sms, int bps) {
   return static_cast<int>(g < 1 ? 1 : g);
 }
 
-// Choice of the two-op configuration per parameter list. All candidates give
-// the same bits; which is fastest depends on the tensor sizes (measured: runs
-// with 3 blocks per SM on the OPT-30B-shaped set, one block per iteration with
-// 4 on the Qwen3-8B-shaped one, runs with 4 on the OPT-1.3B-shaped one, the
-// spread between candidates from 1 % to 12 %). The first calls on a list
-// (keyed by its sizes, dtypes, alignments and device, and by whether the two
-// probes fall in one group of 8 or in two) run the candidates in turn, three
-// rounds each (one for the two-group calls), each call between two events on
-// the caller's stream; once all those events have completed (polled, never
-// waited for), later calls use the candidate with the shortest time (the
-// shortest of its rounds). Calls made while the stream is being captured
-// into a graph, or before a decision, use candidate 0.
-// After a failed runtime call of this file's own bookkeeping (events, capture
-// query): reset the thread's last error only when it is that call's error, so
-// an unrelated error the caller has not collected yet stays pending.
-void clear_own_error(cudaError_t e) {
-  if (e != cudaSuccess && cudaPeekAtLastError() == e) cudaGetLastError();
-}
+thread_local zo::ItemsParams<zo::kItemsFew> tl_items_few;
+thread_local zo::ItemsParams<zo::kItemsSome> tl_items_some;
+thread_local zo::ItemsParams<zo::kItemsMany> tl_items_many;
 
-class TwoOpTuner {
- public:
-  // Candidate for this call; *slot receives the trial index when the call's
-  // launches must be bracketed by that trial's events, else -1.
-  int pick(uint64_t key, int rounds, cudaStream_t s, int* slot) {
-    *slot = -1;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const cudaError_t ce = cudaStreamIsCapturing(s, &cap);
-    if (ce != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      clear_own_error(ce);
-      return 0;
-    }
-    std::lock_guard<std::mutex> lock(mu_);
-    Entry* e = find(key, rounds);
-    if (e == nullptr) return 0;
-    if (e->chosen >= 0) return e->chosen;
-    decide(*e);
-    if (e->chosen >= 0) return e->chosen;
-    if (e->next < e->trials) {
-      *slot = e->next++;
-      return *slot % kTwoOpCandidates;
-    }
-    return 0;
-  }
-
-  void record(uint64_t key, int slot, int which, cudaStream_t s) {
-    std::lock_guard<std::mutex> lock(mu_);
-    Entry* e = find(key, 0);
-    if (e == nullptr || e->ev[slot][which] == nullptr) return;
-    const cudaError_t er = cudaEventRecord(e->ev[slot][which], s);
-    if (er != cudaSuccess) {
-      clear_own_error(er);
-      e->failed = true;
-    }
-  }
-
- private:
-  static constexpr int kMaxRounds = 3;
-  static constexpr int kTrials = kMaxRounds * kTwoOpCandidates;
-
-  struct Entry {
-    uint64_t key = 0;
-    int chosen = -1;
-    int next = 0;  // next trial; trial i runs candidate i % kTwoOpCandidates
-    int trials = kTrials;
-    bool failed = false;
-    cudaEvent_t ev[kTrials][2] = {};
-  };
-
-  // Entry of `key`, created with its events on first use with `rounds` trial
-  // rounds (1..kMaxRounds; rounds = 0 only looks up). nullptr when absent and
-  // not created, the table is full, or events cannot be created: then
-  // candidate 0 is used.
-  Entry* find(uint64_t key, int rounds) {
-    for (Entry& e : entries_)
-      if (e.key == key) return &e;
-    if (rounds < 1 || entries_.size() >= kMaxEntries) return nullptr;
-    Entry e;
-    e.key = key;
-    e.trials = (rounds < kMaxRounds ? rounds : kMaxRounds) * kTwoOpCandidates;
-    for (auto& pair : e.ev)
-      for (cudaEvent_t& ev : pair)
-        if (const cudaError_t ec = cudaEventCreate(&ev); ec != cudaSuccess) {
-          clear_own_error(ec);
-          e.chosen = 0;
-        }
-    entries_.push_back(e);
-    return &entries_.back();
-  }
-
-  void decide(Entry& e) {
-    if (e.failed) {
-      e.chosen = 0;
-      return;
-    }
-    if (e.next < e.trials) return;
-    float best[kTwoOpCandidates];
-    for (int i = 0; i < e.trials; ++i) {
-      if (const cudaError_t q = cudaEventQuery(e.ev[i][1]); q != cudaSuccess) {  // not done yet (or failed)
-        clear_own_error(q);
-        return;
-      }
-      float ms = 0.0f;
-      if (const cudaError_t t = cudaEventElapsedTime(&ms, e.ev[i][0], e.ev[i][1]); t != cudaSuccess) {
-        clear_own_error(t);
-        e.chosen = 0;
-        return;
-      }
-      const int c = i % kTwoOpCandidates;
-      if (i < kTwoOpCandidates || ms < best[c]) best[c] = ms;  // shortest of its rounds
-    }
-    int arg = 0;
-    for (int c = 1; c < kTwoOpCandidates; ++c)
-      if (best[c] < best[arg]) arg = c;
-    e.chosen = arg;
-  }
-
-  static constexpr size_t kMaxEntries = 64;
-  std::mutex mu_;
-  std::vector<Entry> entries_;
+// One perturbation pass over a list.
+struct PerturbPass {
+  RoundKeys keys;
+  zo::PerturbOp op[2];
+  int32_t nops;
+  uint32_t probe;
+  const double* coef;
+  double coef_mul;
+  const int32_t* status;
 };
-TwoOpTuner g_two_op_tuner;
 
-// Hash of what decides the two-op pass's speed: device, sizes, dtypes,
-// 32-byte alignment (an FNV-style multiply-xor per 64-bit word, then a final
-// avalanche; a collision only shares a tuning decision).
-uint64_t list_key(const zo_tensor* params, int32_t n) {
-  uint64_t h = 0xcbf29ce484222325ull;
-  auto mix = [&h](uint64_t v) {
-    h ^= v;
-    h *= 0x100000001b3ull;
-    h ^= h >> 29;
+template <int N>
+void set_pass(zo::ItemsParams<N>& ip, const PerturbPass& pp) {
+  ip.keys = pp.keys;
+  ip.op[0] = pp.op[0];
+  ip.op[1] = pp.op[1];
+  const uint32_t high = static_cast<uint32_t>(static_cast<uint64_t>(ip.e[0].vb) >> 32);
+  ip.g[0] = zo::group_round01(pp.op[0].ctr2, high, pp.keys);
+  ip.g[1] = zo::group_round01(pp.op[1].ctr2, high, pp.keys);
+  ip.nops = pp.nops;
+  ip.probe = pp.probe;
+  ip.coef = pp.coef;
+  ip.coef_mul = pp.coef_mul;
+  ip.status = pp.status;
+}
+
+// Launches over the whole list, each with the smallest table that holds it
+// (kItemsMany per launch when the virtual blocks cross a counter high word).
+int run_perturb(const zo_tensor* params, int32_t n, const PerturbPass& pp, cudaStream_t s) {
+  zo::ItemsCursor cur;
+  const auto launch = [&](auto& ip) -> cudaError_t {
+    const zo::ItemsCursor from = cur;
+    if (zo::fill_items(ip, params, n, cur)) {
+      if (ip.n == 0) return cudaSuccess;
+      set_pass(ip, pp);
+      return zo::launch_perturb_items(ip, s);
+    }
+    cur = from;
+    zo::fill_items(tl_items_many, params, n, cur);
+    set_pass(tl_items_many, pp);
+    return zo::launch_perturb_items_any_high(tl_items_many, s);
   };
-  int dev = 0;
-  cudaGetDevice(&dev);
-  mix(static_cast<uint64_t>(dev));
-  mix(static_cast<uint64_t>(n));
-  for (int32_t t = 0; t < n; ++t) {
-    mix(static_cast<uint64_t>(params[t].numel));
-    mix(static_cast<uint64_t>(params[t].dtype) | (reinterpret_cast<uintptr_t>(params[t].ptr) % 32 == 0 ? 0x100u : 0u));
+  while (cur.t < n) {
+    const int32_t left = n - cur.t;
+    const cudaError_t e = left <= zo::kItemsFew    ? launch(tl_items_few)
+                          : left <= zo::kItemsSome ? launch(tl_items_some)
+                                                   : launch(tl_items_many);
+    if (e != cudaSuccess) return cuda_fail(e, "perturb_items_kernel");
   }
-  h ^= h >> 33;
-  h *= 0xff51afd7ed558ccdull;
-  h ^= h >> 33;
-  return h;
-}
-
-// Enqueue perturb launches over the whole parameter list.
-// Tensors of a perturb launch that are not 32-byte aligned go to
-// perturb_shift_kernel: flag them (kShift). Returns a bit mask of their
-// storage types; *main_work tells whether any other tensor has elements.
-unsigned mark_shift(zo::TensorTable& tab, bool* main_work) {
-  unsigned types = 0;
-  *main_work = false;
-  for (int i = 0; i < tab.n; ++i) {
-    if (tab.numel[i] == 0) continue;
-    if (tab.flags[i] & zo::kVec32) {
-      *main_work = true;
-    } else {
-      tab.flags[i] |= zo::kShift;
-      types |= 1u << (tab.flags[i] & zo::kDtypeMask);
-    }
-  }
-  return types;
-}
-
-// grp_end over the flagged tensors of storage type dt (the others own no
-// group). Returns the number of groups.
-uint32_t shift_groups(const zo::TensorTable& tab, uint8_t dt, uint32_t* grp_end) {
-  uint32_t groups = 0;
-  for (int i = 0; i < tab.n; ++i) {
-    const uint8_t fl = tab.flags[i];
-    if ((fl & zo::kShift) && (fl & zo::kDtypeMask) == dt) {
-      const uint32_t esz = dt == zo::kF32 ? 4 : 2;
-      const int64_t a = static_cast<int64_t>(tab.ptr[i] % 32) / esz;  // 1..15: pointers are element-aligned
-      const int64_t chunks = (tab.numel[i] + a + 15) / 16;
-      groups += static_cast<uint32_t>((chunks + zo::kShiftGroup - 1) / zo::kShiftGroup);
-    }
-    grp_end[i] = groups;
-  }
-  return groups;
-}
-
-thread_local zo::ShiftParams tl_shift;
-
-int run_perturb(const zo_tensor* params, int32_t n, PerturbParams& pp, DeviceInfo* d, cudaStream_t s) {
-  int loop = zo::kLoopBlocks, bps = d->perturb_bps, slot = -1;
-  uint64_t key = 0;
-  if (pp.nops == 2) {
-    // probes in two groups of 8 (two Philox calls per block) run a kernel of
-    // their own, so they get a configuration choice of their own, timed one
-    // round per candidate: such calls come once per 8 probes, and three
-    // rounds would leave a K = 16 step still timing candidates after a few
-    // steps
-    const bool cross = pp.op[0].ctr2 != pp.op[1].ctr2;
-    key = list_key(params, n) ^ (cross ? 0x9E3779B97F4A7C15ull : 0ull);
-    const int c = g_two_op_tuner.pick(key, cross ? 1 : 3, s, &slot);
-    loop = kTwoOpLoop[c];
-    bps = d->two_op_bps[c];
-  }
-  if (slot >= 0) g_two_op_tuner.record(key, slot, 0, s);
-  int64_t blk = 0;
-  for (int32_t t0 = 0; t0 < n;) {
-    int64_t nb = 0;
-    t0 = fill_table(pp.tab, params, t0, n, blk, &nb);
-    if (nb > 0) {
-      bool main_work = false;
-      const unsigned shift_types = mark_shift(pp.tab, &main_work);
-      bool f32v = false;  // aligned fp32 tensors in this launch: pipelined fp32 path (single-op kernel)
-      for (int i = 0; i < pp.tab.n && !f32v; ++i)
-        f32v = (pp.tab.flags[i] & zo::kVec32) && (pp.tab.flags[i] & zo::kDtypeMask) == zo::kF32;
-      if (main_work) {
-        cudaError_t e = zo::launch_perturb(pp, grid_for(pp.tab.blk_total, d->sms, bps), loop, f32v, s);
-        if (e != cudaSuccess) return cuda_fail(e, "perturb_kernel");
-      }
-      if (shift_types) tl_shift.p = pp;
-      for (uint8_t dt = 0; dt < 3; ++dt) {
-        if (!(shift_types & (1u << dt))) continue;
-        const uint32_t groups = shift_groups(pp.tab, dt, tl_shift.grp_end);
-        tl_shift.grp_total = groups;
-        const int64_t want = (static_cast<int64_t>(groups) * 32 + zo::kThreads - 1) / zo::kThreads;
-        const int64_t cap = static_cast<int64_t>(d->sms) * d->shift_bps[pp.nops - 1][dt];
-        cudaError_t e = zo::launch_perturb_shift(tl_shift, dt, static_cast<int>(want < cap ? want : cap), s);
-        if (e != cudaSuccess) return cuda_fail(e, "perturb_shift_kernel");
-      }
-    }
-    blk += nb;
-  }
-  if (slot >= 0) g_two_op_tuner.record(key, slot, 1, s);
   return ZO_OK;
 }
 
@@ -552,7 +350,6 @@ int run_pair_shift(const zo::PairParams& pp, uint8_t dt, bool moved, DeviceInfo*
   return ZO_OK;
 }
 
-thread_local PerturbParams tl_perturb;
 thread_local zo::PairParams tl_pair;
 thread_local zo::SmallUpdateParams tl_update;
 
@@ -593,9 +390,7 @@ int zo_perturb(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint32
   if (rc != ZO_OK) return rc;
   if (!std::isfinite(scale)) return ZO_ERR_ARG;
   if (n_tensors == 0) return ZO_OK;
-  DeviceInfo* d = nullptr;
-  if ((rc = device_info(&d)) != ZO_OK) return rc;
-  PerturbParams& pp = tl_perturb;
+  PerturbPass pp;
   pp.keys = expand_keys(seed);
   pp.probe = probe;
   pp.op[0] = make_op(probe, scale, packing);
@@ -604,7 +399,7 @@ int zo_perturb(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint32
   pp.coef = nullptr;
   pp.coef_mul = 0.0;
   pp.status = nullptr;
-  return run_perturb(params, n_tensors, pp, d, static_cast<cudaStream_t>(stream));
+  return run_perturb(params, n_tensors, pp, static_cast<cudaStream_t>(stream));
 }
 
 int zo_perturb2(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint32_t probe_a, float scale_a,
@@ -614,9 +409,7 @@ int zo_perturb2(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint3
   if (rc != ZO_OK) return rc;
   if (!std::isfinite(scale_a) || !std::isfinite(scale_b)) return ZO_ERR_ARG;
   if (n_tensors == 0) return ZO_OK;
-  DeviceInfo* d = nullptr;
-  if ((rc = device_info(&d)) != ZO_OK) return rc;
-  PerturbParams& pp = tl_perturb;
+  PerturbPass pp;
   pp.keys = expand_keys(seed);
   pp.probe = probe_a;
   pp.op[0] = make_op(probe_a, scale_a, packing);
@@ -625,7 +418,7 @@ int zo_perturb2(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint3
   pp.coef = nullptr;
   pp.coef_mul = 0.0;
   pp.status = nullptr;
-  return run_perturb(params, n_tensors, pp, d, static_cast<cudaStream_t>(stream));
+  return run_perturb(params, n_tensors, pp, static_cast<cudaStream_t>(stream));
 }
 
 int zo_perturb_pair(const zo_tensor* theta, const zo_tensor* plus, const zo_tensor* minus, int32_t n_tensors,
@@ -736,9 +529,7 @@ int zo_update_sequential(const zo_tensor* params, int32_t n_tensors, uint64_t se
   int packing = zo::kPacking1;
   int rc = check_update_args(params, n_tensors, c, K, lr, &packing);
   if (rc != ZO_OK || n_tensors == 0) return rc;
-  DeviceInfo* d = nullptr;
-  if ((rc = device_info(&d)) != ZO_OK) return rc;
-  PerturbParams& pp = tl_perturb;
+  PerturbPass pp;
   pp.keys = expand_keys(seed);
   pp.coef = c;
   pp.coef_mul = -(lr / static_cast<double>(K));
@@ -748,7 +539,7 @@ int zo_update_sequential(const zo_tensor* params, int32_t n_tensors, uint64_t se
     pp.probe = static_cast<uint32_t>(k);
     pp.op[0] = make_op(pp.probe, 0.0f, packing);  // scale read from c on the device
     pp.op[1] = pp.op[0];
-    if ((rc = run_perturb(params, n_tensors, pp, d, static_cast<cudaStream_t>(stream))) != ZO_OK) return rc;
+    if ((rc = run_perturb(params, n_tensors, pp, static_cast<cudaStream_t>(stream))) != ZO_OK) return rc;
   }
   return ZO_OK;
 }

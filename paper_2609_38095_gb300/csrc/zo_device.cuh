@@ -20,7 +20,7 @@ constexpr int kMaxGroups = kMaxProbes / 8;
 constexpr uint8_t kF32 = 0, kBF16 = 1, kF16 = 2;
 constexpr uint8_t kDtypeMask = 0x3;
 constexpr uint8_t kVec32 = 0x80;      // base pointer is 32-byte aligned
-constexpr uint8_t kShift = 0x40;      // not 32-byte aligned: perturbed by perturb_shift_kernel instead
+constexpr uint8_t kShift = 0x40;      // not 32-byte aligned: worked on in aligned chunks
 
 // Elements are addressed by a virtual index g: tensor t starts at a multiple
 // of 16, so each 16-element Philox block lies inside one tensor. Blocks are
@@ -72,37 +72,88 @@ struct PerturbOp {
   uint32_t mul[4];
 };
 
-// Loop of perturb_kernel: one block per iteration, or runs of full blocks.
-constexpr int kLoopBlocks = 0;
-constexpr int kLoopRuns = 1;
+// Tensors off the 32-byte grid are worked on in 32-byte aligned chunks, 31 per
+// warp (lane 0 only generates the block below the first); the pair pass counts
+// them in groups of kShiftGroup chunks.
+constexpr int kShiftLanes = 31;
+constexpr int kShiftSub = 4;                        // rounds of 31 chunks per group
+constexpr int kShiftGroup = kShiftLanes * kShiftSub;
 
-struct PerturbParams {
-  TensorTable tab;
+// Table of a launch of perturb_items_kernel. Work is numbered in 32-byte items
+// (sixteen 16-bit or eight fp32 elements), tensors starting on multiples of 32;
+// a tensor off the 32-byte grid by a elements takes 32 items per 31 of its
+// aligned 32-byte chunks. A tensor's fields lie together, and the tensor of an
+// item is found from a hint per 2^hint_shift items, then by walking on. Three
+// sizes: a launch of few tensors is bound by latency, and 25 KB of parameters
+// cost it 1 us (8 KB: 0.2).
+constexpr int kItemsFew = 64, kItemsSome = 256, kItemsMany = 960;
+constexpr int kItemsHints = 256;
+constexpr uint32_t kItemsCont = 0x20;  // the entry is a later piece of its tensor
+
+struct ItemsEntry {
+  uint64_t base;         // the tensor's address, rounded down to 32 bytes
+  int64_t vb;            // virtual block of its first element
+  uint32_t begin, end;   // its first and one-past-last item
+  uint32_t whole;        // (elements + a) / elements per item: chunks wholly before its end
+  uint32_t meta;         // dtype, kShift and kItemsCont | elements past the whole chunks << 8 | a << 16
+};
+
+// Philox rounds 0-1 as far as they depend on the probe group alone (the
+// launch's virtual blocks sharing the counter's high word).
+struct GroupRound01 {
+  uint32_t x0;    // lo(M1 q) ^ k0[1]
+  uint32_t x2;    // hi(M0 u) ^ k1[1], u = hi(M1 q) ^ bhi ^ k0[0]
+  uint32_t lpa1;  // lo(M0 u)
+};
+
+// Launch item b of its entry: the 32-byte chunk i (from the entry's base) that
+// it works on, and the virtual block (fp32: half block) whose signs its lane
+// generates.
+struct ItemPlace {
+  int32_t i;      // chunk; -1: lane 0 of a tensor's first warp off the grid
+  bool act;       // the lane has elements to change
+  bool full;      // all of the chunk's
+};
+
+__host__ __device__ __forceinline__ ItemPlace item_place(const ItemsEntry& e, uint32_t b) {
+  const bool shift = (e.meta & kShift) != 0;
+  const uint32_t d = b - e.begin, lane = d & 31u;
+  ItemPlace k;
+  // off the grid a warp takes 31 chunks, and lane 0 only generates
+  k.i = static_cast<int32_t>(shift ? (d >> 5) * static_cast<uint32_t>(kShiftLanes) + lane - 1u : d);
+  const bool some = !(shift && lane == 0u);
+  // the first chunk of a tensor off the grid is not full, unless this is a later piece of it
+  k.full = some && k.i < static_cast<int32_t>(e.whole) && (k.i > 0 || !shift || (e.meta & kItemsCont));
+  k.act = some && k.i < static_cast<int32_t>(e.whole) + ((e.meta & 0xFF00u) != 0u ? 1 : 0);
+  return k;
+}
+
+__host__ __device__ __forceinline__ int64_t item_block(const ItemsEntry& e, int32_t i) {
+  return e.vb + ((e.meta & kDtypeMask) == kF32 ? i >> 1 : i);
+}
+
+// An active item's elements lo .. hi - 1 of its chunk.
+__host__ __device__ __forceinline__ void item_range(const ItemsEntry& e, int32_t i, int* lo, int* hi) {
+  *lo = i == 0 && !(e.meta & kItemsCont) ? static_cast<int>(e.meta >> 16) : 0;
+  *hi = i < static_cast<int32_t>(e.whole) ? ((e.meta & kDtypeMask) == kF32 ? 8 : 16)
+                                          : static_cast<int>((e.meta >> 8) & 255u);
+}
+
+template <int N>
+struct ItemsParams {
+  ItemsEntry e[N];       // non-empty tensors
+  uint16_t hint[kItemsHints];
+  int32_t n;
+  int32_t hint_shift;
+  uint32_t total;
   RoundKeys keys;
   PerturbOp op[2];         // applied in order, each rounded to storage; op[1] only when nops == 2
+  GroupRound01 g[2];       // their groups' Philox parts
   int32_t nops;            // 1 or 2
   uint32_t probe;          // probe index k of op[0] (for coef)
   const double* coef;      // optional: op[0]'s scale = fp32(coef_mul * coef[probe])
   double coef_mul;
   const int32_t* status;   // optional: skip everything unless *status == 0
-};
-
-// Tensors of a perturb launch whose base is not 32-byte aligned (views at an
-// element offset) are perturbed by a second kernel that reads and writes
-// them in 32-byte aligned chunks of 16 elements: chunk c of such a tensor
-// holds elements 16c - a .. 16c - a + 15 (a = the base's offset, in
-// elements, from the 32-byte boundary below it), i.e. the tail of Philox
-// block c - 1 and the head of block c. Work is counted in groups of
-// kShiftGroup chunks per warp; grp_end[t] is one past tensor t's last group
-// (tensors without kShift own none).
-constexpr int kShiftLanes = 31;                     // chunks per warp and sub-group (lane 0 only generates)
-constexpr int kShiftSub = 4;                        // rounds of 31 chunks per group
-constexpr int kShiftGroup = kShiftLanes * kShiftSub;
-
-struct ShiftParams {
-  PerturbParams p;         // the launch's table, keys, operations, coefficient and status, as for perturb_kernel
-  uint32_t grp_total;
-  uint32_t grp_end[kMaxTensorsPerLaunch];
 };
 
 // Out-of-place pair of perturbations (zo_perturb_pair): theta is read once
@@ -160,14 +211,6 @@ struct UpdateParams {
   const int32_t* status;   // optional: when *status != 0 only `pre` is applied
 };
 
-// Philox rounds 0-1 as far as they depend on the probe group alone (the
-// launch's virtual blocks sharing the counter's high word).
-struct GroupRound01 {
-  uint32_t x0;    // lo(M1 q) ^ k0[1]
-  uint32_t x2;    // hi(M0 u) ^ k1[1], u = hi(M1 q) ^ bhi ^ k0[0]
-  uint32_t lpa1;  // lo(M0 u)
-};
-
 // The update at one or two probe groups: the groups' and the leading
 // perturbation's Philox parts beside it. In its table launch blocks are
 // 32-byte items: half blocks of fp32 tensors, and 32 per 31 aligned chunks of
@@ -203,6 +246,56 @@ __device__ __forceinline__ uint4 philox10(uint32_t c0, uint32_t c1, uint32_t c2,
 #pragma unroll
   for (int r = 0; r < 10; ++r) philox_round(c0, c1, c2, c3, rk.k0[r], rk.k1[r]);
   return make_uint4(c0, c1, c2, c3);
+}
+
+// Philox4x32-10 with rounds 0 and 1 split by what they depend on, for a
+// launch whose virtual blocks share the counter's high word bhi (every launch
+// below 2^36 weights). The counter is (b_lo, bhi, q, 0). Round 0 multiplies
+// b_lo (per block) and q (per group); round 1 multiplies the word that came
+// from q and bhi (per group) and the one that came from b_lo (per block), so
+// both rounds' products are computed once per group (GroupRound01, shared by
+// every block) and once per block (BlockRound01, shared by the pair's two
+// groups); only their xors and rounds 2-9 are per (block, group). The output
+// equals philox10(b_lo, bhi, q, 0) bit for bit.
+struct BlockRound01 {
+  uint32_t lpa0;  // lo(M0 b_lo)
+  uint32_t hpb1;  // hi(M1 v), v = hi(M0 b_lo) ^ k1[0]
+  uint32_t lpb1;  // lo(M1 v)
+};
+__host__ __device__ __forceinline__ GroupRound01 group_round01(uint32_t q, uint32_t bhi, const RoundKeys& rk) {
+  const uint64_t pb0 = static_cast<uint64_t>(kPhiloxM1) * q;
+  const uint32_t u = static_cast<uint32_t>(pb0 >> 32) ^ bhi ^ rk.k0[0];
+  const uint64_t pa1 = static_cast<uint64_t>(kPhiloxM0) * u;
+  GroupRound01 g;
+  g.x0 = static_cast<uint32_t>(pb0) ^ rk.k0[1];
+  g.x2 = static_cast<uint32_t>(pa1 >> 32) ^ rk.k1[1];
+  g.lpa1 = static_cast<uint32_t>(pa1);
+  return g;
+}
+__device__ __forceinline__ BlockRound01 block_round01(uint32_t blo, const RoundKeys& rk) {
+  const uint64_t pa0 = static_cast<uint64_t>(kPhiloxM0) * blo;
+  const uint32_t v = static_cast<uint32_t>(pa0 >> 32) ^ rk.k1[0];
+  const uint64_t pb1 = static_cast<uint64_t>(kPhiloxM1) * v;
+  BlockRound01 k;
+  k.lpa0 = static_cast<uint32_t>(pa0);
+  k.hpb1 = static_cast<uint32_t>(pb1 >> 32);
+  k.lpb1 = static_cast<uint32_t>(pb1);
+  return k;
+}
+
+// A Philox call after its first two rounds.
+struct PhiloxState {
+  uint32_t c0, c1, c2, c3;
+};
+
+__device__ __forceinline__ uint4 philox_finish(PhiloxState s, const RoundKeys& rk) {
+#pragma unroll
+  for (int r = 2; r < 10; ++r) philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[r], rk.k1[r]);
+  return make_uint4(s.c0, s.c1, s.c2, s.c3);
+}
+
+__device__ __forceinline__ PhiloxState philox_start(const BlockRound01& k, const GroupRound01& g) {
+  return {k.hpb1 ^ g.x0, k.lpb1, g.x2 ^ k.lpa0, g.lpa1};
 }
 
 __device__ __forceinline__ uint32_t word_of(const uint4& x, int m) {
@@ -325,9 +418,40 @@ __device__ __forceinline__ void store_elem(void* base, uint8_t dt, int64_t i, fl
   }
 }
 
+// Elements e0 + i of a tensor, lo <= i < hi <= 16, through f(m, j, value), i =
+// 4 m + j: a block or chunk across an end of its tensor, in place. AHEAD (1, 2
+// or 4) loads are issued before their first store: one by one, each load
+// misses the line that the store before it changed, and up to fifteen round
+// trips to L2 were a fifth of a small list's pass. What AHEAD costs in
+// registers its caller's loop pays, so it is as large as leaves that loop as
+// it was.
+template <int AHEAD, class F>
+__device__ __forceinline__ void map_elements(void* base, uint8_t dt, int64_t e0, int lo, int hi, const F& f) {
+#pragma unroll 1
+  for (int h = lo & ~(AHEAD - 1); h < hi; h += AHEAD) {
+    float v[AHEAD];
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j) v[j] = h + j >= lo && h + j < hi ? load_elem(base, dt, e0 + h + j) : 0.0f;
+#pragma unroll
+    for (int j = 0; j < AHEAD; ++j)
+      if (h + j >= lo && h + j < hi)
+        store_elem(base, dt, e0 + h + j, f(h >> 2, AHEAD == 4 ? j : (h + j) & 3, v[j]));
+  }
+}
+
 // Probe bit of element i (0..15) of a block, moved to bit 31.
 __device__ __forceinline__ uint32_t sign_bit(const uint4& x, int i, uint32_t j) {
   return (word_of(x, i >> 2) << (31u - 8u * static_cast<uint32_t>(i & 3) - j)) & 0x80000000u;
+}
+
+// scale z of the element in byte j of a Philox word: -scale's sign flipped by
+// the probe bit.
+__device__ __forceinline__ float signed_scale_word(uint32_t w, int j, const PerturbOp& op) {
+  return __uint_as_float(op.nscale_bits ^ ((w << (31u - 8u * static_cast<uint32_t>(j) - op.bit)) & 0x80000000u));
+}
+
+__device__ __forceinline__ float add_signed_word(float th, uint32_t w, int j, const PerturbOp& op) {
+  return __fadd_rn(th, signed_scale_word(w, j, op));
 }
 
 // theta + scale z for element i of a block: -scale's sign flipped by the probe bit.
@@ -401,6 +525,25 @@ __device__ __forceinline__ void window16f(const float (&lo)[16], const float (&h
   for (int i = 0; i < 18; ++i) t2[i] = (s & 2u) ? t4[i + 2] : t4[i];
 #pragma unroll
   for (int i = 0; i < 16; ++i) out[i] = (s & 1u) ? t2[i + 1] : t2[i];
+}
+
+// The sign words of a 32-byte item's elements from its Philox block's words
+// (all lanes of a warp, f32 / shift / a the same in all). f32: the item is the
+// block's lower or upper half, its eight bytes come first. shift: a tensor off
+// the 32-byte grid by a elements, whose item holds the tail of the block (f32:
+// half block) below, generated by lane l - 1, and the head of its own.
+__device__ __forceinline__ uint4 item_signs(const uint4& x, bool f32, bool upper, bool shift, uint32_t a) {
+  if (f32) {
+    uint2 y = upper ? make_uint2(x.z, x.w) : make_uint2(x.x, x.y);
+    if (shift) {  // bytes 8 - a .. 15 - a of (the half below) ++ (this half), a = 1..7
+      const uint32_t b0 = __shfl_up_sync(0xFFFFFFFFu, y.x, 1), b1 = __shfl_up_sync(0xFFFFFFFFu, y.y, 1);
+      const uint32_t s = 8u - a, sh = 8u * (s & 3u);
+      const uint32_t w0 = s >= 4u ? b1 : b0, w1 = s >= 4u ? y.x : b1, w2 = s >= 4u ? y.y : y.x;
+      y = make_uint2(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh));
+    }
+    return make_uint4(y.x, y.y, 0u, 0u);
+  }
+  return shift ? window16(shfl_up4(x), x, 16u - a) : x;
 }
 
 }  // namespace zo

@@ -1,0 +1,78 @@
+// zo_items.h -- host-side planning of perturb_items_kernel's tables (ItemsParams).
+#pragma once
+
+#include <cstdint>
+
+#include "zo.h"
+#include "zo_device.cuh"
+
+namespace zo {
+
+// A position in a parameter list: the next tensor, how many of its items are
+// already in earlier entries, and the virtual block of its first element.
+struct ItemsCursor {
+  int32_t t = 0;
+  int64_t done = 0;
+  int64_t v = 0;
+};
+
+// Most items of one entry (an even number, so that a later piece of an fp32
+// tensor starts with a whole block) and of one launch. A longer tensor takes
+// several entries.
+constexpr int64_t kItemsPiece = INT64_C(1) << 30;
+constexpr int64_t kItemsLaunch = INT64_C(1) << 31;
+
+// Fill `ip` from `cur` on, as far as its entries and `launch` items go. Returns
+// whether the launch's virtual blocks share the counter's high word.
+template <int N>
+bool fill_items(ItemsParams<N>& ip, const zo_tensor* params, int32_t n, ItemsCursor& cur, int64_t piece = kItemsPiece,
+                int64_t launch = kItemsLaunch) {
+  ip.n = 0;
+  int64_t b = 0, last = 0;  // items so far, and the last virtual block
+  while (cur.t < n) {
+    const zo_tensor& p = params[cur.t];
+    if (p.numel == 0) {
+      ++cur.t;
+      continue;
+    }
+    if (ip.n == N) break;
+    const int64_t esz = p.dtype == ZO_F32 ? 4 : 2, per = 32 / esz;
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(p.ptr);
+    const int64_t off = static_cast<int64_t>(addr % 32) / esz;
+    const int64_t whole = (p.numel + off) / per, rem = (p.numel + off) % per, items = whole + (rem != 0);
+    const int64_t left = items - cur.done, take = left < piece ? left : piece;
+    const int64_t start = (b + kLaunchAlign - 1) / kLaunchAlign * kLaunchAlign;
+    const int64_t end = start + (off == 0 ? take : (take + kShiftLanes - 1) / kShiftLanes * kLaunchAlign);
+    if (ip.n > 0 && end > launch) break;
+    b = end;
+    ItemsEntry& e = ip.e[ip.n++];
+    e.base = static_cast<uint64_t>(addr - addr % 32) + static_cast<uint64_t>(32 * cur.done);
+    e.vb = cur.v + (p.dtype == ZO_F32 ? cur.done / 2 : cur.done);
+    e.begin = static_cast<uint32_t>(start);
+    e.end = static_cast<uint32_t>(end);
+    e.whole = static_cast<uint32_t>(whole - cur.done < take ? whole - cur.done : take);
+    e.meta = static_cast<uint32_t>(p.dtype) | (off == 0 ? 0u : static_cast<uint32_t>(kShift)) |
+             (cur.done == 0 ? 0u : kItemsCont) | static_cast<uint32_t>(take == left ? rem : 0) << 8 |
+             static_cast<uint32_t>(off) << 16;
+    last = e.vb + take;
+    cur.done += take;
+    if (cur.done == items) {
+      ++cur.t;
+      cur.done = 0;
+      cur.v += (p.numel + 15) / 16;
+    }
+  }
+  ip.total = static_cast<uint32_t>(b);
+  if (ip.n == 0) return true;
+  // hint[k]: the first entry that ends past item k << hint_shift
+  ip.hint_shift = 5;
+  while ((ip.total - 1) >> ip.hint_shift >= static_cast<uint32_t>(kItemsHints)) ++ip.hint_shift;
+  int t = 0;
+  for (uint32_t k = 0; k <= (ip.total - 1) >> ip.hint_shift; ++k) {
+    while (static_cast<uint64_t>(ip.e[t].end) <= static_cast<uint64_t>(k) << ip.hint_shift) ++t;
+    ip.hint[k] = static_cast<uint16_t>(t);
+  }
+  return ip.e[0].vb >> 32 == last >> 32;
+}
+
+}  // namespace zo

@@ -19,10 +19,11 @@ constexpr int kQuadPointsMaxCtas = 256;     // CTAs of the launch that takes a s
 constexpr size_t kQuadPointsMaxSmem = 200 * 1024;  // and its shared memory per CTA
 constexpr int64_t kStaticLossSlice = 2048;  // elements per partial in that variant
 
-// f32v: the launch holds 32-byte aligned fp32 tensors (single-op kernel only).
-cudaError_t launch_perturb(const PerturbParams& p, int grid, int loop, bool f32v, cudaStream_t stream);
-// dt: the storage type of the tensors grp_end counts (one launch per type).
-cudaError_t launch_perturb_shift(const ShiftParams& p, uint8_t dt, int grid, cudaStream_t stream);
+// Perturbation by 32-byte items, one per thread.
+template <int N>
+cudaError_t launch_perturb_items(const ItemsParams<N>& p, cudaStream_t stream);
+// The same when the launch's virtual blocks differ in the counter's high word.
+cudaError_t launch_perturb_items_any_high(const ItemsParams<kItemsMany>& p, cudaStream_t stream);
 cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream);
 // moved: theta at another offset from the 32-byte grid than plus and minus (16-bit only).
 cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, int grid, cudaStream_t stream);
@@ -35,8 +36,6 @@ cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cu
 cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream);
 cudaError_t lut8_prepare();  // raises both kernels' shared-memory limits (once per device)
 bool one_high_word(const TensorTable& tab);  // of the launch's virtual blocks
-cudaError_t perturb_blocks_per_sm(int nops, int loop, int* out);
-cudaError_t shift_blocks_per_sm(int nops, uint8_t dt, int* out);
 cudaError_t pair_blocks_per_sm(int* out);
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,
                                uint8_t* out, int grid, cudaStream_t stream);

@@ -1,17 +1,13 @@
 // zo_stream_kernels.cu -- the HBM-streaming kernels of the 1.5-SPSA step:
 // fused perturb (Algorithm 1, ApplyPackedPerturbation), the out-of-place pair
-// of perturbations, fused K-probe update (Sec. 4.2, Eqs. 5-6) and the debug
-// views of a probe.
+// of perturbations and the debug views of a probe.
 //
-// Work unit: one thread owns one 16-element Philox block at a time (grid-
-// stride over the virtual block space of the launch's tensor table). A block
-// of a 16-bit tensor is 32 bytes: one 256-bit load and one 256-bit store when
-// the tensor is 32-byte aligned, element-wise access for a tensor's last,
-// partial block. The perturbation passes and the update hand tensors that
-// are not 32-byte aligned to perturb_shift_kernel / update_shift_kernel,
-// which work on aligned 32-byte chunks straddling two blocks; the pair pass
-// hands them (and fp32 tensors) to pair_shift_kernel when plus and minus
-// share their offset, and takes narrower accesses otherwise.
+// The perturbation passes work on 32-byte items, one per thread
+// (perturb_items_kernel). The pair pass walks 16-element Philox blocks grid-
+// stride (one 256-bit load and two stores per block of an aligned 16-bit
+// tensor) and hands fp32 tensors and tensors off the 32-byte grid to
+// pair_shift_kernel when plus and minus share their offset, else takes
+// narrower accesses.
 #include "zo_device.cuh"
 
 namespace zo {
@@ -42,421 +38,148 @@ __device__ __forceinline__ float add_signed_mul(float th, const uint4& x, int i,
   return __fadd_rn(th, __uint_as_float(op.nscale_bits ^ sign_bit_mul(x, i, op)));
 }
 
-// Sixteen 16-bit weights in registers (element 2r in the low half of v[r]).
-// CROSS: a two-op pass whose probes fall in two groups of 8 (two Philox calls
-// per block, one pass in eight of the fused schedule). Its adds are packed
-// fp32x2 adds, the same round-to-nearest sum per element: with the second
-// Philox call the loop is issue-bound and the packed adds take it from 20.5
-// to 18.9 ms on the OPT-30B-shaped set, while the one-group pass, bound by
-// HBM, is 1 % slower with them, so it keeps scalar adds.
-template <uint8_t DT, int NOPS, bool CROSS = false>
+// Sixteen 16-bit weights in registers (element 2r in the low half of v[r]),
+// NOPS perturbations one after the other, each rounded to storage. The adds
+// are packed fp32x2 adds, the same round-to-nearest sum per element: 732
+// against 756 us for the two-op pass on the OPT-1.3B-shaped bf16 set, 1156
+// against 1205 us on Qwen3-8B-shaped layers when its probes fall in two groups.
+template <uint8_t DT, int NOPS>
 __device__ __forceinline__ void perturb_regs16(uint32_t (&v)[8], const uint4 (&x)[2], const PerturbOp (&op)[2]) {
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
 #pragma unroll
     for (int o = 0; o < NOPS; ++o) {
-      if constexpr (CROSS) {
-        float2 f = unpack2<DT>(v[r]);
-        fadd2_rn(f.x, f.y, __uint_as_float(op[o].nscale_bits ^ sign_bit_mul(x[o], 2 * r, op[o])),
-                 __uint_as_float(op[o].nscale_bits ^ sign_bit_mul(x[o], 2 * r + 1, op[o])));
-        v[r] = pack2<DT>(f.x, f.y);
-      } else {
-        const float2 f = unpack2<DT>(v[r]);
-        v[r] = pack2<DT>(add_signed_mul(f.x, x[o], 2 * r, op[o]), add_signed_mul(f.y, x[o], 2 * r + 1, op[o]));
-      }
+      float2 f = unpack2<DT>(v[r]);
+      fadd2_rn(f.x, f.y, __uint_as_float(op[o].nscale_bits ^ sign_bit_mul(x[o], 2 * r, op[o])),
+               __uint_as_float(op[o].nscale_bits ^ sign_bit_mul(x[o], 2 * r + 1, op[o])));
+      v[r] = pack2<DT>(f.x, f.y);
     }
   }
 }
 
-// A thread's position in the tensor table. Its blocks only move forward and
-// usually stay inside one tensor, so the table is re-read only when a block
-// leaves the current tensor.
-struct Cursor {
-  int t;           // tensor index
-  uint32_t tb;     // first launch block of tensor t
-  uint32_t te;     // one past its last block
-  uint32_t n16;    // full blocks from tb on that take the pipelined 16-bit path (0 if it does not)
-  uint32_t n32;    // the same for the pipelined fp32 path of the single-op loop
-  uint16_t* tp;    // base pointer
-  uint32_t vd;     // launch block minus virtual block (relative to blk_base) in tensor t
-  uint8_t dt;      // storage dtype
-};
-
-// Launch blocks below tb (padding between tensors) give b - tb >= 2^31, so
-// they fail both n16 and n32 tests and go to perturb_block_other, which skips
-// them.
-__device__ __forceinline__ void cursor_seek(const TensorTable& tab, Cursor& c, uint32_t b) {
-  c.t = advance_tensor(tab, c.t, b);
-  c.tb = tensor_blk_begin(tab, c.t);
-  c.te = tab.blk_end[c.t];
-  const uint8_t fl = tab.flags[c.t];
-  c.dt = fl & kDtypeMask;
-  // pipelined path: full, 32-byte aligned blocks of a 16-bit tensor
-  const uint32_t full = static_cast<uint32_t>(tab.numel[c.t] / 16);
-  c.n16 = ((fl & kVec32) && c.dt != kF32) ? full : 0u;
-  c.n32 = ((fl & kVec32) && c.dt == kF32) ? full : 0u;
-  c.tp = reinterpret_cast<uint16_t*>(tab.ptr[c.t]);
-  c.vd = tab.vdelta[c.t];
-}
-
-// Any other block: fp32, a partial last block, or an unaligned tensor. One
-// instantiation per calling kernel (TAG): ptxas 13.0 crashes when two kernels
-// share this non-inlined function. Blocks of tensors flagged kShift are
-// perturb_shift_kernel's and left alone (the loops above stay exactly as
-// they are for the aligned tensors).
-template <int NOPS, int TAG>
-__device__ __noinline__ void perturb_block_other(const TensorTable& tab, int t, uint32_t b, uint4 x0, uint4 x1,
-                                                 PerturbOp op0, PerturbOp op1) {
-  const uint8_t fl = tab.flags[t];
-  if ((fl & kShift) || b < tensor_blk_begin(tab, t)) return;  // perturb_shift_kernel's, or padding
-  const int64_t e0 = static_cast<int64_t>(b - tensor_blk_begin(tab, t)) * 16;
-  const int64_t cnt = min(static_cast<int64_t>(16), tab.numel[t] - e0);
-  const uint8_t dt = fl & kDtypeMask;
-  void* base = reinterpret_cast<void*>(tab.ptr[t]);
-  if (cnt == 16 && (fl & kVec32) && dt == kF32) {
-    float* p = static_cast<float*>(base) + e0;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t v[8];
-      ld256(p + 8 * half, v);
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        float th = add_signed(__uint_as_float(v[r]), x0, 8 * half + r, op0);
-        if (NOPS == 2) th = add_signed(th, x1, 8 * half + r, op1);
-        v[r] = __float_as_uint(th);
-      }
-      st256(p + 8 * half, v);
-    }
-  } else if (cnt == 16 && dt != kF32) {  // a full block of an unaligned 16-bit tensor
-    uint16_t* p = static_cast<uint16_t*>(base) + e0;
-    uint32_t v[8];
-    ld16x16(p, v);
-    const uint4 x[2] = {x0, x1};
-    const PerturbOp op[2] = {op0, op1};
-    if (dt == kBF16)
-      perturb_regs16<kBF16, NOPS>(v, x, op);
-    else
-      perturb_regs16<kF16, NOPS>(v, x, op);
-    st16x16(p, v);
-  } else {
-    for (int i = 0; i < cnt; ++i) {
-      float th = add_signed(load_elem(base, dt, e0 + i), x0, i, op0);
-      if (NOPS == 2) th = add_signed(round_to_storage(dt, th), x1, i, op1);
-      store_elem(base, dt, e0 + i, th);
-    }
-  }
-}
-
-// A run of n blocks of one 16-bit tensor, all full and 32-byte aligned, at
-// p, p + pstride, ... with virtual blocks vb, vb + stride, ...: a tight,
-// software-pipelined loop (the next block's 256-bit load is issued before the
-// current block is computed and stored, so two loads per thread stay in
-// flight; the pass is HBM-bound and needs the bytes in flight).
-template <int NOPS, uint8_t DT, bool CROSS = false>
-__device__ __forceinline__ void perturb_run16(uint16_t* p, uint32_t n, size_t pstride, int64_t vb,
-                                              uint32_t stride, const PerturbOp (&op)[2], bool same_ctr,
-                                              const RoundKeys& keys) {
-  uint32_t v[8];
-  ld256(p, v);
-  for (uint32_t i = 0; i < n; ++i) {
-    uint16_t* pn = p + pstride;
-    uint32_t vn[8];
-    if (i + 1 < n) ld256(pn, vn);
-    uint4 x[2];
-    x[0] = block_bits(vb, op[0].ctr2, keys);
-    x[1] = x[0];
-    if (NOPS == 2 && (CROSS || !same_ctr)) x[1] = block_bits(vb, op[1].ctr2, keys);
-    perturb_regs16<DT, NOPS, CROSS>(v, x, op);
-    st256(p, v);
-    p = pn;
-    vb += stride;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = vn[r];
-  }
-}
-
-// Grid-stride over the launch's blocks, one block per iteration: the load of
-// the thread's next block (through the cursor, in whatever tensor it lies) is
-// issued before the current block is computed and stored. Every lane of a
-// warp runs the same number of iterations, whatever the tensor sizes. With
-// F32V (single-op launches that contain aligned fp32 tensors) full fp32
-// blocks are pipelined too, as two 256-bit halves; otherwise they go to
-// perturb_block_other, and the 16-bit path keeps its smaller register set.
-enum : int { kBlockOther = 0, kBlock16 = 1, kBlock32 = 2 };
-
-template <bool F32V>
-__device__ __forceinline__ int block_kind(const Cursor& c, uint32_t b) {
-  const uint32_t d = b - c.tb;
-  if (d < c.n16) return kBlock16;
-  if (F32V && d < c.n32) return kBlock32;
-  return kBlockOther;
-}
-
-__device__ __forceinline__ void* block_addr(const Cursor& c, uint32_t b, int kind) {
-  const size_t bytes = kind == kBlock32 ? 64 : 32;
-  return reinterpret_cast<char*>(c.tp) + static_cast<size_t>(b - c.tb) * bytes;
-}
-
-template <int NOPS, bool F32V, bool CROSS = false>
-__device__ __forceinline__ void perturb_blocks(const PerturbParams& P, const PerturbOp (&op)[2], bool same_ctr) {
-  const TensorTable& tab = P.tab;
-  const uint32_t blk_total = tab.blk_total;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;  // launch-relative; < 2^31 + stride never wraps
-  if (b >= blk_total) return;
-  Cursor c;
-  c.t = 0;
-  cursor_seek(tab, c, b);
-  int t = c.t;  // tensor and dtype of the current block
-  uint8_t dt = c.dt;
-  int kind = block_kind<F32V>(c, b);
-  void* p = block_addr(c, b, kind);
-  uint32_t vd = c.vd;
-  uint32_t v[8], w[8];  // the block (16-bit), or its two halves (fp32)
-  if (kind != kBlockOther) ld256(p, v);
-  if (kind == kBlock32) ld256(static_cast<char*>(p) + 32, w);
-  while (true) {
-    const uint32_t bn = b + stride;
-    int kindn = kBlockOther;
-    void* pn = nullptr;
-    uint32_t vn[8], wn[8];
-    if (bn < blk_total) {
-      if (bn >= c.te) cursor_seek(tab, c, bn);
-      kindn = block_kind<F32V>(c, bn);
-      pn = block_addr(c, bn, kindn);
-      if (kindn != kBlockOther) ld256(pn, vn);
-      if (kindn == kBlock32) ld256(static_cast<char*>(pn) + 32, wn);
-    }
-    const int64_t vb = tab.blk_base + (b - vd);  // virtual block: the Philox counter
-    uint4 x[2];
-    x[0] = block_bits(vb, op[0].ctr2, P.keys);
-    x[1] = x[0];
-    if (NOPS == 2 && (CROSS || !same_ctr)) x[1] = block_bits(vb, op[1].ctr2, P.keys);
-    if (kind == kBlock16) {
-      if (dt == kBF16)
-        perturb_regs16<kBF16, NOPS, CROSS>(v, x, op);
-      else
-        perturb_regs16<kF16, NOPS, CROSS>(v, x, op);
-      st256(p, v);
-    } else if (F32V && kind == kBlock32) {
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        v[r] = __float_as_uint(add_signed_mul(__uint_as_float(v[r]), x[0], r, op[0]));
-        w[r] = __float_as_uint(add_signed_mul(__uint_as_float(w[r]), x[0], 8 + r, op[0]));
-      }
-      st256(p, v);
-      st256(static_cast<char*>(p) + 32, w);
-    } else {
-      // each kernel its own copy of the out-of-line routine
-      perturb_block_other<NOPS, F32V ? 2 : (CROSS ? kLoopBlocks + 8 : kLoopBlocks)>(tab, t, b, x[0], x[1], op[0],
-                                                                                   op[1]);
-    }
-    if (bn >= blk_total) break;
-    b = bn;
-    t = c.t;
-    dt = c.dt;
-    vd = c.vd;
-    kind = kindn;
-    p = pn;
+// ---------------------------------------------------------------------------
+// One 32-byte item of theta per thread, every kind of tensor in one launch.
+//
+// Bound: HBM (2 x the list's bytes). A CTA is 256 threads of 32 registers, so
+// an SM holds 2048 threads, each with one 256-bit load and store in flight,
+// and the CTAs come in order, where a persistent grid of 1024 threads per SM
+// had each prefetch its next block. Before -> after, OPT-1.3B-shaped set (2 d B =
+// 5.26 GB in bf16; a plain copy was measured at 6794 GB/s):
+//   one operation    bf16 783 -> 740 us (7110 GB/s), fp32 1650 -> 1474 us
+//   two operations   bf16 807 -> 732 us (7190 GB/s), fp32 1592 -> 1472 us
+//   as slices of one flat buffer, bf16: 860 -> 736 us, two operations 903 -> 809
+// two operations whose probes fall in two groups of 8 (Qwen3-8B-shaped layers)
+// 1192 -> 1156 us; 200 tensors of 40 M bf16 weights 33 -> 23 us, of 1 M 12.9 ->
+// 7.5 us; 12 fp32 tensors of 270 k weights 8.5 -> 5.5 us.
+// What an item costs besides its elements has to be small for that: its tensor
+// is found from a hint (one constant load and a compare; a binary search per
+// warp took 832 us), positions are 32-bit, rounds 0-1 of Philox are split
+// (philox_start), the load is issued before the Philox call, and what only a
+// partial item needs is computed there (1104 against 1031 us for two
+// operations). Not adopted: 4, 8 or 16 items per warp with the next one
+// prefetched (865, 808, 791 us).
+//
+// Tensors off the 32-byte grid (views at an element offset) move in their
+// aligned 32-byte chunks: chunk i holds elements 16 i - a .. 16 i - a + 15 (8 of
+// fp32; a = the base's distance from the boundary below it, in elements), the
+// tail of one block (half block) and the head of the next, whose signs come
+// from the neighbouring lane (item_signs).
+//
+// HIU: the launch's virtual blocks share the counter's high word (any launch
+// below 2^36 weights); otherwise all ten rounds run.
+// ---------------------------------------------------------------------------
+// An item at p. full: its sixteen (eight) elements are in v; otherwise those of
+// the tensor are loaded here, together.
+template <uint8_t DT, int NOPS>
+__device__ __forceinline__ void items_16(char* p, bool full, const ItemsEntry& e, int32_t i, uint32_t (&v)[8],
+                                         const uint4 (&x)[2], const PerturbOp (&op)[2]) {
+  uint16_t* q = reinterpret_cast<uint16_t*>(p);
+  int lo = 0, hi = 0;
+  if (!full) {
+    item_range(e, i, &lo, &hi);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      v[r] = vn[r];
-      w[r] = wn[r];
+      const uint32_t l = 2 * r >= lo && 2 * r < hi ? q[2 * r] : 0u;
+      const uint32_t h = 2 * r + 1 >= lo && 2 * r + 1 < hi ? q[2 * r + 1] : 0u;
+      v[r] = l | (h << 16);
+    }
+  }
+  perturb_regs16<DT, NOPS>(v, x, op);
+  if (full) {
+    st256(p, v);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      if (2 * r >= lo && 2 * r < hi) q[2 * r] = static_cast<uint16_t>(v[r]);
+      if (2 * r + 1 >= lo && 2 * r + 1 < hi) q[2 * r + 1] = static_cast<uint16_t>(v[r] >> 16);
     }
   }
 }
 
-// By runs: while a thread's next blocks (b, b + stride, ... below end) lie in
-// the full, aligned 16-bit region of its current tensor they go through the
-// tight loop of perturb_run16; any other block (fp32, a partial last block,
-// an unaligned tensor) is handled on its own.
-template <int NOPS, int TAG, bool CROSS = false>
-__device__ __forceinline__ void perturb_runs_range(const PerturbParams& P, const PerturbOp (&op)[2], bool same_ctr,
-                                                   uint32_t b, uint32_t end, uint32_t stride) {
-  const TensorTable& tab = P.tab;
-  Cursor c;
-  c.t = 0;
-  bool seeked = false;
-  while (b < end) {
-    if (!seeked || b >= c.te) {
-      cursor_seek(tab, c, b);
-      seeked = true;
-    }
-    const int64_t vb = tab.blk_base + (b - c.vd);  // virtual block: the Philox counter
-    if (b - c.tb < c.n16) {
-      const uint32_t stop = min(c.tb + c.n16, end);
-      const uint32_t n = (stop - b + stride - 1) / stride;  // this thread's blocks in the region
-      uint16_t* p = c.tp + static_cast<size_t>(b - c.tb) * 16;
-      const size_t pstride = static_cast<size_t>(stride) * 16;
-      if (c.dt == kBF16)
-        perturb_run16<NOPS, kBF16, CROSS>(p, n, pstride, vb, stride, op, same_ctr, P.keys);
-      else
-        perturb_run16<NOPS, kF16, CROSS>(p, n, pstride, vb, stride, op, same_ctr, P.keys);
-      b += n * stride;
-    } else {
-      uint4 x[2];
-      x[0] = block_bits(vb, op[0].ctr2, P.keys);
-      x[1] = x[0];
-      if (NOPS == 2 && !same_ctr) x[1] = block_bits(vb, op[1].ctr2, P.keys);
-      perturb_block_other<NOPS, TAG>(tab, c.t, b, x[0], x[1], op[0], op[1]);
-      b += stride;
-    }
+template <int NOPS>
+__device__ __forceinline__ void items_32(char* p, bool full, const ItemsEntry& e, int32_t i, uint32_t (&v)[8],
+                                         const uint4 (&x)[2], const PerturbOp (&op)[2]) {
+  uint32_t* q = reinterpret_cast<uint32_t*>(p);
+  int lo = 0, hi = 0;
+  if (!full) {
+    item_range(e, i, &lo, &hi);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = r >= lo && r < hi ? q[r] : 0u;
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+#pragma unroll
+    for (int o = 0; o < NOPS; ++o) v[r] = __float_as_uint(add_signed_mul(__uint_as_float(v[r]), x[o], r, op[o]));
+  }
+  if (full) {
+    st256(p, v);
+  } else {
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (r >= lo && r < hi) q[r] = v[r];
   }
 }
 
-// Grid-stride by runs. Fewer instructions per block than perturb_blocks, but
-// the lanes of a warp leave a run up to one iteration apart, which costs
-// most where runs are short (tensors of a few blocks per thread).
-template <int NOPS, bool CROSS = false>
-__device__ __forceinline__ void perturb_runs(const PerturbParams& P, const PerturbOp (&op)[2], bool same_ctr) {
-  const uint32_t stride = gridDim.x * blockDim.x;
-  perturb_runs_range<NOPS, CROSS ? kLoopRuns + 8 : kLoopRuns, CROSS>(
-      P, op, same_ctr, blockIdx.x * blockDim.x + threadIdx.x, P.tab.blk_total, stride);
-}
-
-// LOOP selects perturb_blocks (kLoopBlocks) or perturb_runs (kLoopRuns);
-// CROSS marks a two-op launch whose probes fall in two groups of 8. The
-// single-op pass (zo_perturb) always walks block by block (4.99 ms against
-// 5.56 ms by runs on the Qwen3-8B-shaped set, equal elsewhere). For the two-op
-// pass (zo_perturb2) the faster loop and grid depend on the parameter list
-// (OPT-30B-shaped: runs with 3 blocks per SM 18.54 ms, per block with 4
-// 18.72 ms; Qwen3-8B-shaped: 5.96 ms against 5.27 ms), so the host times the
-// candidates on the caller's own list; all give the same bits.
-template <int NOPS, int LOOP, bool F32V = false, bool CROSS = false>
-__global__ void __launch_bounds__(256) perturb_kernel(const __grid_constant__ PerturbParams P) {
+template <int NOPS, bool CROSS, bool HIU, int N>
+__global__ void __launch_bounds__(256) perturb_items_kernel(const __grid_constant__ ItemsParams<N> P) {
   if (P.status != nullptr && *P.status != 0) return;
   PerturbOp op[2] = {P.op[0], P.op[1]};
   if (P.coef != nullptr)
     op[0].nscale_bits = __float_as_uint(__double2float_rn(P.coef_mul * P.coef[P.probe])) ^ 0x80000000u;
-  const bool same_ctr = op[1].ctr2 == op[0].ctr2;
-  if (LOOP == kLoopBlocks)
-    perturb_blocks<NOPS, F32V, CROSS>(P, op, same_ctr);
-  else
-    perturb_runs<NOPS, CROSS>(P, op, same_ctr);
-}
-
-// ---------------------------------------------------------------------------
-// Unaligned tensors (kShift): the same perturbation over 32-byte aligned
-// chunks instead of Philox blocks, so every full chunk moves with 256-bit
-// accesses whatever the tensor's offset. Chunk c (elements 16c - a ..
-// 16c - a + 15) draws its signs from bytes 16 - a .. 31 - a of the 32 bytes
-// Philox(c - 1) ++ Philox(c). In a warp, lane l generates block
-// c0 - 1 + l and works on chunk c0 - 1 + l with the block below taken from
-// lane l - 1 by a shuffle: 32 Philox calls per 31 chunks, lane 0 only
-// generates. Chunks that cross the tensor's ends go element by element.
-// ---------------------------------------------------------------------------
-// A chunk across an end of the tensor, element by element (not inlined: it
-// is rare and would otherwise hold registers in the vector path).
-template <int NOPS, uint8_t DT>
-__device__ __noinline__ void shift_chunk_elements(void* base, int64_t n, int64_t e0, uint4 y0, uint4 y1,
-                                                  PerturbOp op0, PerturbOp op1) {
-  for (int p = 0; p < 16; ++p) {
-    const int64_t e = e0 + p;
-    if (e < 0 || e >= n) continue;
-    float th = add_signed(load_elem(base, DT, e), y0, p, op0);
-    if (NOPS == 2) th = add_signed(round_to_storage(DT, th), y1, p, op1);
-    store_elem(base, DT, e, th);
-  }
-}
-
-// Chunk c is the lane's own (lane > 0) and lies wholly inside the tensor.
-__device__ __forceinline__ bool shift_full(int lane, int64_t c, uint32_t a, int64_t n) {
-  return lane > 0 && c >= 1 && 16 * c - a + 16 <= n;
-}
-
-// One group of kShiftGroup chunks of tensor t (all lanes of the warp), as
-// kShiftSub rounds of 31 chunks. 16-bit chunks are software-pipelined: the
-// load of the lane's next chunk is issued before the current one is
-// computed (two 32-byte loads in flight per lane, as for fp32's two halves).
-template <int NOPS, uint8_t DT>
-__device__ __forceinline__ void shift_group(const PerturbParams& P, const PerturbOp (&op)[2], bool same_ctr, int t,
-                                            int64_t c_first) {
-  constexpr int kElem = DT == kF32 ? 4 : 2;
-  constexpr bool kAhead = DT != kF32;
-  constexpr int kWords = 16 * kElem / 4;  // 32-bit words per chunk: 8 (16-bit) or 16 (fp32)
-  const TensorTable& tab = P.tab;
-  const uintptr_t ptr = tab.ptr[t];
-  const int64_t n = tab.numel[t];
-  const uint32_t a = static_cast<uint32_t>(ptr & 31u) / kElem;  // 1..15 (16-bit) or 1..7 (fp32)
-  char* chunk0 = reinterpret_cast<char*>(ptr - (ptr & 31u));     // 32-byte aligned, a elements before the tensor
-  const int64_t nchunks = (n + a + 15) / 16;
-  const int64_t vb0 = virtual_block(tab, t, tensor_blk_begin(tab, t));  // virtual block of element 0
-  const int lane = static_cast<int>(threadIdx.x & 31u);
-  int64_t c = c_first + lane - 1;  // lane 0: the block below lane 1's chunk, no chunk of its own
-  bool full = shift_full(lane, c, a, n);
-  uint32_t v[kWords];
-  if (kAhead && full) ld256(chunk0 + c * (16 * kElem), *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-#pragma unroll 1
-  for (int s = 0; s < kShiftSub; ++s) {
-    const int64_t cn = c + kShiftLanes;
-    bool fulln = false;
-    uint32_t vn[kWords];
-    if (kAhead && s + 1 < kShiftSub) {
-      fulln = shift_full(lane, cn, a, n);
-      if (fulln) ld256(chunk0 + cn * (16 * kElem), *reinterpret_cast<uint32_t(*)[8]>(&vn[0]));
-    }
-    char* q = chunk0 + c * (16 * kElem);
-    if (!kAhead && full) {
-      ld256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-      ld256(q + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[kWords - 8]));
-    }
-    const int64_t vb = vb0 + c;
-    uint4 x[2], y[2];
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x, wb = b - lane;  // the warp's items lie in one tensor
+  if (wb >= P.total) return;
+  int t = P.hint[wb >> P.hint_shift];
+  while (wb >= P.e[t].end) ++t;
+  const ItemsEntry e = P.e[t];
+  const uint8_t dt = static_cast<uint8_t>(e.meta & kDtypeMask);
+  const bool f32 = dt == kF32, shift = (e.meta & kShift) != 0;
+  const uint32_t a = e.meta >> 16;
+  const ItemPlace k = item_place(e, b);
+  const int64_t vb = item_block(e, k.i);
+  char* p = reinterpret_cast<char*>(e.base) + static_cast<int64_t>(k.i) * 32;
+  uint32_t v[8];
+  // (two Philox calls: the load after them keeps a resident block more)
+  if (!CROSS && k.full) ld256(p, v);
+  uint4 x[2];
+  if constexpr (HIU) {
+    const BlockRound01 r = block_round01(static_cast<uint32_t>(vb), P.keys);
+    x[0] = philox_finish(philox_start(r, P.g[0]), P.keys);
+    x[1] = CROSS ? philox_finish(philox_start(r, P.g[1]), P.keys) : x[0];
+  } else {
     x[0] = block_bits(vb, op[0].ctr2, P.keys);
-    x[1] = x[0];
-    if (NOPS == 2 && !same_ctr) x[1] = block_bits(vb, op[1].ctr2, P.keys);
-    y[0] = window16(shfl_up4(x[0]), x[0], 16u - a);
-    y[1] = y[0];
-    if (NOPS == 2 && !same_ctr) y[1] = window16(shfl_up4(x[1]), x[1], 16u - a);
-    if (full) {
-      if constexpr (DT == kF32) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float th = add_signed_mul(__uint_as_float(v[i]), y[0], i, op[0]);
-          if (NOPS == 2) th = add_signed_mul(th, y[1], i, op[1]);
-          v[i] = __float_as_uint(th);
-        }
-        st256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-        st256(q + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[kWords - 8]));
-      } else {
-        perturb_regs16<DT, NOPS>(*reinterpret_cast<uint32_t(*)[8]>(&v[0]), y, op);
-        st256(q, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-      }
-    } else if (lane > 0 && c >= 0 && c < nchunks) {
-      shift_chunk_elements<NOPS, DT>(reinterpret_cast<void*>(ptr), n, 16 * c - a, y[0], y[1], op[0], op[1]);
-    }
-    c = cn;
-    if (kAhead) {
-      full = fulln;
-#pragma unroll
-      for (int r = 0; r < kWords; ++r) v[r] = vn[r];
-    } else {
-      full = shift_full(lane, c, a, n);
-    }
+    x[1] = CROSS ? block_bits(vb, op[1].ctr2, P.keys) : x[0];
   }
-}
-
-// One kernel per storage type (a shared one would hold the registers of all
-// three paths): the host launches it for each type its unaligned tensors
-// have, with grp_end counting only that type's tensors. Four blocks per SM
-// (64 registers, no spills): measured faster than three (80 registers) for
-// both the single- and the two-op pass.
-template <int NOPS, uint8_t DT>
-__global__ void __launch_bounds__(256, 4) perturb_shift_kernel(const __grid_constant__ ShiftParams S) {
-  const PerturbParams& P = S.p;
-  if (P.status != nullptr && *P.status != 0) return;
-  PerturbOp op[2] = {P.op[0], P.op[1]};
-  if (P.coef != nullptr)
-    op[0].nscale_bits = __float_as_uint(__double2float_rn(P.coef_mul * P.coef[P.probe])) ^ 0x80000000u;
-  const bool same_ctr = op[1].ctr2 == op[0].ctr2;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  int t = 0;
-  for (uint32_t g = warp; g < S.grp_total; g += nwarps) {  // the same g on every lane of the warp
-    while (g >= S.grp_end[t]) ++t;
-    const int64_t c_first = static_cast<int64_t>(g - (t == 0 ? 0u : S.grp_end[t - 1])) * kShiftGroup;
-    shift_group<NOPS, DT>(P, op, same_ctr, t, c_first);
-  }
+  x[0] = item_signs(x[0], f32, (k.i & 1) != 0, shift, a);
+  x[1] = CROSS ? item_signs(x[1], f32, (k.i & 1) != 0, shift, a) : x[0];
+  if (!k.act) return;
+  if (CROSS && k.full) ld256(p, v);
+  if (f32)
+    items_32<NOPS>(p, k.full, e, k.i, v, x, op);
+  else if (dt == kBF16)
+    items_16<kBF16, NOPS>(p, k.full, e, k.i, v, x, op);
+  else
+    items_16<kF16, NOPS>(p, k.full, e, k.i, v, x, op);
 }
 
 // ---------------------------------------------------------------------------
@@ -800,46 +523,37 @@ __global__ void probe_signs_kernel(RoundKeys keys, uint32_t q, uint32_t j, int64
 
 namespace zo {
 
-cudaError_t launch_perturb(const PerturbParams& p, int grid, int loop, bool f32v, cudaStream_t stream) {
-  const bool cross = p.nops == 2 && p.op[0].ctr2 != p.op[1].ctr2;
-  if (p.nops == 1 && f32v)
-    perturb_kernel<1, kLoopBlocks, true><<<grid, kThreads, 0, stream>>>(p);
-  else if (p.nops == 1)
-    perturb_kernel<1, kLoopBlocks><<<grid, kThreads, 0, stream>>>(p);
-  else if (loop == kLoopRuns && cross)
-    perturb_kernel<2, kLoopRuns, false, true><<<grid, kThreads, 0, stream>>>(p);
-  else if (loop == kLoopRuns)
-    perturb_kernel<2, kLoopRuns><<<grid, kThreads, 0, stream>>>(p);
-  else if (cross)
-    perturb_kernel<2, kLoopBlocks, false, true><<<grid, kThreads, 0, stream>>>(p);
+template <bool HIU, int N>
+void launch_items_cfg(const ItemsParams<N>& p, cudaStream_t stream) {
+  const int grid = static_cast<int>((p.total + (kThreads - 1u)) / kThreads);
+  if (p.nops == 1)
+    perturb_items_kernel<1, false, HIU, N><<<grid, kThreads, 0, stream>>>(p);
+  else if (p.op[0].ctr2 == p.op[1].ctr2)
+    perturb_items_kernel<2, false, HIU, N><<<grid, kThreads, 0, stream>>>(p);
   else
-    perturb_kernel<2, kLoopBlocks><<<grid, kThreads, 0, stream>>>(p);
+    perturb_items_kernel<2, true, HIU, N><<<grid, kThreads, 0, stream>>>(p);
+}
+
+template <int N>
+cudaError_t launch_perturb_items(const ItemsParams<N>& p, cudaStream_t stream) {
+  launch_items_cfg<true>(p, stream);
   return cudaGetLastError();
 }
+template cudaError_t launch_perturb_items(const ItemsParams<kItemsFew>& p, cudaStream_t stream);
+template cudaError_t launch_perturb_items(const ItemsParams<kItemsSome>& p, cudaStream_t stream);
+template cudaError_t launch_perturb_items(const ItemsParams<kItemsMany>& p, cudaStream_t stream);
+
+cudaError_t launch_perturb_items_any_high(const ItemsParams<kItemsMany>& p, cudaStream_t stream) {
+  launch_items_cfg<false>(p, stream);
+  return cudaGetLastError();
+}
+static_assert(sizeof(ItemsParams<kItemsMany>) <= 32764, "items table exceeds the kernel parameter space");
 
 static_assert(sizeof(PairParams) <= 32764, "pair table exceeds the kernel parameter space");
-static_assert(sizeof(ShiftParams) <= 32764 && sizeof(PairShiftParams) <= 32764,
+static_assert(sizeof(PairShiftParams) <= 32764,
               "shift table exceeds the kernel parameter space");
-static_assert(sizeof(PerturbParams) <= 32764 && sizeof(SmallUpdateParams) <= 32764,
+static_assert(sizeof(SmallUpdateParams) <= 32764,
               "tensor table exceeds the kernel parameter space");
-
-template <int NOPS>
-void launch_shift_nops(const ShiftParams& p, uint8_t dt, int grid, cudaStream_t stream) {
-  if (dt == kBF16)
-    perturb_shift_kernel<NOPS, kBF16><<<grid, kThreads, 0, stream>>>(p);
-  else if (dt == kF16)
-    perturb_shift_kernel<NOPS, kF16><<<grid, kThreads, 0, stream>>>(p);
-  else
-    perturb_shift_kernel<NOPS, kF32><<<grid, kThreads, 0, stream>>>(p);
-}
-
-cudaError_t launch_perturb_shift(const ShiftParams& p, uint8_t dt, int grid, cudaStream_t stream) {
-  if (p.p.nops == 2)
-    launch_shift_nops<2>(p, dt, grid, stream);
-  else
-    launch_shift_nops<1>(p, dt, grid, stream);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, int grid, cudaStream_t stream) {
   if (dt == kBF16 && moved)
@@ -858,27 +572,6 @@ cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, 
 cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream) {
   perturb_pair_kernel<<<grid, kThreads, 0, stream>>>(p);
   return cudaGetLastError();
-}
-
-cudaError_t perturb_blocks_per_sm(int nops, int loop, int* out) {
-  if (nops == 1)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_kernel<1, kLoopBlocks>, kThreads, 0);
-  if (loop == kLoopRuns)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_kernel<2, kLoopRuns>, kThreads, 0);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_kernel<2, kLoopBlocks>, kThreads, 0);
-}
-
-template <int NOPS>
-cudaError_t shift_bps_nops(uint8_t dt, int* out) {
-  if (dt == kBF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_shift_kernel<NOPS, kBF16>, kThreads, 0);
-  if (dt == kF16)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_shift_kernel<NOPS, kF16>, kThreads, 0);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_shift_kernel<NOPS, kF32>, kThreads, 0);
-}
-
-cudaError_t shift_blocks_per_sm(int nops, uint8_t dt, int* out) {
-  return nops == 2 ? shift_bps_nops<2>(dt, out) : shift_bps_nops<1>(dt, out);
 }
 
 cudaError_t pair_blocks_per_sm(int* out) {

@@ -132,11 +132,15 @@ __device__ __forceinline__ void lut8_apply32(uint32_t (&v)[16], const float (&ac
 __device__ __forceinline__ void lut8_apply_elements(const Lut8Block& k, const float (&acc)[16], const uint4& xp,
                                                     const UpdateParams& P, bool do_sum) {
   const uint8_t dt = k.fl & kDtypeMask;
+  float v[16];  // all loads before the first store: there are registers for it here
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    v[i] = k.e0 + i >= 0 && k.e0 + i < k.numel ? load_elem(k.base, dt, k.e0 + i) : 0.0f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
     const int64_t e = k.e0 + i;
     if (e < 0 || e >= k.numel) continue;
-    float th = load_elem(k.base, dt, e);
+    float th = v[i];
     if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
     if (do_sum) th = __fadd_rn(th, acc[i]);
     store_elem(k.base, dt, e, th);
@@ -266,46 +270,6 @@ __device__ __forceinline__ Lut8Block lut8_block_info(const TensorTable& tab, int
   return k;
 }
 
-// Philox4x32-10 with rounds 0 and 1 split by what they depend on, for a
-// launch whose virtual blocks share the counter's high word bhi (every launch
-// below 2^36 weights). The counter is (b_lo, bhi, q, 0). Round 0 multiplies
-// b_lo (per block) and q (per group); round 1 multiplies the word that came
-// from q and bhi (per group) and the one that came from b_lo (per block), so
-// both rounds' products are computed once per group (GroupRound01, shared by
-// every block) and once per block (BlockRound01, shared by the pair's two
-// groups); only their xors and rounds 2-9 are per (block, group). The output
-// equals philox10(b_lo, bhi, q, 0) bit for bit.
-struct BlockRound01 {
-  uint32_t lpa0;  // lo(M0 b_lo)
-  uint32_t hpb1;  // hi(M1 v), v = hi(M0 b_lo) ^ k1[0]
-  uint32_t lpb1;  // lo(M1 v)
-};
-__host__ __device__ __forceinline__ GroupRound01 group_round01(uint32_t q, uint32_t bhi, const RoundKeys& rk) {
-  const uint64_t pb0 = static_cast<uint64_t>(kPhiloxM1) * q;
-  const uint32_t u = static_cast<uint32_t>(pb0 >> 32) ^ bhi ^ rk.k0[0];
-  const uint64_t pa1 = static_cast<uint64_t>(kPhiloxM0) * u;
-  GroupRound01 g;
-  g.x0 = static_cast<uint32_t>(pb0) ^ rk.k0[1];
-  g.x2 = static_cast<uint32_t>(pa1 >> 32) ^ rk.k1[1];
-  g.lpa1 = static_cast<uint32_t>(pa1);
-  return g;
-}
-__device__ __forceinline__ BlockRound01 block_round01(uint32_t blo, const RoundKeys& rk) {
-  const uint64_t pa0 = static_cast<uint64_t>(kPhiloxM0) * blo;
-  const uint32_t v = static_cast<uint32_t>(pa0 >> 32) ^ rk.k1[0];
-  const uint64_t pb1 = static_cast<uint64_t>(kPhiloxM1) * v;
-  BlockRound01 k;
-  k.lpa0 = static_cast<uint32_t>(pa0);
-  k.hpb1 = static_cast<uint32_t>(pb1 >> 32);
-  k.lpb1 = static_cast<uint32_t>(pb1);
-  return k;
-}
-
-// A Philox call after its first two rounds.
-struct PhiloxState {
-  uint32_t c0, c1, c2, c3;
-};
-
 // A block's part of the counter: HIU, its round-0/1 products; otherwise the
 // counter itself.
 template <bool HIU>
@@ -316,7 +280,7 @@ struct BlockCounter<true> {
   // vr: the block's low word
   __device__ __forceinline__ BlockCounter(uint32_t vr, int64_t, const RoundKeys& rk) : k(block_round01(vr, rk)) {}
   __device__ __forceinline__ PhiloxState start(const GroupRound01& g, uint32_t, const RoundKeys&) const {
-    return {k.hpb1 ^ g.x0, k.lpb1, g.x2 ^ k.lpa0, g.lpa1};
+    return philox_start(k, g);
   }
 };
 template <>
@@ -335,12 +299,6 @@ struct BlockCounter<false> {
     return s;
   }
 };
-
-__device__ __forceinline__ uint4 philox_finish(PhiloxState s, const RoundKeys& rk) {
-#pragma unroll
-  for (int r = 2; r < 10; ++r) philox_round(s.c0, s.c1, s.c2, s.c3, rk.k0[r], rk.k1[r]);
-  return make_uint4(s.c0, s.c1, s.c2, s.c3);
-}
 
 // The words whose byte m holds the signs of probes 8q .. 8q + 7 of element m
 // under packing 8: bit 0 of every byte of eight Philox calls, call i moved to
@@ -920,28 +878,25 @@ template <int PRE, bool TWO, bool ANY>
 __device__ __noinline__ void small_elements(void* base, uint8_t dt, int64_t e0, int64_t numel, uint4 x0, uint4 xl,
                                             uint4 xp, uint32_t f0, uint32_t fl, bool do_sum, PerturbOp pre) {
   const int per = dt == kF32 ? 8 : 16;
-#pragma unroll 1
-  for (int i = 0; i < per; ++i) {
-    const int64_t e = e0 + i;
-    if (e < 0 || e >= numel) continue;
-    const uint32_t sel = 0x7604u | (static_cast<uint32_t>(i & 3) << 4);
-    float th = load_elem(base, dt, e);
-    float a = 0.0f, l = 0.0f, d = 0.0f;
+  const int lo = e0 < 0 ? static_cast<int>(-e0) : 0;
+  const int hi = static_cast<int>(min(static_cast<int64_t>(per), numel - e0));
+  map_elements<2>(base, dt, e0, lo, hi, [&](int m, int j, float v) {
+    float th = v, a = 0.0f, l = 0.0f, d = 0.0f;
     if (do_sum) {
-      if constexpr (TWO) a = lds_f32(__byte_perm(word_of(x0, i >> 2), f0, sel));
-      const uint32_t at = __byte_perm(word_of(xl, i >> 2), fl, sel);
+      const uint32_t sel = 0x7604u | (static_cast<uint32_t>(j) << 4);
+      if constexpr (TWO) a = lds_f32(__byte_perm(word_of(x0, m), f0, sel));
+      const uint32_t at = __byte_perm(word_of(xl, m), fl, sel);
       if constexpr (PRE == kPreTable)
         lds_pair(at, l, d);
       else
         l = lds_f32(at);
     }
     if (PRE != kPreNone) {
-      th = do_sum && PRE == kPreTable ? __fadd_rn(th, d) : add_signed(th, xp, i, pre);
+      th = do_sum && PRE == kPreTable ? __fadd_rn(th, d) : add_signed_word(th, word_of(xp, m), j, pre);
       th = round_to_storage(dt, th);
     }
-    if (do_sum) th = __fadd_rn(th, TWO ? __fadd_rn(a, l) : l);
-    store_elem(base, dt, e, th);
-  }
+    return do_sum ? __fadd_rn(th, TWO ? __fadd_rn(a, l) : l) : th;
+  });
 }
 
 // A warp's position in the table: its 32 items lie in one tensor.
@@ -1008,19 +963,8 @@ __device__ __forceinline__ SmallItem small_item(const TensorTable& tab, const Sm
   return k;
 }
 
-// The sign words of an item's elements from its block's Philox words.
-__device__ __forceinline__ uint4 small_window(const SmallCursor& c, const SmallItem& k, uint4 x) {
-  if ((c.fl & kDtypeMask) == kF32) {  // the same in all lanes
-    uint2 y = k.upper ? make_uint2(x.z, x.w) : make_uint2(x.x, x.y);
-    if (c.fl & kShift) {  // bytes 8 - a .. 15 - a of (the half below) ++ (this half), a = 1..7
-      const uint32_t b0 = __shfl_up_sync(0xFFFFFFFFu, y.x, 1), b1 = __shfl_up_sync(0xFFFFFFFFu, y.y, 1);
-      const uint32_t s = 8u - c.a, sh = 8u * (s & 3u);
-      const uint32_t w0 = s >= 4u ? b1 : b0, w1 = s >= 4u ? y.x : b1, w2 = s >= 4u ? y.y : y.x;
-      y = make_uint2(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh));
-    }
-    return make_uint4(y.x, y.y, 0u, 0u);
-  }
-  return (c.fl & kShift) ? window16(shfl_up4(x), x, 16u - c.a) : x;
+__device__ __forceinline__ uint4 small_window(const SmallCursor& c, const SmallItem& k, const uint4& x) {
+  return item_signs(x, (c.fl & kDtypeMask) == kF32, k.upper, (c.fl & kShift) != 0, c.a);
 }
 
 // ANY: the launch may hold fp32 tensors (numbered in half blocks) and tensors
