@@ -114,7 +114,7 @@ def measured_peaks():
 KERNEL_SOURCES = {
     "perturb_items_kernel<1>": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "perturb_items_kernel<2>": ("zo_device.cuh", "zo_stream_kernels.cu"),
-    "perturb_pair_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
+    "pair_items_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "update_lut8_kernel": ("zo_device.cuh", "zo_update_lut8.cu"),
 }
 
@@ -763,7 +763,7 @@ def run_zo(args):
     K, eps, d = ps.K, ps.eps, ps.d
     params = W.allocate_params(ps, device=dev, view_offset=args.view_offset)
     plist = zo.ParamList(params)
-    shifted = any(t.data_ptr() % 32 for t in params)   # the pair pass uses pair_shift_kernel
+    shifted = any(t.data_ptr() % 32 for t in params)   # views off the 32-byte grid
 
     def like_param(t):
         """A buffer for theta +- eps z_k laid out like t (same offset into its own allocation)."""
@@ -965,9 +965,8 @@ def run_zo(args):
     # the roofline is reported for the kernel with the largest share of the step
     n1, n2 = (K + 1, K - 1) if fused else ((0, 0) if pair else (3 * K, 0))
     if pair:
-        dom_kernel, dom_ms, dom_launches = ("pair_shift_kernel<*> (tensors off the 32-byte grid)" if shifted
-                                            else "perturb_pair_kernel"), pair_ms, my_probes
-        traffic, traffic_how = committed_traffic("perturb_pair_kernel", traffic_key)
+        dom_kernel, dom_ms, dom_launches = "pair_items_kernel", pair_ms, my_probes
+        traffic, traffic_how = committed_traffic("pair_items_kernel", traffic_key)
     elif n2 > 0 and n2 * perturb2_ms > n1 * perturb_ms:
         dom_kernel, dom_ms, dom_launches = "perturb_items_kernel<2> (zo_perturb2)", perturb2_ms, n2
         traffic, traffic_how = committed_traffic("perturb_items_kernel<2>", traffic_key)

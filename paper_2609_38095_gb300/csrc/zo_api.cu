@@ -67,11 +67,6 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
   return op;
 }
 
-// Resident blocks per SM of the pair pass: three of 256 threads stream fastest
-// (4 blocks per SM slower); pair_shift_kernel takes at most 64 registers.
-constexpr int kPairBlocksPerSm = 3;
-constexpr int kShiftBlocksPerSm = 4;
-
 // Packing-1 updates with at most this many probe groups keep both groups'
 // tables in shared memory for the whole launch (update_lut8_small_kernel);
 // all others walk the groups chunk by chunk (update_lut8_kernel).
@@ -80,7 +75,6 @@ constexpr int kSmallGroups = 2;
 // Per-device launch facts, filled once per device.
 struct DeviceInfo {
   int sms = 0;
-  int pair_bps = 0;                       // perturb_pair blocks per SM
   bool lut8_ready = false;                // the update kernels' shared-memory limits are raised
 };
 constexpr int kMaxDevices = 64;
@@ -98,10 +92,6 @@ int device_info(DeviceInfo** out) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
-    int bps = 0;
-    e = zo::pair_blocks_per_sm(&bps);
-    if (e != cudaSuccess) return cuda_fail(e, "occupancy(perturb_pair)");
-    d.pair_bps = bps < 1 ? 1 : (bps < kPairBlocksPerSm ? bps : kPairBlocksPerSm);
     d.sms = sms;
   }
   *out = &d;
@@ -235,13 +225,14 @@ int run_perturb(const zo_tensor* params, int32_t n, const PerturbPass& pp, cudaS
   zo::ItemsCursor cur;
   const auto launch = [&](auto& ip) -> cudaError_t {
     const zo::ItemsCursor from = cur;
-    if (zo::fill_items(ip, params, n, cur)) {
+    const auto no_more = [](auto&, int32_t, int64_t) {};
+    if (zo::fill_items(ip, params, n, cur, no_more)) {
       if (ip.n == 0) return cudaSuccess;
       set_pass(ip, pp);
       return zo::launch_perturb_items(ip, s);
     }
     cur = from;
-    zo::fill_items(tl_items_many, params, n, cur);
+    zo::fill_items(tl_items_many, params, n, cur, no_more);
     set_pass(tl_items_many, pp);
     return zo::launch_perturb_items_any_high(tl_items_many, s);
   };
@@ -255,102 +246,9 @@ int run_perturb(const zo_tensor* params, int32_t n, const PerturbPass& pp, cudaS
   return ZO_OK;
 }
 
-// Fill a pair table with tensors t0, t0+1, ... (same split rules as
-// fill_table).
-int32_t fill_pair_table(zo::PairTable& tab, const zo_tensor* theta, const zo_tensor* plus, const zo_tensor* minus,
-                        int32_t t0, int32_t n, int64_t blk_base, int64_t* nblocks) {
-  tab.n = 0;
-  tab.blk_base = blk_base;
-  int64_t b = 0;
-  int32_t t = t0;
-  for (; t < n && tab.n < zo::kMaxTensorsPerLaunch; ++t) {
-    const int64_t nb = (theta[t].numel + 15) / 16;
-    if (tab.n > 0 && b + nb >= zo::kMaxLaunchBlocks) break;
-    const int i = tab.n++;
-    b += nb;
-    tab.blk_end[i] = static_cast<uint32_t>(b);
-    tab.src[i] = reinterpret_cast<uint64_t>(theta[t].ptr);
-    tab.plus[i] = reinterpret_cast<uint64_t>(plus[t].ptr);
-    tab.minus[i] = reinterpret_cast<uint64_t>(minus[t].ptr);
-    tab.last[i] = static_cast<uint8_t>(theta[t].numel - 16 * (nb > 0 ? nb - 1 : 0));  // 1..16 (0 if empty)
-    uint8_t fl = static_cast<uint8_t>(theta[t].dtype);
-    if ((tab.src[i] | tab.plus[i] | tab.minus[i]) % 32 == 0) fl |= zo::kVec32;
-    tab.flags[i] = fl;
-  }
-  tab.blk_total = static_cast<uint32_t>(b);
-  *nblocks = b;
-  return t;
-}
-
-// Tensors of a pair launch for pair_shift_kernel: fp32 tensors whose three
-// pointers share their offset from the 32-byte grid, and 16-bit tensors not
-// all 32-byte aligned whose plus and minus share theirs (theta may sit at
-// another, the "moved" kernel); the others keep perturb_pair_kernel's paths.
-// Returns a bit mask of (storage type, moved) classes: bit dt + 3 * moved.
-bool pair_moved(const zo::PairTable& tab, int i) { return tab.src[i] % 32 != tab.plus[i] % 32; }
-
-unsigned mark_pair_shift(zo::PairTable& tab, bool* main_work) {
-  unsigned classes = 0;
-  *main_work = false;
-  for (int i = 0; i < tab.n; ++i) {
-    const uint32_t begin = i == 0 ? 0u : tab.blk_end[i - 1];
-    if (tab.blk_end[i] == begin) continue;  // empty
-    const uint8_t dt = tab.flags[i] & zo::kDtypeMask;
-    const bool outs = tab.plus[i] % 32 == tab.minus[i] % 32;
-    const bool moved = pair_moved(tab, i);
-    const bool take = dt == zo::kF32 ? (outs && !moved) : (outs && !(tab.flags[i] & zo::kVec32));
-    if (take) {
-      tab.flags[i] |= zo::kShift;
-      classes |= 1u << (dt + 3 * (moved ? 1 : 0));
-    } else {
-      *main_work = true;
-    }
-  }
-  return classes;
-}
-
-thread_local zo::PairShiftParams tl_pair_shift;
-
-// Launch pair_shift_kernel over the flagged tensors of type dt whose theta
-// is (moved) or is not at another offset than the outputs, in batches of
-// kMaxPairShift entries.
-int run_pair_shift(const zo::PairParams& pp, uint8_t dt, bool moved, DeviceInfo* d, cudaStream_t s) {
-  zo::PairShiftParams& S = tl_pair_shift;
-  S.keys = pp.keys;
-  S.op = pp.op;
-  const zo::PairTable& tab = pp.tab;
-  const uint32_t esz = dt == zo::kF32 ? 4 : 2;
-  int i = 0;
-  while (i < tab.n) {
-    S.n = 0;
-    uint32_t groups = 0;
-    for (; i < tab.n && S.n < zo::kMaxPairShift; ++i) {
-      const uint8_t fl = tab.flags[i];
-      if (!(fl & zo::kShift) || (fl & zo::kDtypeMask) != dt || pair_moved(tab, i) != moved) continue;
-      const uint32_t begin = i == 0 ? 0u : tab.blk_end[i - 1];
-      const int64_t numel = static_cast<int64_t>(tab.blk_end[i] - begin - 1) * 16 + tab.last[i];
-      const int64_t a = static_cast<int64_t>(tab.plus[i] % 32) / esz;  // chunks follow the outputs
-      const int64_t chunks = (numel + a + 15) / 16;
-      const int j = S.n++;
-      S.src[j] = tab.src[i];
-      S.plus[j] = tab.plus[i];
-      S.minus[j] = tab.minus[i];
-      S.numel[j] = numel;
-      S.vb0[j] = tab.blk_base + begin;
-      groups += static_cast<uint32_t>((chunks + zo::kShiftGroup - 1) / zo::kShiftGroup);
-      S.grp_end[j] = groups;
-    }
-    if (S.n == 0) break;
-    S.grp_total = groups;
-    const int64_t want = (static_cast<int64_t>(groups) * 32 + zo::kThreads - 1) / zo::kThreads;
-    const int64_t cap = static_cast<int64_t>(d->sms) * kShiftBlocksPerSm;
-    cudaError_t e = zo::launch_pair_shift(S, dt, moved, static_cast<int>(want < cap ? want : cap), s);
-    if (e != cudaSuccess) return cuda_fail(e, "pair_shift_kernel");
-  }
-  return ZO_OK;
-}
-
-thread_local zo::PairParams tl_pair;
+thread_local zo::PairItemsParams<zo::kItemsFew> tl_pair_few;
+thread_local zo::PairItemsParams<zo::kItemsSome> tl_pair_some;
+thread_local zo::PairItemsParams<zo::kPairItemsMany> tl_pair_many;
 thread_local zo::SmallUpdateParams tl_update;
 
 }  // namespace
@@ -439,30 +337,24 @@ int zo_perturb_pair(const zo_tensor* theta, const zo_tensor* plus, const zo_tens
     if (theta[t].numel > 0 && plus[t].ptr == minus[t].ptr) return ZO_ERR_ARG;
   }
   if (n_tensors == 0) return ZO_OK;
-  DeviceInfo* d = nullptr;
-  if ((rc = device_info(&d)) != ZO_OK) return rc;
-  zo::PairParams& pp = tl_pair;
-  pp.keys = expand_keys(seed);
-  pp.op = make_op(probe, scale, packing);
-  int64_t blk = 0;
-  for (int32_t t0 = 0; t0 < n_tensors;) {
-    int64_t nb = 0;
-    t0 = fill_pair_table(pp.tab, theta, plus, minus, t0, n_tensors, blk, &nb);
-    if (nb > 0) {
-      bool main_work = false;
-      const unsigned shift_types = mark_pair_shift(pp.tab, &main_work);
-      if (main_work) {
-        cudaError_t e = zo::launch_perturb_pair(pp, grid_for(nb, d->sms, d->pair_bps),
-                                                static_cast<cudaStream_t>(stream));
-        if (e != cudaSuccess) return cuda_fail(e, "perturb_pair_kernel");
-      }
-      for (unsigned cls = 0; cls < 6; ++cls) {
-        if (!(shift_types & (1u << cls))) continue;
-        const uint8_t dt = static_cast<uint8_t>(cls % 3);
-        if ((rc = run_pair_shift(pp, dt, cls >= 3, d, static_cast<cudaStream_t>(stream))) != ZO_OK) return rc;
-      }
-    }
-    blk += nb;
+  zo::ItemsCursor cur;
+  const auto launch = [&](auto& ip) -> cudaError_t {
+    const bool one_high = zo::fill_items(ip, plus, n_tensors, cur, [&](auto& e, int32_t t, int64_t bytes) {
+      e.src = static_cast<uint64_t>(reinterpret_cast<uintptr_t>(theta[t].ptr)) + static_cast<uint64_t>(bytes);
+      e.minus = static_cast<uint64_t>(reinterpret_cast<uintptr_t>(minus[t].ptr)) + static_cast<uint64_t>(bytes);
+    });
+    if (ip.n == 0) return cudaSuccess;
+    ip.keys = expand_keys(seed);
+    ip.op = make_op(probe, scale, packing);
+    ip.g = zo::group_round01(ip.op.ctr2, static_cast<uint32_t>(static_cast<uint64_t>(ip.e[0].vb) >> 32), ip.keys);
+    return zo::launch_pair_items(ip, one_high, static_cast<cudaStream_t>(stream));
+  };
+  while (cur.t < n_tensors) {
+    const int32_t left = n_tensors - cur.t;
+    const cudaError_t e = left <= zo::kItemsFew    ? launch(tl_pair_few)
+                          : left <= zo::kItemsSome ? launch(tl_pair_some)
+                                                   : launch(tl_pair_many);
+    if (e != cudaSuccess) return cuda_fail(e, "pair_items_kernel");
   }
   return ZO_OK;
 }

@@ -73,13 +73,10 @@ struct PerturbOp {
 };
 
 // Tensors off the 32-byte grid are worked on in 32-byte aligned chunks, 31 per
-// warp (lane 0 only generates the block below the first); the pair pass counts
-// them in groups of kShiftGroup chunks.
+// warp (lane 0 only generates the block below the first).
 constexpr int kShiftLanes = 31;
-constexpr int kShiftSub = 4;                        // rounds of 31 chunks per group
-constexpr int kShiftGroup = kShiftLanes * kShiftSub;
 
-// Table of a launch of perturb_items_kernel. Work is numbered in 32-byte items
+// Table of a launch by items (perturb_items_kernel). Work is numbered in 32-byte items
 // (sixteen 16-bit or eight fp32 elements), tensors starting on multiples of 32;
 // a tensor off the 32-byte grid by a elements takes 32 items per 31 of its
 // aligned 32-byte chunks. A tensor's fields lie together, and the tensor of an
@@ -141,6 +138,7 @@ __host__ __device__ __forceinline__ void item_range(const ItemsEntry& e, int32_t
 
 template <int N>
 struct ItemsParams {
+  static constexpr int kEntries = N;
   ItemsEntry e[N];       // non-empty tensors
   uint16_t hint[kItemsHints];
   int32_t n;
@@ -156,46 +154,28 @@ struct ItemsParams {
   const int32_t* status;   // optional: skip everything unless *status == 0
 };
 
-// Out-of-place pair of perturbations (zo_perturb_pair): theta is read once
-// and theta + scale z_k, theta - scale z_k are written to two other lists of
-// the same shapes. Three pointer arrays per tensor: to keep 1024 tensors per
-// launch inside the parameter space, a tensor's size is stored as its block
-// range (blk_end) plus the element count of its last block.
-struct PairTable {
-  int32_t n;
-  uint32_t blk_total;
-  int64_t blk_base;
-  uint32_t blk_end[kMaxTensorsPerLaunch];
-  uint64_t src[kMaxTensorsPerLaunch];    // theta
-  uint64_t plus[kMaxTensorsPerLaunch];   // receives rn(theta + scale z)
-  uint64_t minus[kMaxTensorsPerLaunch];  // receives rn(theta - scale z)
-  uint8_t last[kMaxTensorsPerLaunch];    // elements in the tensor's last block, 1..16
-  uint8_t flags[kMaxTensorsPerLaunch];   // dtype | kVec32 (all three pointers 32-byte aligned)
+// Out-of-place pair of perturbations (zo_perturb_pair): theta is read once and
+// theta + scale z_k, theta - scale z_k are written to two other lists of the
+// same shapes. Items are plus's; src and minus are where the same elements of
+// the item at `base` lie in theta and in minus.
+constexpr int kPairItemsMany = 640;
+
+struct PairItemsEntry : ItemsEntry {
+  uint64_t src;
+  uint64_t minus;
 };
 
-// Tensors of a pair launch streamed in 32-byte aligned chunks by
-// pair_shift_kernel (as perturb_shift_kernel): fp32 tensors, and 16-bit
-// tensors whose three pointers are off the 32-byte grid by the same amount.
-// Compact per-tensor entries, one storage type per launch.
-constexpr int kMaxPairShift = 512;
-
-struct PairShiftParams {
+template <int N>
+struct PairItemsParams {
+  static constexpr int kEntries = N;
+  PairItemsEntry e[N];
+  uint16_t hint[kItemsHints];
+  int32_t n;
+  int32_t hint_shift;
+  uint32_t total;
   RoundKeys keys;
   PerturbOp op;
-  int32_t n;
-  uint32_t grp_total;
-  uint64_t src[kMaxPairShift];
-  uint64_t plus[kMaxPairShift];
-  uint64_t minus[kMaxPairShift];
-  int64_t numel[kMaxPairShift];
-  int64_t vb0[kMaxPairShift];       // virtual block of the tensor's element 0
-  uint32_t grp_end[kMaxPairShift];  // one past the tensor's last group of kShiftGroup chunks
-};
-
-struct PairParams {
-  PairTable tab;
-  RoundKeys keys;
-  PerturbOp op;            // probe and +scale's sign flip, as for zo_perturb
+  GroupRound01 g;
 };
 
 struct UpdateParams {
@@ -316,29 +296,8 @@ __device__ __forceinline__ void st256(void* p, const uint32_t (&r)[8]) {
                : "memory");
 }
 
-// Sixteen 16-bit elements at an address that is only 2-byte aligned (a view
-// at an odd offset), element 2r in the low half of v[r]: the widest accesses
-// the address allows, all loads issued before any value is used.
-__device__ __forceinline__ void ld16x16(const uint16_t* p, uint32_t (&v)[8]) {
-  const uintptr_t a = reinterpret_cast<uintptr_t>(p);
-  if ((a & 15u) == 0) {
-    const uint4* q = reinterpret_cast<const uint4*>(p);
-    const uint4 lo = q[0], hi = q[1];
-    v[0] = lo.x; v[1] = lo.y; v[2] = lo.z; v[3] = lo.w;
-    v[4] = hi.x; v[5] = hi.y; v[6] = hi.z; v[7] = hi.w;
-  } else if ((a & 3u) == 0) {
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(p);
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = w[r];
-  } else {
-    uint16_t h[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) h[i] = p[i];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = static_cast<uint32_t>(h[2 * r]) | (static_cast<uint32_t>(h[2 * r + 1]) << 16);
-  }
-}
-
+// Thirty-two bytes to an address that is only 2-byte aligned (a view at an odd
+// offset): the widest accesses it allows.
 __device__ __forceinline__ void st16x16(uint16_t* p, const uint32_t (&v)[8]) {
   const uintptr_t a = reinterpret_cast<uintptr_t>(p);
   if ((a & 15u) == 0) {

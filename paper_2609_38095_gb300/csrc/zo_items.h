@@ -1,4 +1,5 @@
-// zo_items.h -- host-side planning of perturb_items_kernel's tables (ItemsParams).
+// zo_items.h -- host-side planning of the tables of the launches by items
+// (perturb_items_kernel, pair_items_kernel).
 #pragma once
 
 #include <cstdint>
@@ -22,11 +23,14 @@ struct ItemsCursor {
 constexpr int64_t kItemsPiece = INT64_C(1) << 30;
 constexpr int64_t kItemsLaunch = INT64_C(1) << 31;
 
-// Fill `ip` from `cur` on, as far as its entries and `launch` items go. Returns
+// Fill `ip` (ItemsParams, PairItemsParams) from `cur` on, as far as its entries
+// and `launch` items go; more(entry, tensor, bytes) sets what an entry has
+// besides, `bytes` being the entry's base minus the tensor's address. Returns
 // whether the launch's virtual blocks share the counter's high word.
-template <int N>
-bool fill_items(ItemsParams<N>& ip, const zo_tensor* params, int32_t n, ItemsCursor& cur, int64_t piece = kItemsPiece,
-                int64_t launch = kItemsLaunch) {
+template <class Params, class More>
+bool fill_items(Params& ip, const zo_tensor* params, int32_t n, ItemsCursor& cur, const More& more,
+                int64_t piece = kItemsPiece, int64_t launch = kItemsLaunch) {
+  constexpr int N = Params::kEntries;
   ip.n = 0;
   int64_t b = 0, last = 0;  // items so far, and the last virtual block
   while (cur.t < n) {
@@ -45,7 +49,7 @@ bool fill_items(ItemsParams<N>& ip, const zo_tensor* params, int32_t n, ItemsCur
     const int64_t end = start + (off == 0 ? take : (take + kShiftLanes - 1) / kShiftLanes * kLaunchAlign);
     if (ip.n > 0 && end > launch) break;
     b = end;
-    ItemsEntry& e = ip.e[ip.n++];
+    auto& e = ip.e[ip.n++];
     e.base = static_cast<uint64_t>(addr - addr % 32) + static_cast<uint64_t>(32 * cur.done);
     e.vb = cur.v + (p.dtype == ZO_F32 ? cur.done / 2 : cur.done);
     e.begin = static_cast<uint32_t>(start);
@@ -54,6 +58,7 @@ bool fill_items(ItemsParams<N>& ip, const zo_tensor* params, int32_t n, ItemsCur
     e.meta = static_cast<uint32_t>(p.dtype) | (off == 0 ? 0u : static_cast<uint32_t>(kShift)) |
              (cur.done == 0 ? 0u : kItemsCont) | static_cast<uint32_t>(take == left ? rem : 0) << 8 |
              static_cast<uint32_t>(off) << 16;
+    more(e, cur.t, static_cast<int64_t>(e.base - static_cast<uint64_t>(addr)));
     last = e.vb + take;
     cur.done += take;
     if (cur.done == items) {

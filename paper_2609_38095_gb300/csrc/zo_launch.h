@@ -24,9 +24,10 @@ template <int N>
 cudaError_t launch_perturb_items(const ItemsParams<N>& p, cudaStream_t stream);
 // The same when the launch's virtual blocks differ in the counter's high word.
 cudaError_t launch_perturb_items_any_high(const ItemsParams<kItemsMany>& p, cudaStream_t stream);
-cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream);
-// moved: theta at another offset from the 32-byte grid than plus and minus (16-bit only).
-cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, int grid, cudaStream_t stream);
+// The out-of-place pair; one_high: the launch's virtual blocks share the
+// counter's high word.
+template <int N>
+cudaError_t launch_pair_items(const PairItemsParams<N>& p, bool one_high, cudaStream_t stream);
 // Fused update: packing 1, at most two probe groups (K <= 16) and virtual
 // blocks that share the counter's high word; ...
 cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream);
@@ -36,7 +37,6 @@ cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cu
 cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream);
 cudaError_t lut8_prepare();  // raises both kernels' shared-memory limits (once per device)
 bool one_high_word(const TensorTable& tab);  // of the launch's virtual blocks
-cudaError_t pair_blocks_per_sm(int* out);
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,
                                uint8_t* out, int grid, cudaStream_t stream);
 cudaError_t launch_probe_signs(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,

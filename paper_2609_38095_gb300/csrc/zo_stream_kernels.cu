@@ -2,12 +2,8 @@
 // fused perturb (Algorithm 1, ApplyPackedPerturbation), the out-of-place pair
 // of perturbations and the debug views of a probe.
 //
-// The perturbation passes work on 32-byte items, one per thread
-// (perturb_items_kernel). The pair pass walks 16-element Philox blocks grid-
-// stride (one 256-bit load and two stores per block of an aligned 16-bit
-// tensor) and hands fp32 tensors and tensors off the 32-byte grid to
-// pair_shift_kernel when plus and minus share their offset, else takes
-// narrower accesses.
+// All passes work on 32-byte items, one per thread (perturb_items_kernel,
+// pair_items_kernel).
 #include "zo_device.cuh"
 
 namespace zo {
@@ -201,191 +197,6 @@ __device__ __forceinline__ void pair_regs16(const uint32_t (&v)[8], const uint4&
   }
 }
 
-__device__ __noinline__ void pair_block_other(const PairTable& tab, int t, uint32_t b, uint4 x, PerturbOp op) {
-  if (tab.flags[t] & kShift) return;  // pair_shift_kernel's
-  const uint32_t tb = t == 0 ? 0u : tab.blk_end[t - 1];
-  const int64_t e0 = static_cast<int64_t>(b - tb) * 16;
-  const int cnt = b + 1 == tab.blk_end[t] ? tab.last[t] : 16;
-  const uint8_t dt = tab.flags[t] & kDtypeMask;
-  const void* src = reinterpret_cast<const void*>(tab.src[t]);
-  void* pl = reinterpret_cast<void*>(tab.plus[t]);
-  void* mi = reinterpret_cast<void*>(tab.minus[t]);
-  if (cnt == 16 && dt != kF32) {  // a full block with an unaligned pointer among the three
-    uint32_t v[8], m[8];
-    ld16x16(static_cast<const uint16_t*>(src) + e0, v);
-    if (dt == kBF16)
-      pair_regs16<kBF16>(v, x, op, v, m);
-    else
-      pair_regs16<kF16>(v, x, op, v, m);
-    st16x16(static_cast<uint16_t*>(pl) + e0, v);
-    st16x16(static_cast<uint16_t*>(mi) + e0, m);
-    return;
-  }
-  for (int i = 0; i < cnt; ++i) {
-    const float th = load_elem(src, dt, e0 + i);
-    const float d = __uint_as_float(op.nscale_bits ^ sign_bit(x, i, op.bit));
-    store_elem(pl, dt, e0 + i, __fadd_rn(th, d));
-    store_elem(mi, dt, e0 + i, __fsub_rn(th, d));
-  }
-}
-
-// A thread's position in a pair table (as Cursor for TensorTable).
-struct PairCursor {
-  int t;
-  uint32_t tb, te, tfe;  // first block, one past the last, one past the last full vector block (else tb)
-  uint8_t dt;
-};
-
-__device__ __forceinline__ void pair_seek(const PairTable& tab, PairCursor& c, uint32_t b) {
-  while (b >= tab.blk_end[c.t]) ++c.t;
-  c.tb = c.t == 0 ? 0u : tab.blk_end[c.t - 1];
-  c.te = tab.blk_end[c.t];
-  c.dt = tab.flags[c.t] & kDtypeMask;
-  c.tfe = ((tab.flags[c.t] & kVec32) && c.dt != kF32) ? c.te - (tab.last[c.t] < 16 ? 1u : 0u) : c.tb;
-}
-
-// Grid-stride one block per iteration, the next block's theta load issued
-// before the current block is computed (the single-op perturb's loop).
-__global__ void __launch_bounds__(256) perturb_pair_kernel(const __grid_constant__ PairParams P) {
-  const PairTable& tab = P.tab;
-  const PerturbOp op = P.op;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= tab.blk_total) return;
-  PairCursor c;
-  c.t = 0;
-  pair_seek(tab, c, b);
-  int t = c.t;
-  uint8_t dt = c.dt;
-  size_t off = static_cast<size_t>(b - c.tb) * 16;
-  bool vec = b < c.tfe;
-  uint32_t v[8];
-  if (vec) ld256(reinterpret_cast<const uint16_t*>(tab.src[t]) + off, v);
-  while (true) {
-    const uint32_t bn = b + stride;
-    bool vecn = false;
-    size_t offn = 0;
-    uint32_t vn[8];
-    if (bn < tab.blk_total) {
-      if (bn >= c.te) pair_seek(tab, c, bn);
-      vecn = bn < c.tfe;
-      offn = static_cast<size_t>(bn - c.tb) * 16;
-      if (vecn) ld256(reinterpret_cast<const uint16_t*>(tab.src[c.t]) + offn, vn);
-    }
-    const int64_t vb = tab.blk_base + b;
-    const uint4 x = block_bits(vb, op.ctr2, P.keys);
-    if (vec) {
-      uint32_t m[8];
-      if (dt == kBF16)
-        pair_regs16<kBF16>(v, x, op, v, m);
-      else
-        pair_regs16<kF16>(v, x, op, v, m);
-      st256(reinterpret_cast<uint16_t*>(tab.plus[t]) + off, v);
-      st256(reinterpret_cast<uint16_t*>(tab.minus[t]) + off, m);
-    } else {
-      pair_block_other(tab, t, b, x, op);
-    }
-    if (bn >= tab.blk_total) break;
-    b = bn;
-    t = c.t;
-    dt = c.dt;
-    off = offn;
-    vec = vecn;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = vn[r];
-  }
-}
-
-// ---------------------------------------------------------------------------
-// The pair of perturbations in 32-byte aligned chunks (as perturb_shift_kernel;
-// a = 0 for aligned fp32 tensors, whose chunks are the blocks themselves).
-// ---------------------------------------------------------------------------
-template <uint8_t DT>
-__device__ __noinline__ void pair_chunk_elements(const void* src, void* pl, void* mi, int64_t n, int64_t e0, uint4 y,
-                                                 PerturbOp op) {
-  for (int p = 0; p < 16; ++p) {
-    const int64_t e = e0 + p;
-    if (e < 0 || e >= n) continue;
-    const float th = load_elem(src, DT, e);
-    const float d = __uint_as_float(op.nscale_bits ^ sign_bit(y, p, op.bit));
-    store_elem(pl, DT, e, __fadd_rn(th, d));
-    store_elem(mi, DT, e, __fsub_rn(th, d));
-  }
-}
-
-template <uint8_t DT>
-__device__ __forceinline__ void pair_shift_group(const PairShiftParams& S, int t, int64_t c_first) {
-  constexpr int kElem = DT == kF32 ? 4 : 2;
-  constexpr bool kAhead = DT != kF32;
-  constexpr int kWords = 16 * kElem / 4;
-  const PerturbOp& op = S.op;
-  const uintptr_t src = S.src[t];
-  const uint32_t off = static_cast<uint32_t>(src & 31u);  // the same for plus and minus
-  const uint32_t a = off / kElem;                        // 0..15 (16-bit) or 0..7 (fp32)
-  const char* s0 = reinterpret_cast<const char*>(src - off);
-  char* p0 = reinterpret_cast<char*>(S.plus[t] - off);
-  char* m0 = reinterpret_cast<char*>(S.minus[t] - off);
-  const int64_t n = S.numel[t];
-  const int64_t nchunks = (n + a + 15) / 16;
-  const int lane = static_cast<int>(threadIdx.x & 31u);
-  auto full_at = [&](int64_t c) { return lane > 0 && 16 * c >= a && 16 * c - a + 16 <= n; };
-  int64_t c = c_first + lane - 1;
-  bool full = full_at(c);
-  uint32_t v[kWords];
-  if (kAhead && full) ld256(s0 + c * (16 * kElem), *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-#pragma unroll 1
-  for (int s = 0; s < kShiftSub; ++s) {
-    const int64_t cn = c + kShiftLanes;
-    bool fulln = false;
-    uint32_t vn[kWords];
-    if (kAhead && s + 1 < kShiftSub) {
-      fulln = full_at(cn);
-      if (fulln) ld256(s0 + cn * (16 * kElem), *reinterpret_cast<uint32_t(*)[8]>(&vn[0]));
-    }
-    const int64_t cb = c * (16 * kElem);
-    if (!kAhead && full) {
-      ld256(s0 + cb, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-      ld256(s0 + cb + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[kWords - 8]));
-    }
-    const uint4 x = block_bits(S.vb0[t] + c, op.ctr2, S.keys);
-    const uint4 below = shfl_up4(x);
-    const uint4 y = a == 0 ? x : window16(below, x, 16u - a);
-    if (full) {
-      if constexpr (DT == kF32) {
-        uint32_t m[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float th = __uint_as_float(v[i]);
-          const float d = __uint_as_float(op.nscale_bits ^ sign_bit_mul(y, i, op));
-          v[i] = __float_as_uint(__fadd_rn(th, d));
-          m[i] = __float_as_uint(__fsub_rn(th, d));
-        }
-        st256(p0 + cb, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-        st256(p0 + cb + 32, *reinterpret_cast<uint32_t(*)[8]>(&v[8]));
-        st256(m0 + cb, *reinterpret_cast<uint32_t(*)[8]>(&m[0]));
-        st256(m0 + cb + 32, *reinterpret_cast<uint32_t(*)[8]>(&m[8]));
-      } else {
-        uint32_t m[8];
-        pair_regs16<DT>(*reinterpret_cast<uint32_t(*)[8]>(&v[0]), y, op, *reinterpret_cast<uint32_t(*)[8]>(&v[0]),
-                        m);
-        st256(p0 + cb, *reinterpret_cast<uint32_t(*)[8]>(&v[0]));
-        st256(m0 + cb, m);
-      }
-    } else if (lane > 0 && c >= 0 && c < nchunks) {  // a chunk across an end of the tensor
-      pair_chunk_elements<DT>(reinterpret_cast<const void*>(src), reinterpret_cast<void*>(S.plus[t]),
-                              reinterpret_cast<void*>(S.minus[t]), n, 16 * c - a, y, op);
-    }
-    c = cn;
-    if (kAhead) {
-      full = fulln;
-#pragma unroll
-      for (int r = 0; r < kWords; ++r) v[r] = vn[r];
-    } else {
-      full = full_at(c);
-    }
-  }
-}
-
 // Bytes bo .. bo + 31 (bo even, 0..30) of the 64-byte string lo ++ hi.
 __device__ __forceinline__ void window32(const uint32_t (&lo)[8], const uint32_t (&hi)[8], uint32_t bo,
                                          uint32_t (&out)[8]) {
@@ -405,72 +216,95 @@ __device__ __forceinline__ void window32(const uint32_t (&lo)[8], const uint32_t
   for (int i = 0; i < 8; ++i) out[i] = __funnelshift_r(e1[i], e1[i + 1], sh);
 }
 
-// 16-bit tensors whose theta sits at another offset from the 32-byte grid
-// than plus and minus: chunks follow the outputs, and theta's sixteen
-// elements of chunk c are taken from the aligned 32-byte segments of theta
-// that hold them (two, each also read by a neighbouring lane, whose second
-// read hits L1; one when they fill a segment exactly).
-template <uint8_t DT>
-__device__ __forceinline__ void pair_shift_group_moved(const PairShiftParams& S, int t, int64_t c_first) {
-  const PerturbOp& op = S.op;
-  const uintptr_t src = S.src[t];
-  const uint32_t off = static_cast<uint32_t>(S.plus[t] & 31u);  // the outputs' offset, shared by plus and minus
-  const uint32_t a = off / 2, a_src = static_cast<uint32_t>(src & 31u) / 2;
-  // theta element 16c - a sits at position d of theta's aligned segment c + dc
-  const uint32_t d = (a_src + 16u - a) & 15u;
-  const int64_t dc = a_src >= a ? 0 : -1;
-  const char* s0 = reinterpret_cast<const char*>(src - (src & 31u));
-  char* p0 = reinterpret_cast<char*>(S.plus[t] - off);
-  char* m0 = reinterpret_cast<char*>(S.minus[t] - off);
-  const int64_t n = S.numel[t];
-  const int64_t nchunks = (n + a + 15) / 16;
-  const int lane = static_cast<int>(threadIdx.x & 31u);
-#pragma unroll 1
-  for (int s = 0; s < kShiftSub; ++s) {
-    const int64_t c = c_first + s * kShiftLanes + lane - 1;
-    const bool full = lane > 0 && 16 * c >= a && 16 * c - a + 16 <= n;
+// The 32 bytes of theta that belong to an item, at any element offset: the one
+// or two aligned 32-byte segments that hold them (the shared one is also a
+// neighbouring lane's, whose read hits L1).
+__device__ __forceinline__ void ld_item(uint64_t src, uint32_t (&v)[8]) {
+  const uint32_t mis = static_cast<uint32_t>(src & 31u);  // the same in all lanes
+  if (mis == 0u) {
+    ld256(reinterpret_cast<const void*>(src), v);
+  } else {
     uint32_t lo[8], hi[8];
-    if (full) {  // the second segment only when the sixteen elements reach into it (d > 0)
-      const char* q = s0 + (c + dc) * 32;
-      ld256(q, lo);
-      if (d != 0) {
-        ld256(q + 32, hi);
-      } else {
+    ld256(reinterpret_cast<const void*>(src - mis), lo);
+    ld256(reinterpret_cast<const void*>(src - mis + 32u), hi);
+    window32(lo, hi, mis, v);
+  }
+}
+
+template <uint8_t DT>
+__device__ __forceinline__ void pair_item(const PairItemsEntry& e, const ItemPlace& k, const uint32_t (&v)[8],
+                                          const uint4& x, const PerturbOp& op) {
+  const int64_t at = static_cast<int64_t>(k.i) * 32;
+  if (k.full) {
+    uint32_t p[8], m[8];
+    if constexpr (DT == kF32) {
 #pragma unroll
-        for (int r = 0; r < 8; ++r) hi[r] = lo[r];
+      for (int r = 0; r < 8; ++r) {
+        const float d = __uint_as_float(op.nscale_bits ^ sign_bit_mul(x, r, op));
+        p[r] = __float_as_uint(__fadd_rn(__uint_as_float(v[r]), d));
+        m[r] = __float_as_uint(__fsub_rn(__uint_as_float(v[r]), d));
       }
+    } else {
+      pair_regs16<DT>(v, x, op, p, m);
     }
-    const uint4 x = block_bits(S.vb0[t] + c, op.ctr2, S.keys);
-    const uint4 below = shfl_up4(x);
-    const uint4 y = a == 0 ? x : window16(below, x, 16u - a);
-    if (full) {
-      uint32_t v[8], m[8];
-      window32(lo, hi, 2u * d, v);
-      pair_regs16<DT>(v, y, op, v, m);
-      st256(p0 + c * 32, v);
-      st256(m0 + c * 32, m);
-    } else if (lane > 0 && c >= 0 && c < nchunks) {  // a chunk across an end of the tensor
-      pair_chunk_elements<DT>(reinterpret_cast<const void*>(src), reinterpret_cast<void*>(S.plus[t]),
-                              reinterpret_cast<void*>(S.minus[t]), n, 16 * c - a, y, op);
+    st256(reinterpret_cast<void*>(e.base + at), p);
+    if ((e.minus & 31u) == 0u)
+      st256(reinterpret_cast<void*>(e.minus + at), m);
+    else
+      st16x16(reinterpret_cast<uint16_t*>(e.minus + at), m);
+    return;
+  }
+  int lo, hi;
+  item_range(e, k.i, &lo, &hi);
+  const void* src = reinterpret_cast<const void*>(e.src + at);
+#pragma unroll 1
+  for (int h = lo & ~3; h < hi; h += 4) {  // four loads before their first store
+    float th[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) th[j] = h + j >= lo && h + j < hi ? load_elem(src, DT, h + j) : 0.0f;
+    const uint32_t w = word_of(x, h >> 2);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (h + j < lo || h + j >= hi) continue;
+      const float d = signed_scale_word(w, j, op);
+      store_elem(reinterpret_cast<void*>(e.base + at), DT, h + j, __fadd_rn(th[j], d));
+      store_elem(reinterpret_cast<void*>(e.minus + at), DT, h + j, __fsub_rn(th[j], d));
     }
   }
 }
 
-// MOVED: every tensor of the launch has theta at another offset than plus
-// and minus (16-bit only); otherwise all three share it.
-template <uint8_t DT, bool MOVED>
-__global__ void __launch_bounds__(256, 4) pair_shift_kernel(const __grid_constant__ PairShiftParams S) {
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  int t = 0;
-  for (uint32_t g = warp; g < S.grp_total; g += nwarps) {  // the same g on every lane of the warp
-    while (g >= S.grp_end[t]) ++t;
-    const int64_t c_first = static_cast<int64_t>(g - (t == 0 ? 0u : S.grp_end[t - 1])) * kShiftGroup;
-    if constexpr (MOVED)
-      pair_shift_group_moved<DT>(S, t, c_first);
-    else
-      pair_shift_group<DT>(S, t, c_first);
-  }
+// One 32-byte item of plus per thread, as perturb_items_kernel. Bound: HBM (3 x
+// the list's bytes). Before (a persistent grid of three blocks per SM, and a
+// kernel of its own for fp32 and for tensors off the 32-byte grid) -> after:
+// an OPT-30B-shaped fp16 layer and its embedding 902 -> 839 us (7090 GB/s), as
+// slices of flat buffers 953 -> 838, as fp32 1896 -> 1673 us; Qwen3-8B-shaped
+// layers 1640 -> 1521 us.
+template <bool HIU, int N>
+__global__ void __launch_bounds__(256) pair_items_kernel(const __grid_constant__ PairItemsParams<N> P) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x, wb = b - lane;  // the warp's items lie in one tensor
+  if (wb >= P.total) return;
+  int t = P.hint[wb >> P.hint_shift];
+  while (wb >= P.e[t].end) ++t;
+  const PairItemsEntry e = P.e[t];
+  const uint8_t dt = static_cast<uint8_t>(e.meta & kDtypeMask);
+  const ItemPlace k = item_place(e, b);
+  const int64_t vb = item_block(e, k.i);
+  uint32_t v[8];
+  if (k.full) ld_item(e.src + static_cast<int64_t>(k.i) * 32, v);
+  uint4 x;
+  if constexpr (HIU)
+    x = philox_finish(philox_start(block_round01(static_cast<uint32_t>(vb), P.keys), P.g), P.keys);
+  else
+    x = block_bits(vb, P.op.ctr2, P.keys);
+  x = item_signs(x, dt == kF32, (k.i & 1) != 0, (e.meta & kShift) != 0, e.meta >> 16);
+  if (!k.act) return;
+  if (dt == kF32)
+    pair_item<kF32>(e, k, v, x, P.op);
+  else if (dt == kBF16)
+    pair_item<kBF16>(e, k, v, x, P.op);
+  else
+    pair_item<kF16>(e, k, v, x, P.op);
 }
 
 // ---------------------------------------------------------------------------
@@ -547,36 +381,24 @@ cudaError_t launch_perturb_items_any_high(const ItemsParams<kItemsMany>& p, cuda
   launch_items_cfg<false>(p, stream);
   return cudaGetLastError();
 }
-static_assert(sizeof(ItemsParams<kItemsMany>) <= 32764, "items table exceeds the kernel parameter space");
+static_assert(sizeof(ItemsParams<kItemsMany>) <= 32764 && sizeof(PairItemsParams<kPairItemsMany>) <= 32764,
+              "items table exceeds the kernel parameter space");
 
-static_assert(sizeof(PairParams) <= 32764, "pair table exceeds the kernel parameter space");
-static_assert(sizeof(PairShiftParams) <= 32764,
-              "shift table exceeds the kernel parameter space");
 static_assert(sizeof(SmallUpdateParams) <= 32764,
               "tensor table exceeds the kernel parameter space");
 
-cudaError_t launch_pair_shift(const PairShiftParams& p, uint8_t dt, bool moved, int grid, cudaStream_t stream) {
-  if (dt == kBF16 && moved)
-    pair_shift_kernel<kBF16, true><<<grid, kThreads, 0, stream>>>(p);
-  else if (dt == kF16 && moved)
-    pair_shift_kernel<kF16, true><<<grid, kThreads, 0, stream>>>(p);
-  else if (dt == kBF16)
-    pair_shift_kernel<kBF16, false><<<grid, kThreads, 0, stream>>>(p);
-  else if (dt == kF16)
-    pair_shift_kernel<kF16, false><<<grid, kThreads, 0, stream>>>(p);
+template <int N>
+cudaError_t launch_pair_items(const PairItemsParams<N>& p, bool one_high, cudaStream_t stream) {
+  const int grid = static_cast<int>((p.total + (kThreads - 1u)) / kThreads);
+  if (one_high)
+    pair_items_kernel<true, N><<<grid, kThreads, 0, stream>>>(p);
   else
-    pair_shift_kernel<kF32, false><<<grid, kThreads, 0, stream>>>(p);
+    pair_items_kernel<false, N><<<grid, kThreads, 0, stream>>>(p);
   return cudaGetLastError();
 }
-
-cudaError_t launch_perturb_pair(const PairParams& p, int grid, cudaStream_t stream) {
-  perturb_pair_kernel<<<grid, kThreads, 0, stream>>>(p);
-  return cudaGetLastError();
-}
-
-cudaError_t pair_blocks_per_sm(int* out) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, perturb_pair_kernel, kThreads, 0);
-}
+template cudaError_t launch_pair_items(const PairItemsParams<kItemsFew>& p, bool one_high, cudaStream_t stream);
+template cudaError_t launch_pair_items(const PairItemsParams<kItemsSome>& p, bool one_high, cudaStream_t stream);
+template cudaError_t launch_pair_items(const PairItemsParams<kPairItemsMany>& p, bool one_high, cudaStream_t stream);
 
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,
                                uint8_t* out, int grid, cudaStream_t stream) {

@@ -45,7 +45,7 @@ template <int N> int check(int round, std::mt19937& g) {
   const long long launch = round % 2 ? 64 + 2 * piece + pick(5000) : kItemsLaunch;
   static ItemsParams<N> ip;
   while (cur.t < n) {
-    const bool one = fill_items(ip, list.data(), n, cur, piece, launch);
+    const bool one = fill_items(ip, list.data(), n, cur, [](auto&, int32_t, int64_t) {}, piece, launch);
     if (!one) return fail("high word", round, cur.t, 0);
     if (ip.n == 0) { if (cur.t < n) return fail("nothing taken", round, cur.t, 0); break; }
     std::vector<ItemPlace> place(ip.total + 32);
