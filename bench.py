@@ -568,7 +568,7 @@ def run_tiny(args):
     ms_per_step = max_over_ranks(sum(a_.elapsed_time(b_) for a_, b_ in ev) / args.steps, world, dev)
     launches = q.library_launches_per_step()
     if schedule == "onepass":
-        calls = 3                                                            # C-ABI calls per step
+        calls = 2                                                            # C-ABI calls per step
     else:
         calls = 2 * K + 1 + (2 * K if schedule == "fused" else 3 * K) + 2
     host_us_per_call = 1e6 * statistics.median(host_s) / calls

@@ -331,8 +331,11 @@ int zo_perturb_quadratic_loss(float* theta, const float* a, int64_t n, uint64_t 
  * loss, theta <- rn(theta + eps z_k) (Algorithm 1's +eps, -2 eps, +eps per
  * probe), bit for bit the weights that zo_perturb gives on the one-tensor
  * fp32 list {theta, n, ZO_F32, packing}. theta and a are read once, theta is
- * written once; the step's preconditioner and update follow.
+ * written once. With c and status given, the same launch ends with what
+ * zo_precondition writes for these losses (K coefficients and the status word
+ * that zo_update honours); the step's update follows.
  *   losses     device, K rows (L+, L-, L0), the table zo_precondition takes
+ *   c, status  device, K fp64 and one int32, or both null
  *   eps        the scales are (float)eps and (float)(-2 eps)
  *   packing    0 = the process default (zo_set_packing), else 1 or 8
  *   workspace  device scratch of at least
@@ -343,13 +346,14 @@ int zo_perturb_quadratic_loss(float* theta, const float* a, int64_t n, uint64_t 
  * products lie in [2^-100, 2^100), else in fp64, the pairs summed as pairs up
  * to a CTA and in fp64 from there, in a fixed order (bit-reproducible for a
  * given device). The losses differ from zo_quadratic_loss's by rounding only.
- * Errors: ZO_ERR_ARG (n < 0, null pointers, K < 1, a scale not finite,
- * packing not 0/1/8), ZO_ERR_TOO_MANY_PROBES, ZO_ERR_ALIGN (theta, a not
+ * Errors: ZO_ERR_ARG (n < 0, null pointers, K < 1, a scale not finite, c
+ * without status or the reverse, eps <= 0 with c, packing not 0/1/8), ZO_ERR_TOO_MANY_PROBES, ZO_ERR_ALIGN (theta, a not
  * 4-byte aligned), ZO_ERR_WORKSPACE, ZO_ERR_CUDA.
  * ------------------------------------------------------------------------- */
 int64_t zo_quadratic_points_workspace_size(int32_t K);
 int zo_quadratic_points(float* theta, const float* a, int64_t n, uint64_t seed, int32_t packing, int32_t K, double eps,
-                        double* losses, void* workspace, int64_t workspace_bytes, void* stream);
+                        double* losses, double* c, int32_t* status, void* workspace, int64_t workspace_bytes,
+                        void* stream);
 
 /* ---------------------------------------------------------------------------
  * zo_quadratic_loss_static -- zo_quadratic_loss for callers that cannot

@@ -555,8 +555,10 @@ int64_t zo_quadratic_points_workspace_size(int32_t K) {
 }
 
 int zo_quadratic_points(float* theta, const float* a, int64_t n, uint64_t seed, int32_t packing, int32_t K, double eps,
-                        double* losses, void* workspace, int64_t workspace_bytes, void* stream) {
+                        double* losses, double* c, int32_t* status, void* workspace, int64_t workspace_bytes,
+                        void* stream) {
   if (n < 0 || losses == nullptr || (n > 0 && (theta == nullptr || a == nullptr)) || K < 1) return ZO_ERR_ARG;
+  if ((c == nullptr) != (status == nullptr) || (c != nullptr && !(eps > 0.0))) return ZO_ERR_ARG;
   if (K > ZO_MAX_PROBES) return ZO_ERR_TOO_MANY_PROBES;
   if (packing != 0 && packing != zo::kPacking1 && packing != zo::kPacking8) return ZO_ERR_ARG;
   const float scale = static_cast<float>(eps), mscale = static_cast<float>(-2.0 * eps);
@@ -572,7 +574,7 @@ int zo_quadratic_points(float* theta, const float* a, int64_t n, uint64_t seed, 
   uint32_t* ticket =
       reinterpret_cast<uint32_t*>(partial + (2 * static_cast<int64_t>(K) + 1) * zo::kQuadPointsMaxCtas);
   cudaError_t e = zo::launch_quad_points(theta, a, n, expand_keys(seed), packing != 0 ? packing : g_packing.load(), K,
-                                         scale, mscale, losses, partial, ticket, d->sms,
+                                         eps, losses, c, status, partial, ticket, d->sms,
                                          static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? ZO_OK : cuda_fail(e, "quad_points");
 }

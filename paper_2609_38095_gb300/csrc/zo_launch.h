@@ -55,10 +55,10 @@ cudaError_t launch_perturb_quad_loss(float* theta, const float* a, int64_t n, co
                                      double* partial, uint32_t* ticket, int max_partials, int num_sms,
                                      cudaStream_t stream);
 
-// Every forward point of a step: eps, meps the scales +eps and -2 eps; partial:
+// Every forward point of a step, and its coefficients when c is given; partial:
 // (2 K + 1) * kQuadPointsMaxCtas doubles; ticket: as above.
 cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const RoundKeys& keys, int packing, int K,
-                               float eps, float meps, double* losses, double* partial, uint32_t* ticket, int num_sms,
-                               cudaStream_t stream);
+                               double eps, double* losses, double* c, int32_t* status, double* partial,
+                               uint32_t* ticket, int num_sms, cudaStream_t stream);
 
 }  // namespace zo

@@ -16,7 +16,7 @@
 // (Dekker's product by fused multiply-add: a t = p + pe, p t = q + qe, term =
 // q + fma(pe, t, qe)) and summed into an fp32 pair with Knuth's two-sum, two
 // weights per packed fp32x2 operation. The products are exact while a stays
-// in [2^-40, 2^40] and |t| in [2^-30, 2^30] in magnitude; a thread whose
+// in [2^-40, 2^40] or 0 and |t| in [2^-30, 2^30] in magnitude; a thread whose
 // eight weights leave that range at a point (zeros, infinities, tiny or huge
 // weights) redoes the point weight by weight, adding terms whose products
 // leave the exact range in fp64. NaN needs no such care: it reaches the sum
@@ -30,8 +30,11 @@
 // workspace, reset by that CTA) folds the CTAs' fp64 partials in index order
 // and writes the loss table. No CTA waits for another; for a given size every
 // order is fixed, so the losses are bit-reproducible.
+#include <type_traits>
+
 #include "zo_device.cuh"
 #include "zo_launch.h"
+#include "zo_precond.cuh"
 
 namespace zo {
 
@@ -88,40 +91,43 @@ __device__ __forceinline__ Ds ds_sum(Ds a, Ds b) {
 
 constexpr float kMinA = 0x1p-40f, kMaxA = 0x1p40f, kMinT = 0x1p-30f, kMaxT = 0x1p30f;
 
-// The eight terms of one point as a pair; *ok: every |t| in [kMinT, kMaxT].
-// na = -a: the error of a product by one fused multiply-add needs the
-// product's negative, so -p = (-a) t and -q = (-p) t are carried along
-// instead of negating p and q. q is the rounded product p t + 0, with a zero
-// that the compiler cannot see: a packed multiply whose result is only added
-// is fused with those additions (ptxas does so in spite of .rn), and the sums
-// then lose q's rounding error twice over.
+// The eight terms of one point as a pair; with CHECK, *ok: every |t| in [kMinT,
+// kMaxT]. na = -a: the error of a product by one fused multiply-add needs the
+// product's negative, so p and -p are both formed, and the errors come out
+// negated (u = p - a t, w = q - p t, a term's low part is -(u t + w)). q is the
+// rounded product p t + 0, with a zero that the compiler cannot see: a packed
+// multiply whose result is only added is fused with those additions (ptxas
+// does so in spite of .rn), and the sums then lose q's rounding error twice
+// over.
+template <bool CHECK>
 __device__ __forceinline__ Ds point_terms(const f2 (&t)[kItem / 2], const f2 (&a)[kItem / 2], const f2 (&na)[kItem / 2],
                                           f2 zero, bool* ok) {
   f2 s, l;
   float mx = 0.0f, mn = 1.0f;
 #pragma unroll
   for (int i = 0; i < kItem / 2; ++i) {
-    const float2 tv = unpack_f2(t[i]);
-    mx = fmaxf(mx, fmaxf(fabsf(tv.x), fabsf(tv.y)));
-    mn = fminf(mn, fminf(fabsf(tv.x), fabsf(tv.y)));
+    if (CHECK) {
+      const float2 tv = unpack_f2(t[i]);
+      mx = fmaxf(mx, fmaxf(fabsf(tv.x), fabsf(tv.y)));
+      mn = fminf(mn, fminf(fabsf(tv.x), fabsf(tv.y)));
+    }
     const f2 p = mul2(a[i], t[i]);
     const f2 np = mul2(na[i], t[i]);
-    const f2 pe = fma2(a[i], t[i], np);  // a t - p, exact
+    const f2 u = fma2(na[i], t[i], p);
     const f2 q = fma2(p, t[i], zero);
-    const f2 nq = mul2(np, t[i]);
-    const f2 r = fma2(pe, t[i], fma2(p, t[i], nq));  // (a t - p) t + (p t - q)
+    const f2 r = fma2(u, t[i], fma2(np, t[i], q));  // minus the low part
     if (i == 0) {
       s = q;
-      l = r;
+      l = sub2(zero, r);
     } else {
       const f2 sn = add2(s, q);
       const f2 bb = sub2(sn, s);
       const f2 e = add2(sub2(s, sub2(sn, bb)), sub2(q, bb));
-      l = add2(l, add2(e, r));
+      l = add2(l, sub2(e, r));
       s = sn;
     }
   }
-  *ok = mx <= kMaxT && mn >= kMinT;
+  *ok = !CHECK || (mx <= kMaxT && mn >= kMinT);
   const float2 sv = unpack_f2(s), lv = unpack_f2(l);
   return ds_sum({sv.x, lv.x}, {sv.y, lv.y});
 }
@@ -148,6 +154,15 @@ __device__ __noinline__ Ds point_terms_any(const f2 (&t)[kItem / 2], const f2 (&
   }
   *wide = w;
   return sum;
+}
+
+// The coefficient of one probe as zo_precondition forms it (alpha = 0.1,
+// lambda_reg = 1, two-sided); false when a loss, the curvature or it is not
+// finite. Not inlined: pow would take registers from the loop over the probes.
+__device__ __noinline__ bool probe_coefficient(double lp, double lm, double l0, double eps, double* c) {
+  const double cv = probe_curvature(lp, lm, l0, eps);
+  *c = __dmul_rn(probe_weight(cv, 0.1, 1.0), central_difference(lp, lm, eps));
+  return isfinite(lp) && isfinite(lm) && isfinite(l0) && isfinite(cv) && isfinite(*c);
 }
 
 // Sum over a warp, fp64 (fixed tree), in every lane.
@@ -199,6 +214,10 @@ struct QuadPointsParams {
   double* partial;       // (2 K + 1) x gridDim.x
   uint32_t* ticket;      // zero before the launch; the last CTA zeroes it again
   float zero;            // 0.0f
+  float drift;           // (K + 1) 2^-21
+  double eps;            // for the coefficients
+  double* c;             // K coefficients and their status, or null
+  int32_t* status;
 };
 
 template <bool PACK8, bool VEC>
@@ -221,15 +240,19 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
   bool a_ok = true;
   int cnt = 0;
   f2 t[kItem / 2], a[kItem / 2], na[kItem / 2];
-  const auto point = [&](int slot) -> Ds {
+  const auto point = [&](auto check, int slot) -> Ds {
     bool ok;
-    Ds r = point_terms(t, a, na, zero, &ok);
-    ok = ok && a_ok;
-    if (__any_sync(0xFFFFFFFFu, !ok)) {
-      double w = 0.0;
-      if (!ok) r = point_terms_any(t, a, cnt, &w);
-      w = warp_sum(w);
-      if (lane == 0) wide_s[slot * warps + warp] = __dadd_rn(wide_s[slot * warps + warp], w);
+    Ds r = point_terms<decltype(check)::value>(t, a, na, zero, &ok);
+    if constexpr (decltype(check)::value) {
+      ok = ok && a_ok;
+      if (__any_sync(0xFFFFFFFFu, !ok)) {
+        double w = 0.0;
+        if (!ok) r = point_terms_any(t, a, cnt, &w);
+        if (__any_sync(0xFFFFFFFFu, w != 0.0)) {
+          w = warp_sum(w);
+          if (lane == 0) wide_s[slot * warps + warp] = __dadd_rn(wide_s[slot * warps + warp], w);
+        }
+      }
     }
     return r;
   };
@@ -240,8 +263,9 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
   };
 
   const int64_t items = (P.n + kItem - 1) / kItem;
+  // warps take 32 items each, first one per CTA, then a second, ..: few items still use every SM
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x + warp * 32; base < items; base += stride) {
+  for (int64_t base = (static_cast<int64_t>(warp) * gridDim.x + blockIdx.x) * 32; base < items; base += stride) {
     const int64_t item = base + lane;
     const int64_t e0 = item * kItem;
     cnt = static_cast<int>(max(static_cast<int64_t>(0), min(static_cast<int64_t>(kItem), P.n - e0)));
@@ -258,7 +282,8 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     } else {
 #pragma unroll
       for (int i = 0; i < kItem / 2; ++i) {
-        t[i] = pack_f2(2 * i < cnt ? P.theta[e0 + 2 * i] : 0.0f, 2 * i + 1 < cnt ? P.theta[e0 + 2 * i + 1] : 0.0f);
+        // past the end: a = 0, whose terms are exact zeros
+        t[i] = pack_f2(2 * i < cnt ? P.theta[e0 + 2 * i] : 1.0f, 2 * i + 1 < cnt ? P.theta[e0 + 2 * i + 1] : 1.0f);
         a[i] = pack_f2(2 * i < cnt ? P.a[e0 + 2 * i] : 0.0f, 2 * i + 1 < cnt ? P.a[e0 + 2 * i + 1] : 0.0f);
       }
     }
@@ -267,10 +292,11 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     for (int i = 0; i < kItem / 2; ++i) {
       const float2 y = unpack_f2(a[i]);
       na[i] = pack_f2(-y.x, -y.y);
-      a_ok = a_ok && fabsf(y.x) >= kMinA && fabsf(y.x) <= kMaxA && fabsf(y.y) >= kMinA && fabsf(y.y) <= kMaxA;
+      const float ax = fabsf(y.x), ay = fabsf(y.y);
+      a_ok = a_ok && (ax >= kMinA || ax == 0.0f) && ax <= kMaxA && (ay >= kMinA || ay == 0.0f) && ay <= kMaxA;
     }
     {
-      Ds r = point(16 * P.groups);
+      Ds r = point(std::true_type(), 16 * P.groups);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) r = ds_sum(r, shfl_xor_ds(r, off));
       if (lane == 0) store_sum(16 * P.groups, r);
@@ -278,6 +304,7 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     const int64_t b = item >> 1;
     const bool upper = (item & 1) != 0;  // words 2, 3 of the block's Philox output
     uint32_t w0 = 0, w1 = 0;
+    const auto probes = [&](auto check) {
 #pragma unroll 1
     for (int h = 0; 4 * h < P.K; ++h) {  // four probes at a time
       Ds v[8];
@@ -317,14 +344,31 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
           }
         };
         move(0u);
-        v[2 * j] = point(16 * (k >> 3) + 2 * (k & 7));
+        v[2 * j] = point(check, 16 * (k >> 3) + 2 * (k & 7));
         move(P.neps_bits ^ P.nmeps_bits);
-        v[2 * j + 1] = point(16 * (k >> 3) + 2 * (k & 7) + 1);
+        v[2 * j + 1] = point(check, 16 * (k >> 3) + 2 * (k & 7) + 1);
         move(0u);
       }
       const Ds r = butterfly8(v, lane);
       if ((lane & 3) == 0) store_sum(8 * h + (lane >> 2), r);
     }
+    };
+    // The points lie at theta +- eps up to the restores' drift (three roundings
+    // per probe, each at most 2^-24 of |theta| + 2 eps). Far enough from 0 for
+    // all of them, no point needs a check of its own.
+    bool far_ok = a_ok;
+    const float eps = fabsf(__uint_as_float(P.neps_bits)), drift = P.drift;
+#pragma unroll
+    for (int i = 0; i < kItem / 2; ++i) {
+      const float2 x = unpack_f2(t[i]);
+      const float mx = fabsf(x.x) + 2.0f * eps, my = fabsf(x.y) + 2.0f * eps;
+      far_ok = far_ok && fabsf(fabsf(x.x) - eps) >= fmaf(drift, mx, 2.0f * kMinT) && mx <= 0.5f * kMaxT &&
+               fabsf(fabsf(x.y) - eps) >= fmaf(drift, my, 2.0f * kMinT) && my <= 0.5f * kMaxT;
+    }
+    if (__any_sync(0xFFFFFFFFu, !far_ok))
+      probes(std::true_type());
+    else
+      probes(std::false_type());
     if (VEC && cnt == kItem) {
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
@@ -364,6 +408,8 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
   __syncthreads();
   if (!last_s) return;
   __threadfence();
+  double* loss_s = reinterpret_cast<double*>(smem);  // the warps' sums are done with: 2 K + 1 losses, K coefficients
+  double* c_s = loss_s + points;
   for (int p = warp; p < points; p += warps) {
     const double* row = P.partial + static_cast<int64_t>(p) * gridDim.x;
     double s = 0.0;
@@ -374,6 +420,19 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     } else if (lane == 0) {
       P.losses[3 * (p >> 1) + (p & 1)] = f;
     }
+    if (lane == 0) loss_s[p] = f;
+  }
+  if (P.c != nullptr) {
+    __syncthreads();
+    bool bad = false;
+    for (int k = threadIdx.x; k < P.K; k += blockDim.x) {
+      double ck;
+      bad = !probe_coefficient(loss_s[2 * k], loss_s[2 * k + 1], loss_s[2 * P.K], P.eps, &ck) || bad;
+      c_s[k] = ck;
+    }
+    bad = __syncthreads_or(bad);  // one bad probe: nothing but the status is written
+    if (threadIdx.x == 0) *P.status = bad ? static_cast<int32_t>(kStatusNonFinite) : 0;
+    for (int k = threadIdx.x; !bad && k < P.K; k += blockDim.x) P.c[k] = c_s[k];
   }
   if (threadIdx.x == 0) *P.ticket = 0u;
 }
@@ -382,8 +441,8 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
 // needs, then just enough warps for that many, so the last round is not
 // nearly empty. Many probes leave room for fewer warps' sums.
 cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const RoundKeys& keys, int packing, int K,
-                               float eps, float meps, double* losses, double* partial, uint32_t* ticket, int num_sms,
-                               cudaStream_t stream) {
+                               double eps, double* losses, double* c, int32_t* status, double* partial,
+                               uint32_t* ticket, int num_sms, cudaStream_t stream) {
   QuadPointsParams P;
   P.theta = theta;
   P.a = a;
@@ -391,23 +450,27 @@ cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const Ro
   P.keys = keys;
   P.K = K;
   P.groups = (K + 7) / 8;
-  P.neps_bits = __builtin_bit_cast(uint32_t, eps) ^ 0x80000000u;
-  P.nmeps_bits = __builtin_bit_cast(uint32_t, meps) ^ 0x80000000u;
+  P.neps_bits = __builtin_bit_cast(uint32_t, static_cast<float>(eps)) ^ 0x80000000u;
+  P.nmeps_bits = __builtin_bit_cast(uint32_t, static_cast<float>(-2.0 * eps)) ^ 0x80000000u;
   P.losses = losses;
   P.partial = partial;
   P.ticket = ticket;
   P.zero = 0.0f;
+  P.drift = static_cast<float>(K + 1) * 0x1p-21f;
+  P.eps = eps;
+  P.c = c;
+  P.status = status;
   int max_warps = kPointsMaxThreads / 32;
   while (max_warps > 1 && quad_points_smem_bytes(P.groups, max_warps) > kQuadPointsMaxSmem) --max_warps;
   const int64_t items = (n + kItem - 1) / kItem;
   const int64_t cap = static_cast<int64_t>(num_sms) * max_warps * 32;
   const int64_t rounds = items > cap ? (items + cap - 1) / cap : 1;
-  int64_t warps = (items + static_cast<int64_t>(num_sms) * rounds * 32 - 1) / (static_cast<int64_t>(num_sms) * rounds * 32);
-  if (warps < 2 && max_warps >= 2) warps = 2;
+  const int64_t per_round = static_cast<int64_t>(num_sms) * rounds * 32;
+  int64_t warps = (items + per_round - 1) / per_round;
+  if (warps < 8) warps = 8;  // the sums' folds, which take a warp per point
   if (warps > max_warps) warps = max_warps;
-  if (warps < 1) warps = 1;
   const int threads = static_cast<int>(warps) * 32;
-  int64_t grid = (items + threads - 1) / threads;
+  int64_t grid = (items + 31) / 32;
   if (grid < 1) grid = 1;
   if (grid > num_sms) grid = num_sms;
   if (grid > kQuadPointsMaxCtas) grid = kQuadPointsMaxCtas;  // the workspace's partials

@@ -6,6 +6,7 @@
 
 #include "zo_device.cuh"
 #include "zo_launch.h"
+#include "zo_precond.cuh"
 
 namespace zo {
 
@@ -35,7 +36,7 @@ __global__ void precondition_kernel(const double* __restrict__ losses, int K, do
     lp = losses[3 * k + 0];
     lm = losses[3 * k + 1];
     l0 = losses[3 * k + 2];
-    cv = __ddiv_rn(__dadd_rn(__dsub_rn(lp, __dmul_rn(2.0, l0)), lm), __dmul_rn(eps, eps));
+    cv = probe_curvature(lp, lm, l0, eps);
     bad = !isfinite(lp) || !isfinite(lm) || !isfinite(l0) || !isfinite(cv);
   }
   double r = cv;
@@ -58,8 +59,8 @@ __global__ void precondition_kernel(const double* __restrict__ losses, int K, do
   }
   double wk = 0.0, ck = 0.0;
   if (k < K) {
-    wk = __ddiv_rn(1.0, fmax(lambda_reg, pow(fabs(r), alpha)));
-    const double g = one_sided ? __ddiv_rn(__dsub_rn(lp, l0), eps) : __ddiv_rn(__dsub_rn(lp, lm), __dmul_rn(2.0, eps));
+    wk = probe_weight(r, alpha, lambda_reg);
+    const double g = one_sided ? __ddiv_rn(__dsub_rn(lp, l0), eps) : central_difference(lp, lm, eps);
     ck = __dmul_rn(wk, g);
     bad = bad || !isfinite(ck);
   }

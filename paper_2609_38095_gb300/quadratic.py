@@ -10,9 +10,9 @@ table's third column (K doubles).
 
 Schedules (the weights at every forward point and after the step are the
 same bits in all three):
-  onepass  every forward point of the step, the last restore included, in one
-           launch that reads the weights once (zo_quadratic_points), then the
-           preconditioner and the update
+  onepass  every forward point of the step, the last restore included, and the
+           preconditioner in one launch that reads the weights once
+           (zo_quadratic_points), then the update
   fused    the restore of probe k and the +eps of probe k+1 in one pass
            (zo_perturb2), the last restore inside the update pass
            (zo_update_ex); each loss a call of zo_quadratic_loss
@@ -48,7 +48,8 @@ class QuadraticStep:
         self.ws = torch.empty(zo.quadratic_loss_workspace_size(theta.numel()), dtype=torch.uint8, device=dev)
         # the loss with its arguments checked once, and the table cells it writes
         self.loss = zo.QuadraticLoss(theta, a, self.ws)
-        self.points = zo.QuadraticPoints(theta, a, self.losses) if schedule == "onepass" else None
+        self.points = (zo.QuadraticPoints(theta, a, self.losses, out=(self.c, self.status))
+                       if schedule == "onepass" else None)
         row = self.losses.stride(0) * self.losses.element_size()
         base = self.loss.out_address(self.losses)
         self._lp = [base + k * row for k in range(self.K)]                  # L+ of probe k
@@ -60,8 +61,7 @@ class QuadraticStep:
         """Enqueue one step on the current stream (nothing waits)."""
         K, eps = self.K, self.eps
         if self.points is not None:
-            self.points(seed, eps)                             # L0 and every L+, L-; theta restored after each probe
-            zo.precondition(self.losses, eps, out=(self.c, self.status))
+            self.points(seed, eps)   # L0, every L+ and L- (theta restored after each probe), and the preconditioner
             zo.update(self.plist, seed, self.c, self.lr, status=self.status)
             return
         self.loss(self._l0)                                    # clean loss L0 (Algorithm 1)
@@ -88,7 +88,7 @@ class QuadraticStep:
         the loss is two: partial sums, then their fold)."""
         K = self.K
         if self.schedule == "onepass":
-            return 3
+            return 2
         losses = 2 * (2 * K + 1)
         passes = 2 * K if self.schedule == "fused" else 3 * K
         return losses + passes + 2

@@ -85,7 +85,7 @@ def _lib():
             "zo_perturb_quadratic_loss": ([vp, vp, i64, u64, i32, i32, u32, f32, u32, f32, vp, i32, i64, vp, i64, vp],
                                           c.c_int),
             "zo_quadratic_points_workspace_size": ([i32], i64),
-            "zo_quadratic_points": ([vp, vp, i64, u64, i32, i32, f64, vp, vp, i64, vp], c.c_int),
+            "zo_quadratic_points": ([vp, vp, i64, u64, i32, i32, f64, vp, vp, vp, vp, i64, vp], c.c_int),
         }
         for name, (args, res) in sig.items():
             f = getattr(L, name)
@@ -484,10 +484,11 @@ class QuadraticPoints:
     """zo_quadratic_points with theta, a, the loss table and the workspace
     checked once: a call takes theta through every forward point of a step
     (+eps, -2 eps, +eps per probe) and writes the K x 3 loss table, in one
-    launch. The workspace is allocated zero-filled here, as the call requires.
+    launch; with out=(c, status) the launch also does what precondition does.
+    The workspace is allocated zero-filled here, as the call requires.
     packing: None follows the process default."""
 
-    def __init__(self, theta, a, losses, packing=None):
+    def __init__(self, theta, a, losses, packing=None, out=None):
         n = theta.numel()
         if a.numel() != n:
             raise ValueError("theta and a differ in size")
@@ -498,10 +499,16 @@ class QuadraticPoints:
         self.device = theta.device
         K = losses.shape[0]
         workspace = torch.zeros(quadratic_points_workspace_size(K), dtype=torch.uint8, device=self.device)
-        _same_device(self.device, a=a, losses=losses)
-        self._keep = (theta, a, losses, workspace)
+        c, status = out if out is not None else (None, None)
+        if out is not None and (c.numel() < K or status.numel() < 1):
+            raise ValueError("out must be (c with at least K elements, status with at least one)")
+        _same_device(self.device, a=a, losses=losses, c=c, status=status)
+        self._keep = (theta, a, losses, workspace, c, status)
         self._args = (_dev_ptr(theta, torch.float32, "theta"), _dev_ptr(a, torch.float32, "a"), n)
-        self._out = (_dev_ptr(losses, torch.float64, "losses"), _dev_ptr(workspace), workspace.numel())
+        self._out = (_dev_ptr(losses, torch.float64, "losses"),
+                     _dev_ptr(c, torch.float64, "c") if out is not None else None,
+                     _dev_ptr(status, torch.int32, "status") if out is not None else None,
+                     _dev_ptr(workspace), workspace.numel())
         self.K = K
         self.packing = packing or 0
 

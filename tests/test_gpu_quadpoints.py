@@ -119,3 +119,36 @@ def test_points_not_finite(value):
     want_th, want = oracle_points(th, a, W.step_seed(1), 3, 1e-3)
     assert np.array_equal(got_th.view(np.uint32), want_th.view(np.uint32))
     assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+
+
+@pytest.mark.parametrize("n,K", [(5000, 1), (70_001, 8), (3000, 130), (500, zo.ZO_MAX_PROBES)])
+def test_points_with_the_preconditioner(n, K):
+    """c and status from the same launch: bit for bit what zo_precondition
+    gives for the losses written; a loss that is not finite leaves c alone."""
+    rng = np.random.default_rng(n + K)
+    theta = on_device(W.random_storage(rng, n, W.DT_F32), 0)
+    a = on_device((10.0 ** rng.uniform(-2, 2, n)).astype(np.float32), 0)
+    table = torch.empty(K, 3, dtype=torch.float64, device="cuda")
+    c = torch.full((K,), -7.0, dtype=torch.float64, device="cuda")
+    status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+    q = zo.QuadraticPoints(theta, a, table, out=(c, status))
+    q(W.step_seed(2), 1e-3)
+    want, st = zo.precondition(table, 1e-3)
+    assert int(status.item()) == int(st.item()) == zo.ZO_OK
+    assert torch.equal(c, want)
+    theta[n // 2] = float("inf")
+    q(W.step_seed(3), 1e-3)
+    assert int(status.item()) == zo.ZO_ERR_NONFINITE
+    assert torch.equal(c, want)
+
+
+def test_points_at_a_distance_of_eps_from_zero():
+    """Weights within a few roundings of +-eps pass through (almost) zero at a
+    point: they take the checked form of the terms."""
+    eps = 1e-3
+    th = np.full(4099, np.float32(eps), dtype=np.float32)
+    th[1::3] = -np.float32(eps)
+    th[2::7] = np.nextafter(np.float32(eps), np.float32(1))
+    th[5::11] = np.float32(2 * eps)
+    a = (10.0 ** np.random.default_rng(8).uniform(-2, 2, th.size)).astype(np.float32)
+    check(th, a, 6, eps=eps)
