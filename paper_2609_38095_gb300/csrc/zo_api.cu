@@ -72,6 +72,22 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 // all others walk the groups chunk by chunk (update_lut8_kernel).
 constexpr int kSmallGroups = 2;
 
+// Most items per SM of a list that update_items_kernel takes. It does two
+// lookups per element and group where the table-per-lane kernels do one, but
+// copies no tables; the lines lie where the two cross on 12 tensors of bf16
+// weights (us, items against tables):
+//   packing 1   K = 16: 3 M weights 10.5 / 12.9, 8 M 17.1 / 15.8
+//               K = 32: 8 M 23.1 / 23.4, 20 M 45.7 / 43.7
+//               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
+//   packing 8   K = 4: 3 M 10.9 / 15.0, 50 M 80 / 95, 205 M 304 / 353
+//               K = 32: 3 M 27.1 / 31.3, 20 M 132 / 128
+// (3 M weights are 1233 items per SM). Between 1 and 0.05 M all of these take
+// about 9 us here, 11 to 35 with the tables.
+int64_t update_items_per_sm(int packing, int groups) {
+  if (packing == zo::kPacking8) return groups == 1 ? INT64_C(1) << 20 : 4096;
+  return groups == 3 || groups == 4 ? 4096 : 1600;
+}
+
 // Per-device launch facts, filled once per device.
 struct DeviceInfo {
   int sms = 0;
@@ -250,6 +266,9 @@ thread_local zo::PairItemsParams<zo::kItemsFew> tl_pair_few;
 thread_local zo::PairItemsParams<zo::kItemsSome> tl_pair_some;
 thread_local zo::PairItemsParams<zo::kPairItemsMany> tl_pair_many;
 thread_local zo::SmallUpdateParams tl_update;
+thread_local zo::UpdateItemsParams<zo::kItemsFew> tl_update_few;
+thread_local zo::UpdateItemsParams<zo::kItemsSome> tl_update_some;
+thread_local zo::UpdateItemsParams<zo::kItemsMany> tl_update_many;
 
 }  // namespace
 
@@ -393,6 +412,33 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
+  const int64_t most_items = update_items_per_sm(up.packing, up.groups) * d->sms;
+  const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
+    zo::ItemsCursor cur;
+    const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
+                                         most_items);
+    *done = cur.t == n_tensors && one_high && ip.total <= most_items;
+    if (!*done || ip.n == 0) return cudaSuccess;
+    ip.bhi = 0;
+    ip.keys = up.keys;
+    ip.coef = c;
+    ip.coef_mul = up.coef_mul;
+    ip.K = up.K;
+    ip.groups = up.groups;
+    ip.packing = up.packing;
+    ip.has_pre = up.has_pre;
+    ip.pre = up.pre;
+    ip.status = status;
+    return zo::launch_update_items(ip, static_cast<cudaStream_t>(stream));
+  };
+  {
+    bool done = false;
+    const cudaError_t e = n_tensors <= zo::kItemsFew    ? short_list(tl_update_few, &done)
+                          : n_tensors <= zo::kItemsSome ? short_list(tl_update_some, &done)
+                                                        : short_list(tl_update_many, &done);
+    if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
+    if (done) return ZO_OK;
+  }
   const bool few = up.packing == zo::kPacking1 && up.groups <= kSmallGroups;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

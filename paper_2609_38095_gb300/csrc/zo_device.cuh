@@ -505,4 +505,76 @@ __device__ __forceinline__ uint4 item_signs(const uint4& x, bool f32, bool upper
   return shift ? window16(shfl_up4(x), x, 16u - a) : x;
 }
 
+// Helpers of the fused update's kernels.
+__device__ __forceinline__ float lds_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
+// One 4-probe partial ((s0 a0 + s1 a1) + s2 a2) + s3 a3 for sign nibble i.
+__device__ __forceinline__ float quad_partial(const float* a, uint32_t i) {
+  float s = (i & 1u) ? a[0] : -a[0];
+  s = __fadd_rn(s, (i & 2u) ? a[1] : -a[1]);
+  s = __fadd_rn(s, (i & 4u) ? a[2] : -a[2]);
+  s = __fadd_rn(s, (i & 8u) ? a[3] : -a[3]);
+  return s;
+}
+
+// theta pair + the leading perturbation's signed scales, one packed add.
+__device__ __forceinline__ void add_signed2(float2& f, const uint4& x, int i, const PerturbOp& op) {
+  // the probe bit moved to bit 31 by a multiply (PerturbOp::mul): the
+  // multiply-add pipe instead of the integer ALU, the busier one here
+  fadd2_rn(f.x, f.y, __uint_as_float(op.nscale_bits ^ ((word_of(x, i >> 2) * op.mul[i & 3]) & 0x80000000u)),
+           __uint_as_float(op.nscale_bits ^ ((word_of(x, (i + 1) >> 2) * op.mul[(i + 1) & 3]) & 0x80000000u)));
+}
+
+// Sixteen 16-bit weights: the leading perturbation, rounded to storage, then
+// the probe sums.
+template <uint8_t DT>
+__device__ __forceinline__ void update_regs16(uint32_t (&v)[8], const float (&acc)[16], const uint4& xp,
+                                              bool has_pre, const PerturbOp& pre) {
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    float2 f = unpack2<DT>(v[r]);
+    if (has_pre) {
+      add_signed2(f, xp, 2 * r, pre);
+      f = unpack2<DT>(pack2<DT>(f.x, f.y));  // the perturbed value is rounded to storage first
+    }
+    fadd2_rn(f.x, f.y, acc[2 * r], acc[2 * r + 1]);
+    v[r] = pack2<DT>(f.x, f.y);
+  }
+}
+
+// Packing 8: bit 0 of every byte of x to bit i of y's.
+__device__ __forceinline__ void fold_bits(uint4& y, const uint4& x, uint32_t i) {
+  const uint32_t m = 0x01010101u << i;
+  y.x |= (x.x << i) & m;
+  y.y |= (x.y << i) & m;
+  y.z |= (x.z << i) & m;
+  y.w |= (x.w << i) & m;
+}
+
+// The fused update of a short list by items (update_items_kernel): ItemsParams'
+// table, and the update's own arguments as in UpdateParams.
+template <int N>
+struct UpdateItemsParams {
+  static constexpr int kEntries = N;
+  ItemsEntry e[N];
+  uint16_t hint[kItemsHints];
+  int32_t n;
+  int32_t hint_shift;
+  uint32_t total;
+  uint32_t bhi;            // the virtual blocks' counter high word
+  RoundKeys keys;
+  const double* coef;
+  double coef_mul;
+  int32_t K;
+  int32_t groups;
+  int32_t packing;
+  int32_t has_pre;
+  PerturbOp pre;
+  const int32_t* status;
+};
+
 }  // namespace zo

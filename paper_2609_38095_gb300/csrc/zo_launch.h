@@ -37,6 +37,9 @@ cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cu
 cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStream_t stream);
 cudaError_t lut8_prepare();  // raises both kernels' shared-memory limits (once per device)
 bool one_high_word(const TensorTable& tab);  // of the launch's virtual blocks
+// Fused update of a short list; its virtual blocks share the counter's high word.
+template <int N>
+cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream);
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,
                                uint8_t* out, int grid, cudaStream_t stream);
 cudaError_t launch_probe_signs(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,

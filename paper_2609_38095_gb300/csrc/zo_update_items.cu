@@ -1,0 +1,187 @@
+// zo_update_items.cu -- the fused K-probe update of short lists.
+//
+// theta <- rn(fp32(theta) + sum_k a_k z_k[g]), the sums formed from the same
+// 8-probe partials T_lo + T_hi in the same order as in zo_update_lut8.cu, so
+// the bits are the same. What differs is what a launch costs before and after
+// its lookups: the kernels there copy a group's 256-entry table once per lane
+// (32 KB per group, for one lookup per element and group without bank
+// conflicts), which short lists do not repay. Here a group's two 16-entry
+// 4-probe tables lie in 128 bytes as they are: sixteen entries in sixteen
+// banks, so lanes that read different ones do not conflict, and lanes that
+// read the same one share it. Two lookups per element and group, nothing to
+// copy, 128 threads to a CTA so that few items still reach every SM; one
+// 32-byte item per thread, every kind of tensor in one launch
+// (perturb_items_kernel). Bound by its chain of latencies: launch, table,
+// coefficients, one Philox call and sixteen lookups per group, theta. 300 k
+// bf16 weights in 12 tensors, K = 8 / 32 / 64 / 256: 10.5 / 13.5 / 17.0 / 34.5
+// -> 8.7 / 8.2 / 8.8 / 15.1 us; as fp32, K = 32 15.0 -> 8.2; in one flat buffer
+// 23.3 -> 8.6; packing 8, K = 32 14.5 -> 10.2. Not adopted: a grid of 8 to 64
+// CTAs per SM that walks the items (K = 256, 8 M weights 97.5 -> 98-107 us).
+#include "zo_device.cuh"
+#include "zo_launch.h"
+
+namespace zo {
+
+namespace {
+
+constexpr int kItemThreads = 128;
+constexpr uint32_t kFrame = 256;  // bytes from one group's tables to the next's: T_lo at 0, T_hi at 64
+
+__device__ __forceinline__ float lds_f32_hi(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1+64];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
+// Add a group's partial of elements 0 .. 4 WORDS - 1, whose sign bytes are x's.
+template <int WORDS>
+__device__ __forceinline__ void add_group(float (&acc)[16], const uint4& x, uint32_t frame) {
+#pragma unroll
+  for (int m = 0; m < WORDS; ++m) {
+    const uint32_t w = word_of(x, m);
+    const uint32_t lo4 = (w << 2) & 0x3C3C3C3Cu;  // byte j: 4 * low nibble of byte j of w
+    const uint32_t hi4 = (w >> 2) & 0x3C3C3C3Cu;
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) {
+      const uint32_t s0 = 0x7650u | static_cast<uint32_t>(j), s1 = s0 + 1u;
+      float p0 = lds_f32(__byte_perm(lo4, frame, s0)), p1 = lds_f32(__byte_perm(lo4, frame, s1));
+      fadd2_rn(p0, p1, lds_f32_hi(__byte_perm(hi4, frame, s0)), lds_f32_hi(__byte_perm(hi4, frame, s1)));
+      fadd2_rn(acc[4 * m + j], acc[4 * m + j + 1], p0, p1);
+    }
+  }
+}
+
+size_t update_items_smem_bytes(int groups, int packing) {
+  // a_k, the tables on a 256-byte boundary, the counters' group parts
+  return static_cast<size_t>(groups) * (32 + kFrame + 16 * (packing == kPacking8 ? 8 : 1)) + kFrame;
+}
+
+}  // namespace
+
+template <bool PACK8, int N>
+__global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int skip_s;
+  const int G = P.groups;
+  constexpr int kCalls = PACK8 ? 8 : 1;  // Philox calls per group
+  uint4* r01_s = reinterpret_cast<uint4*>(smem);            // kCalls G group parts
+  float* a_s = reinterpret_cast<float*>(r01_s + kCalls * G);  // 8 G coefficients
+  const uint32_t after = static_cast<uint32_t>(__cvta_generic_to_shared(a_s + 8 * G));
+  const uint32_t frame0 = (after + kFrame - 1u) & ~(kFrame - 1u);
+  float* lut = a_s + 8 * G + (frame0 - after) / 4u;
+  if (threadIdx.x == 0) skip_s = (P.status != nullptr && *P.status != 0);
+  for (int k = threadIdx.x; k < 8 * G; k += kItemThreads)
+    a_s[k] = k < P.K ? __double2float_rn(P.coef_mul * P.coef[k]) : 0.0f;
+  for (int k = threadIdx.x; k < kCalls * G; k += kItemThreads) {
+    const GroupRound01 g = group_round01(static_cast<uint32_t>(k), P.bhi, P.keys);
+    r01_s[k] = make_uint4(g.x0, g.x2, g.lpa1, 0u);
+  }
+  // this thread's item, its load on the way while the tables are made
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t b = blockIdx.x * kItemThreads + threadIdx.x, wb = b - lane;
+  const bool here = wb < P.total;  // the same in all lanes
+  int t = here ? P.hint[wb >> P.hint_shift] : 0;
+  while (here && wb >= P.e[t].end) ++t;
+  const ItemsEntry e = P.e[t];
+  const uint8_t dt = static_cast<uint8_t>(e.meta & kDtypeMask);
+  const bool f32 = dt == kF32, shift = (e.meta & kShift) != 0;
+  const uint32_t a = e.meta >> 16;
+  ItemPlace k = item_place(e, b);
+  k.full = k.full && here;
+  k.act = k.act && here;
+  char* p = reinterpret_cast<char*>(e.base) + static_cast<int64_t>(k.i) * 32;
+  uint32_t v[8];
+  if (k.full) ld256(p, v);
+  __syncthreads();
+  const bool do_sum = skip_s == 0;  // a failed preconditioner still gets the leading perturbation
+  if (!do_sum && !P.has_pre) return;
+  for (int i = threadIdx.x; i < 32 * G; i += kItemThreads) {
+    const int h = i >> 4;  // quad of probes
+    lut[(h >> 1) * (kFrame / 4) + (h & 1) * 16 + (i & 15)] = quad_partial(a_s + 4 * h, static_cast<uint32_t>(i) & 15u);
+  }
+  __syncthreads();
+  if (!here) return;
+  const BlockRound01 blk = block_round01(static_cast<uint32_t>(item_block(e, k.i)), P.keys);
+  const auto call = [&](uint32_t c) {
+    const uint4 r = r01_s[c];
+    return philox_finish(philox_start(blk, {r.x, r.y, r.z}), P.keys);
+  };
+  float acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
+  if (do_sum) {
+    uint32_t frame = frame0;
+#pragma unroll 1
+    for (int q = 0; q < G; ++q, frame += kFrame) {
+      uint4 x;
+      if constexpr (PACK8) {
+        x = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 2
+        for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+      } else {
+        x = call(static_cast<uint32_t>(q));
+      }
+      x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
+      if (f32)
+        add_group<2>(acc, x, frame);
+      else
+        add_group<4>(acc, x, frame);
+    }
+  }
+  uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+  if (P.has_pre) {
+    const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
+    xp = item_signs(philox_finish(philox_start(blk, g), P.keys), f32, (k.i & 1) != 0, shift, a);
+  }
+  if (!k.act) return;
+  if (k.full && do_sum) {
+    if (f32) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float th = __uint_as_float(v[i]);
+        if (P.has_pre) th = add_signed(th, xp, i, P.pre);
+        v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
+      }
+    } else if (dt == kBF16) {
+      update_regs16<kBF16>(v, acc, xp, P.has_pre, P.pre);
+    } else {
+      update_regs16<kF16>(v, acc, xp, P.has_pre, P.pre);
+    }
+    st256(p, v);
+    return;
+  }
+  // an item across a tensor's end, or the leading perturbation alone
+  int lo, hi;
+  item_range(e, k.i, &lo, &hi);
+  float th[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) th[i] = i >= lo && i < hi ? load_elem(p, dt, i) : 0.0f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    if (i < lo || i >= hi) continue;
+    if (P.has_pre) th[i] = round_to_storage(dt, add_signed(th[i], xp, i, P.pre));
+    if (do_sum) th[i] = __fadd_rn(th[i], acc[i]);
+    store_elem(p, dt, i, th[i]);
+  }
+}
+
+template <int N>
+cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream) {
+  const int grid = static_cast<int>((p.total + (kItemThreads - 1u)) / kItemThreads);
+  const size_t smem = update_items_smem_bytes(p.groups, p.packing);
+  const auto go = [&](auto kernel) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(update_items_smem_bytes(kMaxGroups, kPacking8)));
+      if (e != cudaSuccess) return e;
+    }
+    kernel<<<grid, kItemThreads, smem, stream>>>(p);
+    return cudaGetLastError();
+  };
+  return p.packing == kPacking8 ? go(update_items_kernel<true, N>) : go(update_items_kernel<false, N>);
+}
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsFew>& p, cudaStream_t stream);
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsSome>& p, cudaStream_t stream);
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsMany>& p, cudaStream_t stream);
+
+}  // namespace zo

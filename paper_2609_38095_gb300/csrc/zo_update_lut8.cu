@@ -25,7 +25,7 @@
 //
 // Loop order. The replicated tables of all groups do not fit in shared memory
 // (32 KB per group), so probe groups are the outer loop: a CTA owns a chunk of
-// 512 * BPT consecutive blocks (BPT = 8 on large launches), accumulates every
+// 512 * BPT consecutive blocks (BPT = 8 but in a launch's last round), accumulates every
 // block's sums over all groups and then applies them to theta (read once,
 // written once). Two regions of 64 KB each hold a pair of groups (one per
 // half): while the lanes look up groups 2p and 2p+1 in one region, they copy
@@ -42,23 +42,8 @@
 namespace zo {
 
 constexpr uint32_t kLut8Region = 65536;   // 256 rows x 256 bytes: the tables of two groups
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-  return v;
-}
-
 __device__ __forceinline__ void sts_f32x4(uint32_t addr, float v) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "f"(v) : "memory");
-}
-
-// One 4-probe partial ((s0 a0 + s1 a1) + s2 a2) + s3 a3 for sign nibble i.
-__device__ __forceinline__ float quad_partial(const float* a, uint32_t i) {
-  float s = (i & 1u) ? a[0] : -a[0];
-  s = __fadd_rn(s, (i & 2u) ? a[1] : -a[1]);
-  s = __fadd_rn(s, (i & 4u) ? a[2] : -a[2]);
-  s = __fadd_rn(s, (i & 8u) ? a[3] : -a[3]);
-  return s;
 }
 
 // Add group q's partial of the 16 elements of a block (Philox output x) to acc,
@@ -92,29 +77,6 @@ struct Lut8Block {
   bool act;        // there are elements here for this lane
   bool vec;        // all sixteen, 32-byte aligned
 };
-
-// theta pair + the leading perturbation's signed scales, one packed add.
-__device__ __forceinline__ void add_signed2(float2& f, const uint4& x, int i, const PerturbOp& op) {
-  // the probe bit moved to bit 31 by a multiply (PerturbOp::mul): the
-  // multiply-add pipe instead of the integer ALU, the busier one here
-  fadd2_rn(f.x, f.y, __uint_as_float(op.nscale_bits ^ ((word_of(x, i >> 2) * op.mul[i & 3]) & 0x80000000u)),
-           __uint_as_float(op.nscale_bits ^ ((word_of(x, (i + 1) >> 2) * op.mul[(i + 1) & 3]) & 0x80000000u)));
-}
-
-template <uint8_t DT>
-__device__ __forceinline__ void lut8_apply16(uint32_t (&v)[8], const float (&acc)[16], const uint4& xp,
-                                             const UpdateParams& P) {
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    float2 f = unpack2<DT>(v[r]);
-    if (P.has_pre) {
-      add_signed2(f, xp, 2 * r, P.pre);
-      f = unpack2<DT>(pack2<DT>(f.x, f.y));  // the perturbed value is rounded to storage first
-    }
-    fadd2_rn(f.x, f.y, acc[2 * r], acc[2 * r + 1]);
-    v[r] = pack2<DT>(f.x, f.y);
-  }
-}
 
 // The same for sixteen fp32 weights: scalar adds, as in every fp32 path.
 __device__ __forceinline__ void lut8_apply32(uint32_t (&v)[16], const float (&acc)[16], const uint4& xp,
@@ -158,6 +120,7 @@ __device__ __forceinline__ void lut8_apply_elements(const Lut8Block& k, const fl
 // tables are 64 KB of shared-memory stores, against 128 KB of lookups per
 // 1024 blocks.
 constexpr int kLut8Threads = 512;
+constexpr int kLut8Bpt = 8;  // most blocks per thread of a chunk
 constexpr uint32_t kTmemCols = 512;
 
 __device__ __forceinline__ void tm_ld16(float (&r)[16], uint32_t taddr) {
@@ -306,14 +269,6 @@ struct BlockCounter<false> {
 // left out: their coefficients are 0 in the tables. A full group's calls run
 // in pairs, two independent chains of multiplies per thread: with the four
 // warps a scheduler has here, one chain leaves the multiply-add pipe waiting.
-__device__ __forceinline__ void fold_bits(uint4& y, const uint4& x, uint32_t i) {
-  const uint32_t m = 0x01010101u << i;
-  y.x |= (x.x << i) & m;
-  y.y |= (x.y << i) & m;
-  y.z |= (x.z << i) & m;
-  y.w |= (x.w << i) & m;
-}
-
 template <bool HIU>
 __device__ __forceinline__ uint4 group_words8(const BlockCounter<HIU>& kb, uint32_t q, uint32_t K, const uint4* r01,
                                               const RoundKeys& keys) {
@@ -433,15 +388,15 @@ __device__ __forceinline__ void lut8_tm_step8(uint32_t ta, const BlockCounter<HI
 // tables (32 per group), under packing 8 the probes' Philox group parts (16
 // bytes each), and the tensors of the chunk's blocks (one per warp and block),
 // below the first region when they fit there, else after the second.
-__host__ __device__ constexpr uint32_t lut8_side_bytes(int groups, int bpt, bool pack8) {
+__host__ __device__ constexpr uint32_t lut8_side_bytes(int groups, bool pack8) {
   return (pack8 ? 288u : 160u) * static_cast<uint32_t>(groups) +
-         4u * static_cast<uint32_t>(kLut8Threads / 32 * bpt);
+         4u * static_cast<uint32_t>(kLut8Threads / 32 * kLut8Bpt);
 }
 // Placed after the second region only when the slack below the first is
 // smaller than it, so the layout ends within 2 * side + 128 KB of the window's
 // start.
 constexpr size_t lut8_smem_bytes(bool pack8) {
-  const size_t after = 2 * static_cast<size_t>(kLut8Region) + 2 * lut8_side_bytes(kMaxGroups, 8, pack8) + 16u;
+  const size_t after = 2 * static_cast<size_t>(kLut8Region) + 2 * lut8_side_bytes(kMaxGroups, pack8) + 16u;
   const size_t below = 3 * static_cast<size_t>(kLut8Region) + 16u;
   return after > below ? after : below;
 }
@@ -458,9 +413,9 @@ static_assert(lut8_smem_bytes(true) <= 226 * 1024, "side data must fit the share
 // K = 1024 on the OPT-1.3B-shaped set: 40.1 -> 39.6 ms), slower below (K = 64:
 // 4.23 -> 4.30 ms on Qwen3-8B-shaped layers), where the two groups' own calls
 // overlap enough and the last pair weighs more.
-template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD>
+template <bool HIU, bool ANY, bool PACK8, bool AHEAD>
 __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __grid_constant__ UpdateParams P) {
-  constexpr int THREADS = kLut8Threads;
+  constexpr int THREADS = kLut8Threads, BPT = kLut8Bpt;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
   __shared__ uint32_t tmem_s;
@@ -468,7 +423,7 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
   const int NP = (G + 1) / 2;  // group pairs: groups 2p, 2p + 1 share one region
   const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
   const uint32_t region0 = (sbase + kLut8Region - 1u) & ~(kLut8Region - 1u);
-  const uint32_t side = lut8_side_bytes(G, BPT, PACK8);
+  const uint32_t side = lut8_side_bytes(G, PACK8);
   const uint32_t hdr = region0 - sbase >= side ? sbase : region0 + 2u * kLut8Region;
   float* a_s = reinterpret_cast<float*>(smem + (hdr - sbase));  // 8 G coefficients
   float* t4 = a_s + 8 * G;                                      // 32 G 4-probe partials
@@ -534,8 +489,8 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
   // TMEM lane 32 (warp mod 4) + lane id, columns from 128 (warp / 4)
   const uint32_t trow = tmem_s + (((warp & 3u) * 32u) << 16) + (warp >> 2) * 128u;
 
-  constexpr uint32_t chunk = static_cast<uint32_t>(THREADS * BPT);
-  const uint32_t per_round = gridDim.x * chunk;
+  const uint32_t row = gridDim.x * static_cast<uint32_t>(THREADS);  // one block per thread of the launch
+  const uint32_t per_round = row * static_cast<uint32_t>(BPT);
   const uint32_t rounds = (tab.blk_total + per_round - 1u) / per_round;
   uint32_t cur = 0;  // region holding the current pair (0 or 1)
   int t = 0;         // tensor of the warp's latest block
@@ -544,15 +499,19 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
   };
 
   for (uint32_t rnd = 0; rnd < rounds; ++rnd) {
-    // this thread's blocks of the chunk: cb, cb + THREADS, ..
-    const uint32_t cb = (rnd * gridDim.x + blockIdx.x) * chunk + threadIdx.x;
+    // this thread's blocks of the chunk: cb, cb + THREADS, .. The last round's chunks are shorter: its blocks
+    // spread over all CTAs (20 M bf16 weights are two rounds and 0.6 %: K = 256 243 -> 185 us, K = 64 80 -> 64;
+    // 3 M, a fraction of one, K = 256 60 -> 44)
+    const uint32_t left = tab.blk_total - rnd * per_round;
+    const int bpt = left >= per_round ? BPT : static_cast<int>((left + row - 1u) / row);
+    const uint32_t cb = rnd * per_round + blockIdx.x * static_cast<uint32_t>(THREADS * bpt) + threadIdx.x;
     int jn = 0;          // blocks of the warp inside the launch
     uint32_t vr[BPT];    // their counter words (registers: 2-6 % faster than shared memory)
 #pragma unroll
     for (int j = 0; j < BPT; ++j) {
       const uint32_t bl = cb + static_cast<uint32_t>(j * THREADS);
       vr[j] = 0u;
-      if (bl - lane < tab.blk_total) {
+      if (j < bpt && bl - lane < tab.blk_total) {
         jn = j + 1;
         t = advance_tensor(tab, t, bl - lane);
         const Lut8Block k = lut8_block_info<ANY>(tab, t, bl);
@@ -689,9 +648,9 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
               lut8_apply32(v, acc, xp, P);
               st256(tp + 32, hi);
             } else if ((k.fl & kDtypeMask) == kBF16) {
-              lut8_apply16<kBF16>(lo, acc, xp, P);
+              update_regs16<kBF16>(lo, acc, xp, P.has_pre, P.pre);
             } else {
-              lut8_apply16<kF16>(lo, acc, xp, P);
+              update_regs16<kF16>(lo, acc, xp, P.has_pre, P.pre);
             }
             st256(tp, lo);
           }
@@ -1083,22 +1042,20 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   }
 }
 
-template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
+template <bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
 cudaError_t launch_lut8_cfg(const UpdateParams& p, int sms, cudaStream_t stream) {
-  // one CTA per chunk of 512 * BPT blocks, at most one per SM
-  const int64_t chunk = static_cast<int64_t>(kLut8Threads) * BPT;
-  const int64_t want = (static_cast<int64_t>(p.tab.blk_total) + chunk - 1) / chunk;
+  // one CTA per SM, or per 512 blocks of a short list
+  const int64_t want = (static_cast<int64_t>(p.tab.blk_total) + kLut8Threads - 1) / kLut8Threads;
   const int grid = static_cast<int>(want < sms ? want : sms);
-  update_lut8_kernel<BPT, HIU, ANY, PACK8, AHEAD><<<grid, kLut8Threads, lut8_smem_bytes(PACK8), stream>>>(p);
+  update_lut8_kernel<HIU, ANY, PACK8, AHEAD><<<grid, kLut8Threads, lut8_smem_bytes(PACK8), stream>>>(p);
   return cudaGetLastError();
 }
 
-template <int BPT, bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
+template <bool HIU, bool ANY, bool PACK8, bool AHEAD = false>
 cudaError_t lut8_limit() {
-  return cudaFuncSetAttribute(update_lut8_kernel<BPT, HIU, ANY, PACK8, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(update_lut8_kernel<HIU, ANY, PACK8, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(lut8_smem_bytes(PACK8)));
 }
-
 
 template <int PRE, bool TWO, bool ANY>
 cudaError_t small_limit() {
@@ -1119,38 +1076,16 @@ cudaError_t lut8_prepare() {
   cudaError_t e = small_limits<kPreNone>();
   if (e == cudaSuccess) e = small_limits<kPreTable>();
   if (e == cudaSuccess) e = small_limits<kPreOwn>();
-  if (e == cudaSuccess) e = lut8_limit<2, true, false, false>();
-  if (e == cudaSuccess) e = lut8_limit<4, true, false, false>();
-  if (e == cudaSuccess) e = lut8_limit<8, true, false, false>();
-  if (e == cudaSuccess) e = lut8_limit<8, true, false, false, true>();
-  if (e == cudaSuccess) e = lut8_limit<2, true, true, false>();
-  if (e == cudaSuccess) e = lut8_limit<4, true, true, false>();
-  if (e == cudaSuccess) e = lut8_limit<8, true, true, false>();
-  if (e == cudaSuccess) e = lut8_limit<8, false, true, false>();
-  if (e == cudaSuccess) e = lut8_limit<2, true, true, true>();
-  if (e == cudaSuccess) e = lut8_limit<4, true, true, true>();
-  if (e == cudaSuccess) e = lut8_limit<8, true, true, true>();
-  if (e == cudaSuccess) e = lut8_limit<8, false, true, true>();
+  if (e == cudaSuccess) e = lut8_limit<true, false, false>();
+  if (e == cudaSuccess) e = lut8_limit<true, false, false, true>();
+  if (e == cudaSuccess) e = lut8_limit<true, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<false, true, false>();
+  if (e == cudaSuccess) e = lut8_limit<true, true, true>();
+  if (e == cudaSuccess) e = lut8_limit<false, true, true>();
   return e;
 }
 
 constexpr int kAheadGroups = 24;  // see AHEAD
-
-// Blocks per thread: the largest of 8, 4, 2 that still gives every SM a chunk.
-int lut8_bpt(uint32_t blk_total, int sms) {
-  for (int bpt = 8; bpt > 2; bpt /= 2)
-    if (static_cast<int64_t>(blk_total) >= static_cast<int64_t>(sms) * kLut8Threads * bpt) return bpt;
-  return 2;
-}
-
-template <bool ANY, bool PACK8>
-cudaError_t launch_lut8_any(const UpdateParams& p, int bpt, int sms, cudaStream_t stream) {
-  switch (bpt) {
-    case 8: return launch_lut8_cfg<8, true, ANY, PACK8>(p, sms, stream);
-    case 4: return launch_lut8_cfg<4, true, ANY, PACK8>(p, sms, stream);
-    default: return launch_lut8_cfg<2, true, ANY, PACK8>(p, sms, stream);
-  }
-}
 
 bool one_high_word(const TensorTable& tab) {
   // every virtual block that a lane sums lies in [blk_base, blk_base + blk_total), except the one below a
@@ -1198,13 +1133,12 @@ cudaError_t launch_update_lut8(const UpdateParams& p, bool any, int sms, cudaStr
   const bool pack8 = p.packing == kPacking8;
   // a launch of one or two groups comes here when the small kernel cannot take it: rare, on the general form
   if (!one_high_word(p.tab) || (!pack8 && p.groups <= 2))
-    return pack8 ? launch_lut8_cfg<8, false, true, true>(p, sms, stream)
-                 : launch_lut8_cfg<8, false, true, false>(p, sms, stream);
-  const int bpt = lut8_bpt(p.tab.blk_total, sms);
-  if (pack8) return launch_lut8_any<true, true>(p, bpt, sms, stream);
-  if (any) return launch_lut8_any<true, false>(p, bpt, sms, stream);
-  if (bpt == 8 && p.groups >= kAheadGroups) return launch_lut8_cfg<8, true, false, false, true>(p, sms, stream);
-  return launch_lut8_any<false, false>(p, bpt, sms, stream);
+    return pack8 ? launch_lut8_cfg<false, true, true>(p, sms, stream)
+                 : launch_lut8_cfg<false, true, false>(p, sms, stream);
+  if (pack8) return launch_lut8_cfg<true, true, true>(p, sms, stream);
+  if (any) return launch_lut8_cfg<true, true, false>(p, sms, stream);
+  return p.groups >= kAheadGroups ? launch_lut8_cfg<true, false, false, true>(p, sms, stream)
+                                  : launch_lut8_cfg<true, false, false>(p, sms, stream);
 }
 
 }  // namespace zo

@@ -1,0 +1,87 @@
+"""The fused update of short lists by items (update_items_kernel): against the
+table-per-lane kernels bit for bit, by padding the same list past the short
+lists' limit with a tensor that both calls share, and against the oracle, over
+every storage type, alignment, packing, probe count and a failed
+preconditioner."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_38095_gb300 import build as zo_build
+from paper_2609_38095_gb300 import workloads as W
+from paper_2609_38095_gb300 import zo
+
+from gpu_helpers import TORCH_TO_DT, assert_update_close, storage_bits, to_torch
+
+pytestmark = pytest.mark.gpu
+
+DTYPES = [torch.bfloat16, torch.float32, torch.float16]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    zo_build.build()
+    oracle.lib()
+
+
+def views_of(host, dtypes, offsets):
+    out = []
+    for h, d, off in zip(host, dtypes, offsets):
+        base = torch.zeros(h.size + off, dtype=d, device="cuda")
+        base[off:].copy_(to_torch(h, d))
+        out.append(base[off:])
+    return out
+
+
+@pytest.mark.parametrize("K,packing", [(1, 1), (8, 1), (16, 1), (17, 1), (64, 1), (384, 1), (1024, 1), (1, 8), (8, 8),
+                                       (9, 8), (130, 8), (1024, 8)])
+@pytest.mark.parametrize("pre,status", [(True, 0), (False, 0), (True, zo.ZO_ERR_NONFINITE),
+                                        (False, zo.ZO_ERR_NONFINITE)])
+def test_short_list(K, packing, pre, status):
+    rng = np.random.default_rng(K * 8 + packing)
+    numels = [1, 15, 16, 17, 31 * 16, 31 * 16 + 1, 500, 8, 7, 1000, 333, 4096]
+    dtypes = [DTYPES[i % 3] for i in range(len(numels))]
+    offsets = [0, 3, 0, 1, 5, 0, 7, 0, 1, 0, 11, 0]
+    dts = [TORCH_TO_DT[d] for d in dtypes]
+    host = [W.random_storage(rng, n, dt) for n, dt in zip(numels, dts)]
+    short, tail = views_of(host, dtypes, offsets), views_of(host, dtypes, offsets)
+    c_np = rng.normal(0, 25, K)
+    c, st = torch.tensor(c_np, device="cuda"), torch.tensor([status], dtype=torch.int32, device="cuda")
+    s, lr, p = W.step_seed(K), 1e-3, (K - 1, 1e-3) if pre else None
+    zo.update(zo.ParamList(short, packing=packing), s, c, lr, status=st, pre=p)
+    with oracle.packing(packing):
+        if pre:
+            oracle.perturb(host, dts, s, K - 1, 1e-3)
+        if not status:
+            oracle.update(host, dts, s, c_np, lr)
+    for i, (v, h, dt) in enumerate(zip(short, host, dts)):
+        if status:
+            assert np.array_equal(storage_bits(v), storage_bits(h)), f"tensor {i}"
+        else:
+            assert_update_close(storage_bits(v), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
+    if packing == 8 and K <= 8:
+        return                                    # update_items_kernel at every size
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    filler = torch.zeros(16 * 4097 * sms, dtype=torch.bfloat16, device="cuda")
+    zo.update(zo.ParamList(tail + [filler], packing=packing), s, c, lr, status=st, pre=p)
+    for i, (x, y) in enumerate(zip(short, tail)):
+        assert torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8)), f"tensor {i}"
+
+
+@pytest.mark.parametrize("n", [64, 65, 256, 257, 960, 961, 2100])
+def test_short_list_of_many_tensors(n):
+    rng = np.random.default_rng(n)
+    numels = [int(x) for x in rng.integers(0, 70, n)]
+    host = [W.random_storage(rng, m, W.DT_BF16) for m in numels]
+    dev = [to_torch(h.copy(), torch.bfloat16) for h in host]
+    K, s, lr = 11, W.step_seed(n), 1e-3
+    c_np = rng.normal(0, 25, K)
+    zo.update(dev, s, torch.tensor(c_np, device="cuda"), lr, pre=(K - 1, 1e-3))
+    oracle.perturb(host, [W.DT_BF16] * n, s, K - 1, 1e-3)
+    oracle.update(host, [W.DT_BF16] * n, s, c_np, lr)
+    for i, (d, h) in enumerate(zip(dev, host)):
+        if h.size:
+            assert_update_close(storage_bits(d), storage_bits(h), W.DT_BF16, c_np, lr, context=f"tensor {i}")
