@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
       t = advance_tensor(tab, t, bl - lane);
       const Lut8Block k = lut8_block_info<ANY>(tab, t, bl);
       uint4 xp = block_bits(k.b, P.pre.ctr2, P.keys);
-      if (ANY && (k.fl & kShift)) xp = window16(shfl_up4(xp), xp, 16u - k.a);
+      if (ANY && (k.fl & kShift)) xp = window16(xp, 16u - k.a);
       if (k.vec && (k.fl & kDtypeMask) != kF32) {
         uint16_t* p = static_cast<uint16_t*>(k.base) + k.e0;
         uint32_t v[8];
@@ -634,14 +634,8 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
           }
           if (pre_at == 3) xp = block_bits(k.b, P.pre.ctr2, P.keys);
           if (ANY && (k.fl & kShift)) {  // the same in all lanes
-            float below[16], own[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              own[i] = acc[i];
-              below[i] = __shfl_up_sync(0xFFFFFFFFu, acc[i], 1);
-            }
-            window16f(below, own, 16u - k.a, acc);
-            xp = window16(shfl_up4(xp), xp, 16u - k.a);
+            window16f(acc, 16u - k.a);
+            if (P.has_pre) xp = window16(xp, 16u - k.a);
           }
           if (k.vec) {
             if (ANY && f32) {
@@ -668,14 +662,8 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
             uint4 xp = make_uint4(0u, 0u, 0u, 0u);
             if (P.has_pre) xp = block_bits(k.b, P.pre.ctr2, P.keys);
             if (ANY && (k.fl & kShift)) {
-              float below[16], own[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                own[i] = acc[i];
-                below[i] = __shfl_up_sync(0xFFFFFFFFu, acc[i], 1);
-              }
-              window16f(below, own, 16u - k.a, acc);
-              xp = window16(shfl_up4(xp), xp, 16u - k.a);
+              window16f(acc, 16u - k.a);
+              xp = window16(xp, 16u - k.a);
             }
             if (mine) lut8_apply_elements(k, acc, xp, P, true);
           }
