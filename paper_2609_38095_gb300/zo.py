@@ -134,42 +134,32 @@ def _check(fn, rc):
         raise ZoError(fn, rc)
 
 
-# The current stream's handle without building a torch Stream object (about
-# 3 us of a 9 us call otherwise); the public route where torch lacks it.
+# The current device and stream by torch's raw calls: torch.cuda's wrappers
+# and a Stream object take about 3 us of a call that is 4 us in all; the
+# public routes where torch lacks them.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
 def _index(device):
     return device.index if device.index is not None else torch.cuda.current_device()
 
 
-def _stream(device):
-    idx = _index(device)
-    if _raw_stream is not None:
-        return ctypes.c_void_p(_raw_stream(idx))
-    return ctypes.c_void_p(torch.cuda.current_stream(idx).cuda_stream)
+def _stream(idx):
+    """The current stream of device `idx`, as an integer handle."""
+    return _raw_stream(idx) if _raw_stream is not None else torch.cuda.current_stream(idx).cuda_stream
 
 
-class _on:
-    """Makes `device` current for a call (the library launches on the current
-    device); a no-op when it already is, the usual case."""
-    __slots__ = ("idx", "prev")
-
-    def __init__(self, device):
-        self.idx = _index(device)
-        self.prev = None
-
-    def __enter__(self):
-        cur = torch.cuda.current_device()
-        if cur != self.idx:
-            self.prev = cur
-            torch.cuda.set_device(self.idx)
-        return self
-
-    def __exit__(self, *exc):
-        if self.prev is not None:
-            torch.cuda.set_device(self.prev)
-        return False
+def _launch(what, idx, f, *args):
+    """f(*args, stream) with device `idx` current (the library launches on the
+    current device); raises unless it returns ZO_OK."""
+    if _raw_device() == idx:
+        rc = f(*args, _stream(idx))
+    else:
+        with torch.cuda.device(idx):
+            rc = f(*args, _stream(idx))
+    if rc != ZO_OK:
+        raise ZoError(what, rc)
 
 
 def _dev_ptr(t, dtype=None, what="tensor"):
@@ -179,7 +169,7 @@ def _dev_ptr(t, dtype=None, what="tensor"):
         raise ValueError(f"{what} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{what} must be {dtype}, got {t.dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _same_device(dev, **tensors):
@@ -219,9 +209,11 @@ class ParamList:
             arr[i].numel = t.numel()
             arr[i].dtype = DTYPE_CODE[t.dtype]
             arr[i].packing = packing or 0
-        self._arr = arr
+        self._arr = arr                          # lives as long as the list
+        self._ptr = ctypes.addressof(arr)
         self.n = n
         self.device = dev if dev is not None else torch.device("cuda", torch.cuda.current_device())
+        self.index = _index(self.device)
 
     @property
     def numels(self):
@@ -238,17 +230,14 @@ def _plist(params):
 def perturb(params, seed: int, probe: int, scale: float):
     """theta <- theta + scale * z_probe in place (zo_perturb)."""
     p = _plist(params)
-    with _on(p.device):
-        _check("zo_perturb", _lib().zo_perturb(p._arr, p.n, seed, probe, scale, _stream(p.device)))
+    _launch("zo_perturb", p.index, _lib().zo_perturb, p._ptr, p.n, seed, probe, scale)
 
 
 def perturb2(params, seed: int, probe_a: int, scale_a: float, probe_b: int, scale_b: float):
     """perturb(probe_a, scale_a) then perturb(probe_b, scale_b), bit for bit, in
     one pass over theta (zo_perturb2)."""
     p = _plist(params)
-    with _on(p.device):
-        _check("zo_perturb2", _lib().zo_perturb2(p._arr, p.n, seed, probe_a, scale_a, probe_b, scale_b,
-                                                 _stream(p.device)))
+    _launch("zo_perturb2", p.index, _lib().zo_perturb2, p._ptr, p.n, seed, probe_a, scale_a, probe_b, scale_b)
 
 
 def perturb_pair(params, plus, minus, seed: int, probe: int, scale: float):
@@ -260,9 +249,7 @@ def perturb_pair(params, plus, minus, seed: int, probe: int, scale: float):
         raise ValueError("plus and minus must have one tensor per parameter")
     if (pl.n and pl.device != p.device) or (mi.n and mi.device != p.device):
         raise ValueError("plus and minus must live on the parameters' device")
-    with _on(p.device):
-        _check("zo_perturb_pair", _lib().zo_perturb_pair(p._arr, pl._arr, mi._arr, p.n, seed, probe, scale,
-                                                         _stream(p.device)))
+    _launch("zo_perturb_pair", p.index, _lib().zo_perturb_pair, p._ptr, pl._ptr, mi._ptr, p.n, seed, probe, scale)
 
 
 def precondition(losses, eps: float, alpha: float = 0.1, lambda_reg: float = 1.0, one_sided: bool = False,
@@ -290,13 +277,9 @@ def precondition(losses, eps: float, alpha: float = 0.1, lambda_reg: float = 1.0
     if with_weights:
         w = torch.empty(K, dtype=torch.float64, device=dev)
         curv = torch.empty(K, dtype=torch.float64, device=dev)
-    with _on(dev):
-        rc = _lib().zo_precondition_ex(lp, K, eps, alpha, lambda_reg, int(flags),
-                                       _dev_ptr(c, torch.float64, "c"),
-                                       _dev_ptr(w, torch.float64) if w is not None else None,
-                                       _dev_ptr(curv, torch.float64) if curv is not None else None,
-                                       _dev_ptr(status, torch.int32, "status"), _stream(dev))
-    _check("zo_precondition", rc)
+    _launch("zo_precondition", _index(dev), _lib().zo_precondition_ex, lp, K, eps, alpha, lambda_reg, int(flags),
+            _dev_ptr(c, torch.float64, "c"), _dev_ptr(w, torch.float64) if w is not None else None,
+            _dev_ptr(curv, torch.float64) if curv is not None else None, _dev_ptr(status, torch.int32, "status"))
     return (c, status, w, curv) if with_weights else (c, status)
 
 
@@ -307,37 +290,29 @@ def update(params, seed: int, c, lr: float, status=None, pre=None):
     p = _plist(params)
     st = _dev_ptr(status, torch.int32, "status") if status is not None else None
     has_pre, pre_probe, pre_scale = (0, 0, 0.0) if pre is None else (1, int(pre[0]), float(pre[1]))
-    with _on(p.device):
-        rc = _lib().zo_update_ex(p._arr, p.n, seed, _dev_ptr(c, torch.float64, "c"), c.numel(), lr, st,
-                                 has_pre, pre_probe, pre_scale, _stream(p.device))
-    _check("zo_update", rc)
+    _launch("zo_update", p.index, _lib().zo_update_ex, p._ptr, p.n, seed, _dev_ptr(c, torch.float64, "c"), c.numel(),
+            lr, st, has_pre, pre_probe, pre_scale)
 
 
 def update_sequential(params, seed: int, c, lr: float, status=None):
     """Algorithm 1's K-pass application, the comparator (zo_update_sequential)."""
     p = _plist(params)
     st = _dev_ptr(status, torch.int32, "status") if status is not None else None
-    with _on(p.device):
-        rc = _lib().zo_update_sequential(p._arr, p.n, seed, _dev_ptr(c, torch.float64, "c"), c.numel(), lr, st,
-                                         _stream(p.device))
-    _check("zo_update_sequential", rc)
+    _launch("zo_update_sequential", p.index, _lib().zo_update_sequential, p._ptr, p.n, seed,
+            _dev_ptr(c, torch.float64, "c"), c.numel(), lr, st)
 
 
 def probe_bytes(seed: int, probe: int, first: int, n: int, device=None):
     """Probe `probe` packed one bit per element (bytes first..first+n-1)."""
     out = torch.empty(n, dtype=torch.uint8, device=device or "cuda")
-    with _on(out.device):
-        rc = _lib().zo_probe_bytes(seed, probe, first, n, ctypes.c_void_p(out.data_ptr()), _stream(out.device))
-    _check("zo_probe_bytes", rc)
+    _launch("zo_probe_bytes", _index(out.device), _lib().zo_probe_bytes, seed, probe, first, n, out.data_ptr())
     return out
 
 
 def probe_signs(seed: int, probe: int, first: int, n: int, device=None):
     """z_probe[g] as int8 for g = first..first+n-1."""
     out = torch.empty(n, dtype=torch.int8, device=device or "cuda")
-    with _on(out.device):
-        rc = _lib().zo_probe_signs(seed, probe, first, n, ctypes.c_void_p(out.data_ptr()), _stream(out.device))
-    _check("zo_probe_signs", rc)
+    _launch("zo_probe_signs", _index(out.device), _lib().zo_probe_signs, seed, probe, first, n, out.data_ptr())
     return out
 
 
@@ -359,11 +334,9 @@ def quadratic_loss(theta, a, out=None, workspace=None):
     if out.numel() < 1:
         raise ValueError("out must hold one float64")
     _same_device(dev, a=a, out=out, workspace=workspace)
-    with _on(dev):
-        rc = _lib().zo_quadratic_loss(_dev_ptr(theta, torch.float32, "theta"), _dev_ptr(a, torch.float32, "a"), n,
-                                      _dev_ptr(out, torch.float64, "out"), _dev_ptr(workspace, what="workspace"),
-                                      workspace.numel() * workspace.element_size(), _stream(dev))
-    _check("zo_quadratic_loss", rc)
+    _launch("zo_quadratic_loss", _index(dev), _lib().zo_quadratic_loss, _dev_ptr(theta, torch.float32, "theta"),
+            _dev_ptr(a, torch.float32, "a"), n, _dev_ptr(out, torch.float64, "out"),
+            _dev_ptr(workspace, what="workspace"), workspace.numel() * workspace.element_size())
     return out
 
 
@@ -378,6 +351,7 @@ class QuadraticLoss:
         if a.numel() != n:
             raise ValueError("theta and a differ in size")
         self.device = theta.device
+        self.index = _index(self.device)
         if workspace is None:
             workspace = torch.empty(quadratic_loss_workspace_size(n), dtype=torch.uint8, device=self.device)
         if workspace.numel() * workspace.element_size() < quadratic_loss_workspace_size(n):
@@ -395,9 +369,7 @@ class QuadraticLoss:
         return out.data_ptr()
 
     def __call__(self, out_address: int):
-        with _on(self.device):
-            rc = _lib().zo_quadratic_loss(*self._args, ctypes.c_void_p(out_address), *self._ws, _stream(self.device))
-        _check("zo_quadratic_loss", rc)
+        _launch("zo_quadratic_loss", self.index, _lib().zo_quadratic_loss, *self._args, out_address, *self._ws)
 
 
 def quadratic_loss_static(theta, a, out=None):
@@ -413,10 +385,9 @@ def quadratic_loss_static(theta, a, out=None):
     if out.numel() < 1:
         raise ValueError("out must hold one float64")
     _same_device(dev, a=a, out=out)
-    with _on(dev):
-        rc = _lib().zo_quadratic_loss_static(_dev_ptr(theta, torch.float32, "theta"), _dev_ptr(a, torch.float32, "a"),
-                                             n, _dev_ptr(out, torch.float64, "out"), _stream(dev))
-    _check("zo_quadratic_loss_static", rc)
+    _launch("zo_quadratic_loss_static", _index(dev), _lib().zo_quadratic_loss_static,
+            _dev_ptr(theta, torch.float32, "theta"), _dev_ptr(a, torch.float32, "a"), n,
+            _dev_ptr(out, torch.float64, "out"))
     return out
 
 
@@ -447,6 +418,7 @@ class QuadraticPass:
         if packing not in (None, 1, 8):
             raise ValueError("packing must be None, 1 or 8")
         self.device = theta.device
+        self.index = _index(self.device)
         size = perturb_quadratic_loss_workspace_size(n)
         if workspace is None:
             workspace = torch.zeros(size, dtype=torch.uint8, device=self.device)
@@ -469,11 +441,8 @@ class QuadraticPass:
         """ops: a list of at most two (probe, scale) pairs applied in order;
         the loss goes to copies float64 cells stride elements apart."""
         nops, pa, sa, pb, sb = _quad_ops(ops)
-        with _on(self.device):
-            rc = _lib().zo_perturb_quadratic_loss(*self._args, seed, self.packing, nops, pa, sa, pb, sb,
-                                                  ctypes.c_void_p(out_address), copies, stride, *self._ws,
-                                                  _stream(self.device))
-        _check("zo_perturb_quadratic_loss", rc)
+        _launch("zo_perturb_quadratic_loss", self.index, _lib().zo_perturb_quadratic_loss, *self._args, seed,
+                self.packing, nops, pa, sa, pb, sb, out_address, copies, stride, *self._ws)
 
 
 def quadratic_points_workspace_size(K: int) -> int:
@@ -497,6 +466,7 @@ class QuadraticPoints:
         if losses.dim() != 2 or losses.shape[1] != 3:
             raise ValueError("losses must have shape (K, 3)")
         self.device = theta.device
+        self.index = _index(self.device)
         K = losses.shape[0]
         workspace = torch.zeros(quadratic_points_workspace_size(K), dtype=torch.uint8, device=self.device)
         c, status = out if out is not None else (None, None)
@@ -513,10 +483,8 @@ class QuadraticPoints:
         self.packing = packing or 0
 
     def __call__(self, seed: int, eps: float):
-        with _on(self.device):
-            rc = _lib().zo_quadratic_points(*self._args, seed, self.packing, self.K, eps, *self._out,
-                                            _stream(self.device))
-        _check("zo_quadratic_points", rc)
+        _launch("zo_quadratic_points", self.index, _lib().zo_quadratic_points, *self._args, seed, self.packing, self.K,
+                eps, *self._out)
 
 
 def perturb_quadratic_loss(theta, a, seed: int, ops, out=None, workspace=None, packing=None):
