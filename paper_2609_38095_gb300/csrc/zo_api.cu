@@ -67,17 +67,12 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
   return op;
 }
 
-// Packing-1 updates with at most this many probe groups keep both groups'
-// tables in shared memory for the whole launch (update_lut8_small_kernel);
-// all others walk the groups chunk by chunk (update_lut8_kernel).
-constexpr int kSmallGroups = 2;
-
 // Most items per SM of a list that update_items_kernel takes. It does two
 // lookups per element and group where the table-per-lane kernels do one, but
 // copies no tables; the lines lie where the two cross on 12 tensors of bf16
 // weights (us, items against tables):
 //   packing 1   K = 16: 3 M weights 10.5 / 12.9, 8 M 17.1 / 15.8
-//               K = 32: 8 M 23.1 / 23.4, 20 M 45.7 / 43.7
+//               K = 20: 5 M 14.7 / 15.1, 8 M 19.2 / 18.8;  K = 32: 16.8 / 17.1, 23.0 / 21.2
 //               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
 //   packing 8   K = 4: 3 M 10.9 / 15.0, 50 M 80 / 95, 205 M 304 / 353
 //               K = 32: 3 M 27.1 / 31.3, 20 M 132 / 128
@@ -85,7 +80,7 @@ constexpr int kSmallGroups = 2;
 // about 9 us here, 11 to 35 with the tables.
 int64_t update_items_per_sm(int packing, int groups) {
   if (packing == zo::kPacking8) return groups == 1 ? INT64_C(1) << 20 : 4096;
-  return groups == 3 || groups == 4 ? 4096 : 1600;
+  return groups == 3 || groups == 4 ? 2400 : 1600;
 }
 
 // Per-device launch facts, filled once per device.
@@ -439,7 +434,12 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
     if (done) return ZO_OK;
   }
-  const bool few = up.packing == zo::kPacking1 && up.groups <= kSmallGroups;
+  int64_t f32 = 0, all = 0;
+  for (int32_t i = 0; i < n_tensors; ++i) {
+    all += params[i].numel;
+    f32 += params[i].dtype == ZO_F32 ? params[i].numel : 0;
+  }
+  const bool few = zo::lut8_small_takes(up, 2 * f32 > all);
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t blk = 0;

@@ -191,13 +191,14 @@ struct UpdateParams {
   const int32_t* status;   // optional: when *status != 0 only `pre` is applied
 };
 
-// The update at one or two probe groups: the groups' and the leading
+// The update at one to kSmallGroups probe groups: the groups' and the leading
 // perturbation's Philox parts beside it. In its table launch blocks are
 // 32-byte items: half blocks of fp32 tensors, and 32 per 31 aligned chunks of
 // tensors off the 32-byte grid (kShift).
+constexpr int kSmallGroups = 4;
 struct SmallUpdateParams {
   UpdateParams u;
-  GroupRound01 g[2];
+  GroupRound01 g[kSmallGroups];
   GroupRound01 gp;
 };
 

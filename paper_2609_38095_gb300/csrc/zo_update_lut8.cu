@@ -32,8 +32,8 @@
 // the next pair's tables into the other; one barrier per pair separates the
 // two. The sums live in tensor memory (TMEM) between pairs, so the chunk is
 // not limited by registers: per pair, each 64 KB table copy and its barrier
-// serve 4096 blocks. With one or two groups (update_lut8_small_kernel) shared
-// memory holds them for the whole launch and there is no chunking.
+// serve 4096 blocks. Up to four groups' tables fit shared memory for the whole
+// launch (update_lut8_small_kernel): no chunks, and the sums stay in registers.
 #include <type_traits>
 
 #include "zo_device.cuh"
@@ -688,12 +688,12 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
 }
 
 // ---------------------------------------------------------------------------
-// One or two probe groups (K <= 16): the tables stay in shared memory for the
+// One to four probe groups (K <= 32): the tables stay in shared memory for the
 // whole launch, so there is no chunking and no barrier. The kernel walks
 // 32-byte items of theta grid-stride like the perturbation passes (sixteen
 // 16-bit or eight fp32 elements, half a Philox block), the next item's 256-bit
 // load issued before the current one is computed: the same sums, in the same
-// order (0 + T8_0 [+ T8_1]), as the chunk kernel.
+// order (0 + T8_0 + T8_1 ...), as the chunk kernel.
 //
 // At K <= 16 the bound is one pass over HBM, 379 cycles per warp and item at
 // 2.07 GHz, and what the SM has to issue in that time: two Philox calls cost
@@ -716,9 +716,18 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
 // weights in one flat buffer, K = 16: 0.749 -> 0.381 ms. Not adopted: a
 // prefetch of the item after the next into L2 (K = 16 -2 %, K = 8 +10 %).
 // ---------------------------------------------------------------------------
-constexpr int kSmallThreads = 1024;
-constexpr size_t small_smem_bytes(bool pairs_and_two) {
-  return (pairs_and_two ? 3 : 2) * static_cast<size_t>(kLut8Region) + 16u;
+// Threads of a CTA: three and four groups' words take more registers than 64
+// (OPT-1.3B-shaped set, ms at 512 / 768 / 1024 threads: three groups 1.107 /
+// 1.122 / 1.219 with the leading perturbation, 1.018 / 1.000 / 1.131 without;
+// four 1.386 / 1.629 / 1.612 and 1.284 / 1.270 / 1.474; 400 M weights in one
+// flat buffer 0.472 / 0.451 / 0.521 and 0.584 / 0.640 / 0.621).
+__host__ __device__ constexpr int small_threads(int G) { return G <= 2 ? 1024 : G == 3 ? 768 : 512; }
+// The last group's (T8, signed scale) pairs fill a region, plain tables half of one.
+__host__ __device__ constexpr uint32_t small_regions(int G, bool pairs) {
+  return pairs ? 1u + static_cast<uint32_t>(G) / 2u : (static_cast<uint32_t>(G) + 1u) / 2u;
+}
+constexpr size_t small_smem_bytes(int G, bool pairs) {
+  return (1 + small_regions(G, pairs)) * static_cast<size_t>(kLut8Region) + 16u;
 }
 
 __device__ __forceinline__ void lds_pair(uint32_t addr, float& a, float& b) {
@@ -732,29 +741,32 @@ __device__ __forceinline__ uint32_t entry_addr(uint32_t w, uint32_t frame) {
 }
 
 // The leading perturbation in the small kernel: none, in the last group's
-// table, or with Philox words of its own.
-constexpr int kPreNone = 0, kPreTable = 1, kPreOwn = 2;
+// table, with Philox words of its own, or with the last group's words (four
+// groups, whose tables leave no room for pairs).
+constexpr int kPreNone = 0, kPreTable = 1, kPreOwn = 2, kPreLast = 3;
 
-// Sum of element I (t), and with kPreTable its leading perturbation (d).
-template <int I, int PRE, bool TWO>
-__device__ __forceinline__ void small_sums(uint32_t w0, uint32_t wl, uint32_t f0, uint32_t fl, float& t0, float& tl,
-                                           float& d) {
-  if constexpr (TWO) t0 = lds_f32(entry_addr<I>(w0, f0));
+// Element I's partial sums, and with kPreTable its leading perturbation (d).
+// x: the groups' words; f0, fl: frames of group 0's and the last group's tables.
+template <int I, int PRE, int G>
+__device__ __forceinline__ void small_sums(const uint4 (&x)[G], uint32_t f0, uint32_t fl, float (&t)[G], float& d) {
+#pragma unroll
+  for (int g = 0; g < G - 1; ++g)
+    t[g] = lds_f32(entry_addr<I>(word_of(x[g], I >> 2), f0 + (g & 1) * 128u + (g >> 1) * kLut8Region));
   if constexpr (PRE == kPreTable)
-    lds_pair(entry_addr<I>(wl, fl), tl, d);
+    lds_pair(entry_addr<I>(word_of(x[G - 1], I >> 2), fl), t[G - 1], d);
   else
-    tl = lds_f32(entry_addr<I>(wl, fl));
+    t[G - 1] = lds_f32(entry_addr<I>(word_of(x[G - 1], I >> 2), fl));
 }
 
-// Sixteen 16-bit elements. x0, xl: words of group 0 and of the last group.
-template <uint8_t DT, int PRE, bool TWO, int R>
-__device__ __forceinline__ void small_pair16(uint32_t& v, const uint4& x0, const uint4& xl, const uint4& xp,
-                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
+// Elements 2R and 2R + 1, 16-bit.
+template <uint8_t DT, int PRE, int G, int R>
+__device__ __forceinline__ void small_pair16(uint32_t& v, const uint4 (&x)[G], const uint4& xp, uint32_t f0,
+                                             uint32_t fl, const UpdateParams& P) {
   constexpr int e = 2 * R;
   float2 f = unpack2<DT>(v);
-  float a0 = 0.0f, a1 = 0.0f, l0, l1, d0 = 0.0f, d1 = 0.0f;
-  small_sums<e, PRE, TWO>(word_of(x0, e >> 2), word_of(xl, e >> 2), f0, fl, a0, l0, d0);
-  small_sums<e + 1, PRE, TWO>(word_of(x0, e >> 2), word_of(xl, e >> 2), f0, fl, a1, l1, d1);
+  float t[G], u[G], d0 = 0.0f, d1 = 0.0f;
+  small_sums<e, PRE, G>(x, f0, fl, t, d0);
+  small_sums<e + 1, PRE, G>(x, f0, fl, u, d1);
   if constexpr (PRE != kPreNone) {
     if constexpr (PRE == kPreTable) {
       f.x = __fadd_rn(f.x, d0);
@@ -764,74 +776,84 @@ __device__ __forceinline__ void small_pair16(uint32_t& v, const uint4& x0, const
     }
     f = unpack2<DT>(pack2<DT>(f.x, f.y));  // the perturbed value is rounded to storage first
   }
+#pragma unroll
+  for (int g = 1; g < G - 1; ++g) fadd2_rn(t[0], u[0], t[g], u[g]);
   if constexpr (PRE == kPreTable) {
-    if constexpr (TWO) {
-      l0 = __fadd_rn(a0, l0);
-      l1 = __fadd_rn(a1, l1);
+    if constexpr (G > 1) {
+      t[0] = __fadd_rn(t[0], t[G - 1]);
+      u[0] = __fadd_rn(u[0], u[G - 1]);
     }
-    f.x = __fadd_rn(f.x, l0);
-    f.y = __fadd_rn(f.y, l1);
-  } else if constexpr (TWO) {
-    fadd2_rn(a0, a1, l0, l1);
-    fadd2_rn(f.x, f.y, a0, a1);
+    f.x = __fadd_rn(f.x, t[0]);
+    f.y = __fadd_rn(f.y, u[0]);
   } else {
-    fadd2_rn(f.x, f.y, l0, l1);
+    if constexpr (G > 1) fadd2_rn(t[0], u[0], t[G - 1], u[G - 1]);
+    fadd2_rn(f.x, f.y, t[0], u[0]);
   }
   v = pack2<DT>(f.x, f.y);
 }
 
-template <uint8_t DT, int PRE, bool TWO>
-__device__ __forceinline__ void small_item16(uint32_t (&v)[8], const uint4& x0, const uint4& xl, const uint4& xp,
-                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
-  small_pair16<DT, PRE, TWO, 0>(v[0], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 1>(v[1], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 2>(v[2], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 3>(v[3], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 4>(v[4], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 5>(v[5], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 6>(v[6], x0, xl, xp, f0, fl, P);
-  small_pair16<DT, PRE, TWO, 7>(v[7], x0, xl, xp, f0, fl, P);
+template <uint8_t DT, int PRE, int G>
+__device__ __forceinline__ void small_item16(uint32_t (&v)[8], const uint4 (&x)[G], const uint4& xp, uint32_t f0,
+                                             uint32_t fl, const UpdateParams& P) {
+  small_pair16<DT, PRE, G, 0>(v[0], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 1>(v[1], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 2>(v[2], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 3>(v[3], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 4>(v[4], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 5>(v[5], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 6>(v[6], x, xp, f0, fl, P);
+  small_pair16<DT, PRE, G, 7>(v[7], x, xp, f0, fl, P);
 }
 
 // One fp32 element (scalar adds, as every fp32 path).
-template <int PRE, bool TWO, int I>
-__device__ __forceinline__ void small_one32(uint32_t& v, const uint4& x0, const uint4& xl, const uint4& xp, uint32_t f0,
-                                            uint32_t fl, const UpdateParams& P) {
+template <int PRE, int G, int I>
+__device__ __forceinline__ void small_one32(uint32_t& v, const uint4 (&x)[G], const uint4& xp, uint32_t f0, uint32_t fl,
+                                            const UpdateParams& P) {
   float th = __uint_as_float(v);
-  float a = 0.0f, l, d = 0.0f;
-  small_sums<I, PRE, TWO>(word_of(x0, I >> 2), word_of(xl, I >> 2), f0, fl, a, l, d);
-  if constexpr (PRE == kPreTable) th = __fadd_rn(th, d);
-  if constexpr (PRE == kPreOwn) th = add_signed(th, xp, I, P.pre);
-  v = __float_as_uint(__fadd_rn(th, TWO ? __fadd_rn(a, l) : l));
+  float t[G], d = 0.0f;
+  small_sums<I, PRE, G>(x, f0, fl, t, d);
+  if constexpr (PRE == kPreTable)
+    th = __fadd_rn(th, d);
+  else if constexpr (PRE != kPreNone)
+    th = add_signed(th, xp, I, P.pre);
+#pragma unroll
+  for (int g = 1; g < G; ++g) t[0] = __fadd_rn(t[0], t[g]);
+  v = __float_as_uint(__fadd_rn(th, t[0]));
 }
 
-template <int PRE, bool TWO>
-__device__ __forceinline__ void small_item32(uint32_t (&v)[8], const uint4& x0, const uint4& xl, const uint4& xp,
-                                             uint32_t f0, uint32_t fl, const UpdateParams& P) {
-  small_one32<PRE, TWO, 0>(v[0], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 1>(v[1], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 2>(v[2], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 3>(v[3], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 4>(v[4], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 5>(v[5], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 6>(v[6], x0, xl, xp, f0, fl, P);
-  small_one32<PRE, TWO, 7>(v[7], x0, xl, xp, f0, fl, P);
+template <int PRE, int G>
+__device__ __forceinline__ void small_item32(uint32_t (&v)[8], const uint4 (&x)[G], const uint4& xp, uint32_t f0,
+                                             uint32_t fl, const UpdateParams& P) {
+  small_one32<PRE, G, 0>(v[0], x, xp, f0, fl, P);
+  small_one32<PRE, G, 1>(v[1], x, xp, f0, fl, P);
+  small_one32<PRE, G, 2>(v[2], x, xp, f0, fl, P);
+  small_one32<PRE, G, 3>(v[3], x, xp, f0, fl, P);
+  small_one32<PRE, G, 4>(v[4], x, xp, f0, fl, P);
+  small_one32<PRE, G, 5>(v[5], x, xp, f0, fl, P);
+  small_one32<PRE, G, 6>(v[6], x, xp, f0, fl, P);
+  small_one32<PRE, G, 7>(v[7], x, xp, f0, fl, P);
 }
 
 // An item across an end of its tensor, element by element (not inlined: it
 // is rare and would otherwise hold registers in the loop). e0: the item's
 // first element; do_sum false: the leading perturbation alone.
-template <int PRE, bool TWO, bool ANY>
+// x0, mid, xl: the groups' words (one group: xl)
+template <int PRE, int G, class... Mid>
 __device__ __noinline__ void small_elements(void* base, uint8_t dt, int64_t e0, int64_t numel, uint4 x0, uint4 xl,
-                                            uint4 xp, uint32_t f0, uint32_t fl, bool do_sum, PerturbOp pre) {
+                                            uint4 xp, uint32_t f0, uint32_t fl, bool do_sum, PerturbOp pre, Mid... mid) {
+  const uint4 x[G > 1 ? G - 1 : 1] = {x0, mid...};
   const int per = dt == kF32 ? 8 : 16;
   const int lo = e0 < 0 ? static_cast<int>(-e0) : 0;
   const int hi = static_cast<int>(min(static_cast<int64_t>(per), numel - e0));
   map_elements<2>(base, dt, e0, lo, hi, [&](int m, int j, float v) {
-    float th = v, a = 0.0f, l = 0.0f, d = 0.0f;
+    float th = v, t = 0.0f, l = 0.0f, d = 0.0f;
     if (do_sum) {
       const uint32_t sel = 0x7604u | (static_cast<uint32_t>(j) << 4);
-      if constexpr (TWO) a = lds_f32(__byte_perm(word_of(x0, m), f0, sel));
+#pragma unroll
+      for (int g = 0; g < G - 1; ++g) {
+        const float p = lds_f32(__byte_perm(word_of(x[g], m), f0 + (g & 1) * 128u + (g >> 1) * kLut8Region, sel));
+        t = g == 0 ? p : __fadd_rn(t, p);
+      }
       const uint32_t at = __byte_perm(word_of(xl, m), fl, sel);
       if constexpr (PRE == kPreTable)
         lds_pair(at, l, d);
@@ -842,7 +864,7 @@ __device__ __noinline__ void small_elements(void* base, uint8_t dt, int64_t e0, 
       th = do_sum && PRE == kPreTable ? __fadd_rn(th, d) : add_signed_word(th, word_of(xp, m), j, pre);
       th = round_to_storage(dt, th);
     }
-    return do_sum ? __fadd_rn(th, TWO ? __fadd_rn(a, l) : l) : th;
+    return do_sum ? __fadd_rn(th, G > 1 ? __fadd_rn(t, l) : l) : th;
   });
 }
 
@@ -916,65 +938,78 @@ __device__ __forceinline__ uint4 small_window(const SmallCursor& c, const SmallI
 
 // ANY: the launch may hold fp32 tensors (numbered in half blocks) and tensors
 // off the 32-byte grid (32 launch items per 31 chunks).
-template <int PRE, bool TWO, bool ANY>
-__global__ void __launch_bounds__(kSmallThreads, 1)
+template <int PRE, int G, bool ANY>
+__global__ void __launch_bounds__(small_threads(G), 1)
     update_lut8_small_kernel(const __grid_constant__ SmallUpdateParams S) {
+  constexpr int kThreads = small_threads(G);
   const UpdateParams& P = S.u;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
-  constexpr int G = TWO ? 2 : 1;
-  constexpr uint32_t kRegions = TWO && PRE == kPreTable ? 2u : 1u;
+  constexpr uint32_t kRegions = small_regions(G, PRE == kPreTable);
   const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
   const uint32_t region0 = (sbase + kLut8Region - 1u) & ~(kLut8Region - 1u);
-  // coefficients and unreplicated tables (2 KB at most) below the region, or after it when the window starts on
+  // coefficients and unreplicated tables (1 KB per group) below the region, or after it when the window starts on
   // a 64 KB boundary
   const uint32_t hdr = region0 - sbase >= 32u * G + 1024u * G ? sbase : region0 + kRegions * kLut8Region;
   float* a_s = reinterpret_cast<float*>(smem + (hdr - sbase));
   float* t8 = a_s + 8 * G;
   if (threadIdx.x == 0) skip_s = (P.status != nullptr && *P.status != 0);
-  for (int k = threadIdx.x; k < 8 * G; k += kSmallThreads)
+  for (int k = threadIdx.x; k < 8 * G; k += kThreads)
     a_s[k] = k < P.K ? __double2float_rn(P.coef_mul * P.coef[k]) : 0.0f;
   __syncthreads();
   const bool do_sum = skip_s == 0;  // a failed preconditioner still gets the leading perturbation
   if (!do_sum && PRE == kPreNone) return;
   if (do_sum) {
-    for (int e = threadIdx.x; e < 256 * G; e += kSmallThreads) {
+    for (int e = threadIdx.x; e < 256 * G; e += kThreads) {
       const float* a = a_s + 8 * (e >> 8);
       const uint32_t n = static_cast<uint32_t>(e) & 255u;
       const float v = __fadd_rn(quad_partial(a, n & 15u), quad_partial(a + 4, n >> 4));
       t8[e] = e < 256 ? __fadd_rn(0.0f, v) : v;
     }
     __syncthreads();
-    // rows of 256 bytes. Pairs: (T8, signed scale) of the last group, lane l in 8-byte word l; plain tables: lane
-    // l in word l of the first (group 0, or the only group) or second (group 1) half of the row
+    // rows of 256 bytes. Pairs: (T8, signed scale) of the last group, lane l in 8-byte word l of the last region;
+    // plain tables: group g in region g / 2, lane l in word l of half g mod 2 of the row
     constexpr int kPieces = 256 * 16;  // 16-byte pieces of a region
-    for (int i = threadIdx.x; i < kPieces; i += kSmallThreads) {
+    for (int i = threadIdx.x; i < kPieces; i += kThreads) {
       const uint32_t n = static_cast<uint32_t>(i) >> 4, piece = static_cast<uint32_t>(i) & 15u;
-      const uint32_t row = region0 + 256u * n + 16u * piece;
-      if constexpr (PRE == kPreTable) {
-        const float v = t8[256 * (G - 1) + n];
-        const float d = __uint_as_float(P.pre.nscale_bits ^ (((n >> P.pre.bit) & 1u) << 31));
-        const uint32_t at = row + (kRegions - 1u) * kLut8Region;
-        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" ::"r"(at), "f"(v), "f"(d) : "memory");
-        if (TWO && piece < 8u) sts_f32x4(row, t8[n]);
-      } else {
-        if (piece < 8u || TWO) sts_f32x4(row, t8[(piece < 8u ? 0 : 256) + n]);
+#pragma unroll
+      for (uint32_t r = 0; r < kRegions; ++r) {
+        const uint32_t row = region0 + r * kLut8Region + 256u * n + 16u * piece;
+        if (PRE == kPreTable && r == kRegions - 1u) {
+          const float v = t8[256 * (G - 1) + n];
+          const float d = __uint_as_float(P.pre.nscale_bits ^ (((n >> P.pre.bit) & 1u) << 31));
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" ::"r"(row), "f"(v), "f"(d) : "memory");
+        } else {
+          const uint32_t g = 2u * r + (piece >> 3);
+          if (g < static_cast<uint32_t>(PRE == kPreTable ? G - 1 : G)) sts_f32x4(row, t8[256u * g + n]);
+        }
       }
     }
     __syncthreads();
   }
   const TensorTable& tab = P.tab;
   const uint32_t total = tab.blk_total;
-  const uint32_t stride = gridDim.x * kSmallThreads;
+  const uint32_t stride = gridDim.x * kThreads;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t f0 = (region0 & 0xFFFF0000u) | (lane << 2);
-  const uint32_t fl = PRE == kPreTable ? ((region0 + (kRegions - 1u) * kLut8Region) & 0xFFFF0000u) | (lane << 3)
-                                       : (TWO ? f0 | 128u : f0);
-  uint32_t b = blockIdx.x * kSmallThreads + threadIdx.x;
+  const uint32_t fl = PRE == kPreTable
+                          ? ((region0 + (kRegions - 1u) * kLut8Region) & 0xFFFF0000u) | (lane << 3)
+                          : f0 + ((G - 1) & 1) * 128u + ((G - 1) >> 1) * kLut8Region;
+  uint32_t b = blockIdx.x * kThreads + threadIdx.x;
   if (b - lane >= total) return;
   SmallCursor c;
   c.t = 0;
   small_seek<ANY>(tab, c, b - lane);
+  const auto edge = [&](const SmallCursor& at, const SmallItem& i, const uint4 (&x)[G], const uint4& xp, bool sum) {
+    const uint8_t dt = at.fl & kDtypeMask;
+    const int64_t n = tab.numel[at.t];
+    if constexpr (G <= 2)
+      small_elements<PRE, G>(at.p, dt, i.e0, n, x[0], x[G - 1], xp, f0, fl, sum, P.pre);
+    else if constexpr (G == 3)
+      small_elements<PRE, G>(at.p, dt, i.e0, n, x[0], x[2], xp, f0, fl, sum, P.pre, x[1]);
+    else
+      small_elements<PRE, G>(at.p, dt, i.e0, n, x[0], x[3], xp, f0, fl, sum, P.pre, x[1], x[2]);
+  };
   if (!do_sum) {
     for (; b - lane < total; b += stride) {
       if (b - lane >= c.te) small_seek<ANY>(tab, c, b - lane);
@@ -982,7 +1017,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       const BlockCounter<true> kb(k.blk, 0, P.keys);
       uint4 xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
       if (ANY) xp = small_window(c, k, xp);
-      if (k.act) small_elements<PRE, TWO, ANY>(c.p, c.fl & kDtypeMask, k.e0, tab.numel[c.t], xp, xp, xp, f0, fl, false, P.pre);
+      uint4 x[G];  // not looked at
+#pragma unroll
+      for (int g = 0; g < G; ++g) x[g] = xp;
+      if (k.act) edge(c, k, x, xp, false);
     }
     return;
   }
@@ -1001,25 +1039,29 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       if (kn.full) ld256(kn.p, vn);
     }
     const BlockCounter<true> kb(k.blk, 0, P.keys);
-    uint4 x0 = philox_finish(kb.start(S.g[0], 0u, P.keys), P.keys);
-    uint4 xl = TWO ? philox_finish(kb.start(S.g[1], 1u, P.keys), P.keys) : x0;
+    uint4 x[G];
+    x[0] = philox_finish(kb.start(S.g[0], 0u, P.keys), P.keys);
+#pragma unroll
+    for (int g = 1; g < G; ++g) x[g] = philox_finish(kb.start(S.g[g], static_cast<uint32_t>(g), P.keys), P.keys);
     uint4 xp = make_uint4(0u, 0u, 0u, 0u);
     if (PRE == kPreOwn) xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
     if (ANY) {
-      x0 = small_window(c, k, x0);
-      xl = TWO ? small_window(c, k, xl) : x0;
+      x[0] = small_window(c, k, x[0]);
+#pragma unroll
+      for (int g = 1; g < G; ++g) x[g] = small_window(c, k, x[g]);
       if (PRE == kPreOwn) xp = small_window(c, k, xp);
     }
+    if (PRE == kPreLast) xp = x[G - 1];
     if (k.full) {
       if (ANY && (c.fl & kDtypeMask) == kF32)
-        small_item32<PRE, TWO>(v, x0, xl, xp, f0, fl, P);
+        small_item32<PRE, G>(v, x, xp, f0, fl, P);
       else if ((c.fl & kDtypeMask) == kBF16)
-        small_item16<kBF16, PRE, TWO>(v, x0, xl, xp, f0, fl, P);
+        small_item16<kBF16, PRE, G>(v, x, xp, f0, fl, P);
       else
-        small_item16<kF16, PRE, TWO>(v, x0, xl, xp, f0, fl, P);
+        small_item16<kF16, PRE, G>(v, x, xp, f0, fl, P);
       st256(k.p, v);
     } else if (k.act) {
-      small_elements<PRE, TWO, ANY>(c.p, c.fl & kDtypeMask, k.e0, tab.numel[c.t], x0, xl, xp, f0, fl, true, P.pre);
+      edge(c, k, x, xp, true);
     }
     if (!more) break;
     b = bn;
@@ -1045,25 +1087,29 @@ cudaError_t lut8_limit() {
                               static_cast<int>(lut8_smem_bytes(PACK8)));
 }
 
-template <int PRE, bool TWO, bool ANY>
+template <int PRE, int G, bool ANY>
 cudaError_t small_limit() {
-  return cudaFuncSetAttribute(update_lut8_small_kernel<PRE, TWO, ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(small_smem_bytes(TWO && PRE == kPreTable)));
+  return cudaFuncSetAttribute(update_lut8_small_kernel<PRE, G, ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(small_smem_bytes(G, PRE == kPreTable)));
 }
 
-template <int PRE>
+template <int PRE, int G>
 cudaError_t small_limits() {
-  cudaError_t e = small_limit<PRE, false, false>();
-  if (e == cudaSuccess) e = small_limit<PRE, true, false>();
-  if (e == cudaSuccess) e = small_limit<PRE, false, true>();
-  if (e == cudaSuccess) e = small_limit<PRE, true, true>();
-  return e;
+  const cudaError_t e = small_limit<PRE, G, false>();
+  return e == cudaSuccess ? small_limit<PRE, G, true>() : e;
 }
 
 cudaError_t lut8_prepare() {
-  cudaError_t e = small_limits<kPreNone>();
-  if (e == cudaSuccess) e = small_limits<kPreTable>();
-  if (e == cudaSuccess) e = small_limits<kPreOwn>();
+  cudaError_t e = small_limits<kPreNone, 1>();
+  if (e == cudaSuccess) e = small_limits<kPreNone, 2>();
+  if (e == cudaSuccess) e = small_limits<kPreNone, 3>();
+  if (e == cudaSuccess) e = small_limits<kPreNone, 4>();
+  if (e == cudaSuccess) e = small_limits<kPreTable, 1>();
+  if (e == cudaSuccess) e = small_limits<kPreTable, 2>();
+  if (e == cudaSuccess) e = small_limits<kPreTable, 3>();
+  if (e == cudaSuccess) e = small_limits<kPreLast, 4>();
+  if (e == cudaSuccess) e = small_limits<kPreOwn, 1>();
+  if (e == cudaSuccess) e = small_limits<kPreOwn, 2>();
   if (e == cudaSuccess) e = lut8_limit<true, false, false>();
   if (e == cudaSuccess) e = lut8_limit<true, false, false, true>();
   if (e == cudaSuccess) e = lut8_limit<true, true, false>();
@@ -1083,37 +1129,50 @@ bool one_high_word(const TensorTable& tab) {
   return (first >> 32) == (last >> 32);
 }
 
-template <int PRE, bool TWO>
-void launch_small_cfg(const SmallUpdateParams& p, bool any, int grid, cudaStream_t stream) {
-  constexpr size_t sm = small_smem_bytes(TWO && PRE == kPreTable);
+template <int PRE, int G>
+void launch_small_cfg(const SmallUpdateParams& p, bool any, int sms, cudaStream_t stream) {
+  constexpr size_t sm = small_smem_bytes(G, PRE == kPreTable);
+  constexpr int threads = small_threads(G);
+  const int64_t want = (static_cast<int64_t>(p.u.tab.blk_total) + threads - 1) / threads;
+  const int grid = static_cast<int>(want < sms ? want : sms);
   if (any)
-    update_lut8_small_kernel<PRE, TWO, true><<<grid, kSmallThreads, sm, stream>>>(p);
+    update_lut8_small_kernel<PRE, G, true><<<grid, threads, sm, stream>>>(p);
   else
-    update_lut8_small_kernel<PRE, TWO, false><<<grid, kSmallThreads, sm, stream>>>(p);
+    update_lut8_small_kernel<PRE, G, false><<<grid, threads, sm, stream>>>(p);
 }
 
-template <int PRE>
-void launch_small_pre(const SmallUpdateParams& p, bool any, int grid, cudaStream_t stream) {
-  if (p.u.groups == 2)
-    launch_small_cfg<PRE, true>(p, any, grid, stream);
-  else
-    launch_small_cfg<PRE, false>(p, any, grid, stream);
+// Which updates the small kernel takes. Three and four groups only with the
+// leading perturbation's probe in the last group, or none: words of its own
+// would be a fifth Philox call's registers. It makes a block's words once per
+// item, so twice for fp32, where the chunk kernel makes them once: with four
+// groups that costs fp32 lists more than the chunks' tables and barriers do
+// (205 M fp32 weights, K = 32: 0.412 ms here, 0.379 there; K = 24: 0.338 and
+// 0.347). Before, K from 17 on walked the chunks: OPT-1.3B-shaped bf16 set with
+// the leading perturbation, K = 24 / 32: 1.612 / 1.857 -> 1.122 / 1.386 ms;
+// 400 M bf16 weights in one flat buffer 0.677 / 0.747 -> 0.451 / 0.584 ms.
+bool lut8_small_takes(const UpdateParams& u, bool mostly_f32) {
+  if (u.packing != kPacking1 || u.groups > kSmallGroups || (u.groups == 4 && mostly_f32)) return false;
+  return u.groups <= 2 || !u.has_pre || u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups);
 }
 
 cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream) {
   const UpdateParams& u = p.u;
   const uint32_t bhi = static_cast<uint32_t>(static_cast<uint64_t>(u.tab.blk_base) >> 32);
-  p.g[0] = group_round01(0u, bhi, u.keys);
-  p.g[1] = group_round01(1u, bhi, u.keys);
+  for (uint32_t g = 0; g < static_cast<uint32_t>(kSmallGroups); ++g) p.g[g] = group_round01(g, bhi, u.keys);
   p.gp = group_round01(u.pre.ctr2, bhi, u.keys);
-  const int64_t want = (static_cast<int64_t>(u.tab.blk_total) + kSmallThreads - 1) / kSmallThreads;
-  const int grid = static_cast<int>(want < sms ? want : sms);
-  if (!u.has_pre)
-    launch_small_pre<kPreNone>(p, any, grid, stream);
-  else if (u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups))
-    launch_small_pre<kPreTable>(p, any, grid, stream);
+  const bool last = u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups);
+  if (u.groups == 1)
+    !u.has_pre ? launch_small_cfg<kPreNone, 1>(p, any, sms, stream)
+    : last     ? launch_small_cfg<kPreTable, 1>(p, any, sms, stream)
+               : launch_small_cfg<kPreOwn, 1>(p, any, sms, stream);
+  else if (u.groups == 2)
+    !u.has_pre ? launch_small_cfg<kPreNone, 2>(p, any, sms, stream)
+    : last     ? launch_small_cfg<kPreTable, 2>(p, any, sms, stream)
+               : launch_small_cfg<kPreOwn, 2>(p, any, sms, stream);
+  else if (u.groups == 3)
+    !u.has_pre ? launch_small_cfg<kPreNone, 3>(p, any, sms, stream) : launch_small_cfg<kPreTable, 3>(p, any, sms, stream);
   else
-    launch_small_pre<kPreOwn>(p, any, grid, stream);
+    !u.has_pre ? launch_small_cfg<kPreNone, 4>(p, any, sms, stream) : launch_small_cfg<kPreLast, 4>(p, any, sms, stream);
   return cudaGetLastError();
 }
 
