@@ -69,17 +69,26 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 
 // Most items per SM of a list that update_items_kernel takes. It does two
 // lookups per element and group where the table-per-lane kernels do one, but
-// copies no tables; the lines lie where the two cross on 12 tensors of bf16
-// weights (us, items against tables):
+// copies no tables; the lines lie where the two cross on 12 or 24 tensors (us,
+// items against tables):
 //   packing 1   K = 16: 3 M weights 10.5 / 12.9, 8 M 17.1 / 15.8
 //               K = 20: 5 M 14.7 / 15.1, 8 M 19.2 / 18.8;  K = 32: 16.8 / 17.1, 23.0 / 21.2
 //               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
-//   packing 8   K = 4: 3 M 10.9 / 15.0, 50 M 80 / 95, 205 M 304 / 353
-//               K = 32: 3 M 27.1 / 31.3, 20 M 132 / 128
-// (3 M weights are 1233 items per SM). Between 1 and 0.05 M all of these take
-// about 9 us here, 11 to 35 with the tables.
-int64_t update_items_per_sm(int packing, int groups) {
-  if (packing == zo::kPacking8) return groups == 1 ? INT64_C(1) << 20 : 4096;
+// (3 M weights are 1233 items per SM). Under packing 8 generating the bits is
+// most of the work and full occupancy does it best, whatever the size, but for
+// long lists of many groups; fp32 items hold half a block each and make its
+// words twice:
+//   16 bits     K = 3: 5 M 13.8 / 20.3, 205 M 279 / 317;  K = 24: 29.2 / 38.0, 872 / 907
+//               K = 64: 60 M 628 / 633, 205 M 2116 / 2091;  K = 128: 1212 / 1207, 4109 / 4021
+//   fp32        K = 3: 3 M 12.9 / 15.0, 6 M 21.1 / 19.8;  K = 24: 1 M 14.7 / 15.0, 3 M 31.2 / 27.0
+//               K = 64: 1 M 27.2 / 23.2
+// (1 M fp32 weights are 822 items per SM). Between 1 and 0.05 M weights of
+// packing 1 all of these take about 9 us here, 11 to 35 with the tables.
+int64_t update_items_per_sm(int packing, int groups, bool mostly_f32) {
+  if (packing == zo::kPacking8) {
+    if (mostly_f32) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
+    return groups < 8 ? INT64_C(1) << 20 : 24000;
+  }
   return groups == 3 || groups == 4 ? 2400 : 1600;
 }
 
@@ -407,13 +416,23 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  const int64_t most_items = update_items_per_sm(up.packing, up.groups) * d->sms;
+  int64_t f32 = 0, all = 0;
+  for (int32_t i = 0; i < n_tensors; ++i) {
+    all += params[i].numel;
+    f32 += params[i].dtype == ZO_F32 ? params[i].numel : 0;
+  }
+  const bool mostly_f32 = 2 * f32 > all;
+  const int64_t most_items = update_items_per_sm(up.packing, up.groups, mostly_f32) * d->sms;
   const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
     zo::ItemsCursor cur;
     const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
                                          most_items);
     *done = cur.t == n_tensors && one_high && ip.total <= most_items;
     if (!*done || ip.n == 0) return cudaSuccess;
+    // packing 8: several items per thread where ten waves of CTAs remain, which spread a CTA's tables over more
+    // work (205 M bf16 weights, K = 8, one / eight items: 396 / 376 us; 20 M: 44 / 48)
+    const int64_t waves = ip.total / (INT64_C(8) * 128 * 10 * d->sms);
+    ip.rounds = static_cast<uint32_t>(waves < 1 ? 1 : waves > 8 ? 8 : waves);
     ip.bhi = 0;
     ip.keys = up.keys;
     ip.coef = c;
@@ -434,12 +453,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
     if (done) return ZO_OK;
   }
-  int64_t f32 = 0, all = 0;
-  for (int32_t i = 0; i < n_tensors; ++i) {
-    all += params[i].numel;
-    f32 += params[i].dtype == ZO_F32 ? params[i].numel : 0;
-  }
-  const bool few = zo::lut8_small_takes(up, 2 * f32 > all);
+  const bool few = zo::lut8_small_takes(up, mostly_f32);
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t blk = 0;

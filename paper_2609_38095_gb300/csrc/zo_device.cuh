@@ -581,6 +581,7 @@ struct UpdateItemsParams {
   int32_t n;
   int32_t hint_shift;
   uint32_t total;
+  uint32_t rounds;         // packing 8: items a thread takes, one CTA apart
   uint32_t bhi;            // the virtual blocks' counter high word
   RoundKeys keys;
   const double* coef;

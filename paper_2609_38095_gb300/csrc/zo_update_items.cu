@@ -17,6 +17,15 @@
 // -> 8.7 / 8.2 / 8.8 / 15.1 us; as fp32, K = 32 15.0 -> 8.2; in one flat buffer
 // 23.3 -> 8.6; packing 8, K = 32 14.5 -> 10.2. Not adopted: a grid of 8 to 64
 // CTAs per SM that walks the items (K = 256, 8 M weights 97.5 -> 98-107 us).
+//
+// Packing 8 has eight Philox calls per group and is bound by them (85 to 90
+// cycles per warp and call on an SM's quarter). A full group's calls are
+// unrolled, several chains in flight per thread, and a thread of a long list
+// takes up to eight items: 205 M bf16 weights, K = 8 / 24 / 32: 417 / 907 /
+// 1130 -> 374 / 872 / 1120 us (a persistent grid with plain Philox calls took
+// 378 / 880 / 1130), 20 M 46.7 / 105 / 128 -> 44.4 / 93.8 / 117.5. Not adopted:
+// the calls in twos or fours (K = 8 445 / 432 us), registers capped at 40 for
+// more warps (spills; 409), CTAs of 256 threads (406).
 #include "zo_device.cuh"
 #include "zo_launch.h"
 
@@ -78,20 +87,32 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
   }
   // this thread's item, its load on the way while the tables are made
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t b = blockIdx.x * kItemThreads + threadIdx.x, wb = b - lane;
-  const bool here = wb < P.total;  // the same in all lanes
-  int t = here ? P.hint[wb >> P.hint_shift] : 0;
-  while (here && wb >= P.e[t].end) ++t;
-  const ItemsEntry e = P.e[t];
-  const uint8_t dt = static_cast<uint8_t>(e.meta & kDtypeMask);
-  const bool f32 = dt == kF32, shift = (e.meta & kShift) != 0;
-  const uint32_t a = e.meta >> 16;
-  ItemPlace k = item_place(e, b);
-  k.full = k.full && here;
-  k.act = k.act && here;
-  char* p = reinterpret_cast<char*>(e.base) + static_cast<int64_t>(k.i) * 32;
+  uint32_t b = blockIdx.x * (kItemThreads * (PACK8 ? P.rounds : 1u)) + threadIdx.x;
+  bool here = false;  // the same in all lanes
+  ItemsEntry e;
+  uint8_t dt = 0;
+  bool f32 = false, shift = false;
+  uint32_t a = 0;
+  ItemPlace k;
+  char* p = nullptr;
   uint32_t v[8];
-  if (k.full) ld256(p, v);
+  const auto seek = [&] {
+    const uint32_t wb = b - lane;
+    here = wb < P.total;
+    int t = here ? P.hint[wb >> P.hint_shift] : 0;
+    while (here && wb >= P.e[t].end) ++t;
+    e = P.e[t];
+    dt = static_cast<uint8_t>(e.meta & kDtypeMask);
+    f32 = dt == kF32;
+    shift = (e.meta & kShift) != 0;
+    a = e.meta >> 16;
+    k = item_place(e, b);
+    k.full = k.full && here;
+    k.act = k.act && here;
+    p = reinterpret_cast<char*>(e.base) + static_cast<int64_t>(k.i) * 32;
+    if (k.full) ld256(p, v);
+  };
+  seek();
   __syncthreads();
   const bool do_sum = skip_s == 0;  // a failed preconditioner still gets the leading perturbation
   if (!do_sum && !P.has_pre) return;
@@ -101,73 +122,90 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
   }
   __syncthreads();
   if (!here) return;
-  const BlockRound01 blk = block_round01(static_cast<uint32_t>(item_block(e, k.i)), P.keys);
-  const auto call = [&](uint32_t c) {
-    const uint4 r = r01_s[c];
-    return philox_finish(philox_start(blk, {r.x, r.y, r.z}), P.keys);
-  };
-  float acc[16];
+  const auto item = [&] {
+    const BlockRound01 blk = block_round01(static_cast<uint32_t>(item_block(e, k.i)), P.keys);
+    const auto call = [&](uint32_t c) {
+      const uint4 r = r01_s[c];
+      return philox_finish(philox_start(blk, {r.x, r.y, r.z}), P.keys);
+    };
+    float acc[16];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
-  if (do_sum) {
-    uint32_t frame = frame0;
+    for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
+    if (do_sum) {
+      uint32_t frame = frame0;
 #pragma unroll 1
-    for (int q = 0; q < G; ++q, frame += kFrame) {
-      uint4 x;
-      if constexpr (PACK8) {
-        x = make_uint4(0u, 0u, 0u, 0u);
+      for (int q = 0; q < G; ++q, frame += kFrame) {
+        uint4 x;
+        if constexpr (PACK8) {
+          x = make_uint4(0u, 0u, 0u, 0u);
+          if (8 * q + 8 <= P.K) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+          } else {
 #pragma unroll 2
-        for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+            for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+          }
+        } else {
+          x = call(static_cast<uint32_t>(q));
+        }
+        x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
+        if (f32)
+          add_group<2>(acc, x, frame);
+        else
+          add_group<4>(acc, x, frame);
+      }
+    }
+    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+    if (P.has_pre) {
+      const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
+      xp = item_signs(philox_finish(philox_start(blk, g), P.keys), f32, (k.i & 1) != 0, shift, a);
+    }
+    if (!k.act) return;
+    if (k.full && do_sum) {
+      if (f32) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float th = __uint_as_float(v[i]);
+          if (P.has_pre) th = add_signed(th, xp, i, P.pre);
+          v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
+        }
+      } else if (dt == kBF16) {
+        update_regs16<kBF16>(v, acc, xp, P.has_pre, P.pre);
       } else {
-        x = call(static_cast<uint32_t>(q));
+        update_regs16<kF16>(v, acc, xp, P.has_pre, P.pre);
       }
-      x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
-      if (f32)
-        add_group<2>(acc, x, frame);
-      else
-        add_group<4>(acc, x, frame);
+      st256(p, v);
+      return;
     }
-  }
-  uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-  if (P.has_pre) {
-    const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
-    xp = item_signs(philox_finish(philox_start(blk, g), P.keys), f32, (k.i & 1) != 0, shift, a);
-  }
-  if (!k.act) return;
-  if (k.full && do_sum) {
-    if (f32) {
+    // an item across a tensor's end, or the leading perturbation alone
+    int lo, hi;
+    item_range(e, k.i, &lo, &hi);
+    float th[16];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float th = __uint_as_float(v[i]);
-        if (P.has_pre) th = add_signed(th, xp, i, P.pre);
-        v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
-      }
-    } else if (dt == kBF16) {
-      update_regs16<kBF16>(v, acc, xp, P.has_pre, P.pre);
-    } else {
-      update_regs16<kF16>(v, acc, xp, P.has_pre, P.pre);
+    for (int i = 0; i < 16; ++i) th[i] = i >= lo && i < hi ? load_elem(p, dt, i) : 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < lo || i >= hi) continue;
+      if (P.has_pre) th[i] = round_to_storage(dt, add_signed(th[i], xp, i, P.pre));
+      if (do_sum) th[i] = __fadd_rn(th[i], acc[i]);
+      store_elem(p, dt, i, th[i]);
     }
-    st256(p, v);
-    return;
-  }
-  // an item across a tensor's end, or the leading perturbation alone
-  int lo, hi;
-  item_range(e, k.i, &lo, &hi);
-  float th[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) th[i] = i >= lo && i < hi ? load_elem(p, dt, i) : 0.0f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    if (i < lo || i >= hi) continue;
-    if (P.has_pre) th[i] = round_to_storage(dt, add_signed(th[i], xp, i, P.pre));
-    if (do_sum) th[i] = __fadd_rn(th[i], acc[i]);
-    store_elem(p, dt, i, th[i]);
+  };
+  if constexpr (PACK8) {
+    for (uint32_t left = P.rounds; here; seek()) {
+      item();
+      if (--left == 0u) break;
+      b += kItemThreads;
+    }
+  } else {
+    item();
   }
 }
 
 template <int N>
 cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream) {
-  const int grid = static_cast<int>((p.total + (kItemThreads - 1u)) / kItemThreads);
+  const uint32_t per = kItemThreads * (p.packing == kPacking8 ? p.rounds : 1u);
+  const int grid = static_cast<int>((static_cast<uint64_t>(p.total) + (per - 1u)) / per);
   const size_t smem = update_items_smem_bytes(p.groups, p.packing);
   const auto go = [&](auto kernel) -> cudaError_t {
     if (smem > 48 * 1024) {

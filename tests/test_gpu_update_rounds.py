@@ -1,0 +1,47 @@
+"""The fused update under packing 8 on a list long enough that a thread of the
+item kernel takes several items, with a full and a partial probe group: the
+long tensor ends inside an item, the short ones hold fp32 and views. Against
+the oracle within the derived bound."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2609_38095_gb300 import build as zo_build
+from paper_2609_38095_gb300 import workloads as W
+from paper_2609_38095_gb300 import zo
+
+from gpu_helpers import TORCH_TO_DT, assert_update_close, storage_bits, to_torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    zo_build.build()
+    oracle.lib()
+
+
+@pytest.mark.parametrize("rounds,pre", [(2, True), (3, False)])
+def test_several_items_per_thread(rounds, pre):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    K, seed, lr = 9, W.step_seed(rounds), 1e-3
+    numels = [16 * 8 * 128 * 10 * sms * rounds + 7, 1, 1000, 4099]
+    dtypes = [torch.bfloat16, torch.float16, torch.float32, torch.bfloat16]
+    rng = np.random.default_rng(rounds)
+    dts = [TORCH_TO_DT[d] for d in dtypes]
+    host = [W.random_storage(rng, n, dt) for n, dt in zip(numels, dts)]
+    dev = [to_torch(h.copy(), d) for h, d in zip(host, dtypes)]
+    view = torch.zeros(numels[-1] + 16, dtype=dtypes[-1], device="cuda")[3:3 + numels[-1]]
+    view.copy_(dev[-1])
+    dev[-1] = view
+    c_np = rng.normal(0, 25, K)
+    zo.update(zo.ParamList(dev, packing=8), seed, torch.tensor(c_np, device="cuda"), lr, pre=(K - 1, 1e-3) if pre else None)
+    with oracle.packing(8):
+        if pre:
+            oracle.perturb(host, dts, seed, K - 1, 1e-3)
+        oracle.update(host, dts, seed, c_np, lr)
+    for i, (x, h, dt) in enumerate(zip(dev, host, dts)):
+        assert_update_close(storage_bits(x), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
