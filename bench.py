@@ -83,12 +83,12 @@ def parse_args():
     ap.add_argument("--no-pair", action="store_true",
                     help="skip the extra measurement of the out-of-place pair schedule")
     ap.add_argument("--no-other-sets", action="store_true",
-                    help="skip the short timings of the other parameter sets (and of the aligned-chunk kernels)")
+                    help="skip the short timings of the other parameter sets (and of views off the 32-byte grid)")
     ap.add_argument("--no-sequential", action="store_true",
                     help="skip timing Algorithm 1's K sequential update passes against the fused update")
     ap.add_argument("--view-offset", type=int, default=0,
                     help="every parameter a view this many elements into its own allocation (e.g. 1: off the "
-                         "32-byte grid, the perturbation passes run the aligned-chunk kernel)")
+                         "32-byte grid)")
     args = ap.parse_args()
     if args.steps is None:
         args.steps = W.TINY_STEPS if args.config == "tiny" else 2
@@ -717,9 +717,6 @@ def time_kernels_on_set(key, dev, hbm_peak, alu_peak, view_offset=0):
             torch.cuda.synchronize(dev)
             return e0.elapsed_time(e1) / n
 
-        for i in range(12):                       # the two-op tuner's trials, then its choice
-            zo.perturb2(plist, seed, i, eps, i + 1, eps)
-        torch.cuda.synchronize(dev)
         zo.perturb2(plist, seed, 0, eps, 1, eps)
         zo.update(plist, seed, c, eps, pre=(K - 1, eps))
         p1 = ms_of(lambda i: zo.perturb(plist, seed, i, eps if i % 2 else -eps), 6)
@@ -976,7 +973,7 @@ def run_zo(args):
     dom_bytes = pair_bytes if pair else perturb_bytes
     # the update's DRAM bytes (one read and one write of theta, whatever K): the
     # 8-probe-table kernel's committed capture when it is the one this K runs
-    if args.packing == 1 and K > 16 and not shifted:
+    if args.packing == 1 and K > 32 and not shifted:
         upd_traffic, upd_traffic_how = committed_traffic("update_lut8_kernel", traffic_key)
     else:
         upd_traffic, upd_traffic_how = None, "no capture committed for the update kernel this K runs"

@@ -28,8 +28,8 @@ cudaError_t launch_perturb_items_any_high(const ItemsParams<kItemsMany>& p, cuda
 // counter's high word.
 template <int N>
 cudaError_t launch_pair_items(const PairItemsParams<N>& p, bool one_high, cudaStream_t stream);
-// Fused update: packing 1, at most two probe groups (K <= 16) and virtual
-// blocks that share the counter's high word; ...
+// Fused update: what lut8_small_takes (packing 1, at most kSmallGroups probe
+// groups) with virtual blocks that share the counter's high word; ...
 bool lut8_small_takes(const UpdateParams& u, bool mostly_f32);
 cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream);
 // ... and every other one. any: the launch holds fp32 tensors or tensors off

@@ -980,8 +980,8 @@ __global__ void __launch_bounds__(small_threads(G), 1)
           const float d = __uint_as_float(P.pre.nscale_bits ^ (((n >> P.pre.bit) & 1u) << 31));
           asm volatile("st.shared.v4.f32 [%0], {%1, %2, %1, %2};" ::"r"(row), "f"(v), "f"(d) : "memory");
         } else {
-          const uint32_t g = 2u * r + (piece >> 3);
-          if (g < static_cast<uint32_t>(PRE == kPreTable ? G - 1 : G)) sts_f32x4(row, t8[256u * g + n]);
+          const int g = static_cast<int>(2u * r + (piece >> 3));
+          if (g < (PRE == kPreTable ? G - 1 : G)) sts_f32x4(row, t8[256 * g + static_cast<int>(n)]);
         }
       }
     }
