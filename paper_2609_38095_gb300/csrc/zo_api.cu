@@ -75,18 +75,20 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 //               K = 20: 5 M 14.7 / 15.1, 8 M 19.2 / 18.8;  K = 32: 16.8 / 17.1, 23.0 / 21.2
 //               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
 // (3 M weights are 1233 items per SM). Under packing 8 generating the bits is
-// most of the work and full occupancy does it best, whatever the size, but for
-// long lists of many groups; fp32 items hold half a block each and make its
-// words twice:
+// most of the work and many small CTAs do it best, whatever the size, but for
+// long lists of many groups:
 //   16 bits     K = 3: 5 M 13.8 / 20.3, 205 M 279 / 317;  K = 24: 29.2 / 38.0, 872 / 907
 //               K = 64: 60 M 628 / 633, 205 M 2116 / 2091;  K = 128: 1212 / 1207, 4109 / 4021
-//   fp32        K = 3: 3 M 12.9 / 15.0, 6 M 21.1 / 19.8;  K = 24: 1 M 14.7 / 15.0, 3 M 31.2 / 27.0
-//               K = 64: 1 M 27.2 / 23.2
-// (1 M fp32 weights are 822 items per SM). Between 1 and 0.05 M weights of
-// packing 1 all of these take about 9 us here, 11 to 35 with the tables.
-int64_t update_items_per_sm(int packing, int groups, bool mostly_f32) {
+//   fp32        K = 8: 3 M 12.9 / 17.0, 100 M 193 / 206;  K = 24: 21.7 / 27.0, 432 / 458
+//               K = 64: 3 M 43.8 / 48.5, 100 M 1034 / 1039
+//   fp32 views  K = 3: 3 M 14.7 / 17.0, 6 M 23.1 / 21.3;  K = 24: 1 M 14.8 / 17.0, 3 M 31.4 / 28.2
+//               K = 64: 1 M 27.3 / 24.8
+// (1 M fp32 weights are 822 items per SM; those off the 32-byte grid make a
+// block's words twice). Between 1 and 0.05 M weights of packing 1 all of these
+// take about 9 us here, 11 to 35 with the tables.
+int64_t update_items_per_sm(int packing, int groups, bool f32_views) {
   if (packing == zo::kPacking8) {
-    if (mostly_f32) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
+    if (f32_views) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
     return groups < 8 ? INT64_C(1) << 20 : 24000;
   }
   return groups == 3 || groups == 4 ? 2400 : 1600;
@@ -416,13 +418,15 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  int64_t f32 = 0, all = 0;
+  int64_t f32 = 0, f32_off = 0, all = 0;  // elements: fp32, fp32 off the 32-byte grid, all
   for (int32_t i = 0; i < n_tensors; ++i) {
     all += params[i].numel;
-    f32 += params[i].dtype == ZO_F32 ? params[i].numel : 0;
+    if (params[i].dtype != ZO_F32) continue;
+    f32 += params[i].numel;
+    if (reinterpret_cast<uintptr_t>(params[i].ptr) % 32 != 0) f32_off += params[i].numel;
   }
-  const bool mostly_f32 = 2 * f32 > all;
-  const int64_t most_items = update_items_per_sm(up.packing, up.groups, mostly_f32) * d->sms;
+  const bool mostly_f32 = 2 * f32 > all, f32_blocks = 2 * (f32 - f32_off) > all;
+  const int64_t most_items = update_items_per_sm(up.packing, up.groups, 2 * f32_off > all) * d->sms;
   const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
     zo::ItemsCursor cur;
     const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
@@ -432,7 +436,9 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     // packing 8: several items per thread where ten waves of CTAs remain, which spread a CTA's tables over more
     // work (205 M bf16 weights, K = 8, one / eight items: 396 / 376 us; 20 M: 44 / 48)
     const int64_t waves = ip.total / (INT64_C(8) * 128 * 10 * d->sms);
+    ip.f32_blocks = f32_blocks;
     ip.rounds = static_cast<uint32_t>(waves < 1 ? 1 : waves > 8 ? 8 : waves);
+    if (f32_blocks && ip.rounds % 2 == 1) ++ip.rounds;  // fp32: whole blocks, two items each
     ip.bhi = 0;
     ip.keys = up.keys;
     ip.coef = c;

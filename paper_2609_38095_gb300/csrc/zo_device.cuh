@@ -581,7 +581,8 @@ struct UpdateItemsParams {
   int32_t n;
   int32_t hint_shift;
   uint32_t total;
-  uint32_t rounds;         // packing 8: items a thread takes, one CTA apart
+  uint32_t rounds;         // packing 8: items a thread takes
+  int32_t f32_blocks;      // packing 8: mostly fp32 on the 32-byte grid
   uint32_t bhi;            // the virtual blocks' counter high word
   RoundKeys keys;
   const double* coef;

@@ -25,7 +25,11 @@
 // 1130 -> 374 / 872 / 1120 us (a persistent grid with plain Philox calls took
 // 378 / 880 / 1130), 20 M 46.7 / 105 / 128 -> 44.4 / 93.8 / 117.5. Not adopted:
 // the calls in twos or fours (K = 8 445 / 432 us), registers capped at 40 for
-// more warps (spills; 409), CTAs of 256 threads (406).
+// more warps (spills; 409), CTAs of 256 threads (406). Aligned fp32 is taken by
+// whole blocks, two items of a lane at a time (an instantiation of its own: 90
+// registers), so that a block's words are made once: 100 M fp32 weights, K = 3 /
+// 8 / 24: 162 / 206 / 458 us in the chunk kernel, 230 / 325 / 782 by single
+// items, 150 / 193 / 432 so.
 #include "zo_device.cuh"
 #include "zo_launch.h"
 
@@ -67,10 +71,14 @@ size_t update_items_smem_bytes(int groups, int packing) {
 
 }  // namespace
 
-template <bool PACK8, int N>
+// What a launch holds: packing 1, packing 8, or packing 8 and mostly fp32 on the 32-byte grid.
+constexpr int kPlain = 0, kBytes = 1, kBytesF32 = 2;
+
+template <int KIND, int N>
 __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
+  constexpr bool PACK8 = KIND != kPlain, WIDE = KIND == kBytesF32;
   const int G = P.groups;
   constexpr int kCalls = PACK8 ? 8 : 1;  // Philox calls per group
   uint4* r01_s = reinterpret_cast<uint4*>(smem);            // kCalls G group parts
@@ -87,7 +95,8 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
   }
   // this thread's item, its load on the way while the tables are made
   const uint32_t lane = threadIdx.x & 31u;
-  uint32_t b = blockIdx.x * (kItemThreads * (PACK8 ? P.rounds : 1u)) + threadIdx.x;
+  uint32_t left = PACK8 ? P.rounds : 1u;  // a warp's items are consecutive
+  uint32_t b = (blockIdx.x * (kItemThreads / 32u) + (threadIdx.x >> 5)) * 32u * left + lane;
   bool here = false;  // the same in all lanes
   ItemsEntry e;
   uint8_t dt = 0;
@@ -95,7 +104,9 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
   uint32_t a = 0;
   ItemPlace k;
   char* p = nullptr;
-  uint32_t v[8];
+  uint32_t v[8], v2[8];
+  bool pairs = WIDE;
+  bool wide = false;  // WIDE: lane l takes items 2 l and 2 l + 1 of the next 64, an fp32 block (the same in all lanes)
   const auto seek = [&] {
     const uint32_t wb = b - lane;
     here = wb < P.total;
@@ -106,16 +117,22 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
     f32 = dt == kF32;
     shift = (e.meta & kShift) != 0;
     a = e.meta >> 16;
-    k = item_place(e, b);
+    wide = pairs && here && f32 && !shift && left >= 2u && wb - e.begin + 64u <= e.whole;
+    k = item_place(e, wide ? b + lane : b);
     k.full = k.full && here;
     k.act = k.act && here;
     p = reinterpret_cast<char*>(e.base) + static_cast<int64_t>(k.i) * 32;
     if (k.full) ld256(p, v);
+    if (WIDE && wide) ld256(p + 32, v2);
   };
   seek();
   __syncthreads();
   const bool do_sum = skip_s == 0;  // a failed preconditioner still gets the leading perturbation
   if (!do_sum && !P.has_pre) return;
+  if (WIDE && !do_sum) {  // element by element, below
+    pairs = false;
+    seek();
+  }
   for (int i = threadIdx.x; i < 32 * G; i += kItemThreads) {
     const int h = i >> 4;  // quad of probes
     lut[(h >> 1) * (kFrame / 4) + (h & 1) * 16 + (i & 15)] = quad_partial(a_s + 4 * h, static_cast<uint32_t>(i) & 15u);
@@ -148,8 +165,8 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
         } else {
           x = call(static_cast<uint32_t>(q));
         }
-        x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
-        if (f32)
+        if (!(WIDE && wide)) x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
+        if (f32 && !(WIDE && wide))
           add_group<2>(acc, x, frame);
         else
           add_group<4>(acc, x, frame);
@@ -158,7 +175,8 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
     uint4 xp = make_uint4(0u, 0u, 0u, 0u);
     if (P.has_pre) {
       const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
-      xp = item_signs(philox_finish(philox_start(blk, g), P.keys), f32, (k.i & 1) != 0, shift, a);
+      xp = philox_finish(philox_start(blk, g), P.keys);
+      if (!(WIDE && wide)) xp = item_signs(xp, f32, (k.i & 1) != 0, shift, a);
     }
     if (!k.act) return;
     if (k.full && do_sum) {
@@ -168,6 +186,15 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
           float th = __uint_as_float(v[i]);
           if (P.has_pre) th = add_signed(th, xp, i, P.pre);
           v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
+        }
+        if (WIDE && wide) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float th = __uint_as_float(v2[i]);
+            if (P.has_pre) th = add_signed(th, xp, 8 + i, P.pre);
+            v2[i] = __float_as_uint(__fadd_rn(th, acc[8 + i]));
+          }
+          st256(p + 32, v2);
         }
       } else if (dt == kBF16) {
         update_regs16<kBF16>(v, acc, xp, P.has_pre, P.pre);
@@ -192,10 +219,13 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
     }
   };
   if constexpr (PACK8) {
-    for (uint32_t left = P.rounds; here; seek()) {
+    while (here) {
       item();
-      if (--left == 0u) break;
-      b += kItemThreads;
+      const uint32_t took = WIDE && wide ? 2u : 1u;
+      left -= took;
+      if (left == 0u) break;
+      b += 32u * took;
+      seek();
     }
   } else {
     item();
@@ -216,7 +246,8 @@ cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stre
     kernel<<<grid, kItemThreads, smem, stream>>>(p);
     return cudaGetLastError();
   };
-  return p.packing == kPacking8 ? go(update_items_kernel<true, N>) : go(update_items_kernel<false, N>);
+  if (p.packing != kPacking8) return go(update_items_kernel<kPlain, N>);
+  return p.f32_blocks ? go(update_items_kernel<kBytesF32, N>) : go(update_items_kernel<kBytes, N>);
 }
 template cudaError_t launch_update_items(const UpdateItemsParams<kItemsFew>& p, cudaStream_t stream);
 template cudaError_t launch_update_items(const UpdateItemsParams<kItemsSome>& p, cudaStream_t stream);

@@ -1,7 +1,9 @@
 """The fused update under packing 8 on a list long enough that a thread of the
 item kernel takes several items, with a full and a partial probe group: the
-long tensor ends inside an item, the short ones hold fp32 and views. Against
-the oracle within the derived bound."""
+long tensor ends inside an item, the short ones hold fp32 and views. Lists of
+mostly fp32 take whole blocks of 64 bytes: sizes around a warp's 64 items, a
+partial last block, views in between, and a failed preconditioner's leading
+perturbation alone. Against the oracle within the derived bound."""
 import numpy as np
 import pytest
 import torch
@@ -45,3 +47,33 @@ def test_several_items_per_thread(rounds, pre):
         oracle.update(host, dts, seed, c_np, lr)
     for i, (x, h, dt) in enumerate(zip(dev, host, dts)):
         assert_update_close(storage_bits(x), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
+
+
+@pytest.mark.parametrize("K,pre,status", [(9, True, 0), (17, False, 0), (8, True, zo.ZO_ERR_NONFINITE)])
+@pytest.mark.parametrize("big", [20_011, 3_000_017])
+def test_blocks_of_fp32(K, pre, status, big):
+    numels = [big, 512, 511, 513, 256, 8, 1024, 2051, 40, 1040]
+    offsets = [0, 0, 0, 0, 0, 0, 0, 3, 0, 0]
+    dtypes = [torch.float32] * 8 + [torch.bfloat16, torch.float16]
+    rng = np.random.default_rng(K)
+    seed, lr = W.step_seed(K), 1e-3
+    dts = [TORCH_TO_DT[d] for d in dtypes]
+    host = [W.random_storage(rng, n, dt) for n, dt in zip(numels, dts)]
+    bases = [torch.full((n + 32,), 3.0, dtype=d, device="cuda") for n, d in zip(numels, dtypes)]
+    dev = [b[o:o + n] for b, o, n in zip(bases, offsets, numels)]
+    for x, h, d in zip(dev, host, dtypes):
+        x.copy_(to_torch(h, d))
+    c_np = rng.normal(0, 25, K)
+    zo.update(zo.ParamList(dev, packing=8), seed, torch.tensor(c_np, device="cuda"), lr,
+              status=torch.tensor([status], dtype=torch.int32, device="cuda"), pre=(K - 1, 1e-3) if pre else None)
+    with oracle.packing(8):
+        if pre:
+            oracle.perturb(host, dts, seed, K - 1, 1e-3)
+        if status == 0:
+            oracle.update(host, dts, seed, c_np, lr)
+    for i, (x, h, dt) in enumerate(zip(dev, host, dts)):
+        if status == 0:
+            assert_update_close(storage_bits(x), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
+        else:
+            assert np.array_equal(storage_bits(x), storage_bits(h)), f"tensor {i}"
+        assert torch.all(bases[i][:offsets[i]] == 3.0) and torch.all(bases[i][offsets[i] + numels[i]:] == 3.0)
