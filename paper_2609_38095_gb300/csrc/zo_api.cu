@@ -418,15 +418,14 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  int64_t f32 = 0, f32_off = 0, all = 0;  // elements: fp32, fp32 off the 32-byte grid, all
+  int64_t f32 = 0, f32_off = 0, all = 0;  // elements: fp32 on and off the 32-byte grid, all
   for (int32_t i = 0; i < n_tensors; ++i) {
     all += params[i].numel;
     if (params[i].dtype != ZO_F32) continue;
-    f32 += params[i].numel;
-    if (reinterpret_cast<uintptr_t>(params[i].ptr) % 32 != 0) f32_off += params[i].numel;
+    (reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0 ? f32 : f32_off) += params[i].numel;
   }
-  const bool mostly_f32 = 2 * f32 > all, f32_blocks = 2 * (f32 - f32_off) > all;
-  const int64_t most_items = update_items_per_sm(up.packing, up.groups, 2 * f32_off > all) * d->sms;
+  const bool f32_blocks = 2 * f32 > all, f32_views = 2 * f32_off > all;
+  const int64_t most_items = update_items_per_sm(up.packing, up.groups, f32_views) * d->sms;
   const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
     zo::ItemsCursor cur;
     const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
@@ -459,7 +458,8 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
     if (done) return ZO_OK;
   }
-  const bool few = zo::lut8_small_takes(up, mostly_f32);
+  const bool few = zo::lut8_small_takes(up, f32_views);
+  tl_update.f32_blocks = f32_blocks;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t blk = 0;

@@ -200,6 +200,7 @@ struct SmallUpdateParams {
   UpdateParams u;
   GroupRound01 g[kSmallGroups];
   GroupRound01 gp;
+  int32_t f32_blocks;  // mostly fp32 on the 32-byte grid
 };
 
 // ---------------------------------------------------------------------------

@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(kLut8Threads, 1) update_lut8_kernel(const __gr
 // the leading perturbation: K = 8 0.845 -> 0.787 ms, K = 16 0.941 -> 0.903 ms
 // (fp16 0.962 -> 0.880); without it 0.822 -> 0.780 and 0.880 -> 0.810 ms. fp32
 // and tensors off the 32-byte grid ran element by element or in a kernel of
-// their own before: 205 M fp32 weights, K = 16: 0.332 -> 0.260 ms; 400 M bf16
+// their own before: 205 M fp32 weights, K = 16: 0.332 -> 0.249 ms; 400 M bf16
 // weights in one flat buffer, K = 16: 0.749 -> 0.381 ms. Not adopted: a
 // prefetch of the item after the next into L2 (K = 16 -2 %, K = 8 +10 %).
 // ---------------------------------------------------------------------------
@@ -936,9 +936,36 @@ __device__ __forceinline__ uint4 small_window(const SmallCursor& c, const SmallI
   return item_signs(x, (c.fl & kDtypeMask) == kF32, k.upper, (c.fl & kShift) != 0, c.a);
 }
 
+// The groups' words of an aligned fp32 item. Lanes 2 j and 2 j + 1 hold the
+// halves of one block, so of every two groups each lane makes one's words and
+// hands the other lane the half that it needs. 205 M fp32 weights, K = 16 / 24 /
+// 32 (the last in the chunk kernel before): 265 / 337 / 379 -> 249 / 291 / 336 us;
+// 40 M, K = 24: 72 -> 64 us.
+template <int G>
+__device__ __forceinline__ void small_pair_words(uint4 (&x)[G], const BlockCounter<true>& kb,
+                                                 const GroupRound01 (&gs)[kSmallGroups], bool upper,
+                                                 const RoundKeys& keys) {
+#pragma unroll
+  for (int g = 0; g + 1 < G; g += 2) {
+    const GroupRound01 mine = {upper ? gs[g + 1].x0 : gs[g].x0, upper ? gs[g + 1].x2 : gs[g].x2,
+                               upper ? gs[g + 1].lpa1 : gs[g].lpa1};
+    const uint4 y = philox_finish(kb.start(mine, 0u, keys), keys);
+    const uint32_t a = __shfl_xor_sync(0xFFFFFFFFu, upper ? y.x : y.z, 1);
+    const uint32_t b = __shfl_xor_sync(0xFFFFFFFFu, upper ? y.y : y.w, 1);
+    x[g] = make_uint4(upper ? a : y.x, upper ? b : y.y, 0u, 0u);
+    x[g + 1] = make_uint4(upper ? y.z : a, upper ? y.w : b, 0u, 0u);
+  }
+  if (G & 1) {
+    const uint4 y = philox_finish(kb.start(gs[G - 1], 0u, keys), keys);
+    x[G - 1] = upper ? make_uint4(y.z, y.w, 0u, 0u) : make_uint4(y.x, y.y, 0u, 0u);
+  }
+}
+
 // ANY: the launch may hold fp32 tensors (numbered in half blocks) and tensors
-// off the 32-byte grid (32 launch items per 31 chunks).
-template <int PRE, int G, bool ANY>
+// off the 32-byte grid (32 launch items per 31 chunks). BLOCKS: mostly aligned
+// fp32, whose words a pair of lanes makes once (small_pair_words); in the
+// general instantiation that code costs views 4 % (586 -> 607 us, K = 32).
+template <int PRE, int G, bool ANY, bool BLOCKS>
 __global__ void __launch_bounds__(small_threads(G), 1)
     update_lut8_small_kernel(const __grid_constant__ SmallUpdateParams S) {
   constexpr int kThreads = small_threads(G);
@@ -1040,16 +1067,21 @@ __global__ void __launch_bounds__(small_threads(G), 1)
     }
     const BlockCounter<true> kb(k.blk, 0, P.keys);
     uint4 x[G];
-    x[0] = philox_finish(kb.start(S.g[0], 0u, P.keys), P.keys);
-#pragma unroll
-    for (int g = 1; g < G; ++g) x[g] = philox_finish(kb.start(S.g[g], static_cast<uint32_t>(g), P.keys), P.keys);
     uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-    if (PRE == kPreOwn) xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
-    if (ANY) {
-      x[0] = small_window(c, k, x[0]);
+    if (BLOCKS && (c.fl & kDtypeMask) == kF32 && !(c.fl & kShift)) {
+      small_pair_words<G>(x, kb, S.g, k.upper, P.keys);
+      if (PRE == kPreOwn) xp = small_window(c, k, philox_finish(kb.start(S.gp, 0u, P.keys), P.keys));
+    } else {
+      x[0] = philox_finish(kb.start(S.g[0], 0u, P.keys), P.keys);
 #pragma unroll
-      for (int g = 1; g < G; ++g) x[g] = small_window(c, k, x[g]);
-      if (PRE == kPreOwn) xp = small_window(c, k, xp);
+      for (int g = 1; g < G; ++g) x[g] = philox_finish(kb.start(S.g[g], static_cast<uint32_t>(g), P.keys), P.keys);
+      if (PRE == kPreOwn) xp = philox_finish(kb.start(S.gp, 0u, P.keys), P.keys);
+      if (ANY) {
+        x[0] = small_window(c, k, x[0]);
+#pragma unroll
+        for (int g = 1; g < G; ++g) x[g] = small_window(c, k, x[g]);
+        if (PRE == kPreOwn) xp = small_window(c, k, xp);
+      }
     }
     if (PRE == kPreLast) xp = x[G - 1];
     if (k.full) {
@@ -1087,16 +1119,19 @@ cudaError_t lut8_limit() {
                               static_cast<int>(lut8_smem_bytes(PACK8)));
 }
 
-template <int PRE, int G, bool ANY>
+template <int PRE, int G, bool ANY, bool BLOCKS = false>
 cudaError_t small_limit() {
-  return cudaFuncSetAttribute(update_lut8_small_kernel<PRE, G, ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(update_lut8_small_kernel<PRE, G, ANY, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(small_smem_bytes(G, PRE == kPreTable)));
 }
 
 template <int PRE, int G>
 cudaError_t small_limits() {
-  const cudaError_t e = small_limit<PRE, G, false>();
-  return e == cudaSuccess ? small_limit<PRE, G, true>() : e;
+  cudaError_t e = small_limit<PRE, G, false>();
+  if (e == cudaSuccess) e = small_limit<PRE, G, true>();
+  if constexpr (G > 1)
+    if (e == cudaSuccess) e = small_limit<PRE, G, true, true>();
+  return e;
 }
 
 cudaError_t lut8_prepare() {
@@ -1135,23 +1170,29 @@ void launch_small_cfg(const SmallUpdateParams& p, bool any, int sms, cudaStream_
   constexpr int threads = small_threads(G);
   const int64_t want = (static_cast<int64_t>(p.u.tab.blk_total) + threads - 1) / threads;
   const int grid = static_cast<int>(want < sms ? want : sms);
+  if constexpr (G > 1) {
+    if (any && p.f32_blocks) {
+      update_lut8_small_kernel<PRE, G, true, true><<<grid, threads, sm, stream>>>(p);
+      return;
+    }
+  }
   if (any)
-    update_lut8_small_kernel<PRE, G, true><<<grid, threads, sm, stream>>>(p);
+    update_lut8_small_kernel<PRE, G, true, false><<<grid, threads, sm, stream>>>(p);
   else
-    update_lut8_small_kernel<PRE, G, false><<<grid, threads, sm, stream>>>(p);
+    update_lut8_small_kernel<PRE, G, false, false><<<grid, threads, sm, stream>>>(p);
 }
 
 // Which updates the small kernel takes. Three and four groups only with the
 // leading perturbation's probe in the last group, or none: words of its own
-// would be a fifth Philox call's registers. It makes a block's words once per
-// item, so twice for fp32, where the chunk kernel makes them once: with four
-// groups that costs fp32 lists more than the chunks' tables and barriers do
-// (205 M fp32 weights, K = 32: 0.412 ms here, 0.379 there; K = 24: 0.338 and
-// 0.347). Before, K from 17 on walked the chunks: OPT-1.3B-shaped bf16 set with
-// the leading perturbation, K = 24 / 32: 1.612 / 1.857 -> 1.122 / 1.386 ms;
-// 400 M bf16 weights in one flat buffer 0.677 / 0.747 -> 0.451 / 0.584 ms.
-bool lut8_small_takes(const UpdateParams& u, bool mostly_f32) {
-  if (u.packing != kPacking1 || u.groups > kSmallGroups || (u.groups == 4 && mostly_f32)) return false;
+// would be a fifth Philox call's registers. Views of fp32 make a block's words
+// twice here, once per half, where the chunk kernel makes them once: with four
+// groups that costs them more than the chunks' tables and barriers do (205 M
+// fp32 weights in one flat buffer, K = 32: 0.450 ms here, 0.425 there; K = 24:
+// 0.363 and 0.386). Before, K from 17 on walked the chunks: OPT-1.3B-shaped bf16
+// set with the leading perturbation, K = 24 / 32: 1.612 / 1.857 -> 1.122 / 1.386
+// ms; 400 M bf16 weights in one flat buffer 0.677 / 0.747 -> 0.451 / 0.584 ms.
+bool lut8_small_takes(const UpdateParams& u, bool f32_views) {
+  if (u.packing != kPacking1 || u.groups > kSmallGroups || (u.groups == 4 && f32_views)) return false;
   return u.groups <= 2 || !u.has_pre || u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups);
 }
 
