@@ -1,4 +1,4 @@
-"""The fused update with three and four probe groups, lists long enough for the
+"""The fused update with three and four probe groups (two of fp32), lists long enough for the
 kernel that keeps every group's table in shared memory: each place its leading
 perturbation's signs come from (none, the last group, another group), each
 storage type, aligned and in views, tensors that end inside an item or hold
@@ -65,6 +65,11 @@ def long_list(dtype):
 @pytest.mark.parametrize("dtype", [BF16, F32], ids=["bf16", "f32"])
 def test_three_and_four_groups(K, pre_probe, dtype):
     check([long_list(dtype), 1, 15, 513, 77], [dtype, F16, F32, BF16, F16], [0, 0, 3, 5, 0], K, pre_probe, seed=K)
+
+
+@pytest.mark.parametrize("K,pre_probe", [(9, None), (16, 15), (12, 3)])
+def test_two_groups_of_fp32_blocks(K, pre_probe):
+    check([long_list(F32), 8, 7, 1023, 65], [F32, F32, F32, F32, BF16], [0, 0, 0, 3, 1], K, pre_probe, seed=K)
 
 
 @pytest.mark.parametrize("K", [20, 32])
