@@ -77,7 +77,9 @@ bool fill_items(Params& ip, const zo_tensor* params, int32_t n, ItemsCursor& cur
     while (static_cast<uint64_t>(ip.e[t].end) <= static_cast<uint64_t>(k) << ip.hint_shift) ++t;
     ip.hint[k] = static_cast<uint16_t>(t);
   }
-  return ip.e[0].vb >> 32 == last >> 32;
+  // the first block: of a later piece off the grid, the one below, whose tail is the piece's first elements
+  const bool below = (ip.e[0].meta & kItemsCont) && (ip.e[0].meta & kShift);
+  return (ip.e[0].vb - (below ? 1 : 0)) >> 32 == last >> 32;
 }
 
 }  // namespace zo

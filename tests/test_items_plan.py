@@ -90,8 +90,42 @@ template <int N> int check(int round, std::mt19937& g) {
       if (hits[t][e] != 1) return fail("not changed exactly once", round, t, static_cast<long long>(e));
   return 0;
 }
+// Lists past 2^32 blocks: a launch that fill_items calls one of a single counter high word uses no block of another,
+// in the first and the last warp of each entry.
+static int check_high_words(const std::vector<long long>& blocks, const std::vector<int>& offsets) {
+  static ItemsParams<kItemsMany> ip;
+  const int n = static_cast<int>(blocks.size());
+  std::vector<zo_tensor> list(n);
+  for (int t = 0; t < n; ++t)
+    list[t] = {reinterpret_cast<void*>((t + 1) * (1ll << 44) + 2 * offsets[t]), 16 * blocks[t], ZO_BF16, 1};
+  ItemsCursor cur;
+  for (int l = 0; cur.t < n; ++l) {
+    if (!fill_items(ip, list.data(), n, cur, [](auto&, int32_t, int64_t) {})) continue;
+    const int64_t high = ip.e[0].vb >> 32;
+    for (int t = 0; t < ip.n; ++t) {
+      const ItemsEntry& e = ip.e[t];
+      for (uint32_t wb : {e.begin, e.begin + (e.end - 1 - e.begin) / 32 * 32})
+        for (uint32_t b = wb; b < wb + 32 && b < e.end; ++b) {
+          const ItemPlace k = item_place(e, b);
+          if (!k.act) continue;
+          int lo, hi;
+          item_range(e, k.i, &lo, &hi);
+          const int a = static_cast<int>(e.meta >> 16);
+          if (hi > a && item_block(e, k.i) >> 32 != high) return fail("high word", l, t, b);
+          if (lo < a && item_block(e, item_place(e, b - 1).i) >> 32 != high) return fail("high word below", l, t, b);
+        }
+    }
+  }
+  return 0;
+}
 int main() {
   std::mt19937 g(12345);
+  const long long b30 = 1ll << 30;
+  for (int off : {0, 1, 9}) {
+    if (check_high_words({b30, b30, b30, 2 * b30 - 100}, {0, 0, 0, off})) return 1;
+    if (check_high_words({b30, b30, b30 - 5, 2 * b30 - 100}, {0, 0, 0, off})) return 1;
+    if (check_high_words({2 * b30 - 1, 2 * b30 - 1, 2, 700}, {off, off, off, off})) return 1;
+  }
   for (int r = 0; r < 600; ++r)
     if (check<kItemsFew>(r, g)) return 1;
   for (int r = 0; r < 20; ++r)
