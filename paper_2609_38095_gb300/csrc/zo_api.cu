@@ -56,14 +56,20 @@ void probe_counter(uint32_t k, int packing, uint32_t* ctr2, uint32_t* bit) {
   }
 }
 
+// An operand's sign taken from bit `bit` of a weight's byte.
+void set_bit(zo::PerturbOp& op, uint32_t bit) {
+  op.bit = bit;
+  for (uint32_t m = 0; m < 4; ++m) op.mul[m] = 1u << (31u - 8u * m - bit);
+}
+
 // theta <- rn(theta + scale z_k) as a kernel operand.
 zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
   zo::PerturbOp op;
-  probe_counter(k, packing, &op.ctr2, &op.bit);
-  uint32_t u;
+  uint32_t bit = 0, u;
+  probe_counter(k, packing, &op.ctr2, &bit);
+  set_bit(op, bit);
   std::memcpy(&u, &scale, sizeof(u));
   op.nscale_bits = u ^ 0x80000000u;  // -scale: the probe bit flips it to +scale
-  for (uint32_t m = 0; m < 4; ++m) op.mul[m] = 1u << (31u - 8u * m - op.bit);
   return op;
 }
 
@@ -432,11 +438,12 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
                                          most_items);
     *done = cur.t == n_tensors && one_high && ip.total <= most_items;
     if (!*done || ip.n == 0) return cudaSuccess;
-    // packing 8: several items per thread where ten waves of CTAs remain, which spread a CTA's tables over more
-    // work (205 M bf16 weights, K = 8, one / eight items: 396 / 376 us; 20 M: 44 / 48)
-    const int64_t waves = ip.total / (INT64_C(8) * 128 * 10 * d->sms);
+    // packing 8: several items per thread where about eight waves of CTAs remain, which spread a CTA's tables over
+    // more work (205 M bf16 weights, K = 8, one / eight / ten items: 396 / 317 / 315 us; as fp32 with 32 / 64 at most
+    // 326 / 322; 30 M bf16 weights one / two 58.4 / 55.7)
+    const int64_t unit = INT64_C(8) * 128 * 8 * d->sms, waves = (ip.total + unit / 2) / unit, cap = f32_blocks ? 64 : 16;
     ip.f32_blocks = f32_blocks;
-    ip.rounds = static_cast<uint32_t>(waves < 1 ? 1 : waves > 8 ? 8 : waves);
+    ip.rounds = static_cast<uint32_t>(waves < 1 ? 1 : waves > cap ? cap : waves);
     if (f32_blocks && ip.rounds % 2 == 1) ++ip.rounds;  // fp32: whole blocks, two items each
     ip.bhi = 0;
     ip.keys = up.keys;
@@ -447,6 +454,9 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     ip.packing = up.packing;
     ip.has_pre = up.has_pre;
     ip.pre = up.pre;
+    ip.pre_last = up.has_pre && up.packing == zo::kPacking8 && pre_probe < static_cast<uint32_t>(K) &&
+                  pre_probe / 8u + 1u == static_cast<uint32_t>(up.groups);
+    if (ip.pre_last) set_bit(ip.pre, pre_probe & 7u);
     ip.status = status;
     return zo::launch_update_items(ip, static_cast<cudaStream_t>(stream));
   };

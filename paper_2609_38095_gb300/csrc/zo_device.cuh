@@ -592,6 +592,7 @@ struct UpdateItemsParams {
   int32_t groups;
   int32_t packing;
   int32_t has_pre;
+  int32_t pre_last;        // packing 8: pre's probe is one of the last group's, pre.bit its place in it
   PerturbOp pre;
   const int32_t* status;
 };

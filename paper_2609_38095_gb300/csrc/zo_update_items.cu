@@ -21,15 +21,24 @@
 // Packing 8 has eight Philox calls per group and is bound by them (85 to 90
 // cycles per warp and call on an SM's quarter). A full group's calls are
 // unrolled, several chains in flight per thread, and a thread of a long list
-// takes up to eight items: 205 M bf16 weights, K = 8 / 24 / 32: 417 / 907 /
-// 1130 -> 374 / 872 / 1120 us (a persistent grid with plain Philox calls took
-// 378 / 880 / 1130), 20 M 46.7 / 105 / 128 -> 44.4 / 93.8 / 117.5. Not adopted:
-// the calls in twos or fours (K = 8 445 / 432 us), registers capped at 40 for
-// more warps (spills; 409), CTAs of 256 threads (406). Aligned fp32 is taken by
-// whole blocks, two items of a lane at a time (an instantiation of its own: 90
-// registers), so that a block's words are made once: 100 M fp32 weights, K = 3 /
-// 8 / 24: 162 / 206 / 458 us in the chunk kernel, 230 / 325 / 782 by single
-// items, 150 / 193 / 432 so.
+// takes several items. A leading perturbation whose probe is one of the last
+// group's, as a step's restore has it, takes that group's words instead of a
+// call of its own. 205 M bf16 weights, K = 4 / 8 / 16, without / with it: 249 /
+// 315 / 562 and 284 / 346 / 593 us (a persistent grid with plain Philox calls
+// took 312 / 312 / 564 and 380 / 379 / 632; a call of its own 313 / 377 / 627);
+// 60 M, K = 24: 245 and 255 (247 and 268; 264). Not adopted: the calls in twos
+// or fours (K = 8 445 / 432 us), registers capped at 40 for more warps (spills;
+// 409), CTAs of 256 threads (406), the counters' group parts computed instead of
+// read (60 M, K = 8 99 -> 105).
+//
+// Aligned fp32 is taken by whole blocks, two items of a lane at a time (an
+// instantiation of its own, 88 registers), so that a block's words are made
+// once, its calls' bits folded where the lookups take them (16-bit items would
+// pay for that when they are views: 100 M, K = 24 426 -> 438). 205 M fp32
+// weights, K = 4 / 8 / 16, without / with the leading perturbation: 278 / 322 /
+// 562 and 296 / 348 / 591 us (the persistent grid: 321 / 322 / 562 and 364 / 364 /
+// 610). Not adopted there: 76 registers, six CTAs to an SM (K = 16 580), theta
+// loaded after the calls (100 M, K = 8 164 -> 177).
 #include "zo_device.cuh"
 #include "zo_launch.h"
 
@@ -46,14 +55,26 @@ __device__ __forceinline__ float lds_f32_hi(uint32_t addr) {
   return v;
 }
 
-// Add a group's partial of elements 0 .. 4 WORDS - 1, whose sign bytes are x's.
+// Four times the low and the high nibbles of x's bytes, in its bytes.
+__device__ __forceinline__ uint4 low_offsets(const uint4& x) {
+  return make_uint4((x.x << 2) & 0x3C3C3C3Cu, (x.y << 2) & 0x3C3C3C3Cu, (x.z << 2) & 0x3C3C3C3Cu,
+                    (x.w << 2) & 0x3C3C3C3Cu);
+}
+__device__ __forceinline__ uint4 high_offsets(const uint4& x) {
+  return make_uint4((x.x >> 2) & 0x3C3C3C3Cu, (x.y >> 2) & 0x3C3C3C3Cu, (x.z >> 2) & 0x3C3C3C3Cu,
+                    (x.w >> 2) & 0x3C3C3C3Cu);
+}
+__device__ __forceinline__ uint4 shift_left(const uint4& x, uint32_t n) {
+  return make_uint4(x.x << n, x.y << n, x.z << n, x.w << n);
+}
+
+// Add a group's partial of elements 0 .. 4 WORDS - 1, whose bytes of lo and hi hold four times the signs of the
+// group's probes 0-3 and 4-7.
 template <int WORDS>
-__device__ __forceinline__ void add_group(float (&acc)[16], const uint4& x, uint32_t frame) {
+__device__ __forceinline__ void add_group(float (&acc)[16], const uint4& lo, const uint4& hi, uint32_t frame) {
 #pragma unroll
   for (int m = 0; m < WORDS; ++m) {
-    const uint32_t w = word_of(x, m);
-    const uint32_t lo4 = (w << 2) & 0x3C3C3C3Cu;  // byte j: 4 * low nibble of byte j of w
-    const uint32_t hi4 = (w >> 2) & 0x3C3C3C3Cu;
+    const uint32_t lo4 = word_of(lo, m), hi4 = word_of(hi, m);
 #pragma unroll
     for (int j = 0; j < 4; j += 2) {
       const uint32_t s0 = 0x7650u | static_cast<uint32_t>(j), s1 = s0 + 1u;
@@ -74,8 +95,10 @@ size_t update_items_smem_bytes(int groups, int packing) {
 // What a launch holds: packing 1, packing 8, or packing 8 and mostly fp32 on the 32-byte grid.
 constexpr int kPlain = 0, kBytes = 1, kBytesF32 = 2;
 
-template <int KIND, int N>
-__global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
+// LAST: packing 8, the leading perturbation's probe is one of the last group's, whose words it takes. The second launch
+// bound (5 CTAs of kBytesF32) leaves its calls the registers that they were interleaved with.
+template <int KIND, bool LAST, int N>
+__global__ void __launch_bounds__(kItemThreads, KIND == kBytesF32 ? 5 : 0) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
   constexpr bool PACK8 = KIND != kPlain, WIDE = KIND == kBytesF32;
@@ -145,6 +168,8 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
       const uint4 r = r01_s[c];
       return philox_finish(philox_start(blk, {r.x, r.y, r.z}), P.keys);
     };
+    const auto own = [&](const uint4& x) { return item_signs(x, f32, (k.i & 1) != 0, shift, a); };
+    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
     float acc[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
@@ -152,31 +177,60 @@ __global__ void __launch_bounds__(kItemThreads) update_items_kernel(const __grid
       uint32_t frame = frame0;
 #pragma unroll 1
       for (int q = 0; q < G; ++q, frame += kFrame) {
-        uint4 x;
-        if constexpr (PACK8) {
-          x = make_uint4(0u, 0u, 0u, 0u);
+        uint4 lo, hi;  // the lookups' offsets
+        if constexpr (WIDE) {
+          // the bits folded where the lookups take them
+          lo = hi = make_uint4(0u, 0u, 0u, 0u);
           if (8 * q + 8 <= P.K) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+            for (int i = 0; i < 8; ++i) fold_bits(i < 4 ? lo : hi, call(static_cast<uint32_t>(8 * q + i)), i & 3);
           } else {
-#pragma unroll 2
-            for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+#pragma unroll 1
+            for (int i = 0; i < 4 && 8 * q + i < P.K; ++i) fold_bits(lo, call(static_cast<uint32_t>(8 * q + i)), i);
+#pragma unroll 1
+            for (int i = 4; i < 8 && 8 * q + i < P.K; ++i) fold_bits(hi, call(static_cast<uint32_t>(8 * q + i)), i & 3);
+          }
+          if (wide) {
+            if (LAST) xp = make_uint4(lo.x + (hi.x << 4), lo.y + (hi.y << 4), lo.z + (hi.z << 4), lo.w + (hi.w << 4));
+            lo = shift_left(lo, 2u);
+            hi = shift_left(hi, 2u);
+          } else {
+            const uint4 up = shift_left(hi, 4u);
+            const uint4 x = own(make_uint4(lo.x + up.x, lo.y + up.y, lo.z + up.z, lo.w + up.w));
+            lo = low_offsets(x);
+            hi = high_offsets(x);
+            if (LAST) xp = x;
           }
         } else {
-          x = call(static_cast<uint32_t>(q));
+          uint4 x;
+          if constexpr (PACK8) {
+            x = make_uint4(0u, 0u, 0u, 0u);
+            if (8 * q + 8 <= P.K) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+            } else {
+#pragma unroll 2
+              for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
+            }
+          } else {
+            x = call(static_cast<uint32_t>(q));
+          }
+          x = own(x);
+          lo = low_offsets(x);
+          hi = high_offsets(x);
+          if (LAST) xp = x;
         }
-        if (!(WIDE && wide)) x = item_signs(x, f32, (k.i & 1) != 0, shift, a);
         if (f32 && !(WIDE && wide))
-          add_group<2>(acc, x, frame);
+          add_group<2>(acc, lo, hi, frame);
         else
-          add_group<4>(acc, x, frame);
+          add_group<4>(acc, lo, hi, frame);
       }
     }
-    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
-    if (P.has_pre) {
+    if (P.has_pre && !(LAST && do_sum)) {
       const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
       xp = philox_finish(philox_start(blk, g), P.keys);
-      if (!(WIDE && wide)) xp = item_signs(xp, f32, (k.i & 1) != 0, shift, a);
+      if (LAST) xp = shift_left(xp, P.pre.bit);
+      if (!(WIDE && wide)) xp = own(xp);
     }
     if (!k.act) return;
     if (k.full && do_sum) {
@@ -246,8 +300,10 @@ cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stre
     kernel<<<grid, kItemThreads, smem, stream>>>(p);
     return cudaGetLastError();
   };
-  if (p.packing != kPacking8) return go(update_items_kernel<kPlain, N>);
-  return p.f32_blocks ? go(update_items_kernel<kBytesF32, N>) : go(update_items_kernel<kBytes, N>);
+  if (p.packing != kPacking8) return go(update_items_kernel<kPlain, false, N>);
+  if (p.pre_last != 0)
+    return p.f32_blocks ? go(update_items_kernel<kBytesF32, true, N>) : go(update_items_kernel<kBytes, true, N>);
+  return p.f32_blocks ? go(update_items_kernel<kBytesF32, false, N>) : go(update_items_kernel<kBytes, false, N>);
 }
 template cudaError_t launch_update_items(const UpdateItemsParams<kItemsFew>& p, cudaStream_t stream);
 template cudaError_t launch_update_items(const UpdateItemsParams<kItemsSome>& p, cudaStream_t stream);
