@@ -20,8 +20,8 @@ LIB = os.path.join(HERE, "libzo.so")
 STAMP = LIB + ".arch"   # architecture the library was linked for
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["zo_api.cu", "zo_stream_kernels.cu", "zo_update_lut8.cu", "zo_small_kernels.cu",
-           "zo_quad_step.cu", "zo_update_items.cu"]
-HEADERS = ["zo_device.cuh", "zo_items.h", "zo_launch.h", "zo_precond.cuh"]
+           "zo_quad_step.cu", "zo_update_items.cu", "zo_update_blocks.cu"]
+HEADERS = ["zo_blocks.cuh", "zo_device.cuh", "zo_items.h", "zo_launch.h", "zo_precond.cuh"]
 
 
 def nvcc() -> str:

@@ -468,7 +468,8 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
     if (done) return ZO_OK;
   }
-  const bool few = zo::lut8_small_takes(up, f32_views);
+  const bool blocks = f32_views && zo::update_blocks_takes(up, f32_off, d->sms);
+  const bool few = !blocks && zo::lut8_small_takes(up, f32_views);
   tl_update.f32_blocks = f32_blocks;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -485,9 +486,11 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     for (int i = 0; i < up.tab.n && !any; ++i)
       any = up.tab.numel[i] > 0 &&
             ((up.tab.flags[i] & zo::kShift) || (up.tab.flags[i] & zo::kDtypeMask) == zo::kF32);
-    const cudaError_t e = small ? zo::launch_update_lut8_small(tl_update, any, d->sms, s)
-                                : zo::launch_update_lut8(up, any, d->sms, s);
-    if (e != cudaSuccess) return cuda_fail(e, small ? "update_lut8_small_kernel" : "update_lut8_kernel");
+    const cudaError_t e = blocks  ? zo::launch_update_blocks(up, d->sms, s)
+                          : small ? zo::launch_update_lut8_small(tl_update, any, d->sms, s)
+                                  : zo::launch_update_lut8(up, any, d->sms, s);
+    if (e != cudaSuccess)
+      return cuda_fail(e, blocks ? "update_blocks_kernel" : small ? "update_lut8_small_kernel" : "update_lut8_kernel");
   }
   return ZO_OK;
 }

@@ -36,6 +36,7 @@
 // launch (update_lut8_small_kernel): no chunks, and the sums stay in registers.
 #include <type_traits>
 
+#include "zo_blocks.cuh"
 #include "zo_device.cuh"
 #include "zo_launch.h"
 
@@ -63,22 +64,7 @@ __device__ __forceinline__ void lut8_lookup(float (&acc)[16], const uint4& x, ui
   }
 }
 
-// A thread's block of the current chunk, or, of a tensor off the 32-byte grid
-// (kShift), its 32-byte aligned chunk of sixteen elements: chunk c holds
-// elements 16c - a .. 16c - a + 15 (a = the base's offset from the boundary
-// below it, in elements), the tail of block c - 1 and the head of block c.
-struct Lut8Block {
-  int64_t b;       // virtual block whose probes the lane sums (Philox counter)
-  int64_t e0;      // first element of the block or chunk inside its tensor (below 0 in a tensor's first chunk)
-  int64_t numel;   // elements of the tensor
-  void* base;      // tensor base pointer
-  uint32_t a;      // chunks: a; blocks: 0
-  uint8_t fl;      // tensor flags
-  bool act;        // there are elements here for this lane
-  bool vec;        // all sixteen, 32-byte aligned
-};
-
-// The same for sixteen fp32 weights: scalar adds, as in every fp32 path.
+// Sixteen fp32 weights: the leading perturbation, then the probe sums (scalar adds, as in every fp32 path).
 __device__ __forceinline__ void lut8_apply32(uint32_t (&v)[16], const float (&acc)[16], const uint4& xp,
                                              const UpdateParams& P) {
 #pragma unroll
@@ -86,26 +72,6 @@ __device__ __forceinline__ void lut8_apply32(uint32_t (&v)[16], const float (&ac
     float th = __uint_as_float(v[i]);
     if (P.has_pre) th = add_signed(th, xp, i, P.pre);
     v[i] = __float_as_uint(__fadd_rn(th, acc[i]));
-  }
-}
-
-// The same element by element, for a block or chunk across an end of its
-// tensor; do_sum false: the leading perturbation alone.
-__device__ __forceinline__ void lut8_apply_elements(const Lut8Block& k, const float (&acc)[16], const uint4& xp,
-                                                    const UpdateParams& P, bool do_sum) {
-  const uint8_t dt = k.fl & kDtypeMask;
-  float v[16];  // all loads before the first store: there are registers for it here
-#pragma unroll
-  for (int i = 0; i < 16; ++i)
-    v[i] = k.e0 + i >= 0 && k.e0 + i < k.numel ? load_elem(k.base, dt, k.e0 + i) : 0.0f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const int64_t e = k.e0 + i;
-    if (e < 0 || e >= k.numel) continue;
-    float th = v[i];
-    if (P.has_pre) th = round_to_storage(dt, add_signed(th, xp, i, P.pre));
-    if (do_sum) th = __fadd_rn(th, acc[i]);
-    store_elem(k.base, dt, e, th);
   }
 }
 
@@ -199,38 +165,6 @@ __device__ __forceinline__ void lut8_replicate4(uint32_t t4, uint32_t dst_t, int
 #pragma unroll
     for (int p = 0; p < S; ++p) sts_f32x4(dst_t + 128u + p * kRowStep * 256u, v1[p]);
   }
-}
-
-// Launch block bl, of tensor t: its place. (t of the warp's first block: every
-// tensor starts on a multiple of 32 launch blocks, so the 32 blocks of a warp
-// lie in one tensor or in the padding after it.) ANY: the launch may hold
-// kShift tensors. Of those each warp takes 31 chunks: lane l sums block
-// 31 w + l - 1 of the tensor and works on the chunk of that number, with the
-// sums of the block below from lane l - 1; lane 0 only sums.
-template <bool ANY>
-__device__ __forceinline__ Lut8Block lut8_block_info(const TensorTable& tab, int t, uint32_t bl) {
-  Lut8Block k;
-  const uint32_t tb = tensor_blk_begin(tab, t);
-  const uint32_t d = bl - tb;
-  k.fl = tab.flags[t];
-  k.numel = tab.numel[t];
-  k.base = reinterpret_cast<void*>(tab.ptr[t]);
-  k.a = 0u;
-  if (ANY && (k.fl & kShift)) {
-    const uint32_t lane = d & 31u;
-    k.a = static_cast<uint32_t>(tab.ptr[t] & 31u) / ((k.fl & kDtypeMask) == kF32 ? 4u : 2u);
-    const int64_t c = static_cast<int64_t>(d >> 5) * 31 + lane - 1;
-    k.b = virtual_block(tab, t, tb) + c;
-    k.e0 = 16 * c - k.a;
-    k.act = lane > 0 && k.e0 < k.numel;
-    k.vec = k.act && k.e0 >= 0 && k.e0 + 16 <= k.numel;
-  } else {
-    k.b = virtual_block(tab, t, bl);
-    k.e0 = static_cast<int64_t>(d) * 16;
-    k.act = bl < tab.blk_end[t];
-    k.vec = k.act && k.e0 + 16 <= k.numel && (k.fl & kVec32);
-  }
-  return k;
 }
 
 // A block's part of the counter: HIU, its round-0/1 products; otherwise the

@@ -2,7 +2,8 @@
 kernel that keeps every group's table in shared memory: each place its leading
 perturbation's signs come from (none, the last group, another group), each
 storage type, aligned and in views, tensors that end inside an item or hold
-less than one. Views are compared bit for bit with the same values in aligned
+less than one; and lists of mostly fp32 views without a leading perturbation,
+which a kernel of their own takes by blocks. Views are compared bit for bit with the same values in aligned
 tensors, everything with the oracle within the derived bound."""
 import numpy as np
 import pytest
@@ -75,3 +76,19 @@ def test_two_groups_of_fp32_blocks(K, pre_probe):
 @pytest.mark.parametrize("K", [20, 32])
 def test_whole_list_in_views(K):
     check([long_list(BF16), 31 * 16, 16], [BF16, F16, F32], [1, 9, 2], K, K - 1, seed=K + 1)
+
+
+@pytest.mark.parametrize("K,per_sm", [(17, 0), (24, 0), (32, 0), (39, 0), (41, 0), (56, 0), (80, 0), (5, 200_050)])
+def test_fp32_views_by_blocks(K, per_sm):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = per_sm * sms + 3 if per_sm else long_list(F32)
+    numels = [n, 16 * 31 - 3, 16 * 31 - 2, 16 * 62 - 2, 9, 1, 513, 77, 4096, 130]
+    check(numels, [F32] * 6 + [F16, BF16, F32, BF16], [3, 3, 2, 2, 7, 1, 5, 0, 0, 0], K, None, seed=K)
+
+
+def test_fp32_views_after_a_failed_preconditioner():
+    theta = torch.randn(long_list(F32) + 1, device="cuda")
+    before = theta.clone()
+    zo.update([theta[1:]], 3, torch.ones(32, dtype=torch.float64, device="cuda"), 1e-3,
+              status=torch.tensor([zo.ZO_ERR_NONFINITE], dtype=torch.int32, device="cuda"))
+    assert torch.equal(theta, before)
