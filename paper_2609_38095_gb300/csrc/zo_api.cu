@@ -82,22 +82,26 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 //               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
 // (3 M weights are 1233 items per SM). Under packing 8 generating the bits is
 // most of the work and many small CTAs do it best, whatever the size, but for
-// long lists of many groups:
-//   16 bits     K = 3: 5 M 13.8 / 20.3, 205 M 279 / 317;  K = 24: 29.2 / 38.0, 872 / 907
-//               K = 64: 60 M 628 / 633, 205 M 2116 / 2091;  K = 128: 1212 / 1207, 4109 / 4021
-//   fp32        K = 8: 3 M 12.9 / 17.0, 100 M 193 / 206;  K = 24: 21.7 / 27.0, 432 / 458
-//               K = 64: 3 M 43.8 / 48.5, 100 M 1034 / 1039
-//   fp32 views  K = 3: 3 M 14.7 / 17.0, 6 M 23.1 / 21.3;  K = 24: 1 M 14.8 / 17.0, 3 M 31.4 / 28.2
-//               K = 64: 1 M 27.3 / 24.8
+// 16-bit lists of many groups:
+//   fp32          K = 3: 100 M 150 / 162;  K = 24: 399 / 458;  K = 64: 50 M 506 / 531, 205 M 2010 / 2081
+//                 K = 256: 50 M 1944 / 1978, 205 M 7800 / 7880
+//   16 bits       K = 3: 205 M 279 / 317;  K = 24: 872 / 907;  K = 64: 50 M 512 / 522, 205 M 2049 / 2047
+//                 K = 96: 50 M 756 / 763, 80 M 1203 / 1199;  K = 256: 20 M 804 / 832, 50 M 1977 / 1967
+//   16-bit views  K = 64: 20 M 224 / 227, 205 M 2179 / 2154;  K = 128: 10 M 224 / 233, 20 M 434 / 429, 50 M 1070 / 1040
+//   fp32 views    K = 3: 3 M 14.7 / 17.0, 6 M 23.1 / 21.3;  K = 24: 1 M 14.8 / 17.0, 3 M 31.4 / 28.2
+//                 K = 64: 1 M 27.3 / 24.8
 // (1 M fp32 weights are 822 items per SM; those off the 32-byte grid make a
-// block's words twice). Between 1 and 0.05 M weights of packing 1 all of these
-// take about 9 us here, 11 to 35 with the tables.
-int64_t update_items_per_sm(int packing, int groups, bool f32_views) {
-  if (packing == zo::kPacking8) {
-    if (f32_views) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
-    return groups < 8 ? INT64_C(1) << 20 : 24000;
-  }
-  return groups == 3 || groups == 4 ? 2400 : 1600;
+// block's words twice. With a leading perturbation, whose words the items have
+// for nothing, they gain up to 1 %: K = 64, 205 M 2076 / 2100.) Between 1 and
+// 0.05 M weights of packing 1 all of these take about 9 us here, 11 to 35 with
+// the tables. f32, views: mostly so, by weights.
+int64_t update_items_per_sm(int packing, int groups, bool f32, bool views) {
+  if (packing != zo::kPacking8) return groups == 3 || groups == 4 ? 2400 : 1600;
+  constexpr int64_t any = INT64_C(1) << 20;
+  if (f32 && views) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
+  if (f32 || groups < 8) return any;
+  if (views) return groups == 8 ? 24000 : 8000;
+  return groups == 8 ? any : 24000;
 }
 
 // Per-device launch facts, filled once per device.
@@ -424,14 +428,17 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  int64_t f32 = 0, f32_off = 0, all = 0;  // elements: fp32 on and off the 32-byte grid, all
+  int64_t f32 = 0, f32_off = 0, off = 0, all = 0;  // weights: fp32 on and off the 32-byte grid, any off it, all
   for (int32_t i = 0; i < n_tensors; ++i) {
+    const bool on = reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0;
     all += params[i].numel;
-    if (params[i].dtype != ZO_F32) continue;
-    (reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0 ? f32 : f32_off) += params[i].numel;
+    if (!on) off += params[i].numel;
+    if (params[i].dtype == ZO_F32) (on ? f32 : f32_off) += params[i].numel;
   }
   const bool f32_blocks = 2 * f32 > all, f32_views = 2 * f32_off > all;
-  const int64_t most_items = update_items_per_sm(up.packing, up.groups, f32_views) * d->sms;
+  const int64_t most_items =
+      update_items_per_sm(up.packing, up.groups, f32_blocks || f32_views, f32_views || (!f32_blocks && 2 * off > all)) *
+      d->sms;
   const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
     zo::ItemsCursor cur;
     const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
