@@ -73,7 +73,9 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
   return op;
 }
 
-// Most items per SM of a list that update_items_kernel takes. It does two
+// Most items per SM of a list that update_items_kernel takes, in as many
+// launches as its tensors fill tables (packing 8, K = 8, 1000 tensors of 1 M bf16
+// weights in all: 42 -> 21 us). It does two
 // lookups per element and group where the table-per-lane kernels do one, but
 // copies no tables; the lines lie where the two cross on 12 or 24 tensors (us,
 // items against tables):
@@ -97,7 +99,7 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 // the tables. f32, views: mostly so, by weights.
 int64_t update_items_per_sm(int packing, int groups, bool f32, bool views) {
   if (packing != zo::kPacking8) return groups == 3 || groups == 4 ? 2400 : 1600;
-  constexpr int64_t any = INT64_C(1) << 20;
+  constexpr int64_t any = INT64_C(1) << 40;
   if (f32 && views) return groups == 1 ? 3000 : groups <= 4 ? 1200 : 400;
   if (f32 || groups < 8) return any;
   if (views) return groups == 8 ? 24000 : 8000;
@@ -429,8 +431,10 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
   int64_t f32 = 0, f32_off = 0, off = 0, all = 0;  // weights: fp32 on and off the 32-byte grid, any off it, all
+  int64_t items = 0;                               // of the list by items
   for (int32_t i = 0; i < n_tensors; ++i) {
     const bool on = reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0;
+    items += zo::tensor_items(params[i]);
     all += params[i].numel;
     if (!on) off += params[i].numel;
     if (params[i].dtype == ZO_F32) (on ? f32 : f32_off) += params[i].numel;
@@ -439,12 +443,10 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   const int64_t most_items =
       update_items_per_sm(up.packing, up.groups, f32_blocks || f32_views, f32_views || (!f32_blocks && 2 * off > all)) *
       d->sms;
-  const auto short_list = [&](auto& ip, bool* done) -> cudaError_t {
-    zo::ItemsCursor cur;
-    const bool one_high = zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {}, zo::kItemsPiece,
-                                         most_items);
-    *done = cur.t == n_tensors && one_high && ip.total <= most_items;
-    if (!*done || ip.n == 0) return cudaSuccess;
+  zo::ItemsCursor cur;
+  const auto by_items = [&](auto& ip) -> cudaError_t {
+    zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {});
+    if (ip.n == 0) return cudaSuccess;
     // packing 8: several items per thread where about eight waves of CTAs remain, which spread a CTA's tables over
     // more work (205 M bf16 weights, K = 8, one / eight / ten items: 396 / 317 / 315 us; as fp32 with 32 / 64 at most
     // 326 / 322; 30 M bf16 weights one / two 58.4 / 55.7)
@@ -467,16 +469,18 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     ip.status = status;
     return zo::launch_update_items(ip, static_cast<cudaStream_t>(stream));
   };
-  {
-    bool done = false;
-    const cudaError_t e = n_tensors <= zo::kItemsFew    ? short_list(tl_update_few, &done)
-                          : n_tensors <= zo::kItemsSome ? short_list(tl_update_some, &done)
-                                                        : short_list(tl_update_many, &done);
-    if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
-    if (done) return ZO_OK;
+  if (items <= most_items && all / 16 + n_tensors <= INT64_C(1) << 32) {  // the blocks' counter high word is 0
+    while (cur.t < n_tensors) {
+      const int32_t left = n_tensors - cur.t;
+      const cudaError_t e = left <= zo::kItemsFew    ? by_items(tl_update_few)
+                            : left <= zo::kItemsSome ? by_items(tl_update_some)
+                                                     : by_items(tl_update_many);
+      if (e != cudaSuccess) return cuda_fail(e, "update_items_kernel");
+    }
+    return ZO_OK;
   }
-  const bool blocks = f32_views && zo::update_blocks_takes(up, f32_off, d->sms);
-  const bool few = !blocks && zo::lut8_small_takes(up, f32_views);
+  const bool by_blocks = f32_views && zo::update_blocks_takes(up, f32_off, d->sms);
+  const bool few = !by_blocks && zo::lut8_small_takes(up, f32_views);
   tl_update.f32_blocks = f32_blocks;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -493,11 +497,11 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     for (int i = 0; i < up.tab.n && !any; ++i)
       any = up.tab.numel[i] > 0 &&
             ((up.tab.flags[i] & zo::kShift) || (up.tab.flags[i] & zo::kDtypeMask) == zo::kF32);
-    const cudaError_t e = blocks  ? zo::launch_update_blocks(up, d->sms, s)
-                          : small ? zo::launch_update_lut8_small(tl_update, any, d->sms, s)
-                                  : zo::launch_update_lut8(up, any, d->sms, s);
+    const cudaError_t e = by_blocks ? zo::launch_update_blocks(up, d->sms, s)
+                          : small   ? zo::launch_update_lut8_small(tl_update, any, d->sms, s)
+                                    : zo::launch_update_lut8(up, any, d->sms, s);
     if (e != cudaSuccess)
-      return cuda_fail(e, blocks ? "update_blocks_kernel" : small ? "update_lut8_small_kernel" : "update_lut8_kernel");
+      return cuda_fail(e, by_blocks ? "update_blocks_kernel" : small ? "update_lut8_small_kernel" : "update_lut8_kernel");
   }
   return ZO_OK;
 }

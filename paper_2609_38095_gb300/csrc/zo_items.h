@@ -17,6 +17,20 @@ struct ItemsCursor {
   int64_t v = 0;
 };
 
+// log2 of a storage type's bytes (a division by a variable costs a long list's
+// call more than the rest of its loop).
+inline int size_shift(int32_t dtype) { return dtype == ZO_F32 ? 2 : 1; }
+
+// Items of a tensor in a launch's numbering, up to the next tensor's start.
+inline int64_t tensor_items(const zo_tensor& p) {
+  if (p.numel == 0) return 0;
+  const int sh = size_shift(p.dtype);
+  const int64_t off = static_cast<int64_t>(reinterpret_cast<uintptr_t>(p.ptr) % 32) >> sh;
+  const int64_t items = (p.numel + off + (32 >> sh) - 1) >> (5 - sh);
+  return off == 0 ? (items + kLaunchAlign - 1) / kLaunchAlign * kLaunchAlign
+                  : (items + kShiftLanes - 1) / kShiftLanes * kLaunchAlign;
+}
+
 // Most items of one entry (an even number, so that a later piece of an fp32
 // tensor starts with a whole block) and of one launch. A longer tensor takes
 // several entries.
@@ -40,10 +54,11 @@ bool fill_items(Params& ip, const zo_tensor* params, int32_t n, ItemsCursor& cur
       continue;
     }
     if (ip.n == N) break;
-    const int64_t esz = p.dtype == ZO_F32 ? 4 : 2, per = 32 / esz;
+    const int sh = size_shift(p.dtype);
     const uintptr_t addr = reinterpret_cast<uintptr_t>(p.ptr);
-    const int64_t off = static_cast<int64_t>(addr % 32) / esz;
-    const int64_t whole = (p.numel + off) / per, rem = (p.numel + off) % per, items = whole + (rem != 0);
+    const int64_t off = static_cast<int64_t>(addr % 32) >> sh;
+    const int64_t whole = (p.numel + off) >> (5 - sh), rem = (p.numel + off) & ((32 >> sh) - 1);
+    const int64_t items = whole + (rem != 0);
     const int64_t left = items - cur.done, take = left < piece ? left : piece;
     const int64_t start = (b + kLaunchAlign - 1) / kLaunchAlign * kLaunchAlign;
     const int64_t end = start + (off == 0 ? take : (take + kShiftLanes - 1) / kShiftLanes * kLaunchAlign);

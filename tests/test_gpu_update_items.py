@@ -85,3 +85,24 @@ def test_short_list_of_many_tensors(n):
     for i, (d, h) in enumerate(zip(dev, host)):
         if h.size:
             assert_update_close(storage_bits(d), storage_bits(h), W.DT_BF16, c_np, lr, context=f"tensor {i}")
+
+
+@pytest.mark.parametrize("n", [961, 1985])
+@pytest.mark.parametrize("K,packing", [(19, 1), (9, 8)])
+def test_more_tensors_than_a_launch_holds(n, K, packing):
+    rng = np.random.default_rng(n + K)
+    numels = [int(x) for x in rng.integers(0, 90, n)]
+    numels[7], numels[n - 3] = 70_001, 5000
+    dtypes = [DTYPES[i % 3] for i in range(n)]
+    offsets = [int(x) for x in rng.integers(0, 4, n)]
+    dts = [TORCH_TO_DT[d] for d in dtypes]
+    host = [W.random_storage(rng, m, dt) for m, dt in zip(numels, dts)]
+    dev = views_of(host, dtypes, offsets)
+    s, lr, c_np = W.step_seed(n), 1e-3, rng.normal(0, 25, K)
+    zo.update(zo.ParamList(dev, packing=packing), s, torch.tensor(c_np, device="cuda"), lr, pre=(K - 1, 1e-3))
+    with oracle.packing(packing):
+        oracle.perturb(host, dts, s, K - 1, 1e-3)
+        oracle.update(host, dts, s, c_np, lr)
+    for i, (d, h, dt) in enumerate(zip(dev, host, dts)):
+        if h.size:
+            assert_update_close(storage_bits(d), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
