@@ -343,9 +343,10 @@ int zo_perturb_quadratic_loss(float* theta, const float* a, int64_t n, uint64_t 
  *              ZERO-FILLED before its first use (it holds a counter that every
  *              call leaves at zero), not shared with concurrent calls.
  * Each loss term is carried as an exact pair of fp32 values while its partial
- * products lie in [2^-100, 2^100), else in fp64, the pairs summed as pairs up
- * to a CTA and in fp64 from there, in a fixed order (bit-reproducible for a
- * given device). The losses differ from zo_quadratic_loss's by rounding only.
+ * products lie in [2^-100, 2^100), else in fp64, the pairs summed as pairs in a
+ * warp, as three fp32 values up to a CTA and in fp64 from there, in a fixed
+ * order (bit-reproducible for a given device). The losses differ from
+ * zo_quadratic_loss's by rounding only.
  * Errors: ZO_ERR_ARG (n < 0, null pointers, K < 1, a scale not finite, c
  * without status or the reverse, eps <= 0 with c, packing not 0/1/8), ZO_ERR_TOO_MANY_PROBES, ZO_ERR_ALIGN (theta, a not
  * 4-byte aligned), ZO_ERR_WORKSPACE, ZO_ERR_CUDA.

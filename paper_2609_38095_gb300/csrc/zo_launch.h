@@ -16,7 +16,7 @@ constexpr int kMaxLossPartials = 2048;
 constexpr int kStaticLossPartials = 4096;   // fixed scratch of the allocation-free loss (32 KB)
 constexpr int kMaxQuadPassPartials = 4096;  // CTAs of the one-pass perturbation + loss
 constexpr int kQuadPointsMaxCtas = 256;     // CTAs of the launch that takes a step through all its forward points
-constexpr size_t kQuadPointsMaxSmem = 200 * 1024;  // and its shared memory per CTA
+constexpr size_t kQuadPointsMaxSmem = 224 * 1024;  // and its shared memory per CTA
 constexpr int64_t kStaticLossSlice = 2048;  // elements per partial in that variant
 
 // Perturbation by 32-byte items, one per thread.

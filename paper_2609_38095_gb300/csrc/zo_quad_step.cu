@@ -24,12 +24,16 @@
 //
 // Reduction. A thread ends four probes with eight pairs, which a warp's
 // butterfly folds by halving the values as it doubles the lanes (9 exchanges
-// for the 8 values; a tree for each would be 40). The pairs are added per
-// warp in shared memory over the launch's rounds, then over the CTA's warps
-// in order, and the CTA that finishes last (a ticket counter in the
-// workspace, reset by that CTA) folds the CTAs' fp64 partials in index order
-// and writes the loss table. No CTA waits for another; for a given size every
-// order is fixed, so the losses are bit-reproducible.
+// for the 8 values; a tree for each would be 40). From the warp on, over its
+// rounds in shared memory and over the CTA's warps, eight lanes to a point, a
+// sum is three fp32 values that carry the pairs' rounding errors: two alone put
+// a loss 1.6 times as far from the exact sum as a launch per point does, whose
+// sums are fp64 from the warp on (root mean square over 60 losses 1.9e-16, 1.2e-16
+// so and there); fp64 here took the slow pipe 2 us (d = 2^20, K = 8: 31 -> 33).
+// The CTA that finishes last (a ticket counter in the workspace, reset by that
+// CTA) folds the CTAs' fp64 partials in index order and writes the loss table.
+// No CTA waits for another; for a given size every order is fixed, so the
+// losses are bit-reproducible.
 #include <type_traits>
 
 #include "zo_device.cuh"
@@ -87,6 +91,28 @@ __device__ __forceinline__ Ds ds_sum(Ds a, Ds b) {
   const float bb = __fsub_rn(s, a.s);
   const float e = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, bb)), __fsub_rn(b.s, bb));
   return {s, __fadd_rn(a.l, __fadd_rn(e, b.l))};
+}
+
+// x <- fl(x + y); its rounding error.
+__device__ __forceinline__ float two_sum(float& x, float y) {
+  const float s = __fadd_rn(x, y);
+  const float bb = __fsub_rn(s, x);
+  const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(y, bb));
+  x = s;
+  return e;
+}
+
+struct Ts {  // s + l + m
+  float s, l, m;
+};
+
+// a + b, the errors of the first two parts' sums kept.
+__device__ __forceinline__ Ts ts_sum(Ts a, Ts b) {
+  const float e = two_sum(a.s, b.s);
+  const float f = two_sum(a.l, b.l);
+  const float g = two_sum(a.l, e);
+  a.m = __fadd_rn(__fadd_rn(a.m, b.m), __fadd_rn(f, g));
+  return a;
 }
 
 constexpr float kMinA = 0x1p-40f, kMaxA = 0x1p40f, kMinT = 0x1p-30f, kMaxT = 0x1p30f;
@@ -196,10 +222,11 @@ __device__ __forceinline__ Ds butterfly8(Ds (&v)[8], int lane) {
 
 }  // namespace
 
-// Shared memory per warp: fp32 pairs and fp64 parts of 16 points per group of
-// 8 probes, then of the clean loss (slot 16 G).
-size_t quad_points_smem_bytes(int groups, int warps) {
-  return static_cast<size_t>(warps) * (16u * static_cast<size_t>(groups) + 1u) * 16u;
+// Shared memory per warp: the sums' fp32 values (in launches of several rounds
+// a third one, below 2^-46 of the first, as bf16) and fp64 parts of 16 points per
+// group of 8 probes, then of the clean loss (slot 16 G).
+size_t quad_points_smem_bytes(int groups, int warps, bool several) {
+  return static_cast<size_t>(warps) * (16u * static_cast<size_t>(groups) + 1u) * (several ? 18u : 16u);
 }
 
 struct QuadPointsParams {
@@ -215,6 +242,7 @@ struct QuadPointsParams {
   uint32_t* ticket;      // zero before the launch; the last CTA zeroes it again
   float zero;            // 0.0f
   float drift;           // (K + 1) 2^-21
+  int32_t several;       // rounds
   double eps;            // for the coefficients
   double* c;             // K coefficients and their status, or null
   int32_t* status;
@@ -228,9 +256,11 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
   const int slots = 16 * P.groups + 1;
   double* wide_s = reinterpret_cast<double*>(smem);                     // [slots][warps]
   float2* pair_s = reinterpret_cast<float2*>(wide_s + slots * warps);   // [slots][warps]
+  __nv_bfloat16* third_s = reinterpret_cast<__nv_bfloat16*>(pair_s + slots * warps);  // [slots][warps]
   for (int i = threadIdx.x; i < slots * warps; i += blockDim.x) {
     wide_s[i] = 0.0;
     pair_s[i] = make_float2(0.0f, 0.0f);
+    if (P.several) third_s[i] = __float2bfloat16_rn(0.0f);
   }
   __syncthreads();
 
@@ -256,10 +286,17 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     }
     return r;
   };
+  bool again = false;  // not the warp's first round
   const auto store_sum = [&](int slot, Ds v) {
     float2& c = pair_s[slot * warps + warp];
-    const Ds r = ds_sum({c.x, c.y}, v);
+    if (!again) {
+      c = make_float2(v.s, v.l);
+      return;
+    }
+    __nv_bfloat16& m = third_s[slot * warps + warp];
+    const Ts r = ts_sum({c.x, c.y, __bfloat162float(m)}, {v.s, v.l, 0.0f});
     c = make_float2(r.s, r.l);
+    m = __float2bfloat16_rn(r.m);
   };
 
   const int64_t items = (P.n + kItem - 1) / kItem;
@@ -295,12 +332,10 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
       const float ax = fabsf(y.x), ay = fabsf(y.y);
       a_ok = a_ok && (ax >= kMinA || ax == 0.0f) && ax <= kMaxA && (ay >= kMinA || ay == 0.0f) && ay <= kMaxA;
     }
-    {
-      Ds r = point(std::true_type(), 16 * P.groups);
+    Ds clean = point(std::true_type(), 16 * P.groups);
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) r = ds_sum(r, shfl_xor_ds(r, off));
-      if (lane == 0) store_sum(16 * P.groups, r);
-    }
+    for (int off = 16; off > 0; off >>= 1) clean = ds_sum(clean, shfl_xor_ds(clean, off));
+    Ds mine = {0.0f, 0.0f};
     const int64_t b = item >> 1;
     const bool upper = (item & 1) != 0;  // words 2, 3 of the block's Philox output
     uint32_t w0 = 0, w1 = 0;
@@ -349,8 +384,16 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
         v[2 * j + 1] = point(check, 16 * (k >> 3) + 2 * (k & 7) + 1);
         move(0u);
       }
+      // of eight probes' sums, lanes 4 i take the first four's, lanes 4 i + 1 the others', and with the last ones
+      // lane 2 the clean loss: one store
       const Ds r = butterfly8(v, lane);
-      if ((lane & 3) == 0) store_sum(8 * h + (lane >> 2), r);
+      if ((lane & 3) == (h & 1)) mine = r;
+      const bool last = 4 * (h + 1) >= P.K;
+      if ((h & 1) != 0 || last) {
+        const bool c = last && lane == 2;
+        if (c) mine = clean;
+        if ((lane & 3) <= (h & 1) || c) store_sum(c ? 16 * P.groups : 8 * ((h & ~1) + (lane & 3)) + (lane >> 2), mine);
+      }
     }
     };
     // The points lie at theta +- eps up to the restores' drift (three roundings
@@ -369,6 +412,7 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
       probes(std::true_type());
     else
       probes(std::false_type());
+    again = true;
     if (VEC && cnt == kItem) {
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
@@ -385,22 +429,31 @@ __global__ void __launch_bounds__(kPointsMaxThreads, 1) quad_points_kernel(const
     }
   }
   __syncthreads();
-  // the CTA's sums: lane i takes warp i's, a fixed tree over the lanes
+  // the CTA's sums: of each eight lanes, lane i takes warps i, i + 8, .., then a fixed tree over the lanes (rolled: a
+  // launch this short waits for every line of code)
   const int points = 2 * P.K + 1;
-  for (int p = warp; p < points; p += warps) {
-    const int at = (p == 2 * P.K ? 16 * P.groups : p) * warps + lane;
-    Ds r = {0.0f, 0.0f};
+  for (int p0 = 4 * warp; p0 < points; p0 += 4 * warps) {
+    const int p = p0 + (lane >> 3), row = (p == 2 * P.K ? 16 * P.groups : p) * warps;
+    Ts r = {0.0f, 0.0f, 0.0f};
     double w = 0.0;
-    if (lane < warps) {
-      r = {pair_s[at].x, pair_s[at].y};
-      w = wide_s[at];
+#pragma unroll 1
+    for (int i = lane & 7; p < points && i < warps; i += 8) {
+      r = ts_sum(r, {pair_s[row + i].x, pair_s[row + i].y, P.several ? __bfloat162float(third_s[row + i]) : 0.0f});
+      const double x = wide_s[row + i];
+      if (__double_as_longlong(x) != 0) w = __dadd_rn(w, x);
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) r = ds_sum(r, shfl_xor_ds(r, off));
-    if (__any_sync(0xFFFFFFFFu, w != 0.0)) w = warp_sum(w);
-    if (lane == 0)
-      P.partial[static_cast<int64_t>(p) * gridDim.x + blockIdx.x] =
-          __dadd_rn(__dadd_rn(static_cast<double>(r.s), static_cast<double>(r.l)), w);
+#pragma unroll 1
+    for (int off = 4; off > 0; off >>= 1)
+      r = ts_sum(r, {__shfl_xor_sync(0xFFFFFFFFu, r.s, off), __shfl_xor_sync(0xFFFFFFFFu, r.l, off),
+                     __shfl_xor_sync(0xFFFFFFFFu, r.m, off)});
+    const bool any_wide = __any_sync(0xFFFFFFFFu, __double_as_longlong(w) != 0);
+#pragma unroll 1
+    for (int off = any_wide ? 4 : 0; off > 0; off >>= 1) w = __dadd_rn(w, __shfl_xor_sync(0xFFFFFFFFu, w, off));
+    if (p < points && (lane & 7) == 0) {
+      double sum = __dadd_rn(static_cast<double>(r.s), __dadd_rn(static_cast<double>(r.l), static_cast<double>(r.m)));
+      if (any_wide) sum = __dadd_rn(sum, w);
+      P.partial[static_cast<int64_t>(p) * gridDim.x + blockIdx.x] = sum;
+    }
   }
   __threadfence();  // the partials are visible before the ticket counts them
   __syncthreads();
@@ -461,7 +514,7 @@ cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const Ro
   P.c = c;
   P.status = status;
   int max_warps = kPointsMaxThreads / 32;
-  while (max_warps > 1 && quad_points_smem_bytes(P.groups, max_warps) > kQuadPointsMaxSmem) --max_warps;
+  while (max_warps > 1 && quad_points_smem_bytes(P.groups, max_warps, true) > kQuadPointsMaxSmem) --max_warps;
   const int64_t items = (n + kItem - 1) / kItem;
   const int64_t cap = static_cast<int64_t>(num_sms) * max_warps * 32;
   const int64_t rounds = items > cap ? (items + cap - 1) / cap : 1;
@@ -475,7 +528,8 @@ cudaError_t launch_quad_points(float* theta, const float* a, int64_t n, const Ro
   if (grid > num_sms) grid = num_sms;
   if (grid > kQuadPointsMaxCtas) grid = kQuadPointsMaxCtas;  // the workspace's partials
   const bool vec = reinterpret_cast<uintptr_t>(theta) % 16 == 0 && reinterpret_cast<uintptr_t>(a) % 16 == 0;
-  const size_t smem = quad_points_smem_bytes(P.groups, static_cast<int>(warps));
+  P.several = items > grid * warps * 32;
+  const size_t smem = quad_points_smem_bytes(P.groups, static_cast<int>(warps), P.several != 0);
   const auto go = [&](auto kernel) -> cudaError_t {
     if (smem > 48 * 1024) {
       cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -1,9 +1,12 @@
 """zo_quadratic_points: every forward point of a step of the small workload in
 one launch, against the oracle's perturbations (bit for bit) and its fp64
 losses. Each loss is a sum of n exact or 2^-47-accurate terms, added as fp32
-pairs (relative error at most 2^-45 per addition of at most 8 + 40 in a
-thread, warp and CTA, and one per round), so 1e-12 of the sum of |terms| holds
-with room at these sizes."""
+pairs in a warp (relative error at most 2^-45 per addition of at most 8 + 5),
+then as three fp32 values and in fp64, so 1e-12 of the sum of |terms| holds with
+room at these sizes. Against exact sums its losses are no further off than those of a launch
+per point (zo_perturb_quadratic_loss)."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -152,3 +155,39 @@ def test_points_at_a_distance_of_eps_from_zero():
     th[5::11] = np.float32(2 * eps)
     a = (10.0 ** np.random.default_rng(8).uniform(-2, 2, th.size)).astype(np.float32)
     check(th, a, 6, eps=eps)
+
+
+def exact_loss(th, a):
+    """1/2 sum a theta^2 of fp32 arrays, rounded once: a t is exact in fp64, (a t) t is split into two fp64 values."""
+    t = th.astype(np.float64)
+    p = a.astype(np.float64) * t
+    q = p * t
+    high = p * 134217729.0                     # Veltkamp's split: 26 bits and the rest
+    high = high - (high - p)
+    return 0.5 * math.fsum(np.concatenate([q, (high * t - q) + (p - high) * t]).tolist())
+
+
+def test_points_as_close_to_exact_sums_as_a_launch_per_point():
+    """Root mean square over 60 losses, of the same theta and a at every point. Both round a sum of some hundred fp64
+    partials, each good to 2^-53 or so; a quarter is left for the two orders' chance. Sums held as fp32 pairs up to the
+    CTA are 1.6 times as far off."""
+    K, eps, err = 2, 1e-3, {"points": [], "launches": []}
+    for n, seeds in ((1 << 20, 8), (2_500_007, 4)):
+        for sd in range(seeds):
+            rng = np.random.default_rng(sd)
+            th = (rng.standard_normal(n) * 0.02).astype(np.float32)
+            a = (10.0 ** rng.uniform(-2, 2, n)).astype(np.float32)
+            seed, x, v, ad = W.step_seed(sd), on_device(th, 0), on_device(th, 0), on_device(a, 0)
+            table = torch.empty(K, 3, dtype=torch.float64, device="cuda")
+            zo.QuadraticPoints(x, ad, table)(seed, eps)
+            table = table.cpu().numpy()
+            one, out = zo.QuadraticPass(v, ad), torch.empty(1, dtype=torch.float64, device="cuda")
+            for ops, mine in (((), table[0, 2]), ([(0, eps)], table[0, 0]), ([(0, -2 * eps)], table[0, 1]),
+                              ([(0, eps), (1, eps)], table[1, 0]), ([(1, -2 * eps)], table[1, 1])):
+                one(seed, ops, one.out_address(out))
+                theirs = float(out.item())
+                want = exact_loss(v.cpu().numpy(), a)
+                err["points"].append((mine - want) / want)
+                err["launches"].append((theirs - want) / want)
+    rms = {k: float(np.sqrt(np.mean(np.square(e)))) for k, e in err.items()}
+    assert rms["points"] <= 1.25 * rms["launches"], rms
