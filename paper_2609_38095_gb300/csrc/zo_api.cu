@@ -480,7 +480,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     return ZO_OK;
   }
   const bool by_blocks = f32_views && zo::update_blocks_takes(up, f32_off, d->sms);
-  const bool few = !by_blocks && zo::lut8_small_takes(up, f32_views);
+  const bool few = !by_blocks && zo::lut8_small_takes(up, f32_blocks, f32_views);
   tl_update.f32_blocks = f32_blocks;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -30,7 +30,7 @@ template <int N>
 cudaError_t launch_pair_items(const PairItemsParams<N>& p, bool one_high, cudaStream_t stream);
 // Fused update: what lut8_small_takes (packing 1, at most kSmallGroups probe
 // groups) with virtual blocks that share the counter's high word; ...
-bool lut8_small_takes(const UpdateParams& u, bool f32_views);  // f32_views: mostly fp32 off the 32-byte grid
+bool lut8_small_takes(const UpdateParams& u, bool f32_blocks, bool f32_views);  // mostly fp32 on, off the 32-byte grid
 cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream);
 // ... and every other one. any: the launch holds fp32 tensors or tensors off
 // the 32-byte grid (those flagged kShift, in slots of 32 launch blocks per 31

@@ -675,9 +675,9 @@ __device__ __forceinline__ uint32_t entry_addr(uint32_t w, uint32_t frame) {
 }
 
 // The leading perturbation in the small kernel: none, in the last group's
-// table, with Philox words of its own, or with the last group's words (four
-// groups, whose tables leave no room for pairs).
-constexpr int kPreNone = 0, kPreTable = 1, kPreOwn = 2, kPreLast = 3;
+// table, with Philox words of its own, with the last group's words (four
+// groups, whose tables leave no room for pairs), or with another group's.
+constexpr int kPreNone = 0, kPreTable = 1, kPreOwn = 2, kPreLast = 3, kPreGroup = 4;
 
 // Element I's partial sums, and with kPreTable its leading perturbation (d).
 // x: the groups' words; f0, fl: frames of group 0's and the last group's tables.
@@ -1018,6 +1018,12 @@ __global__ void __launch_bounds__(small_threads(G), 1)
       }
     }
     if (PRE == kPreLast) xp = x[G - 1];
+    if constexpr (PRE == kPreGroup) {  // the same group in all lanes
+      xp = x[0];
+#pragma unroll
+      for (int g = 1; g + 1 < G; ++g)
+        if (P.pre.ctr2 == static_cast<uint32_t>(g)) xp = x[g];
+    }
     if (k.full) {
       if (ANY && (c.fl & kDtypeMask) == kF32)
         small_item32<PRE, G>(v, x, xp, f0, fl, P);
@@ -1059,11 +1065,14 @@ cudaError_t small_limit() {
                               static_cast<int>(small_smem_bytes(G, PRE == kPreTable)));
 }
 
+// Whether there is a BLOCKS instantiation (see lut8_small_takes).
+constexpr bool small_has_blocks(int pre, int G) { return G > 1 && !(pre == kPreGroup && G == 4); }
+
 template <int PRE, int G>
 cudaError_t small_limits() {
   cudaError_t e = small_limit<PRE, G, false>();
   if (e == cudaSuccess) e = small_limit<PRE, G, true>();
-  if constexpr (G > 1)
+  if constexpr (small_has_blocks(PRE, G))
     if (e == cudaSuccess) e = small_limit<PRE, G, true, true>();
   return e;
 }
@@ -1079,6 +1088,9 @@ cudaError_t lut8_prepare() {
   if (e == cudaSuccess) e = small_limits<kPreLast, 4>();
   if (e == cudaSuccess) e = small_limits<kPreOwn, 1>();
   if (e == cudaSuccess) e = small_limits<kPreOwn, 2>();
+  if (e == cudaSuccess) e = small_limits<kPreGroup, 2>();
+  if (e == cudaSuccess) e = small_limits<kPreGroup, 3>();
+  if (e == cudaSuccess) e = small_limits<kPreGroup, 4>();
   if (e == cudaSuccess) e = lut8_limit<true, false, false>();
   if (e == cudaSuccess) e = lut8_limit<true, false, false, true>();
   if (e == cudaSuccess) e = lut8_limit<true, true, false>();
@@ -1104,7 +1116,7 @@ void launch_small_cfg(const SmallUpdateParams& p, bool any, int sms, cudaStream_
   constexpr int threads = small_threads(G);
   const int64_t want = (static_cast<int64_t>(p.u.tab.blk_total) + threads - 1) / threads;
   const int grid = static_cast<int>(want < sms ? want : sms);
-  if constexpr (G > 1) {
+  if constexpr (small_has_blocks(PRE, G)) {
     if (any && p.f32_blocks) {
       update_lut8_small_kernel<PRE, G, true, true><<<grid, threads, sm, stream>>>(p);
       return;
@@ -1117,17 +1129,23 @@ void launch_small_cfg(const SmallUpdateParams& p, bool any, int sms, cudaStream_
 }
 
 // Which updates the small kernel takes. Three and four groups only with the
-// leading perturbation's probe in the last group, or none: words of its own
-// would be a fifth Philox call's registers. Views of fp32 make a block's words
+// leading perturbation's probe in one of them, or none: words of its own
+// would be a fifth Philox call's registers. (Its probe in another group than the
+// last: 400 M bf16 weights, K = 16 / 24 / 32: 322 / 584 / 664 us with a call of its
+// own or in the chunk kernel -> 284 / 362 / 448; in one flat buffer 475 / 753 / 827 ->
+// 370 / 472 / 634; fp32 699 / 676 -> 495 / 571, but with four groups 754 -> 797, so
+// those stay.) Views of fp32 make a block's words
 // twice here, once per half, where the chunk kernel makes them once: with four
 // groups that costs them more than the chunks' tables and barriers do (205 M
 // fp32 weights in one flat buffer, K = 32: 0.450 ms here, 0.425 there; K = 24:
 // 0.363 and 0.386). Before, K from 17 on walked the chunks: OPT-1.3B-shaped bf16
 // set with the leading perturbation, K = 24 / 32: 1.612 / 1.857 -> 1.122 / 1.386
 // ms; 400 M bf16 weights in one flat buffer 0.677 / 0.747 -> 0.451 / 0.584 ms.
-bool lut8_small_takes(const UpdateParams& u, bool f32_views) {
+bool lut8_small_takes(const UpdateParams& u, bool f32_blocks, bool f32_views) {
   if (u.packing != kPacking1 || u.groups > kSmallGroups || (u.groups == 4 && f32_views)) return false;
-  return u.groups <= 2 || !u.has_pre || u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups);
+  const uint32_t groups = static_cast<uint32_t>(u.groups);
+  if (u.groups <= 2 || !u.has_pre || u.pre.ctr2 + 1u == groups) return true;
+  return u.pre.ctr2 < groups && !(u.groups == 4 && f32_blocks);
 }
 
 cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cudaStream_t stream) {
@@ -1136,6 +1154,7 @@ cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cu
   for (uint32_t g = 0; g < static_cast<uint32_t>(kSmallGroups); ++g) p.g[g] = group_round01(g, bhi, u.keys);
   p.gp = group_round01(u.pre.ctr2, bhi, u.keys);
   const bool last = u.pre.ctr2 + 1u == static_cast<uint32_t>(u.groups);
+  const bool group = !last && u.pre.ctr2 < static_cast<uint32_t>(u.groups);
   if (u.groups == 1)
     !u.has_pre ? launch_small_cfg<kPreNone, 1>(p, any, sms, stream)
     : last     ? launch_small_cfg<kPreTable, 1>(p, any, sms, stream)
@@ -1143,11 +1162,16 @@ cudaError_t launch_update_lut8_small(SmallUpdateParams& p, bool any, int sms, cu
   else if (u.groups == 2)
     !u.has_pre ? launch_small_cfg<kPreNone, 2>(p, any, sms, stream)
     : last     ? launch_small_cfg<kPreTable, 2>(p, any, sms, stream)
+    : group    ? launch_small_cfg<kPreGroup, 2>(p, any, sms, stream)
                : launch_small_cfg<kPreOwn, 2>(p, any, sms, stream);
   else if (u.groups == 3)
-    !u.has_pre ? launch_small_cfg<kPreNone, 3>(p, any, sms, stream) : launch_small_cfg<kPreTable, 3>(p, any, sms, stream);
+    !u.has_pre ? launch_small_cfg<kPreNone, 3>(p, any, sms, stream)
+    : last     ? launch_small_cfg<kPreTable, 3>(p, any, sms, stream)
+               : launch_small_cfg<kPreGroup, 3>(p, any, sms, stream);
   else
-    !u.has_pre ? launch_small_cfg<kPreNone, 4>(p, any, sms, stream) : launch_small_cfg<kPreLast, 4>(p, any, sms, stream);
+    !u.has_pre ? launch_small_cfg<kPreNone, 4>(p, any, sms, stream)
+    : last     ? launch_small_cfg<kPreLast, 4>(p, any, sms, stream)
+               : launch_small_cfg<kPreGroup, 4>(p, any, sms, stream);
   return cudaGetLastError();
 }
 

@@ -62,20 +62,21 @@ def long_list(dtype):
     return sms * 2400 * per + 3 * per + 1
 
 
-@pytest.mark.parametrize("K,pre_probe", [(17, 16), (24, None), (25, 24), (32, 31), (32, None), (31, 3)])
+@pytest.mark.parametrize("K,pre_probe", [(17, 16), (24, None), (25, 24), (32, 31), (32, None), (31, 3), (24, 2), (20, 13),
+                                         (30, 9), (27, 17), (27, 40)])
 @pytest.mark.parametrize("dtype", [BF16, F32], ids=["bf16", "f32"])
 def test_three_and_four_groups(K, pre_probe, dtype):
     check([long_list(dtype), 1, 15, 513, 77], [dtype, F16, F32, BF16, F16], [0, 0, 3, 5, 0], K, pre_probe, seed=K)
 
 
-@pytest.mark.parametrize("K,pre_probe", [(9, None), (16, 15), (12, 3)])
+@pytest.mark.parametrize("K,pre_probe", [(9, None), (16, 15), (12, 3), (12, 20)])
 def test_two_groups_of_fp32_blocks(K, pre_probe):
     check([long_list(F32), 8, 7, 1023, 65], [F32, F32, F32, F32, BF16], [0, 0, 0, 3, 1], K, pre_probe, seed=K)
 
 
-@pytest.mark.parametrize("K", [20, 32])
-def test_whole_list_in_views(K):
-    check([long_list(BF16), 31 * 16, 16], [BF16, F16, F32], [1, 9, 2], K, K - 1, seed=K + 1)
+@pytest.mark.parametrize("K,pre_probe", [(20, 19), (32, 31), (16, 5), (24, 9), (32, 12)])
+def test_whole_list_in_views(K, pre_probe):
+    check([long_list(BF16), 31 * 16, 16], [BF16, F16, F32], [1, 9, 2], K, pre_probe, seed=K + 1)
 
 
 @pytest.mark.parametrize("K,per_sm", [(17, 0), (24, 0), (32, 0), (39, 0), (41, 0), (56, 0), (80, 0), (5, 200_050)])
