@@ -106,6 +106,38 @@ int64_t update_items_per_sm(int packing, int groups, bool f32, bool views) {
   return groups == 8 ? any : 24000;
 }
 
+// Which kernel an update's list goes to.
+enum UpdateRoute { kByItems, kByBlocks, kResidentTables, kByChunks };
+
+struct UpdatePlan {
+  UpdateRoute route;
+  bool f32_blocks;  // mostly fp32 on the 32-byte grid
+};
+
+UpdatePlan plan_update(const zo_tensor* params, int32_t n, const UpdateParams& up, int sms) {
+  int64_t f32 = 0, f32_off = 0, off = 0, all = 0;  // weights: fp32 on and off the 32-byte grid, any off it, all
+  int64_t items = 0;                               // of the list by items
+  for (int32_t i = 0; i < n; ++i) {
+    const bool on = reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0;
+    items += zo::tensor_items(params[i]);
+    all += params[i].numel;
+    if (!on) off += params[i].numel;
+    if (params[i].dtype == ZO_F32) (on ? f32 : f32_off) += params[i].numel;
+  }
+  const bool f32_blocks = 2 * f32 > all, f32_views = 2 * f32_off > all;
+  const int64_t most_items =
+      update_items_per_sm(up.packing, up.groups, f32_blocks || f32_views, f32_views || (!f32_blocks && 2 * off > all)) *
+      sms;
+  UpdatePlan p = {kByChunks, f32_blocks};
+  if (items <= most_items && all / 16 + n <= INT64_C(1) << 32)  // the items' counter high word is 0
+    p.route = kByItems;
+  else if (f32_views && zo::update_blocks_takes(up, f32_off, sms))
+    p.route = kByBlocks;
+  else if (zo::lut8_small_takes(up, f32_blocks, f32_views))
+    p.route = kResidentTables;
+  return p;
+}
+
 // Per-device launch facts, filled once per device.
 struct DeviceInfo {
   int sms = 0;
@@ -430,19 +462,8 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
   up.has_pre = has_pre != 0;
   up.pre = make_op(pre_probe, has_pre != 0 ? pre_scale : 0.0f, up.packing);
   up.status = status;
-  int64_t f32 = 0, f32_off = 0, off = 0, all = 0;  // weights: fp32 on and off the 32-byte grid, any off it, all
-  int64_t items = 0;                               // of the list by items
-  for (int32_t i = 0; i < n_tensors; ++i) {
-    const bool on = reinterpret_cast<uintptr_t>(params[i].ptr) % 32 == 0;
-    items += zo::tensor_items(params[i]);
-    all += params[i].numel;
-    if (!on) off += params[i].numel;
-    if (params[i].dtype == ZO_F32) (on ? f32 : f32_off) += params[i].numel;
-  }
-  const bool f32_blocks = 2 * f32 > all, f32_views = 2 * f32_off > all;
-  const int64_t most_items =
-      update_items_per_sm(up.packing, up.groups, f32_blocks || f32_views, f32_views || (!f32_blocks && 2 * off > all)) *
-      d->sms;
+  const UpdatePlan plan = plan_update(params, n_tensors, up, d->sms);
+  const bool f32_blocks = plan.f32_blocks;
   zo::ItemsCursor cur;
   const auto by_items = [&](auto& ip) -> cudaError_t {
     zo::fill_items(ip, params, n_tensors, cur, [](auto&, int32_t, int64_t) {});
@@ -469,7 +490,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     ip.status = status;
     return zo::launch_update_items(ip, static_cast<cudaStream_t>(stream));
   };
-  if (items <= most_items && all / 16 + n_tensors <= INT64_C(1) << 32) {  // the blocks' counter high word is 0
+  if (plan.route == kByItems) {
     while (cur.t < n_tensors) {
       const int32_t left = n_tensors - cur.t;
       const cudaError_t e = left <= zo::kItemsFew    ? by_items(tl_update_few)
@@ -479,8 +500,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
     }
     return ZO_OK;
   }
-  const bool by_blocks = f32_views && zo::update_blocks_takes(up, f32_off, d->sms);
-  const bool few = !by_blocks && zo::lut8_small_takes(up, f32_blocks, f32_views);
+  const bool by_blocks = plan.route == kByBlocks, few = plan.route == kResidentTables;
   tl_update.f32_blocks = f32_blocks;
   if ((rc = lut8_ready(d)) != ZO_OK) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -504,6 +524,19 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
       return cuda_fail(e, by_blocks ? "update_blocks_kernel" : small ? "update_lut8_small_kernel" : "update_lut8_kernel");
   }
   return ZO_OK;
+}
+
+// Not part of the public interface: the kernel that zo_update_ex sends a list to
+// on a device of `sms` SMs (UpdateRoute), for the tests of each kernel.
+int zo_internal_update_route(const zo_tensor* params, int32_t n_tensors, int32_t K, int32_t has_pre,
+                             uint32_t pre_probe, int32_t sms) {
+  UpdateParams& up = tl_update.u;
+  int rc = validate_params(params, n_tensors, &up.packing);
+  if (rc != ZO_OK) return rc;
+  up.groups = (K + 7) / 8;
+  up.has_pre = has_pre != 0;
+  up.pre = make_op(pre_probe, 0.0f, up.packing);
+  return plan_update(params, n_tensors, up, sms).route;
 }
 
 int zo_update_sequential(const zo_tensor* params, int32_t n_tensors, uint64_t seed, const double* c, int32_t K,

@@ -1,11 +1,37 @@
 """Helpers shared by the GPU parity tests: storage round-trips between torch
 tensors and the oracle's numpy storage arrays, ulp distances and bounds."""
+import ctypes
+
 import numpy as np
 import torch
 
 from paper_2609_38095_gb300 import workloads as W
+from paper_2609_38095_gb300 import zo
 
 TORCH_TO_DT = {torch.float32: W.DT_F32, torch.bfloat16: W.DT_BF16, torch.float16: W.DT_F16}
+
+
+UPDATE_ROUTES = ("items", "blocks", "tables", "chunks")
+
+
+def update_route(plist, K, pre_probe=None):
+    """The kernel that zo.update sends a list to: update_items_kernel,
+    update_blocks_kernel, update_lut8_small_kernel or update_lut8_kernel."""
+    f = zo._lib().zo_internal_update_route
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_uint32, ctypes.c_int32]
+    f.restype = ctypes.c_int
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    r = f(plist._ptr, plist.n, K, int(pre_probe is not None), pre_probe or 0, sms)
+    assert r >= 0, r
+    return UPDATE_ROUTES[r]
+
+
+def filler(items_per_sm, dtype, offset=0):
+    """A tensor of at least that many 32-byte items per SM, `offset` elements into its allocation: last in a list, it
+    makes the list long without moving the other tensors' probes."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = sms * items_per_sm * (32 // torch.empty(0, dtype=dtype).element_size()) + 5
+    return torch.zeros(n + offset, dtype=dtype, device="cuda")[offset:]
 
 
 def storage_np(t: torch.Tensor) -> np.ndarray:

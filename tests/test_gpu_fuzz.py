@@ -1,9 +1,8 @@
 """Seeded fuzzing of the parameter-list handling: random lists (empty, tiny,
 odd-sized and large tensors, all three dtypes, views at random element
 offsets, so every alignment class) driven through random sequences of
-zo_perturb, zo_perturb2 (every tuned configuration: each list starts with ten
-two-op calls), zo_perturb_pair and zo_update_ex, each result checked
-against the oracle: bit-exact for the perturbations, within the derived
+zo_perturb, zo_perturb2 (ten of them first), zo_perturb_pair and zo_update_ex,
+each result checked against the oracle: bit-exact for the perturbations, within the derived
 tolerance for the update."""
 import numpy as np
 import pytest
@@ -69,7 +68,7 @@ def test_fuzz_lists_and_sequences(case):
     packing = int(rng.choice([1, 8]))
     with oracle.packing(packing), zo.packing(packing):
         for step in range(22):
-            op = 0.5 if step < 10 else rng.random()   # ten two-op calls first: every tuned configuration
+            op = 0.5 if step < 10 else rng.random()   # ten two-op calls first
             k = int(rng.integers(0, 1024))
             scale = float(rng.choice([1e-3, -2e-3, 0.25, -3e-7]))
             if op < 0.25:

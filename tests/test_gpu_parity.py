@@ -15,7 +15,7 @@ from paper_2609_38095_gb300 import build as zo_build
 from paper_2609_38095_gb300 import workloads as W
 from paper_2609_38095_gb300 import zo
 
-from gpu_helpers import (TORCH_TO_DT, assert_update_close, bits_to_f64, storage_bits, storage_np, to_torch,
+from gpu_helpers import (TORCH_TO_DT, assert_update_close, bits_to_f64, storage_bits, storage_np, to_torch, update_route,
                          ulp_distance16)
 
 pytestmark = pytest.mark.gpu
@@ -175,9 +175,9 @@ def test_perturb_every_unaligned_offset(dtype, ops, prefix, packing_mode):
 @pytest.mark.parametrize("K", [5, 16, 64])
 @pytest.mark.parametrize("pre", [False, True])
 def test_update_every_unaligned_offset(dtype, K, pre, packing_mode):
-    """The fused update of unaligned views (aligned chunks, probe sums taken
-    from the neighbouring lane) gives bit for bit what update_kernel gives
-    for the same values in aligned tensors, is within the derived bound of
+    """The fused update of unaligned views (aligned chunks, the signs of the
+    block below taken from the neighbouring lane) gives bit for bit what the
+    same values in aligned tensors give, is within the derived bound of
     the oracle, and writes nothing outside the views."""
     bases, views, host = unaligned_list(dtype, seed=80 + K)
     dts = [TORCH_TO_DT[dtype]] * len(views)
@@ -352,37 +352,38 @@ def test_update_within_tolerance(K, packing_mode):
             print(f"K={K} tensor {i}: {st}")
 
 
-@pytest.mark.parametrize("bpt,K,pre", [(8, 24, True), (8, 40, False), (4, 24, False), (4, 40, True),
-                                       (2, 64, True), (2, 200, False)])
-def test_update_every_chunk_size(bpt, K, pre):
-    """The 8-probe-table update (packing 1, 16 < K <= 384) gives each CTA a
-    chunk of 512 x BPT blocks, BPT = 8, 4 or 2 by launch size (every SM gets
-    a chunk). Lists sized for each BPT on this device, with bf16, fp16 and
+@pytest.mark.parametrize("rows,K,pre", [(4, 40, True), (4, 64, False), (5, 100, True), (8, 40, False), (9, 48, True),
+                                        (10, 36, False)])
+def test_update_every_chunk_size(rows, K, pre):
+    """The chunk kernel (packing 1, more than four probe groups) gives each CTA a chunk of
+    512 blocks a row, eight rows but in the last round, whose rows are what is
+    left. Lists of one and two rounds on this device, with bf16, fp16 and
     fp32 tensors, partial last blocks, a zero-length tensor and a view off the
-    32-byte grid (its blocks skipped by the kernel and done by
-    update_shift_kernel), against the oracle element by element."""
+    32-byte grid, against the oracle element by element."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    blocks = sms * 512 * bpt + 3 * 512 + 7            # just above this BPT's threshold
+    blocks = sms * 512 * rows - 3 * 512 - 7           # the last row not quite full
     numels = [blocks * 16 - 9 * 4096 - 3001 - 17, 4096 * 9 + 5, 0, 3001, 17]
     dtypes = [torch.bfloat16, torch.float16, torch.bfloat16, torch.float32, torch.float16]
-    host, dev = make_list(numels, dtypes, seed=bpt * 1000 + K)
+    host, dev = make_list(numels, dtypes, seed=rows * 1000 + K)
     # the fp16 tensor as a view one element into its own allocation
     base = torch.empty(numels[1] + 1, dtype=torch.float16, device="cuda")
     dev[1] = base[1:]
     dev[1].copy_(to_torch(host[1], torch.float16))
     dts = [TORCH_TO_DT[d] for d in dtypes]
-    c_np = np.random.default_rng(K + bpt).normal(0, 25, K)
+    c_np = np.random.default_rng(K + rows).normal(0, 25, K)
     c = torch.tensor(c_np, dtype=torch.float64, device="cuda")
-    seed, lr, eps = W.step_seed(K + bpt), 1e-3, 1e-3
-    zo.update(dev, seed, c, lr, pre=(K - 1, eps) if pre else None)
+    seed, lr, eps = W.step_seed(K + rows), 1e-3, 1e-3
+    plist = zo.ParamList(dev, packing=1)
+    assert update_route(plist, K, K - 1 if pre else None) == "chunks"
+    zo.update(plist, seed, c, lr, pre=(K - 1, eps) if pre else None)
     if pre:
         oracle.perturb(host, dts, seed, K - 1, eps)
     oracle.update(host, dts, seed, c_np, lr)
     for i, (d, h, dt) in enumerate(zip(dev, host, dts)):
         if h.size:
             st = assert_update_close(storage_bits(d), storage_bits(h), dt, c_np, lr,
-                                     context=f"BPT={bpt} K={K} tensor {i}")
-            print(f"BPT={bpt} K={K} tensor {i}: {st}")
+                                     context=f"rows={rows} K={K} tensor {i}")
+            print(f"rows={rows} K={K} tensor {i}: {st}")
 
 
 @pytest.mark.parametrize("n_alias", [32, 45])
@@ -691,13 +692,9 @@ def test_perturb2_is_two_perturbs(a, b, packing_mode):
     assert_storage_equal(dev, host)
 
 
-def test_perturb2_every_tuned_configuration():
-    """zo_perturb2 times its three candidate configurations on the first nine
-    calls for a parameter list with both probes in one group of 8 (three
-    rounds), and on the first three with the probes in two groups (one
-    round, a kernel of its own), then keeps the fastest of each: 12 calls of
-    the first kind and 6 of the second on one list run every candidate and
-    the chosen one, each bit-exact with the oracle."""
+def test_perturb2_many_pairs_on_one_list():
+    """zo_perturb2 on one list again and again, its probes in one group of 8
+    and in two: every call bit-exact with the oracle."""
     rng = np.random.default_rng(606)
     numels = [int(x) for x in rng.integers(1, 70000, 40)] + [4096 * 300, 17]
     dtypes = [DTS[int(x)] for x in rng.integers(0, 3, len(numels))]
@@ -724,7 +721,7 @@ def test_fused_step_in_a_cuda_graph():
     dts = [TORCH_TO_DT[d] for d in MIXED_DTYPES]
     rng = np.random.default_rng(809)
     for dtype, off, n in ((torch.bfloat16, 3, 5000), (torch.float32, 1, 777), (torch.float16, 5, 40)):
-        h = W.random_storage(rng, n, TORCH_TO_DT[dtype])       # views off the 32-byte grid: the chunk kernels
+        h = W.random_storage(rng, n, TORCH_TO_DT[dtype])       # views off the 32-byte grid
         v = torch.empty(n + off, dtype=dtype, device="cuda")[off:]
         v.copy_(to_torch(h, dtype))
         host.append(h.copy())
@@ -776,8 +773,8 @@ def test_fused_step_in_a_cuda_graph():
 def test_concurrent_host_threads_on_their_own_streams():
     """Two host threads, each with its own parameter list and stream, call the
     library at the same time (the binding releases the GIL in every call):
-    the per-thread launch state, the device table and the two-op tuner keep
-    them apart, and each list matches the oracle."""
+    the per-thread launch state and the device table keep them apart, and each
+    list matches the oracle."""
     import threading
     K, eps, iters = 6, 1e-3, 20
     jobs = []

@@ -4,7 +4,7 @@ Weights: every bf16 and every fp16 bit pattern (signed zeros, subnormals,
 the largest finite values, infinities, every NaN), and for fp32 storage the
 same classes (NaNs with payloads, quiet and signalling) plus seeded random
 bit patterns. Each list holds the patterns three times: an aligned tensor
-(the 256-bit block path), a view one element in (the aligned-chunk kernels)
+(256-bit accesses), a view one element in (aligned chunks across two blocks)
 and a short tail (the element-wise path).
 
 Scales: small and large ones of both signs, one that lands every weight of
@@ -26,7 +26,7 @@ from paper_2609_38095_gb300 import build as zo_build
 from paper_2609_38095_gb300 import workloads as W
 from paper_2609_38095_gb300 import zo
 
-from gpu_helpers import assert_update_close, storage_bits, storage_np, to_torch
+from gpu_helpers import assert_update_close, filler, storage_bits, storage_np, to_torch, update_route
 
 pytestmark = pytest.mark.gpu
 
@@ -141,6 +141,33 @@ def test_update_special_values(name, K, pre, packing_mode):
     for i, (d, h) in enumerate(zip(dev, host)):
         st = assert_update_close(storage_bits(d), storage_bits(h), dt, c_np, lr, context=f"{name} K={K} tensor {i}")
         print(f"specials update {name} K={K} pre={pre} tensor {i}: {st}")
+
+
+# Lists that a long last tensor sends to the kernels of long lists: every instantiation of the leading perturbation in
+# the kernel with resident tables (with 16-bit majorities and, for its blocks of fp32, an fp32 one), the chunk kernel
+# under both packings, the kernel by blocks.
+@pytest.mark.parametrize("name", list(CASES))
+@pytest.mark.parametrize("K,pre_probe,packing,long,route",
+                         [(8, None, 1, "bf16", "tables"), (16, 15, 1, "bf16", "tables"), (16, 3, 1, "bf16", "tables"),
+                          (16, 99, 1, "bf16", "tables"), (24, 23, 1, "f32", "tables"), (32, 31, 1, "bf16", "tables"),
+                          (32, 9, 1, "bf16", "tables"), (32, 31, 1, "f32", "tables"), (64, 63, 1, "bf16", "chunks"),
+                          (200, 199, 1, "bf16", "chunks"), (64, None, 1, "bf16", "chunks"), (32, None, 1, "view", "blocks"),
+                          (8, 7, 8, "view", "chunks"), (64, None, 8, "view", "chunks")])
+def test_update_special_values_in_long_lists(name, K, pre_probe, packing, long, route):
+    seed, lr = W.step_seed(47), 1e-2
+    c_np = np.random.default_rng(K).normal(0, 5, K)
+    c = torch.tensor(c_np, dtype=torch.float64, device="cuda")
+    host, dev, dt = make(name)
+    last = {"bf16": (2401, torch.bfloat16, 0), "f32": (2501, torch.float32, 0), "view": (3001, torch.float32, 1)}[long]
+    plist = zo.ParamList(dev + [filler(*last)], packing=packing)
+    assert update_route(plist, K, pre_probe) == route
+    zo.update(plist, seed, c, lr, pre=None if pre_probe is None else (pre_probe, 1e-3))
+    with oracle.packing(packing):
+        if pre_probe is not None:
+            oracle.perturb(host, [dt] * 3, seed, pre_probe, 1e-3)
+        oracle.update(host, [dt] * 3, seed, c_np, lr)
+    for i, (d, h) in enumerate(zip(dev, host)):
+        assert_update_close(storage_bits(d), storage_bits(h), dt, c_np, lr, context=f"{name} K={K} tensor {i}")
 
 
 @pytest.mark.parametrize("name", list(CASES))

@@ -14,7 +14,7 @@ from paper_2609_38095_gb300 import build as zo_build
 from paper_2609_38095_gb300 import workloads as W
 from paper_2609_38095_gb300 import zo
 
-from gpu_helpers import TORCH_TO_DT, assert_update_close, storage_bits, to_torch
+from gpu_helpers import TORCH_TO_DT, assert_update_close, storage_bits, to_torch, update_route
 
 pytestmark = pytest.mark.gpu
 
@@ -29,9 +29,9 @@ def _built():
     oracle.lib()
 
 
-def check(numels, dtypes, offsets, K, pre_probe, seed):
+def check(numels, dtypes, offsets, K, pre_probe, seed, route="tables"):
     """One update of views `offsets` elements into their allocations (0:
-    aligned), against aligned copies and the oracle."""
+    aligned), on the given route, against aligned copies and the oracle."""
     rng = np.random.default_rng(seed)
     dts = [TORCH_TO_DT[d] for d in dtypes]
     host = [W.random_storage(rng, n, dt) for n, dt in zip(numels, dts)]
@@ -43,7 +43,9 @@ def check(numels, dtypes, offsets, K, pre_probe, seed):
     c_np = rng.normal(0, 25, K)
     c = torch.tensor(c_np, device="cuda")
     s, lr, p = W.step_seed(seed), 1e-3, None if pre_probe is None else (pre_probe, 1e-3)
-    zo.update(zo.ParamList(views, packing=1), s, c, lr, pre=p)
+    plist = zo.ParamList(views, packing=1)
+    assert update_route(plist, K, pre_probe) == route
+    zo.update(plist, s, c, lr, pre=p)
     zo.update(zo.ParamList(aligned, packing=1), s, c, lr, pre=p)
     with oracle.packing(1):
         if pre_probe is not None:
@@ -66,7 +68,11 @@ def long_list(dtype):
                                          (30, 9), (27, 17), (27, 40)])
 @pytest.mark.parametrize("dtype", [BF16, F32], ids=["bf16", "f32"])
 def test_three_and_four_groups(K, pre_probe, dtype):
-    check([long_list(dtype), 1, 15, 513, 77], [dtype, F16, F32, BF16, F16], [0, 0, 3, 5, 0], K, pre_probe, seed=K)
+    # fp32 of four groups keeps to the last group's words; a probe of no group has none here
+    last = pre_probe is None or pre_probe // 8 == (K - 1) // 8
+    chunks = pre_probe is not None and pre_probe >= 8 * ((K + 7) // 8) or (dtype == F32 and K > 24 and not last)
+    check([long_list(dtype), 1, 15, 513, 77], [dtype, F16, F32, BF16, F16], [0, 0, 3, 5, 0], K, pre_probe, seed=K,
+          route="chunks" if chunks else "tables")
 
 
 @pytest.mark.parametrize("K,pre_probe", [(9, None), (16, 15), (12, 3), (12, 20)])
@@ -84,7 +90,8 @@ def test_fp32_views_by_blocks(K, per_sm):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n = per_sm * sms + 3 if per_sm else long_list(F32)
     numels = [n, 16 * 31 - 3, 16 * 31 - 2, 16 * 62 - 2, 9, 1, 513, 77, 4096, 130]
-    check(numels, [F32] * 6 + [F16, BF16, F32, BF16], [3, 3, 2, 2, 7, 1, 5, 0, 0, 0], K, None, seed=K)
+    check(numels, [F32] * 6 + [F16, BF16, F32, BF16], [3, 3, 2, 2, 7, 1, 5, 0, 0, 0], K, None, seed=K,
+          route="blocks")
 
 
 def test_fp32_views_after_a_failed_preconditioner():

@@ -1,6 +1,6 @@
 """The fused update of short lists by items (update_items_kernel): against the
-table-per-lane kernels bit for bit, by padding the same list past the short
-lists' limit with a tensor that both calls share, and against the oracle, over
+kernels of long lists bit for bit (the route asserted), by padding the same list
+past the short lists' limit with a last tensor, and against the oracle, over
 every storage type, alignment, packing, probe count and a failed
 preconditioner."""
 import numpy as np
@@ -12,7 +12,7 @@ from paper_2609_38095_gb300 import build as zo_build
 from paper_2609_38095_gb300 import workloads as W
 from paper_2609_38095_gb300 import zo
 
-from gpu_helpers import TORCH_TO_DT, assert_update_close, storage_bits, to_torch
+from gpu_helpers import TORCH_TO_DT, assert_update_close, filler, storage_bits, to_torch, update_route
 
 pytestmark = pytest.mark.gpu
 
@@ -47,7 +47,7 @@ def test_short_list(K, packing, pre, status):
     offsets = [0, 3, 0, 1, 5, 0, 7, 0, 1, 0, 11, 0]
     dts = [TORCH_TO_DT[d] for d in dtypes]
     host = [W.random_storage(rng, n, dt) for n, dt in zip(numels, dts)]
-    short, tail = views_of(host, dtypes, offsets), views_of(host, dtypes, offsets)
+    short, copies = views_of(host, dtypes, offsets), [h.copy() for h in host]
     c_np = rng.normal(0, 25, K)
     c, st = torch.tensor(c_np, device="cuda"), torch.tensor([status], dtype=torch.int32, device="cuda")
     s, lr, p = W.step_seed(K), 1e-3, (K - 1, 1e-3) if pre else None
@@ -62,13 +62,16 @@ def test_short_list(K, packing, pre, status):
             assert np.array_equal(storage_bits(v), storage_bits(h)), f"tensor {i}"
         else:
             assert_update_close(storage_bits(v), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
-    if packing == 8 and K <= 8:
-        return                                    # update_items_kernel at every size
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    filler = torch.zeros(16 * 4097 * sms, dtype=torch.bfloat16, device="cuda")
-    zo.update(zo.ParamList(tail + [filler], packing=packing), s, c, lr, status=st, pre=p)
-    for i, (x, y) in enumerate(zip(short, tail)):
-        assert torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8)), f"tensor {i}"
+    # sixteen-bit weights for the kernels of packing 1 with a table per lane, fp32 views for the rest
+    for long in ([filler(4097, torch.bfloat16)] if packing == 1 else []) + [filler(4097, torch.float32, 1)]:
+        tail = views_of(copies, dtypes, offsets)
+        plist = zo.ParamList(tail + [long], packing=packing)
+        assert update_route(zo.ParamList(tail, packing=packing), K, K - 1 if pre else None) == "items"
+        route = update_route(plist, K, K - 1 if pre else None)
+        assert route != "items" and (packing == 1 or route == "chunks")
+        zo.update(plist, s, c, lr, status=st, pre=p)
+        for i, (x, y) in enumerate(zip(short, tail)):
+            assert torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8)), f"{route}: tensor {i}"
 
 
 @pytest.mark.parametrize("n", [64, 65, 256, 257, 960, 961, 2100])
