@@ -340,7 +340,7 @@ const char* zo_status_string(int status) {
 
 const char* zo_last_cuda_error(void) { return g_last_cuda_error; }
 
-int zo_version(void) { return 10400; }
+int zo_version(void) { return 10500; }
 
 int zo_set_packing(int32_t bits_per_value) {
   if (bits_per_value != zo::kPacking1 && bits_per_value != zo::kPacking8) return ZO_ERR_ARG;

@@ -45,11 +45,14 @@ class QuadraticStep:
         self.losses = torch.empty(self.K, 3, dtype=torch.float64, device=dev)
         self.c = torch.empty(self.K, dtype=torch.float64, device=dev)
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
+        # onepass: every forward point and the preconditioner in one call; else a loss with its arguments checked
+        # once, and the table cells that it writes
+        self.onepass = self.ws = self.loss = None
+        if schedule == "onepass":
+            self.onepass = zo.QuadraticPoints(theta, a, self.losses, out=(self.c, self.status))
+            return
         self.ws = torch.empty(zo.quadratic_loss_workspace_size(theta.numel()), dtype=torch.uint8, device=dev)
-        # the loss with its arguments checked once, and the table cells it writes
         self.loss = zo.QuadraticLoss(theta, a, self.ws)
-        self.points = (zo.QuadraticPoints(theta, a, self.losses, out=(self.c, self.status))
-                       if schedule == "onepass" else None)
         row = self.losses.stride(0) * self.losses.element_size()
         base = self.loss.out_address(self.losses)
         self._lp = [base + k * row for k in range(self.K)]                  # L+ of probe k
@@ -60,8 +63,8 @@ class QuadraticStep:
     def step(self, seed: int):
         """Enqueue one step on the current stream (nothing waits)."""
         K, eps = self.K, self.eps
-        if self.points is not None:
-            self.points(seed, eps)   # L0, every L+ and L- (theta restored after each probe), and the preconditioner
+        if self.onepass is not None:
+            self.onepass(seed, eps)  # L0, every L+ and L- (theta restored after each probe), and the preconditioner
             zo.update(self.plist, seed, self.c, self.lr, status=self.status)
             return
         self.loss(self._l0)                                    # clean loss L0 (Algorithm 1)

@@ -34,7 +34,7 @@ def test_exports_every_declared_symbol(L):
 
 
 def test_version_and_strings(L):
-    assert zo.version() == 10400
+    assert zo.version() == 10500
     for s in (0, -1, -2, -3, -4, -5, -6, -7):
         assert zo.status_string(s).startswith("ZO_")
     assert "unknown" in zo.status_string(99)
@@ -227,7 +227,7 @@ def test_header_is_plain_c_and_links_from_c(tmp_path, L):
         "#include <stdio.h>\n#include <string.h>\n#include \"zo.h\"\n"
         "int main(void) {\n"
         "  zo_tensor t = {0, 0, ZO_BF16, 0};\n"
-        "  if (zo_version() != 10400) return 1;\n"
+        "  if (zo_version() != 10500) return 1;\n"
         "  if (strncmp(zo_status_string(ZO_ERR_ARG), \"ZO_ERR_ARG\", 10) != 0) return 2;\n"
         "  if (zo_perturb(&t, -1, 1, 0, 1e-3f, NULL) != ZO_ERR_ARG) return 3;\n"
         "  if (zo_set_packing(3) != ZO_ERR_ARG) return 4;\n"

@@ -15,6 +15,7 @@ import oracle
 from paper_2609_38095_gb300 import build as zo_build
 from paper_2609_38095_gb300 import workloads as W
 from paper_2609_38095_gb300 import zo
+from paper_2609_38095_gb300.quadratic import QuadraticStep
 
 pytestmark = pytest.mark.gpu
 
@@ -191,3 +192,10 @@ def test_points_as_close_to_exact_sums_as_a_launch_per_point():
                 err["launches"].append((theirs - want) / want)
     rms = {k: float(np.sqrt(np.mean(np.square(e)))) for k, e in err.items()}
     assert rms["points"] <= 1.25 * rms["launches"], rms
+
+
+def test_step_holds_what_its_schedule_uses():
+    theta, a = torch.ones(100, device="cuda"), torch.ones(100, device="cuda")
+    one, fused = (QuadraticStep(theta, a, 2, 1e-3, 1e-3, schedule=s) for s in ("onepass", "fused"))
+    assert isinstance(one.onepass, zo.QuadraticPoints) and one.loss is None and one.ws is None
+    assert fused.onepass is None and isinstance(fused.loss, zo.QuadraticLoss)
