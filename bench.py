@@ -115,7 +115,7 @@ KERNEL_SOURCES = {
     "perturb_items_kernel<1>": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "perturb_items_kernel<2>": ("zo_device.cuh", "zo_stream_kernels.cu"),
     "pair_items_kernel": ("zo_device.cuh", "zo_stream_kernels.cu"),
-    "update_lut8_kernel": ("zo_device.cuh", "zo_update_lut8.cu"),
+    "update_lut8_kernel": ("zo_blocks.cuh", "zo_device.cuh", "zo_update_lut8.cu"),
 }
 
 
@@ -774,7 +774,9 @@ def run_zo(args):
     c = torch.empty(K, dtype=torch.float64, device=dev)
     status = torch.zeros(1, dtype=torch.int32, device=dev)
     stream = torch.cuda.current_stream(dev)
-    chunks = (len(params) + 959) // 960   # tensors per launch
+    # launches of a pass: tensors per table of perturb_items_kernel, pair_items_kernel and the update's kernels
+    chunks, pair_chunks = (len(params) + 959) // 960, (len(params) + 639) // 640
+    update_chunks = (len(params) + 1023) // 1024 if args.packing == 1 else chunks
     pp = args.probe_parallel
     pair = args.schedule == "pair" or pp
     my_probes = K          # probes whose passes this rank runs
@@ -854,11 +856,11 @@ def run_zo(args):
     passes = K + 1 if pair else (2 * K + 1 if fused else 3 * K + 1)   # sweeps over the weights, update included
     if pp:
         passes = my_probes + 1                                            # on each rank
-        launches = args.steps * (my_probes * chunks + 1 + chunks)
+        launches = args.steps * (my_probes * pair_chunks + 1 + update_chunks)
     elif pair:
-        launches = args.steps * (K * chunks + 1 + chunks)
+        launches = args.steps * (K * pair_chunks + 1 + update_chunks)
     else:
-        launches = args.steps * ((passes - 1) * chunks + 1 + chunks)
+        launches = args.steps * ((passes - 1) * chunks + 1 + update_chunks)
 
     def avg_ms(key):
         v = [a.elapsed_time(b) for a, b in timing[key]]
@@ -970,7 +972,11 @@ def run_zo(args):
     else:
         dom_kernel, dom_ms, dom_launches = "perturb_items_kernel<1> (zo_perturb)", perturb_ms, n1
         traffic, traffic_how = committed_traffic("perturb_items_kernel<1>", traffic_key)
+    # a pass may be several launches; the committed traffic is a pass's
+    dom_per_pass = pair_chunks if pair else chunks
     dom_bytes = pair_bytes if pair else perturb_bytes
+    if traffic is not None and dom_per_pass > 1:
+        traffic, traffic_how = traffic / dom_per_pass, f"{traffic_how}; a pass's traffic over its {dom_per_pass} launches"
     # the update's DRAM bytes (one read and one write of theta, whatever K): the
     # 8-probe-table kernel's committed capture when it is the one this K runs
     if args.packing == 1 and K > 32 and not shifted:
@@ -1014,8 +1020,8 @@ def run_zo(args):
                      f"{args.schedule} ({passes} passes over the weights per step)"),
         "roofline": {"bound": "hbm", "kernel": dom_kernel, "achieved": dom_achieved, "peak": hbm_peak,
                      "unit": "GB/s", "frac": dom_achieved / hbm_peak, "traffic": traffic, "traffic_source": traffic_how,
-                     "peak_source": f"{peak_kind} hbm_gbs", "bytes_per_launch": dom_bytes,
-                     "launches_per_step": dom_launches * chunks,
+                     "peak_source": f"{peak_kind} hbm_gbs", "bytes_per_launch": dom_bytes / dom_per_pass,
+                     "launches_per_step": dom_launches * dom_per_pass,
                      "step_share": dom_launches * dom_ms / ms_per_step},
         "kernels": {
             "perturb": ({"ms": perturb_ms, "GB/s": achieved, "frac_of_measured_hbm": achieved / hbm_peak,
@@ -1023,7 +1029,7 @@ def run_zo(args):
                          "launches_per_step": (K + 1 if fused else 3 * K) * chunks} if not pair else None),
             "pair": ({"ms": pair_ms, "GB/s": pair_bytes / (pair_ms * 1e-3) / 1e9,
                       "frac_of_measured_hbm": pair_bytes / (pair_ms * 1e-3) / 1e9 / hbm_peak,
-                      "bytes_per_pass": pair_bytes, "launches_per_step": my_probes * chunks} if pair else None),
+                      "bytes_per_pass": pair_bytes, "launches_per_step": my_probes * pair_chunks} if pair else None),
             "perturb2": ({"ms": perturb2_ms, "GB/s": perturb_bytes / (perturb2_ms * 1e-3) / 1e9,
                           "frac_of_measured_hbm": perturb_bytes / (perturb2_ms * 1e-3) / 1e9 / hbm_peak,
                           "launches_per_step": (K - 1) * chunks} if fused and K > 1 else None),

@@ -18,11 +18,10 @@
  * Memory. Every array argument is DEVICE memory of the current CUDA device,
  * owned by the caller, except the zo_tensor descriptor array itself (host
  * memory, read during the call only). The library allocates no device
- * memory: the tensor table travels inside the kernel launch parameters. Its
- * only CUDA objects are the timing events of zo_perturb2's launch
- * configuration choice (18 per parameter list, at most 64 lists, kept until
- * the process exits). Host side, each calling thread keeps its launch
- * parameter blocks (about 150 KB of thread-local storage).
+ * memory and creates no CUDA objects: the tensor table travels inside the
+ * kernel launch parameters. Nothing is kept about a parameter list between
+ * calls. Host side, each calling thread keeps its launch parameter blocks
+ * (about 160 KB of thread-local storage).
  *
  * Streams. `stream` is a cudaStream_t (NULL = legacy default stream). Every
  * call only enqueues work on it and returns; results are visible to later
@@ -41,10 +40,7 @@
  * Tensors may mix dtypes. numel may be 0 and at most 16 * (2^31 - 1) - 1
  * (ZO_ERR_ARG beyond). ptr must be aligned to its element size. Any such
  * alignment gives the same results; a tensor whose ptr is not 32-byte aligned
- * is streamed in 32-byte aligned chunks by a second kernel of the same call
- * (zo_perturb, zo_perturb2, zo_update, zo_update_ex, zo_update_sequential;
- * zo_perturb_pair when plus and minus share their offset), otherwise with
- * narrower accesses.
+ * is streamed in 32-byte aligned chunks, in the same launch as the others.
  *
  * Probes. z_k is Rademacher, one bit per parameter per probe (Sec. 2, Sec. 4.3
  * "Bit-Packed perturbations"; unpack rule of Appendix F: bit 1 -> +1, bit 0 ->
@@ -148,14 +144,6 @@ int zo_perturb(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint32
  * forward pass runs between probe k's restore (+eps) and probe k+1's first
  * perturbation (+eps), so a step can apply them together:
  * zo_perturb2(k, +eps, k + 1, +eps). Errors as zo_perturb.
- * Launch configuration: the first nine calls on a parameter list (identified
- * by device, sizes, dtypes and 32-byte alignments) with both probes in one
- * group of 8 (k / 8 equal; packing 1) each run one of three loop / grid
- * configurations between two CUDA events recorded on `stream`, and so do the
- * first three calls with the probes in two groups (a kernel of its own);
- * later calls of each kind use the fastest. The results never depend on the
- * configuration. Calls made while `stream` is being captured into a CUDA
- * graph use the first configuration and record no event.
  * ------------------------------------------------------------------------- */
 int zo_perturb2(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint32_t probe_a, float scale_a,
                 uint32_t probe_b, float scale_b, void* stream);
@@ -174,10 +162,11 @@ int zo_perturb2(const zo_tensor* params, int32_t n_tensors, uint64_t seed, uint3
  * theta's: the probes are theta's). plus[t] may be theta[t]
  * itself (then theta becomes theta + scale z) and so may minus[t]; plus[t]
  * and minus[t] must be different, and any other overlap is undefined.
- * Access paths (same results): 256-bit blocks when all three pointers of a
- * 16-bit tensor are 32-byte aligned; 32-byte aligned chunks when plus and
- * minus share their offset from that grid (theta at any offset) and for fp32
- * tensors whose three pointers share it; narrower accesses otherwise.
+ * Access paths (same results): plus is written in 32-byte aligned chunks,
+ * theta is read at any offset in the aligned 32-byte segments that hold a
+ * chunk's elements, and minus is written in 32-byte chunks when it shares
+ * plus's offset from that grid, otherwise by the widest stores (16, 4 or 2
+ * bytes) that its address allows.
  * Errors: ZO_ERR_ARG (also for mismatched lists or plus[t] == minus[t]),
  * ZO_ERR_DTYPE, ZO_ERR_ALIGN, ZO_ERR_CUDA. No counterpart in the paper as a
  * kernel: it trades device memory for HBM traffic. */

@@ -85,11 +85,12 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 // (3 M weights are 1233 items per SM). Under packing 8 generating the bits is
 // most of the work and many small CTAs do it best, whatever the size, but for
 // 16-bit lists of many groups:
-//   fp32          K = 3: 100 M 150 / 162;  K = 24: 399 / 458;  K = 64: 50 M 506 / 531, 205 M 2010 / 2081
+//   fp32          K = 3: 100 M 134 / 151;  K = 24: 399 / 450;  K = 64: 50 M 506 / 531, 205 M 2010 / 2081
 //                 K = 256: 50 M 1944 / 1978, 205 M 7800 / 7880
-//   16 bits       K = 3: 205 M 279 / 317;  K = 24: 872 / 907;  K = 64: 50 M 512 / 522, 205 M 2049 / 2047
+//   16 bits       K = 3: 205 M 219 / 268;  K = 24: 809 / 862;  K = 64: 50 M 512 / 522, 205 M 2049 / 2047
 //                 K = 96: 50 M 756 / 763, 80 M 1203 / 1199;  K = 256: 20 M 804 / 832, 50 M 1977 / 1967
-//   16-bit views  K = 64: 20 M 224 / 227, 205 M 2179 / 2154;  K = 128: 10 M 224 / 233, 20 M 434 / 429, 50 M 1070 / 1040
+//   16-bit views  K = 3: 205 M 235 / 316;  K = 48: 1650 / 1649;  K = 64: 20 M 224 / 227, 205 M 2179 / 2154
+//                 K = 128: 10 M 224 / 233, 20 M 434 / 429, 50 M 1070 / 1040
 //   fp32 views    K = 3: 3 M 14.7 / 17.0, 6 M 23.1 / 21.3;  K = 24: 1 M 14.8 / 17.0, 3 M 31.4 / 28.2
 //                 K = 64: 1 M 27.3 / 24.8
 // (1 M fp32 weights are 822 items per SM; those off the 32-byte grid make a

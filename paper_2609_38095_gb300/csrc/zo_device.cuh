@@ -572,7 +572,7 @@ __device__ __forceinline__ void fold_bits(uint4& y, const uint4& x, uint32_t i) 
   y.w |= (x.w << i) & m;
 }
 
-// The fused update of a short list by items (update_items_kernel): ItemsParams'
+// The fused update by items (update_items_kernel): ItemsParams'
 // table, and the update's own arguments as in UpdateParams.
 template <int N>
 struct UpdateItemsParams {

@@ -1,5 +1,5 @@
 // zo_items.h -- host-side planning of the tables of the launches by items
-// (perturb_items_kernel, pair_items_kernel).
+// (perturb_items_kernel, pair_items_kernel, update_items_kernel).
 #pragma once
 
 #include <cstdint>

@@ -41,7 +41,7 @@ bool one_high_word(const TensorTable& tab);  // of the launch's virtual blocks
 // Fused update of fp32 views without a leading perturbation (weights: of the list's, those fp32 off the 32-byte grid).
 bool update_blocks_takes(const UpdateParams& u, int64_t weights, int sms);
 cudaError_t launch_update_blocks(const UpdateParams& p, int sms, cudaStream_t stream);
-// Fused update of a short list; its virtual blocks share the counter's high word.
+// Fused update by items; its virtual blocks share the counter's high word.
 template <int N>
 cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream);
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,

@@ -9,8 +9,9 @@
 // (theta and a are read once, theta written once) and only the 2 K + 1 sums
 // cross threads.
 //
-// Bound: fp32 arithmetic (13 operations per weight and point, below) and the
-// grid's size; d = 2^20 and K = 8 are 17.8 M terms.
+// Bound: fp32 arithmetic (seven packed operations per weight and point, below,
+// and an addition and a sign flip per weight and move) and the grid's size; d =
+// 2^20 and K = 8 are 17.8 M terms.
 //
 // Sums. Each term a t^2 is formed without rounding as a pair of fp32 values
 // (Dekker's product by fused multiply-add: a t = p + pe, p t = q + qe, term =

@@ -8,8 +8,8 @@
 // and a view's sums are then moved over two lanes once, where the kernels with
 // a table per lane move every group's words, and for fp32 make a block's words
 // twice. 64 registers, so 32 warps to an SM with nothing held but the sums:
-// theta is read after them. Bound by issue (72 % of it, ALU 63 %) from three
-// groups on, by HBM below.
+// theta is read after them. Bound by issue (69 % of it, ALU 59 %, K = 32)
+// from three groups on, by HBM below.
 //
 // fp32 views, us here / in the table-per-lane kernels: 221 M weights, K = 8 273 /
 // 290, K = 24 364 / 387, K = 32 433 / 455, K = 40 505 / 516; 45 M, K = 8 62 / 66,

@@ -1,4 +1,5 @@
-// zo_update_items.cu -- the fused K-probe update of short lists.
+// zo_update_items.cu -- the fused K-probe update by 32-byte items: short lists,
+// and most of packing 8.
 //
 // theta <- rn(fp32(theta) + sum_k a_k z_k[g]), the sums formed from the same
 // 8-probe partials T_lo + T_hi in the same order as in zo_update_lut8.cu, so
