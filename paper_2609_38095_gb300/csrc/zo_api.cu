@@ -82,7 +82,8 @@ zo::PerturbOp make_op(uint32_t k, float scale, int packing) {
 //   packing 1   K = 16: 3 M weights 10.5 / 12.9, 8 M 17.1 / 15.8
 //               K = 20: 5 M 14.7 / 15.1, 8 M 19.2 / 18.8;  K = 32: 16.8 / 17.1, 23.0 / 21.2
 //               K = 64: 3 M 16.8 / 19.1, 8 M 33.4 / 31.6;  K = 256: 43.6 / 43.6, 97 / 80
-// (3 M weights are 1233 items per SM). Under packing 8 generating the bits is
+// (3 M weights are 1233 items per SM; the items' side before kPlain's launch bound,
+// which takes 3 to 7 % off K = 64 and more). Under packing 8 generating the bits is
 // most of the work and many small CTAs do it best, whatever the size, but for
 // 16-bit lists of many groups:
 //   fp32          K = 3: 100 M 134 / 151;  K = 24: 399 / 450;  K = 64: 50 M 506 / 531, 205 M 2010 / 2081
@@ -489,7 +490,7 @@ int zo_update_ex(const zo_tensor* params, int32_t n_tensors, uint64_t seed, cons
                   pre_probe / 8u + 1u == static_cast<uint32_t>(up.groups);
     if (ip.pre_last) set_bit(ip.pre, pre_probe & 7u);
     ip.status = status;
-    return zo::launch_update_items(ip, static_cast<cudaStream_t>(stream));
+    return zo::launch_update_items(ip, d->sms, static_cast<cudaStream_t>(stream));
   };
   if (plan.route == kByItems) {
     while (cur.t < n_tensors) {

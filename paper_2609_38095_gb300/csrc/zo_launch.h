@@ -43,7 +43,7 @@ bool update_blocks_takes(const UpdateParams& u, int64_t weights, int sms);
 cudaError_t launch_update_blocks(const UpdateParams& p, int sms, cudaStream_t stream);
 // Fused update by items; its virtual blocks share the counter's high word.
 template <int N>
-cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream);
+cudaError_t launch_update_items(const UpdateItemsParams<N>& p, int sms, cudaStream_t stream);
 cudaError_t launch_probe_bytes(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,
                                uint8_t* out, int grid, cudaStream_t stream);
 cudaError_t launch_probe_signs(const RoundKeys& keys, uint32_t ctr2, uint32_t bit, int64_t first, int64_t n,

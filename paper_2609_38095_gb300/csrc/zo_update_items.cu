@@ -16,7 +16,8 @@
 // coefficients, one Philox call and sixteen lookups per group, theta. 300 k
 // bf16 weights in 12 tensors, K = 8 / 32 / 64 / 256: 10.5 / 13.5 / 17.0 / 34.5
 // -> 8.7 / 8.2 / 8.8 / 15.1 us; as fp32, K = 32 15.0 -> 8.2; in one flat buffer
-// 23.3 -> 8.6; packing 8, K = 32 14.5 -> 10.2. Not adopted: a grid of 8 to 64
+// 23.3 -> 8.6; packing 8, K = 32 14.5 -> 10.2 (calls back to back 5.5 / 6.0 / 6.2 /
+// 12.3; 5.3; 6.4; 8.3). Not adopted: a grid of 8 to 64
 // CTAs per SM that walks the items (K = 256, 8 M weights 97.5 -> 98-107 us).
 //
 // Packing 8 has eight Philox calls per group and is bound by them (85 to 90
@@ -56,34 +57,31 @@ __device__ __forceinline__ float lds_f32_hi(uint32_t addr) {
   return v;
 }
 
-// Four times the low and the high nibbles of x's bytes, in its bytes.
-__device__ __forceinline__ uint4 low_offsets(const uint4& x) {
-  return make_uint4((x.x << 2) & 0x3C3C3C3Cu, (x.y << 2) & 0x3C3C3C3Cu, (x.z << 2) & 0x3C3C3C3Cu,
-                    (x.w << 2) & 0x3C3C3C3Cu);
-}
-__device__ __forceinline__ uint4 high_offsets(const uint4& x) {
-  return make_uint4((x.x >> 2) & 0x3C3C3C3Cu, (x.y >> 2) & 0x3C3C3C3Cu, (x.z >> 2) & 0x3C3C3C3Cu,
-                    (x.w >> 2) & 0x3C3C3C3Cu);
-}
 __device__ __forceinline__ uint4 shift_left(const uint4& x, uint32_t n) {
   return make_uint4(x.x << n, x.y << n, x.z << n, x.w << n);
 }
 
-// Add a group's partial of elements 0 .. 4 WORDS - 1, whose bytes of lo and hi hold four times the signs of the
+// Add a group's partial of elements 4 M .. 4 M + 3: their bytes of lo4 and hi4 hold four times the signs of the
 // group's probes 0-3 and 4-7.
-template <int WORDS>
-__device__ __forceinline__ void add_group(float (&acc)[16], const uint4& lo, const uint4& hi, uint32_t frame) {
+template <int M>
+__device__ __forceinline__ void add_word(float (&acc)[16], uint32_t lo4, uint32_t hi4, uint32_t frame) {
 #pragma unroll
-  for (int m = 0; m < WORDS; ++m) {
-    const uint32_t lo4 = word_of(lo, m), hi4 = word_of(hi, m);
-#pragma unroll
-    for (int j = 0; j < 4; j += 2) {
-      const uint32_t s0 = 0x7650u | static_cast<uint32_t>(j), s1 = s0 + 1u;
-      float p0 = lds_f32(__byte_perm(lo4, frame, s0)), p1 = lds_f32(__byte_perm(lo4, frame, s1));
-      fadd2_rn(p0, p1, lds_f32_hi(__byte_perm(hi4, frame, s0)), lds_f32_hi(__byte_perm(hi4, frame, s1)));
-      fadd2_rn(acc[4 * m + j], acc[4 * m + j + 1], p0, p1);
-    }
+  for (int j = 0; j < 4; j += 2) {
+    const uint32_t s0 = 0x7650u | static_cast<uint32_t>(j), s1 = s0 + 1u;
+    float p0 = lds_f32(__byte_perm(lo4, frame, s0)), p1 = lds_f32(__byte_perm(lo4, frame, s1));
+    fadd2_rn(p0, p1, lds_f32_hi(__byte_perm(hi4, frame, s0)), lds_f32_hi(__byte_perm(hi4, frame, s1)));
+    fadd2_rn(acc[4 * M + j], acc[4 * M + j + 1], p0, p1);
   }
+}
+
+// The same of the first WORDS words of sign bytes.
+template <int WORDS>
+__device__ __forceinline__ void add_group(float (&acc)[16], const uint4& x, uint32_t frame) {
+  add_word<0>(acc, (x.x << 2) & 0x3C3C3C3Cu, (x.x >> 2) & 0x3C3C3C3Cu, frame);
+  add_word<1>(acc, (x.y << 2) & 0x3C3C3C3Cu, (x.y >> 2) & 0x3C3C3C3Cu, frame);
+  if (WORDS == 2) return;
+  add_word<2>(acc, (x.z << 2) & 0x3C3C3C3Cu, (x.z >> 2) & 0x3C3C3C3Cu, frame);
+  add_word<3>(acc, (x.w << 2) & 0x3C3C3C3Cu, (x.w >> 2) & 0x3C3C3C3Cu, frame);
 }
 
 size_t update_items_smem_bytes(int groups, int packing) {
@@ -93,16 +91,20 @@ size_t update_items_smem_bytes(int groups, int packing) {
 
 }  // namespace
 
-// What a launch holds: packing 1, packing 8, or packing 8 and mostly fp32 on the 32-byte grid.
-constexpr int kPlain = 0, kBytes = 1, kBytesF32 = 2;
+// What a launch holds: packing 1, packing 8, packing 8 and mostly fp32 on the 32-byte grid, or packing 1 with at most
+// two groups on more CTAs than 7 per SM.
+constexpr int kPlain = 0, kBytes = 1, kBytesF32 = 2, kPlainMany = 3;
 
 // LAST: packing 8, the leading perturbation's probe is one of the last group's, whose words it takes. The second launch
-// bound (5 CTAs of kBytesF32) leaves its calls the registers that they were interleaved with.
+// bound leaves a group's calls and lookups the registers that they are interleaved with: 5 CTAs of kBytesF32, 7 of
+// kPlain (70 registers). Without it kPlain takes 56 and holds 9 CTAs, us: 24 tensors, 2 M bf16 weights, K = 16 / 96 /
+// 520 5.8 / 13.3 / 55.7, with it 5.7 / 13.0 / 54.3; 0.03 M, K = 520 23.5, with it 18.0. Only a second wave costs more
+// where little is left to interleave, 3 M bf16 weights, K = 8 / 16: 6.2 / 7.1 in place of kPlainMany's 5.8 / 6.9.
 template <int KIND, bool LAST, int N>
-__global__ void __launch_bounds__(kItemThreads, KIND == kBytesF32 ? 5 : 0) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
+__global__ void __launch_bounds__(kItemThreads, KIND == kPlain ? 7 : KIND == kBytesF32 ? 5 : 0) update_items_kernel(const __grid_constant__ UpdateItemsParams<N> P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int skip_s;
-  constexpr bool PACK8 = KIND != kPlain, WIDE = KIND == kBytesF32;
+  constexpr bool PACK8 = KIND == kBytes || KIND == kBytesF32, WIDE = KIND == kBytesF32;
   const int G = P.groups;
   constexpr int kCalls = PACK8 ? 8 : 1;  // Philox calls per group
   uint4* r01_s = reinterpret_cast<uint4*>(smem);            // kCalls G group parts
@@ -170,18 +172,18 @@ __global__ void __launch_bounds__(kItemThreads, KIND == kBytesF32 ? 5 : 0) updat
       return philox_finish(philox_start(blk, {r.x, r.y, r.z}), P.keys);
     };
     const auto own = [&](const uint4& x) { return item_signs(x, f32, (k.i & 1) != 0, shift, a); };
-    uint4 xp = make_uint4(0u, 0u, 0u, 0u);
+    uint4 last = make_uint4(0u, 0u, 0u, 0u);  // LAST: the last group's sign bytes
     float acc[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
     if (do_sum) {
       uint32_t frame = frame0;
+      uint4 lo, hi;  // WIDE: the bits of probes 0-3 and 4-7, where the lookups take them
 #pragma unroll 1
       for (int q = 0; q < G; ++q, frame += kFrame) {
-        uint4 lo, hi;  // the lookups' offsets
+        uint4 x = make_uint4(0u, 0u, 0u, 0u);  // the sign bytes of this lane's elements
         if constexpr (WIDE) {
-          // the bits folded where the lookups take them
-          lo = hi = make_uint4(0u, 0u, 0u, 0u);
+          lo = hi = x;
           if (8 * q + 8 <= P.K) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) fold_bits(i < 4 ? lo : hi, call(static_cast<uint32_t>(8 * q + i)), i & 3);
@@ -191,42 +193,41 @@ __global__ void __launch_bounds__(kItemThreads, KIND == kBytesF32 ? 5 : 0) updat
 #pragma unroll 1
             for (int i = 4; i < 8 && 8 * q + i < P.K; ++i) fold_bits(hi, call(static_cast<uint32_t>(8 * q + i)), i & 3);
           }
+          if (!wide) x = make_uint4(lo.x + (hi.x << 4), lo.y + (hi.y << 4), lo.z + (hi.z << 4), lo.w + (hi.w << 4));
           if (wide) {
-            if (LAST) xp = make_uint4(lo.x + (hi.x << 4), lo.y + (hi.y << 4), lo.z + (hi.z << 4), lo.w + (hi.w << 4));
             lo = shift_left(lo, 2u);
             hi = shift_left(hi, 2u);
+            add_word<0>(acc, lo.x, hi.x, frame);
+            add_word<1>(acc, lo.y, hi.y, frame);
+            add_word<2>(acc, lo.z, hi.z, frame);
+            add_word<3>(acc, lo.w, hi.w, frame);
+          }
+        } else if constexpr (PACK8) {
+          if (8 * q + 8 <= P.K) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
           } else {
-            const uint4 up = shift_left(hi, 4u);
-            const uint4 x = own(make_uint4(lo.x + up.x, lo.y + up.y, lo.z + up.z, lo.w + up.w));
-            lo = low_offsets(x);
-            hi = high_offsets(x);
-            if (LAST) xp = x;
+#pragma unroll 2
+            for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
           }
         } else {
-          uint4 x;
-          if constexpr (PACK8) {
-            x = make_uint4(0u, 0u, 0u, 0u);
-            if (8 * q + 8 <= P.K) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
-            } else {
-#pragma unroll 2
-              for (int i = 0; i < 8 && 8 * q + i < P.K; ++i) fold_bits(x, call(static_cast<uint32_t>(8 * q + i)), i);
-            }
-          } else {
-            x = call(static_cast<uint32_t>(q));
-          }
-          x = own(x);
-          lo = low_offsets(x);
-          hi = high_offsets(x);
-          if (LAST) xp = x;
+          x = call(static_cast<uint32_t>(q));
         }
-        if (f32 && !(WIDE && wide))
-          add_group<2>(acc, lo, hi, frame);
-        else
-          add_group<4>(acc, lo, hi, frame);
+        if (!(WIDE && wide)) {
+          x = own(x);
+          if (f32)
+            add_group<2>(acc, x, frame);
+          else
+            add_group<4>(acc, x, frame);
+        }
+        if (LAST && !(WIDE && wide)) last = x;
+      }
+      if constexpr (LAST && WIDE) {
+        if (wide)  // both were shifted for the lookups
+          last = make_uint4((lo.x >> 2) + (hi.x << 2), (lo.y >> 2) + (hi.y << 2), (lo.z >> 2) + (hi.z << 2), (lo.w >> 2) + (hi.w << 2));
       }
     }
+    uint4 xp = last;
     if (P.has_pre && !(LAST && do_sum)) {
       const GroupRound01 g = group_round01(P.pre.ctr2, P.bhi, P.keys);
       xp = philox_finish(philox_start(blk, g), P.keys);
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(kItemThreads, KIND == kBytesF32 ? 5 : 0) updat
 }
 
 template <int N>
-cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stream) {
+cudaError_t launch_update_items(const UpdateItemsParams<N>& p, int sms, cudaStream_t stream) {
   const uint32_t per = kItemThreads * (p.packing == kPacking8 ? p.rounds : 1u);
   const int grid = static_cast<int>((static_cast<uint64_t>(p.total) + (per - 1u)) / per);
   const size_t smem = update_items_smem_bytes(p.groups, p.packing);
@@ -301,13 +302,14 @@ cudaError_t launch_update_items(const UpdateItemsParams<N>& p, cudaStream_t stre
     kernel<<<grid, kItemThreads, smem, stream>>>(p);
     return cudaGetLastError();
   };
-  if (p.packing != kPacking8) return go(update_items_kernel<kPlain, false, N>);
+  if (p.packing != kPacking8)
+    return p.groups <= 2 && grid > 7 * sms ? go(update_items_kernel<kPlainMany, false, N>) : go(update_items_kernel<kPlain, false, N>);
   if (p.pre_last != 0)
     return p.f32_blocks ? go(update_items_kernel<kBytesF32, true, N>) : go(update_items_kernel<kBytes, true, N>);
   return p.f32_blocks ? go(update_items_kernel<kBytesF32, false, N>) : go(update_items_kernel<kBytes, false, N>);
 }
-template cudaError_t launch_update_items(const UpdateItemsParams<kItemsFew>& p, cudaStream_t stream);
-template cudaError_t launch_update_items(const UpdateItemsParams<kItemsSome>& p, cudaStream_t stream);
-template cudaError_t launch_update_items(const UpdateItemsParams<kItemsMany>& p, cudaStream_t stream);
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsFew>& p, int sms, cudaStream_t stream);
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsSome>& p, int sms, cudaStream_t stream);
+template cudaError_t launch_update_items(const UpdateItemsParams<kItemsMany>& p, int sms, cudaStream_t stream);
 
 }  // namespace zo

@@ -109,3 +109,23 @@ def test_more_tensors_than_a_launch_holds(n, K, packing):
     for i, (d, h, dt) in enumerate(zip(dev, host, dts)):
         if h.size:
             assert_update_close(storage_bits(d), storage_bits(h), dt, c_np, lr, context=f"tensor {i}")
+
+
+@pytest.mark.parametrize("items_per_sm", [880, 896])  # just below and above 7 CTAs of 128 items per SM
+@pytest.mark.parametrize("K", [1, 16, 17])
+@pytest.mark.parametrize("pre", [True, False])
+def test_lists_of_two_waves(items_per_sm, K, pre):
+    rng = np.random.default_rng(items_per_sm + K)
+    dtypes, offsets = [torch.bfloat16, torch.float32, torch.float16], [0, 3, 1]
+    host = [W.random_storage(rng, 1001, TORCH_TO_DT[d]) for d in dtypes]
+    c = torch.tensor(rng.normal(0, 25, K), device="cuda")
+    p = (K - 1, 1e-3) if pre else None
+    got = []
+    for per_sm, route in ((items_per_sm, "items"), (4097, "tables")):
+        ws = views_of(host, dtypes, offsets) + [filler(per_sm, torch.bfloat16)]
+        plist = zo.ParamList(ws, packing=1)
+        assert update_route(plist, K, K - 1 if pre else None) == route
+        zo.update(plist, W.step_seed(K), c, 1e-3, pre=p)
+        got.append(ws)
+    for i, (x, y) in enumerate(zip(*got)):
+        assert torch.equal(x.contiguous().view(torch.uint8), y[:x.numel()].contiguous().view(torch.uint8)), f"tensor {i}"
