@@ -129,3 +129,28 @@ def test_lists_of_two_waves(items_per_sm, K, pre):
         got.append(ws)
     for i, (x, y) in enumerate(zip(*got)):
         assert torch.equal(x.contiguous().view(torch.uint8), y[:x.numel()].contiguous().view(torch.uint8)), f"tensor {i}"
+
+
+@pytest.mark.parametrize("K", [64, 65, 520])  # eight groups and more
+def test_last_words_by_length(K):
+    rng = np.random.default_rng(K)
+    host = [W.random_storage(rng, n, W.DT_F32) for n in (4099, 16, 131)]
+    copies = [h.copy() for h in host]
+    dtypes = [torch.float32] * len(host)
+    c_np = rng.normal(0, 25, K)
+    c, s, lr = torch.tensor(c_np, device="cuda"), W.step_seed(K), 1e-3
+    got = []
+    for per_sm in (0, 490, 500, 4097):  # fp32 items per SM of the last tensor: one wave of many groups, and more
+        ws = views_of(copies, dtypes, [0] * len(host)) + ([filler(per_sm, torch.float32)] if per_sm else [])
+        plist = zo.ParamList(ws, packing=8)
+        assert update_route(plist, K, K - 1) == "items"
+        zo.update(plist, s, c, lr, pre=(K - 1, 1e-3))
+        got.append(ws)
+    with oracle.packing(8):
+        oracle.perturb(host, [W.DT_F32] * len(host), s, K - 1, 1e-3)
+        oracle.update(host, [W.DT_F32] * len(host), s, c_np, lr)
+    for i, h in enumerate(host):
+        assert_update_close(storage_bits(got[0][i]), storage_bits(h), W.DT_F32, c_np, lr, context=f"tensor {i}")
+    for a, b in zip(got, got[1:]):
+        for i, (x, y) in enumerate(zip(a, b)):
+            assert torch.equal(x.view(torch.uint8), y[:x.numel()].view(torch.uint8)), f"tensor {i}"
