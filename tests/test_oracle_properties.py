@@ -94,8 +94,9 @@ def test_precondition_invariants(L, eps, alpha, lam, one_sided, relative):
     assert rc == oracle.OK
     assert np.all(w > 0) and np.all(w <= 1.0 / lam * (1 + 1e-15))
     d = (L[:, 0] - L[:, 2]) / eps if one_sided else (L[:, 0] - L[:, 1]) / (2 * eps)
-    assert np.all(np.sign(c) == np.sign(d) * (w > 0))
-    assert np.all(np.abs(c) <= np.abs(d) / lam * (1 + 1e-12))
+    # zero only where w |d| lies below the smallest fp64 number, 2^-1074
+    assert np.all((np.sign(c) == np.sign(d)) | ((c == 0) & (np.abs(d) <= 2.0**-1074 / w)))
+    assert np.all(np.abs(c) <= np.abs(d) / lam * (1 + 1e-12) + 2.0**-1074)
     if not relative:
         order = np.argsort(np.abs(cv), kind="stable")
         assert np.all(np.diff(w[order]) <= 1e-15 * w[order][1:])
